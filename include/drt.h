@@ -311,7 +311,7 @@ drt_status drt_synthesize_H_retraced(drt_ctx *ctx, uint64_t link, const drt_time
  * stage.  Extrapolation and synthesis stream through a record buffer of at most 4 GiB in waves of
  * links.  The chunk length per link comes from a phase-error model, shortened by a factor 1, 2 or 4
  * chosen by timing the first wave's preparation and extrapolation (drt_batch_tuning), and the
- * synthesis frequency tile (bins per thread) from timing its variants on the batch (autotuning,
+ * synthesis frequency tile (bins) from timing its variants on the batch (autotuning,
  * done synchronously inside drt_batch_create).  Scratch is allocated once per batch within the HBM budget.  The links
  * must stay loaded and the H buffers valid while the batch exists.
  * drt_batch_run launches the batch on `stream`; with use_graph != 0 the first run is captured into
@@ -323,7 +323,7 @@ drt_status drt_batch_create(drt_ctx *ctx, int32_t n_links, const uint64_t *links
                             const drt_time_grid *tgrids, const drt_freq_grid *fgrids, void *const *H,
                             int32_t precision, drt_batch **out);
 drt_status drt_batch_run(drt_ctx *ctx, drt_batch *batch, int32_t use_graph, void *stream);
-/* chosen synthesis variant (frequency tile of 0: 8, 1: 16, 2: 32 bins per thread), scratch
+/* chosen synthesis variant (frequency tile of 0: 128, 1: 256, 2: 512 bins), scratch
  * bytes, the autotuner's best sample time (ms) and the path-steps of the last run that FP32 could
  * not resolve and the FP64 redo kernel recomputed (reading it waits for the device); any output
  * may be NULL.  With redo_steps non-NULL the call returns DRT_ENOMEM when a wave of the last run

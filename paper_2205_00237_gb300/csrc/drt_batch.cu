@@ -12,13 +12,13 @@
 //   stage 4  FP32-bulk extrapolation      (link, path, 32 consecutive steps: one warp), one unit
 //            range and launch per chain length 0..3, per length 2 and 3 of the multi-diffraction
 //            chains, and one for the rest (each path of it running the instance for its length)
-//   stage 5  H synthesis                  (link, 32 consecutive (step, bin tile) pairs: one block)
+//   stage 5  H synthesis                  (link, consecutive (step, bin tile) items: one block)
 // All stages run in waves of links whose per-path-step records (20 B each) fit one record buffer and
 // whose poses, warm starts and anchors fit one scratch region, both reused by the next wave, so a
 // batch of any size streams through a bounded scratch.  Links are ordered by decreasing work so the
 // largest units are claimed first.  Steps FP32 cannot resolve go to an FP64 redo kernel at the end
 // of their wave, which adds their contribution to H with atomics.  The frequency tile
-// width of stage 5 (8, 16 or 32 bins per thread) is autotuned on the batch.  The whole sequence can
+// width of stage 5 (128, 256 or 512 bins) is autotuned on the batch.  The whole sequence can
 // be captured in a CUDA graph.
 #include <cuda_runtime.h>
 
@@ -33,71 +33,57 @@
 #include <vector>
 
 #include "drt_batch.cuh"
+#include "drt_synth.cuh"
 
 namespace drt {
 
-// stage 5: a block takes (link, SYNTH_U consecutive (step, tile of KT bins) pairs), as in the
-// single-link synthesis: lane l owns pair l, the SYNTH_PG warps split the paths and add their
-// partial sums in shared memory; exact FP32 seed per (pair, path), complex rotation across the tile
+// stage 5: a unit (one block) is synth_run consecutive (step, tile of bins) items of one link, each a tile of
+// the tensor-core synthesis (drt_synth.cuh) whose paths the block's warps split, adding their sums in shared
+// memory; in links of at most SYNTH_SOLO paths, SYNTH_W times as many items, each warp taking its own whole
+template <int VI> struct SynthShape;
+template <> struct SynthShape<0> { typedef SynthTile<1, 1> T; };
+template <> struct SynthShape<1> { typedef SynthTile<1, 2> T; };
+template <> struct SynthShape<2> { typedef SynthTile<2, 2> T; };
+
 template <int VI>
-__global__ void __launch_bounds__(SYNTH_U * SYNTH_PG) k_batch_synth(const BatchDev B) {
-    constexpr int KT = SYNTH_KT[VI];
-    __shared__ float2 part[SYNTH_PG][KT][SYNTH_U + 1];
+__global__ void __launch_bounds__(32 * SYNTH_W, 4) k_batch_synth(const BatchDev B) {
+    typedef typename SynthShape<VI>::T Tile;
+    static_assert(Tile::BINS == SYNTH_BINS[VI], "tile of the variant");
+    __shared__ float2 part[SYNTH_W][Tile::BINS];
     const long long it = blockIdx.x;   // one unit per block (a plain grid: no claim loop needed here)
     if (it >= B.n_items) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int w = threadIdx.x >> 5;
     const int li = find_link(B, ST_SYNTH + VI, it);
     const BatchLink &BL = B.links[li];
-    const int F = BL.fg.n_bins, P = BL.L.n_paths, T = BL.tg.n_steps;
-    const int ntile = (F + KT - 1) / KT;
-    const long long pair = (it - BL.it0[ST_SYNTH + VI]) * SYNTH_U + lane;
-    const bool live = pair < (long long)T * ntile;
-    const int ti = live ? (int)(pair / ntile) : 0, k0 = live ? (int)(pair % ntile) * KT : 0;
-    const float kf = (float)k0;
-    float2 acc[KT];
+    const int F = BL.fg.n_bins, P = BL.L.n_paths, ntile = (F + Tile::BINS - 1) / Tile::BINS;
+    const long long items = (long long)BL.tg.n_steps * ntile, unit = it - BL.it0[ST_SYNTH + VI];
+    const bool solo = P <= SYNTH_SOLO;
+    for (int i = 0; i < B.synth_run; ++i) {
+        const long long item = solo ? (unit * B.synth_run + i) * SYNTH_W + w : unit * B.synth_run + i;
+        if (item >= items) break;   // uniform over the block unless solo, which has no barrier
+        const int ti = (int)(item / ntile), k0 = (int)(item % ntile) * Tile::BINS;
+        const size_t row = BL.rec0 + (size_t)ti * P;
+        float2 *out = BL.H + (size_t)ti * F + k0;
+        Tile tile;
+        tile.run(B.rec_a + row, B.rec_b + row, P, solo ? 0 : w, solo ? 1 : SYNTH_W, k0);
+        if (solo) {
+            tile.each([&](int k, float2 v) {
+                if (k0 + k < F) out[k] = v;
+            });
+            continue;
+        }
+        if (i) __syncthreads();   // the last item's sums have been read
+        tile.each([&](int k, float2 v) { part[w][k] = v; });
+        __syncthreads();
+        for (int k = threadIdx.x; k < Tile::BINS && k0 + k < F; k += 32 * SYNTH_W) {
+            float2 v = part[0][k];
 #pragma unroll
-    for (int j = 0; j < KT; ++j) acc[j] = make_float2(0.f, 0.f);
-    if (live) {
-        const float4 *__restrict__ ra = B.rec_a + BL.rec0 + (size_t)ti * P;
-        const float *__restrict__ rb = B.rec_b + BL.rec0 + (size_t)ti * P;
-        // the next path's record is loaded one iteration ahead (its latency hides behind the terms)
-        float4 rn = w < P ? __ldg(ra + w) : make_float4(0.f, 0.f, 0.f, 0.f);
-        float lon = w < P ? __ldg(rb + w) : 0.f;
-        for (int p = w; p < P; p += SYNTH_PG) {
-            const float4 r = rn;
-            const float lo = lon;
-            if (p + SYNTH_PG < P) {
-                rn = __ldg(ra + p + SYNTH_PG);
-                lon = __ldg(rb + p + SYNTH_PG);
+            for (int g = 1; g < SYNTH_W; ++g) {
+                v.x += part[g][k].x;
+                v.y += part[g][k].y;
             }
-            if (r.x == 0.f && r.y == 0.f) continue;
-            float ph = kf * r.w;   // exact: the step's high part has 12 significant bits, k0 < 4096
-            ph -= floorf(ph);
-            ph += r.z + kf * lo;
-            ph -= rintf(ph);       // cycles in [-1/2, 1/2]
-            float st = r.w + lo;
-            st -= rintf(st);
-            float sn, cs, ws, wc;   // hardware sine / cosine on [-pi, pi] (abs. error ~4e-7)
-            __sincosf(6.28318530717958648f * ph, &sn, &cs);
-            __sincosf(6.28318530717958648f * st, &ws, &wc);
-            const float zr = fmaf(r.x, cs, r.y * sn), zi = fmaf(r.y, cs, -r.x * sn);
-            add_geometric<KT>(acc, zr, zi, wc, -ws);
+            out[k] = v;
         }
-    }
-#pragma unroll
-    for (int j = 0; j < KT; ++j) part[w][j][lane] = acc[j];
-    __syncthreads();
-    if (!live) return;
-    float2 *out = BL.H + (size_t)ti * F + k0;
-#pragma unroll
-    for (int j = w; j < KT; j += SYNTH_PG) {
-        float2 v = part[0][j][lane];
-#pragma unroll
-        for (int g = 1; g < SYNTH_PG; ++g) {
-            v.x += part[g][j][lane].x;
-            v.y += part[g][j][lane].y;
-        }
-        if (k0 + j < F) out[j] = v;
     }
 }
 
@@ -124,6 +110,7 @@ struct BatchPlan {
     bool dual = false;  // some link asks for Doppler outputs: carry the rates
     bool any_out = false;   // some link asks for per-path-step records (all units then run generic code)
     bool any_pair = false;  // some entries form carrier pairs
+    int synth_run = 1;      // items in turn per synthesis block (see k_batch_synth)
     cudaGraphExec_t graph = nullptr;
     cudaStream_t capture = nullptr;   // private stream the graph is captured on (any caller stream,
                                       // the legacy default stream included, can then launch it)
@@ -147,6 +134,7 @@ static BatchDev dev_view(const BatchPlan &P, int l0, int l1, long long n_items, 
     B.counter = reinterpret_cast<unsigned long long *>(P.mem) + k;
     B.rec_a = reinterpret_cast<float4 *>(P.mem + P.off_rec);
     B.rec_b = reinterpret_cast<float *>(P.mem + P.off_rec + P.rec_count * sizeof(float4));
+    B.synth_run = P.synth_run;
     B.redo.count = reinterpret_cast<int *>(P.mem + P.off_redo);
     B.redo.items = reinterpret_cast<int4 *>(P.mem + P.off_redo + 256);
     B.redo.cap = (int)std::min<size_t>((P.redo_bytes - 256) / sizeof(int4), 0x7fffffff);
@@ -155,9 +143,9 @@ static BatchDev dev_view(const BatchPlan &P, int l0, int l1, long long n_items, 
 
 static cudaError_t launch_synth_variant(int v, const BatchDev &B, int grid, cudaStream_t s) {
     switch (v) {
-    case 0: k_batch_synth<0><<<grid, SYNTH_U * SYNTH_PG, 0, s>>>(B); break;
-    case 2: k_batch_synth<2><<<grid, SYNTH_U * SYNTH_PG, 0, s>>>(B); break;
-    default: k_batch_synth<1><<<grid, SYNTH_U * SYNTH_PG, 0, s>>>(B); break;
+    case 0: k_batch_synth<0><<<grid, 32 * SYNTH_W, 0, s>>>(B); break;
+    case 2: k_batch_synth<2><<<grid, 32 * SYNTH_W, 0, s>>>(B); break;
+    default: k_batch_synth<1><<<grid, 32 * SYNTH_W, 0, s>>>(B); break;
     }
     return cudaGetLastError();
 }
@@ -312,6 +300,11 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
     }
     std::vector<int> pos(n);
     for (int k = 0; k < n; ++k) pos[order[k]] = k;
+    {   // the link search of a synthesis block is shared by several items where there are many waves of blocks
+        long long steps = 0;
+        for (int i = 0; i < n; ++i) steps += tgs[i].n_steps;
+        P->synth_run = (int)std::max<long long>(1, std::min<long long>(4, steps / (sm_count() * 64)));
+    }
     P->host.resize(n);
     size_t off = 0;   // scratch offsets; made absolute in batch_bind
     auto take = [&](size_t b) {
@@ -396,9 +389,10 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
             if (!second && !P->any_out) W.n_bulkd[k] += (long long)(B.L.multi_start[k + 1] - B.L.multi_start[k]) * nbw;
         }
         for (int v = 0; v < 3; ++v) {   // a link without paths gets H = 0
-            const long long pairs = T * ((fgs[i].n_bins + SYNTH_KT[v] - 1) / SYNTH_KT[v]);
+            const long long items = T * ((fgs[i].n_bins + SYNTH_BINS[v] - 1) / SYNTH_BINS[v]);
+            const long long per = (long long)P->synth_run * (Pn <= SYNTH_SOLO ? SYNTH_W : 1);
             B.it0[ST_SYNTH + v] = W.n_synth[v];
-            W.n_synth[v] += (pairs + SYNTH_U - 1) / SYNTH_U;
+            W.n_synth[v] += (items + per - 1) / per;
         }
     }
     if (n) close_wave(n);
@@ -468,7 +462,8 @@ cudaError_t batch_autotune(BatchPlan *P, cudaStream_t s, float *best_ms) {
     if (e == cudaSuccess) e = cudaMemsetAsync(P->mem + P->off_redo, 0, 24, s);
     if (e == cudaSuccess) e = run_prep(*P, 0, s);
     if (e == cudaSuccess) e = run_wave_bulk(*P, 0, s);
-    const long long sample = (long long)sm_count() * 256;   // units of each variant timed
+    // the same share of the wave in every variant, whose units differ in their bins
+    const double share = std::min(1.0, (double)sm_count() * 64 / (double)std::max<long long>(1, P->waves[0].n_synth[2]));
     float best = 1e30f;
     int pick = 1;
     for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep)   // first pass warms up
@@ -477,7 +472,7 @@ cudaError_t batch_autotune(BatchPlan *P, cudaStream_t s, float *best_ms) {
             e = cudaMemsetAsync(P->mem + counter_of(0, 9) * sizeof(unsigned long long), 0,
                                 sizeof(unsigned long long), s);
             cudaEventRecord(a, s);
-            if (e == cudaSuccess) e = run_wave_synth(*P, 0, s, sample);
+            if (e == cudaSuccess) e = run_wave_synth(*P, 0, s, (long long)std::ceil(share * P->waves[0].n_synth[v]));
             cudaEventRecord(b, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);
             float ms = 0.f;

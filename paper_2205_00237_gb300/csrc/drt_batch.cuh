@@ -12,9 +12,9 @@ namespace drt {
 enum { ST_POSEB = 0, ST_POSE64 = 1, ST_WARM = 2, ST_BASE = 3, ST_BULK = 4, ST_SYNTH = 8, ST_BULKM = 11, ST_BULKD = 12,
        N_STAGES = 14 };
 constexpr int BULK_W = 32;                // time steps per extrapolation unit (one warp's lanes)
-constexpr int SYNTH_U = 32;               // (step, tile) pairs per synthesis unit (one block) ...
-constexpr int SYNTH_PG = 4;               // ... whose warps split the paths
-constexpr int SYNTH_KT[3] = {8, 16, 32};
+constexpr int SYNTH_W = 4;                // warps of a synthesis block: they split the paths of its (step, tile) items,
+constexpr int SYNTH_SOLO = 64;            // or, in links of at most this many paths, take an item each
+constexpr int SYNTH_BINS[3] = {128, 256, 512};   // bins of a tile per variant
 constexpr size_t REC_BYTES = sizeof(float4) + sizeof(float);   // one synthesis record
 constexpr size_t REC_CAP = (size_t)4 << 30;                    // record buffer of one wave (bytes)
 constexpr size_t SCRATCH_CAP = (size_t)8 << 30;                // poses, warm starts, anchors of one wave
@@ -51,6 +51,7 @@ struct BatchDev {
     unsigned long long *counter;
     float4 *rec_a;
     float *rec_b;
+    int synth_run;       // items a synthesis block (or, in small links, each of its warps) takes in turn
     RedoList redo;   // items (link, path, step)
 };
 

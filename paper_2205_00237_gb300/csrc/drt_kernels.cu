@@ -4,13 +4,14 @@
 //   k_power_bin      power-Doppler / power-delay profiles
 //   k_step_power, k_toggle, k_select, k_window_mask
 //                    multipath-lifetime expiry and T_C windows
-//   k_synth          a9: H(t, f) = sum_p a_p exp(-j 2 pi f tau_p); one thread per (time-step,
-//                    16-bin frequency tile, path group), sincos seed per tile and a complex
-//                    rotation recurrence inside it, FP32 FMA accumulation, groups added in
-//                    shared memory
+//   k_synth_mma      a9: H(t, f) = sum_p a_p exp(-j 2 pi f tau_p) on the tensor cores (drt_synth.cuh)
+//   k_synth          the same for at most 16 bins: one thread per (time-step, path group), sincos seed
+//                    and a complex rotation recurrence, FP32 FMA accumulation, groups added in shared
+//                    memory
 //   k_probe          FMA issue-rate probe for the roofline denominators
 #include <algorithm>
 #include "drt_launch.cuh"
+#include "drt_synth.cuh"
 
 namespace drt {
 
@@ -289,14 +290,69 @@ k_synth(const float4 *__restrict__ rec_a, const float *__restrict__ rec_b, int n
     }
 }
 
+// The same on the tensor cores (drt_synth.cuh): an item is one instant's tile of SynthTile<MT, NJ>::BINS
+// bins; PG warps split its paths and add their sums in shared memory (PG = 1: a warp per item, four to a
+// block).
+template <int MT, int NJ, int PG>
+__global__ void __launch_bounds__(PG == 1 ? 128 : 32 * PG, PG == 8 ? 2 : 4)
+k_synth_mma(const float4 *__restrict__ rec_a, const float *__restrict__ rec_b, int n_paths, int n_steps, int n_bins,
+            float2 *__restrict__ H, int ld) {
+    typedef SynthTile<MT, NJ> Tile;
+    const int w = threadIdx.x >> 5, ntile = (n_bins + Tile::BINS - 1) / Tile::BINS;
+    const long long item = PG == 1 ? 4ll * blockIdx.x + w : blockIdx.x;
+    if (item >= (long long)n_steps * ntile) return;
+    const int ti = (int)(item / ntile), k0 = (int)(item % ntile) * Tile::BINS;
+    Tile tile;
+    tile.run(rec_a + (size_t)ti * n_paths, rec_b + (size_t)ti * n_paths, n_paths, PG == 1 ? 0 : w, PG, k0);
+    float2 *out = H + (size_t)ti * ld + k0;
+    if constexpr (PG == 1) {
+        tile.each([&](int k, float2 v) {
+            if (k0 + k < n_bins) out[k] = v;
+        });
+    } else {
+        __shared__ float2 part[PG][Tile::BINS];
+        tile.each([&](int k, float2 v) { part[w][k] = v; });
+        __syncthreads();
+        for (int k = threadIdx.x; k < Tile::BINS && k0 + k < n_bins; k += 32 * PG) {
+            float2 v = part[0][k];
+#pragma unroll
+            for (int g = 1; g < PG; ++g) {
+                v.x += part[g][k].x;
+                v.y += part[g][k].y;
+            }
+            out[k] = v;
+        }
+    }
+}
+
+template <int MT, int NJ>
+static void launch_synth_mma(const RecD &rec, int n_paths, int n_steps, int n_bins, float2 *H, int ld, cudaStream_t s) {
+    const long long items = (long long)n_steps * ((n_bins + SynthTile<MT, NJ>::BINS - 1) / SynthTile<MT, NJ>::BINS);
+    // Warps per item: one where items alone fill the SMs' 16 warps (measured at 64 paths x 5000 steps x 256 bins: 14 us,
+    // 18 us with four) and short paths leave little to split; eight where there are too few of them for four (300
+    // steps x 512 paths x 512 bins: 12 us, 14 us with four; 2000 steps: 49 us, 45 us with four)
+    if (n_paths <= 16 || (items >= 152 * 16 && n_paths <= 320) || items >= 152 * 64)
+        k_synth_mma<MT, NJ, 1><<<(unsigned)((items + 3) / 4), 128, 0, s>>>(rec.rec_a, rec.rec_b, n_paths, n_steps, n_bins, H, ld);
+    else if (items >= 152 * 8 || n_paths <= 64)
+        k_synth_mma<MT, NJ, 4><<<(unsigned)items, 128, 0, s>>>(rec.rec_a, rec.rec_b, n_paths, n_steps, n_bins, H, ld);
+    else
+        k_synth_mma<MT, NJ, 8><<<(unsigned)items, 256, 0, s>>>(rec.rec_a, rec.rec_b, n_paths, n_steps, n_bins, H, ld);
+}
+
 cudaError_t launch_synth(const RecD &rec, int32_t n_paths, const TimeGridD &tg, const FreqGridD &fg, float2 *H,
                          cudaStream_t s, int ld) {
     if (ld < 0) ld = fg.n_bins;
-    int ntile = (fg.n_bins + KT - 1) / KT;
-    long long pairs = (long long)tg.n_steps * ntile;
+    const int F = fg.n_bins;
+    long long pairs = (long long)tg.n_steps * ((F + KT - 1) / KT);
     if (pairs == 0) return cudaSuccess;
-    k_synth<<<(unsigned)((pairs + SYN_PAIRS - 1) / SYN_PAIRS), SYN_PAIRS * PG, 0, s>>>(rec.rec_a, rec.rec_b, n_paths,
-                                                                                     tg.n_steps, fg.n_bins, H, ld);
+    // one tile of the term-by-term kernel costs less than the smallest matrix tile (128 bins); two cost more
+    // (300 paths x 3000 steps x 32 bins: 28 us against 22 us)
+    if (F <= KT)
+        k_synth<<<(unsigned)((pairs + SYN_PAIRS - 1) / SYN_PAIRS), SYN_PAIRS * PG, 0, s>>>(rec.rec_a, rec.rec_b, n_paths,
+                                                                                         tg.n_steps, F, H, ld);
+    else if (F <= 128) launch_synth_mma<1, 1>(rec, n_paths, tg.n_steps, F, H, ld, s);
+    else if (F <= 256) launch_synth_mma<1, 2>(rec, n_paths, tg.n_steps, F, H, ld, s);
+    else launch_synth_mma<2, 2>(rec, n_paths, tg.n_steps, F, H, ld, s);
     return cudaGetLastError();
 }
 

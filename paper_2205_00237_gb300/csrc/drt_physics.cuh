@@ -1237,13 +1237,9 @@ DRT_HD void write_record(const RecD &r, size_t ri, double tau, cx<double> a, uin
     double y = df * tau;
     double st = y - floor(y);
     double hi = ldexp(rint(ldexp(st, 12)), -12);
-    float4 v;
-    v.x = fl ? 0.f : (float)a.re;
-    v.y = fl ? 0.f : (float)a.im;
-    v.z = (float)phi0;
-    v.w = (float)hi;
-    r.rec_a[ri] = v;
-    r.rec_b[ri] = (float)(st - hi);
+    // a path that does not exist has an all-zero record: its phases may not be finite
+    r.rec_a[ri] = fl ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4((float)a.re, (float)a.im, (float)phi0, (float)hi);
+    r.rec_b[ri] = fl ? 0.f : (float)(st - hi);
 }
 
 // FP64 (path, time-step) core: primitives from `load(j, type, idx)`; FP64 outputs (amp double[2],
@@ -2011,11 +2007,8 @@ DRT_HD bool bulk_eval(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg
         x -= floorf(x);
         float ph = Bk.ph0 + x;
         ph -= floorf(ph);
-        r.ar = fl ? 0.f : ak.re;
-        r.ai = fl ? 0.f : ak.im;
-        r.ph = ph;
-        r.hi = Bk.st_hi;
-        r.lo = fmaf(g.dfc, dd_len, Bk.st_lo);
+        // a path that does not exist has an all-zero record: its phases may not be finite
+        r = fl ? Rec5{0.f, 0.f, 0.f, 0.f, 0.f} : Rec5{ak.re, ak.im, ph, Bk.st_hi, fmaf(g.dfc, dd_len, Bk.st_lo)};
     };
     phase_record(fg, B, a, rec);
     if (fg2) {
