@@ -307,6 +307,15 @@ Link *find_link(drt_ctx *c, uint64_t id) {
 TimeGridD tgd(const drt_time_grid *g, int chunk = 16) { return make_tgrid(g->t_start, g->dt, g->n_steps, chunk); }
 FreqGridD fgd(const drt_freq_grid *g) { return make_fgrid(g->fc, g->bandwidth, g->n_bins); }
 
+// Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
+// is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
+// as checked at load.  Beyond that the records are computed in FP64.
+bool ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
+    const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
+    const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T);
+    return v.ff_range && reach * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
+}
+
 // bracket one launch with events when tracing is on
 template <class F> drt_status traced(drt_ctx *c, int kind, cudaStream_t s, F &&launch) {
     if (!c->profiling) {
@@ -382,11 +391,35 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
                 return st;
         return DRT_OK;
     }
-    size_t pose_bytes = (size_t)tg->n_steps * L.dev.n_bodies * POSE_W * sizeof(double);
+    const bool outs = out.tau || out.amp || out.doppler || out.angles || out.flags || out.points;
+    const bool two = !outs && rec.rec_a && ff_applies(L.view, *tg, *fg);
+    size_t pose_bytes = two ? pose_ff_bytes(L.dev, t) : (size_t)tg->n_steps * L.dev.n_bodies * POSE_W * sizeof(double);
     if (drt_status st = ensure(c, c->pose, pose_bytes)) return st;
     if (drt_status st = ensure(c, c->warm, warm_bytes(L.dev, t))) return st;
     double *pose = reinterpret_cast<double *>(c->pose.ptr);
     double *warm = reinterpret_cast<double *>(c->warm.ptr);
+    if (two) {
+        // side[1]: warm starts, the chains that wait for them; side[0]: lengths 2 and 0; s: lengths 3 and 1
+        if (drt_status st = traced(c, 0, s, [&] { return launch_pose_ff(L.dev, t, pose, s); })) return st;
+        return traced(c, 1, s, [&] {
+            const LinkDev &D = L.dev;
+            cudaStream_t s0 = c->side[0], s1 = c->side[1];
+            cudaError_t e = cudaEventRecord(c->ev_fork, s);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, c->ev_fork, 0);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s1, c->ev_fork, 0);
+            if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1);
+            if (e == cudaSuccess) e = launch_extrapolate_ff_generic(D, t, f, pose, rec, warm, s1);
+            if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 2, warm, s0);
+            if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 0, warm, s0);
+            if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 3, warm, s);
+            if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 1, warm, s);
+            if (e == cudaSuccess) e = cudaEventRecord(c->ev_join[0], s0);
+            if (e == cudaSuccess) e = cudaEventRecord(c->ev_join[1], s1);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join[0], 0);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->ev_join[1], 0);
+            return e;
+        });
+    }
     if (drt_status st = traced(c, 0, s, [&] { return launch_pose(L.dev, t, pose, s); })) return st;
     // The FP64 kernels all wait on the FP64 pipe, so the launches of one call run side by side on three
     // streams: every launch's last wave of blocks then shares the SMs with the others instead of
@@ -458,7 +491,26 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
     if (drt_status st = validate(s, ps)) return st;
     {
         auto n3 = [](const double *x) { return std::sqrt(dot3(x, x)); };
-        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0};
+        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0, 0.0, true};
+        auto reach = [&](const double *x) { v.extent = std::max(v.extent, n3(x)); };
+        reach(s->tx.r);
+        reach(s->rx.r);
+        for (int i = 0; i < s->n_bodies; ++i) reach(s->bodies[i].o);
+        // a rotating primitive stays within |o| + |rel| <= 2 |o| + |c|
+        auto prim = [&](int body, const double *x) {
+            v.extent = std::max(v.extent, 2 * n3(s->bodies[body].o) + n3(x));
+        };
+        for (int i = 0; i < s->n_faces; ++i) prim(s->faces[i].body, s->faces[i].c);
+        for (int i = 0; i < s->n_edges; ++i) {
+            prim(s->edges[i].body, s->edges[i].a);
+            prim(s->edges[i].body, s->edges[i].b);
+        }
+        for (int i = 0; i < s->n_tiles; ++i) {
+            prim(s->tiles[i].body, s->tiles[i].c);
+            v.ff_range = v.ff_range && s->tiles[i].area < 1e8;
+        }
+        for (int i = 0; i < s->n_materials; ++i)
+            v.ff_range = v.ff_range && s->materials[i].eps_r < 1e6 && s->materials[i].sigma < 1e8;
         for (int i = 0; i < s->n_bodies; ++i) {
             const drt_body &b = s->bodies[i];
             v.vmax = std::max(v.vmax, n3(b.v));
@@ -542,7 +594,67 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
     for (int i = 0; i < s->n_materials; ++i) {
         const drt_material &m = s->materials[i];
         const double spec = std::sqrt(std::max(0.0, 1.0 - m.rough_s * m.rough_s));   // specular scale of a rough face
-        mats[i] = MatD{m.eps_r, m.sigma, spec, m.pec, (float)m.eps_r, (float)m.sigma, (float)spec, (float)m.pec};
+        mats[i] = MatD{m.eps_r, m.sigma, spec, m.pec, (float)m.eps_r, (float)m.sigma, (float)spec, (float)m.pec,
+                       ff_host(m.eps_r), ff_host(m.sigma), ff_host(spec)};
+    }
+    // two-float copies
+    auto q3 = [](ff *d, const double *x) {
+        for (int j = 0; j < 3; ++j) d[j] = ff_host(x[j]);
+    };
+    auto placed = [&](int body, ff *d, const double *rel) {   // the index a two-float primitive keeps: -1 at rest
+        const bool fixed = H.body_fixed[body] != 0;
+        for (int j = 0; j < 3; ++j) d[j] = ff_host(fixed ? bodies[body].o[j] + rel[j] : rel[j]);
+        return fixed ? -1 : body;
+    };
+    H.facesQ.resize(s->n_faces);
+    for (int i = 0; i < s->n_faces; ++i) {
+        const FaceD &g = faces[i];
+        FaceQ &h = H.facesQ[i];
+        h.body = placed(g.body, h.c, g.c);
+        q3(h.n, g.n);
+        q3(h.u, g.u);
+        h.hu = ff_host(g.hu);
+        h.hw = ff_host(g.hw);
+        h.mat = g.mat;
+    }
+    H.edgesQ.resize(s->n_edges);
+    for (int i = 0; i < s->n_edges; ++i) {
+        const EdgeD &g = edges[i];
+        EdgeQ &h = H.edgesQ[i];
+        h.body = placed(g.body, h.a, g.a);
+        q3(h.e, g.e);
+        q3(h.t0, g.t0);
+        q3(h.n0, g.n0);
+        h.len = ff_host(g.len);
+        h.wn = ff_host(g.wn);
+        h.snp = ff_host(g.snp);
+        h.cnp = ff_host(g.cnp);
+        h.mat = g.mat;
+    }
+    H.tilesQ.resize(s->n_tiles);
+    for (int i = 0; i < s->n_tiles; ++i) {
+        const TileD &g = tiles[i];
+        TileQ &h = H.tilesQ[i];
+        h.body = placed(g.body, h.c, g.c);
+        q3(h.n, g.n);
+        h.area = ff_host(g.area);
+        h.s = ff_host(g.s);
+        h.cph = ff_host(g.cph);
+        h.sph = ff_host(g.sph);
+        h.alpha = (int32_t)g.alpha;
+        h.mat = g.mat;
+        h.pad = 0;
+    }
+    H.bodiesQ.resize(s->n_bodies);
+    for (int i = 0; i < s->n_bodies; ++i) {
+        const BodyD &g = bodies[i];
+        BodyQ &h = H.bodiesQ[i];
+        q3(h.o, g.o);
+        q3(h.v, g.v);
+        q3(h.a, g.a);
+        q3(h.k, g.k);
+        h.w0 = ff_host(g.w0);
+        h.wdot = ff_host(g.wdot);
     }
     auto f3 = [](float *d, const double *x) {
         for (int j = 0; j < 3; ++j) d[j] = (float)x[j];
@@ -757,6 +869,10 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     L.n_paths = ps->n_paths;
     LinkDev &d = L.dev;
     LinkImage img;
+    auto bytes = [](const auto &...v) { return ((v.size() * sizeof(v[0]) + 256) + ...); };
+    img.host.reserve(bytes(H.bodies, H.body_fixed, H.faces, H.edges, H.tiles, H.mats, H.facesF, H.edgesF, H.tilesF, H.facesQ,
+                           H.edgesQ, H.tilesQ, H.bodiesQ, H.ptypes, H.pprims, H.ps0, H.perm) +
+                     (size_t)(d.n_paths - d.n_bulk) * 2 * MAXI * sizeof(double) + 256);
     img.add(H.bodies, &d.bodies);
     img.add(H.body_fixed, &d.body_fixed);
     img.add(H.faces, &d.faces);
@@ -766,6 +882,10 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     img.add(H.facesF, &d.facesF);
     img.add(H.edgesF, &d.edgesF);
     img.add(H.tilesF, &d.tilesF);
+    img.add(H.facesQ, &d.facesQ);
+    img.add(H.edgesQ, &d.edgesQ);
+    img.add(H.tilesQ, &d.tilesQ);
+    img.add(H.bodiesQ, &d.bodiesQ);
     img.add(H.ptypes, &d.ptypes);
     img.add(H.pprims, &d.pprims);
     img.add(H.ps0, &d.ps0);

@@ -5,11 +5,13 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <cmath>
 #include <memory>
 #include <string>
 #include <vector>
 
 #include "../../include/drt.h"
+#include "drt_ff.cuh"
 
 namespace drt {
 
@@ -21,11 +23,17 @@ constexpr int POSE_W = 18;   // doubles per (time, body) pose record: R (3x3 row
 struct FaceD { double c[3], n[3], u[3], hu, hw; int32_t body, mat; };                       // 96 B
 struct EdgeD { double a[3], e[3], t0[3], n0[3], len, wn, snp, cnp; int32_t body, mat, pad0, pad1; };  // 144 B: snp, cnp = sin, cos(wn pi)
 struct TileD { double c[3], n[3], area, s, alpha, cph, sph; int32_t body, mat; };          // 96 B: cph + j sph = exp(j phase)
-struct MatD { double eps_r, sigma, spec, pec; float eps_rf, sigmaf, specf, pecf; };         // 48 B: spec = sqrt(1 - S^2)
+struct MatD { double eps_r, sigma, spec, pec; float eps_rf, sigmaf, specf, pecf; ff eps_rq, sigmaq, specq; };   // spec = sqrt(1 - S^2)
 // FP32 copies for the FP32-bulk form (same meaning, no FP64 conversions in its kernels)
 struct FaceF { float c[3], n[3], u[3], hu, hw; int32_t body, mat, pad0, pad1, pad2; };          // 64 B
 struct EdgeF { float a[3], e[3], t0[3], n0[3], len, wn, snp, cnp; int32_t body, mat; };      // 72 B
 struct TileF { float c[3], n[3], area, s, alpha, cph, sph; int32_t body, mat; };            // 52 B
+// two-float copies (drt_ff.cuh) for the records of H in the FP64 form; a primitive of a body at rest holds its place in the world
+// and body = -1, the others their place relative to the body's rotation centre
+struct FaceQ { ff c[3], n[3], u[3], hu, hw; int32_t body, mat; };
+struct EdgeQ { ff a[3], e[3], t0[3], n0[3], len, wn, snp, cnp; int32_t body, mat; };
+struct TileQ { ff c[3], n[3], area, s, cph, sph; int32_t alpha, body, mat, pad; };
+struct BodyQ { ff o[3], v[3], a[3], k[3], w0, wdot; };
 struct TermD { double r[3], v[3], a[3]; };
 struct BodyD { double o[3], v[3], a[3], k[3], w0, wdot; };
 
@@ -50,6 +58,10 @@ struct LinkDev {
     const FaceF *facesF;
     const EdgeF *edgesF;
     const TileF *tilesF;
+    const FaceQ *facesQ;
+    const EdgeQ *edgesQ;
+    const TileQ *tilesQ;
+    const BodyQ *bodiesQ;
     // paths in internal (signature-sorted) order
     const uint32_t *ptypes;   // byte j = type of vertex j (0 past the chain)
     const int4 *pprims;       // primitive index of vertex j
@@ -75,16 +87,32 @@ struct FreqGridD {
     float fcf;        // fc
     float f0c, dfc;   // (fc - B/2) / c and B / (n_bins c): first bin and bin step over c (1/m)
     float disp_lim;   // interaction-point displacement since the chunk base past which a step is redone in FP64 (m)
+    ff kq, iskq, iepsq, lamq;   // FieldK of the two-float form
+    ff f0c_q, dfc_q;            // f0 / c, df / c
     double f0, df;    // first bin fc - B/2 and bin step B / n_bins (Hz), so that no kernel divides per step
 };
 inline TimeGridD make_tgrid(double t_start, double dt, int32_t n_steps, int32_t chunk) {
     return TimeGridD{t_start, dt, n_steps, chunk, (float)dt};
 }
 inline FreqGridD make_fgrid(double fc, double bandwidth, int32_t n_bins) {
-    const double c0 = 299792458.0;
-    return FreqGridD{fc, bandwidth, n_bins, (float)fc, (float)((fc - 0.5 * bandwidth) / c0),
-                     (float)(bandwidth / n_bins / c0), (float)(0.8 * 60e9 / fc), fc - 0.5 * bandwidth,
-                     n_bins > 0 ? bandwidth / n_bins : 0.0};
+    const double c0 = 299792458.0, pi = 3.14159265358979323846, eps0 = 8.8541878128e-12, k = 2 * pi * fc / c0;
+    FreqGridD g{};
+    g.fc = fc;
+    g.bandwidth = bandwidth;
+    g.n_bins = n_bins;
+    g.fcf = (float)fc;
+    g.f0c = (float)((fc - 0.5 * bandwidth) / c0);
+    g.dfc = (float)(bandwidth / n_bins / c0);
+    g.disp_lim = (float)(0.8 * 60e9 / fc);
+    g.f0 = fc - 0.5 * bandwidth;
+    g.df = n_bins > 0 ? bandwidth / n_bins : 0.0;
+    g.kq = ff_host(k);
+    g.iskq = ff_host(1.0 / std::sqrt(2 * pi * k));
+    g.iepsq = ff_host(1.0 / (2 * pi * fc * eps0));
+    g.lamq = ff_host(c0 / (4 * pi * fc));
+    g.f0c_q = ff_host(g.f0 / c0);
+    g.dfc_q = ff_host(g.df / c0);
+    return g;
 }
 
 // user-visible outputs (caller order), any may be null
@@ -106,7 +134,8 @@ struct RecD { float4 *rec_a; float *rec_b; };
 
 // kinematic bounds of a link used by the batch planner's chunk model: fastest terminal / body
 // translation speed (m/s), largest acceleration (m/s^2), largest angular speed (rad/s)
-struct drt_scene_view { double vmax, amax, wmax; };
+// and extent, the largest coordinate at t0 (m); ff_range: every length and material constant lies in the range of the two-float form
+struct drt_scene_view { double vmax, amax, wmax, extent; bool ff_range; };
 
 // a10 batch plans (drt_batch.cu)
 struct BatchPlan;
@@ -163,6 +192,10 @@ struct PackedLink {
     std::vector<FaceF> facesF;
     std::vector<EdgeF> edgesF;
     std::vector<TileF> tilesF;
+    std::vector<FaceQ> facesQ;
+    std::vector<EdgeQ> edgesQ;
+    std::vector<TileQ> tilesQ;
+    std::vector<BodyQ> bodiesQ;
     std::vector<uint32_t> ptypes;
     std::vector<int4> pprims;
     std::vector<double> ps0;
@@ -182,6 +215,14 @@ cudaError_t launch_extrapolate_fp64(const LinkDev &L, const TimeGridD &tg, const
                                     cudaStream_t s, int p0 = 0, int p1 = -1, bool f32out = false,
                                     double *warm = nullptr, cudaStream_t s_multi = nullptr);
 size_t warm_bytes(const LinkDev &L, const TimeGridD &tg);
+// the FP64 form's synthesis records in two-float numbers (values only): poses and terminal positions per step into mem
+// (pose_ff_bytes), then the chains of length n < MAXI with at most one diffraction per segment, and the others
+size_t pose_ff_bytes(const LinkDev &L, const TimeGridD &tg);
+cudaError_t launch_pose_ff(const LinkDev &L, const TimeGridD &tg, void *mem, cudaStream_t s);
+cudaError_t launch_extrapolate_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const void *mem,
+                                  const RecD &rec, int n, const double *warm, cudaStream_t s);
+cudaError_t launch_extrapolate_ff_generic(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const void *mem,
+                                          const RecD &rec, const double *warm, cudaStream_t s);
 // the warm-start table of the multi-diffraction chains (FP64 dual-number solves at the chunk bases)
 // edge parameters and rates at t = 0 of the multi-diffraction paths (LinkDev::t0par), at load
 cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s);

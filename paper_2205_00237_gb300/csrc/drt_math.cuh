@@ -129,6 +129,8 @@ template <class E> DRT_HD v3<E> cross(v3<E> a, v3<E> b) {
     return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
 
+template <class S> DRT_HD v3<S> axpy(v3<S> X, v3<S> n, S s) { return X + n * s; }   // overloaded for two-float numbers
+
 // value / derivative parts of a vector of scalars, and promotion of a plain vector
 template <class S> DRT_HD v3<typename ST<S>::R> val(v3<S> a) { return {sval(a.x), sval(a.y), sval(a.z)}; }
 template <class S> DRT_HD v3<typename ST<S>::R> der(v3<S> a) { return {srate(a.x), srate(a.y), srate(a.z)}; }
@@ -194,6 +196,7 @@ template <class T> DRT_HD c3<T> operator+(c3<T> a, c3<T> b) { return {a.x + b.x,
 template <class T> DRT_HD c3<T> cscale(v3<T> e, cx<T> s) { return {s * e.x, s * e.y, s * e.z}; }
 template <class T> DRT_HD c3<T> cscale(c3<T> E, cx<T> s) { return {E.x * s, E.y * s, E.z * s}; }
 template <class T> DRT_HD cx<T> cdot(c3<T> E, v3<T> e) { return E.x * e.x + E.y * e.y + E.z * e.z; }
+template <class T> DRT_HD c3<T> mix(v3<T> a, cx<T> s, v3<T> b, cx<T> t) { return cscale(a, s) + cscale(b, t); }
 template <class T> DRT_HD T cnorm(c3<T> E) { return sqrt(cabs2(E.x) + cabs2(E.y) + cabs2(E.z)); }
 
 // acc[j] += z w^j, j < KT, for |w| = 1 (one path's terms across a frequency tile).  Where |Im w| >= 1/4

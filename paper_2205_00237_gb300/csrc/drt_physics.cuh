@@ -11,6 +11,7 @@
 #include <type_traits>
 #include "drt_internal.h"
 #include "drt_fnodes.h"
+#include "drt_ff.cuh"
 #include "drt_math.cuh"
 
 namespace drt {
@@ -89,15 +90,30 @@ template <class S> DRT_HD v3<S> refl_point(v3<S> Sv, v3<S> Rv, v3<S> c, v3<S> n)
     v3<S> Q = Sv + (Rv - Sv) * g;
     return Q - n * dot(Q - c, n);
 }
+template <class S> DRT_HD S twice(S h) { return h + h; }
 // image of X across the wall (c, n)
 template <class S> DRT_HD v3<S> mirror(v3<S> X, v3<S> c, v3<S> n) {
     S h = dot(X - c, n);
-    return X - n * (h + h);
+    return X - n * twice(h);
 }
 template <class S> DRT_HD v3<S> mirror_dir(v3<S> d, v3<S> n) {
     S h = dot(d, n);
-    return d - n * (h + h);
+    return d - n * twice(h);
 }
+
+// Two-float arithmetic is 7 to 31 instructions an operation: inlined at every vertex, the code of a chain outgrows the
+// instruction caches (7 to 11 no-instruction stalls per issue, 28 % of the issue slots used).  Its helpers are one copy each.
+#define DRT_NOINL __host__ __device__ __noinline__
+#define DRT_NOINL1 inline DRT_NOINL   // not a template
+DRT_NOINL1 v3<ff> refl_point_ff(v3<ff> Sv, v3<ff> Rv, v3<ff> c, v3<ff> n) { 
+    const v3<ff> u = Sv - c;
+    const ff hs = dot(u, n), hr = dot(Rv - c, n), g = hs / (hs + hr);
+    const v3<ff> Q = axpy(Sv, Rv - Sv, g);
+    return axpy(Q, n, -dot(Q - c, n));
+}
+DRT_NOINL1 v3<ff> mirror_ff(v3<ff> X, v3<ff> c, v3<ff> n) { return axpy(X, n, twice(-dot(X - c, n))); }
+DRT_HD v3<ff> refl_point(v3<ff> Sv, v3<ff> Rv, v3<ff> c, v3<ff> n) { return refl_point_ff(Sv, Rv, c, n); }
+DRT_HD v3<ff> mirror(v3<ff> X, v3<ff> c, v3<ff> n) { return mirror_ff(X, c, n); }
 
 // posed primitives of one chain vertex
 template <class S> struct Prim {
@@ -228,10 +244,28 @@ DRT_HD S keller_s(v3<S> Sv, v3<S> Rv, const Prim<S> &e, uint32_t &fl) {
         fl |= F_DEGEN;
         return sa;
     }
+    // two-float numbers: within 1 um of the edge line
+    if constexpr (std::is_same<T, ff>::value)
+        if (!(ra2.h > 1e-12f) || !(rb2.h > 1e-12f)) fl |= F_REDO64;
     // near grazing (a virtual terminal within 1 mm of the edge line) FP32 cannot resolve the cone
     if (sizeof(T) == 4 && (ra2 < T(1e-6) || rb2 < T(1e-6))) fl |= F_REDO64;
     S ra = norm(pa), rb = norm(pb);
     return sa + (sb - sa) * ra / (ra + rb);
+}
+
+struct KellerFF { ff s; uint32_t fl; };
+DRT_NOINL1 KellerFF keller_s_ff(v3<ff> Sv, v3<ff> Rv, v3<ff> p, v3<ff> a) {
+    Prim<ff> e;
+    e.p = p;
+    e.a = a;
+    KellerFF r{ff(0.f), 0};
+    r.s = keller_s<ff>(Sv, Rv, e, r.fl);
+    return r;
+}
+DRT_HD ff keller_s(v3<ff> Sv, v3<ff> Rv, const Prim<ff> &e, uint32_t &fl) {
+    const KellerFF r = keller_s_ff(Sv, Rv, e.p, e.a);
+    fl |= r.fl;
+    return r.s;
 }
 
 template <class S> DRT_HD void clamp_positive(S &x, typename ST<S>::R eps);
@@ -242,6 +276,9 @@ template <> DRT_HD void clamp_positive<double>(double &x, double eps) {
     if (!(x > eps)) x = eps;
 }
 template <> DRT_HD void clamp_positive<float>(float &x, float eps) {
+    if (!(x > eps)) x = eps;
+}
+template <> DRT_HD void clamp_positive<ff>(ff &x, ff eps) {
     if (!(x > eps)) x = eps;
 }
 template <> DRT_HD void clamp_positive<de>(de &x, float eps) {
@@ -260,6 +297,7 @@ template <> DRT_HD void clamp_positive<dd>(dd &x, float eps) {
 // Newton start for an edge parameter from its value `base` + `delta` and rate: for delta numbers
 // the base part is `base` (the chunk-base solution) and the delta `delta`
 template <class S> DRT_HD S newton_start(double base, double delta, double rate);
+template <> DRT_HD ff newton_start<ff>(double base, double delta, double) { return from_double(base + delta); }
 template <> DRT_HD double newton_start<double>(double base, double delta, double) { return base + delta; }
 template <> DRT_HD float newton_start<float>(double base, double delta, double) { return (float)(base + delta); }
 template <> DRT_HD dl<double> newton_start<dl<double>>(double base, double delta, double rate) {
@@ -274,6 +312,7 @@ template <> DRT_HD dd newton_start<dd>(double base, double delta, double rate) {
 template <class S> DRT_HD S newton_start_f(double base, float delta, float rate);
 template <> DRT_HD de newton_start_f<de>(double base, float delta, float) { return {(float)base, delta}; }
 template <> DRT_HD dd newton_start_f<dd>(double base, float delta, float rate) { return {(float)base, delta, rate}; }
+template <> DRT_HD ff newton_start_f<ff>(double base, float delta, float) { return from_double(base) + ff(delta); }
 
 // chain length of path p (vertices before the first empty type byte)
 DRT_HD int chain_length(const LinkDev &L, int p) {
@@ -311,7 +350,7 @@ DRT_HD void place_keller(const Prim<S> *pr, v3<S> *V, uint32_t &fl, const bool *
 #pragma unroll
     for (int i = N; i >= 1; --i) {
         const Prim<S> &q = pr[i - 1];
-        if (q.type == T_D && !(nv && nv[i])) V[i] = q.p + q.a * keller_s(img[i - 1], cur, q, fl);
+        if (q.type == T_D && !(nv && nv[i])) V[i] = axpy(q.p, q.a, keller_s(img[i - 1], cur, q, fl));
         else if (q.type == T_R) cur = mirror(cur, q.p, q.a);
         else cur = V[i];
     }
@@ -360,7 +399,8 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
                                 const D *rate0, uint32_t &fl) {
     typedef typename ST<S>::R T;
     // convergence threshold on the Newton step (m): near round-off of the working precision
-    const T tol = sizeof(T) == 8 ? T(1e-10) : T(1e-4);
+    // (two-float numbers stop at a step of 1 um: the next one would be ~1e-12 / leg length, below their resolution)
+    const T tol = std::is_same<T, ff>::value ? T(1e-6) : sizeof(T) == 8 ? T(1e-10) : T(1e-4);
     // below this step (m) the length change of a Newton step is at round-off of the ~100 m path
     // length, so the backtracking test is only applied to larger steps
     const T ls_min = sizeof(T) == 8 ? T(1e-4) : T(1e-2);
@@ -589,6 +629,15 @@ template <int N> constexpr int len_min() { return N == LEN_GEN ? 2 : 0; }
 // of the form exact outside the 1e-9 m band of the FP64 form.  F_NEAR100 marks margins within 100x
 // that bound (the FP32-bulk step uses it to keep the FP32 flags of invalid steps that moved far).
 template <class T> DRT_HD T amax3(v3<T> a) { return fmax(fmax(fabs(a.x), fabs(a.y)), fabs(a.z)); }
+DRT_HD float amax3(v3<ff> a) { return fmaxf(fmaxf(fabsf(a.x.h), fabsf(a.y.h)), fabsf(a.z.h)); }
+// The two-float form (H of the FP64 form) leaves margins within 2^-36 of the coordinates (1.5e-9 m at 100 m: ~2000 times the
+// rounding of a coordinate) to FP64 in the same way.
+DRT_HD float ff_margin_tol(float scale) { return 1.4551915e-11f * (scale + 1.f); }
+// the margin b - |a| (b may be infinite) and the sign-exact value of a normalised number
+DRT_HD float ff_within(ff a, ff b) {
+    const ff m = fabs(a);
+    return (b.h - m.h) + (b.l - m.l);
+}
 // bound on the FP32 error of a margin computed from positions of magnitude `scale` (m): 2e-6 of the
 // scale is ~17 ulp of the largest coordinate; the FP32 flags of the canyon, link and highway workloads
 // were found exact outside 1e-4 m of every boundary without this test (coordinates up to ~600 m)
@@ -602,6 +651,41 @@ DRT_HD float fp32_margin_tol(float scale) { return 2e-6f * (scale + 1.f); }
 // error bound.  (Called out of line in the FP32 kernels it measured no faster, unlike the field
 // updates, so it stays inline.)
 template <class T> struct VertexCheck { uint32_t fl; T m; };
+DRT_NOINL1 VertexCheck<float> vertex_validity_inl(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
+                                              v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
+    uint32_t fl = 0;
+    float m, scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), amax3(Pi));
+    if (ty == T_D) {
+        scale = fmaxf(scale, amax3(c));
+        const ff s = dot(Pi - c, nn);
+        const float up = (h1.h - s.h) + (h1.l - s.l);
+        if (s.h < 0.f || up < 0.f) fl |= F_EDGE;
+        m = fminf(fabsf(s.h), fabsf(up));
+#pragma unroll
+        for (int side = -1; side <= 1; side += 2) {   // see the general form below
+            const v3<ff> r = (side < 0 ? Pm : Pp) - Pi;
+            const v3<ff> rp = axpy(r, nn, -dot(r, nn));
+            const ff y = dot(rp, cc), x = dot(rp, b);
+            const float sn = det2(h3, x, h4, y).h;
+            if (!(y.h > 0.f) && !(sn > 0.f)) fl |= F_SIDE;   // zero of either is within the margin
+            m = fminf(m, fminf(fabsf(y.h), fabsf(sn)));
+        }
+    } else {
+        m = 1e30f;
+        if (ty == T_R) {
+            scale = fmaxf(scale, amax3(c));
+            const v3<ff> r = Pi - c;
+            const float mu = ff_within(dot(r, b), h1), mw = ff_within(dot(r, cross(b, nn)), h2);
+            if (mu < 0.f || mw < 0.f) fl |= F_FACE;
+            m = fminf(fabsf(mu), fabsf(mw));
+        }
+        const float dp = dot(Pm - c, nn).h, dn = dot(Pp - c, nn).h;   // a tile is its own point
+        if (!(dp > 0.f) || !(dn > 0.f)) fl |= F_SIDE;
+        m = fminf(m, fminf(fabsf(dp), fabsf(dn)));
+    }
+    // written so that a margin that is not a number is inside the bound
+    return VertexCheck<float>{fl, m > ff_margin_tol(scale) ? 2.f : 0.f};
+}
 template <class T>
 DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3<T> cc, T h1, T h2, T h3, T h4,
                                           v3<T> Pm, v3<T> Pi, v3<T> Pp) {
@@ -659,10 +743,11 @@ DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3
 template <int N = -1, class S>
 DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P) {
     typedef typename ST<S>::R T;
-    constexpr bool F32 = sizeof(T) == 4;
+    constexpr bool F32 = sizeof(T) == 4, FF = std::is_same<T, ff>::value;
+    typedef std::conditional_t<FF, float, T> M;
     const int nv = N >= 0 ? N : n;
     uint32_t fl = 0;
-    T mmin = T(1e30);    // FP32 only: the smallest margin over its bound
+    M mmin = M(1e30);    // FP32 and two-float only: the smallest margin over its bound
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI + 1; ++i) {
         if (i > nv + 1) break;
@@ -673,7 +758,7 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
     for (int i = 1; i <= MAXI; ++i) {
         if (i > nv) break;
         const Prim<S> &q = pr[i - 1];
-        const VertexCheck<T> v =
+        const VertexCheck<M> v =
             vertex_validity_inl(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
         fl |= v.fl;
         mmin = fmin(mmin, v.m);
@@ -682,6 +767,8 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         if (mmin < T(1)) fl |= F_REDO64;
         if (mmin < T(100)) fl |= F_NEAR100;
     }
+    if constexpr (FF)
+        if (mmin < 1.f) fl |= F_REDO64;
     return fl;
 }
 
@@ -691,6 +778,7 @@ template <class T> struct MatV { T eps_r, sigma, spec; bool pec; };   // spec = 
 template <class T> DRT_HD MatV<T> matv(const MatD &m);
 template <> DRT_HD MatV<double> matv<double>(const MatD &m) { return {m.eps_r, m.sigma, m.spec, m.pec != 0.0}; }
 template <> DRT_HD MatV<float> matv<float>(const MatD &m) { return {m.eps_rf, m.sigmaf, m.specf, m.pecf != 0.f}; }
+template <> DRT_HD MatV<ff> matv<ff>(const MatD &m) { return {m.eps_rq, m.sigmaq, m.specq, m.pec != 0.0}; }
 template <class T> struct TileV { T area, s, cph, sph; int alpha; };   // cph + j sph = exp(j phase)
 template <class T> DRT_HD TileV<T> tilev(const LinkDev &L, int idx);
 template <> DRT_HD TileV<double> tilev<double>(const LinkDev &L, int idx) {
@@ -700,6 +788,11 @@ template <> DRT_HD TileV<double> tilev<double>(const LinkDev &L, int idx) {
 template <> DRT_HD TileV<float> tilev<float>(const LinkDev &L, int idx) {
     const TileF &t = L.tilesF[idx];
     return {t.area, t.s, t.cph, t.sph, (int)t.alpha};
+}
+
+template <> DRT_HD TileV<ff> tilev<ff>(const LinkDev &L, int idx) {
+    const TileQ &t = L.tilesQ[idx];
+    return {t.area, t.s, t.cph, t.sph, t.alpha};
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -721,6 +814,29 @@ DRT_HD void fresnel(const MatV<T> &m, T ieps, T ct, cx<T> &rte, cx<T> &rtm) {
     const T n1 = cabs2(b1), n2 = cabs2(b2), r = T(1) / (n1 * n2), i1 = n2 * r, i2 = n1 * r;
     rte = C<T>(fma(a1.re, b1.re, a1.im * b1.im) * i1, fma(a1.im, b1.re, -a1.re * b1.im) * i1);
     rtm = C<T>(fma(a2.re, b2.re, a2.im * b2.im) * i2, fma(a2.im, b2.re, -a2.re * b2.im) * i2);
+}
+
+struct FresnelFF { cx<ff> te, tm; };
+DRT_NOINL1 FresnelFF fresnel_ff(MatV<ff> m, ff ieps, ff ct) {
+    FresnelFF r;
+    if (m.pec) {
+        r.te = C<ff>(ff(-1.f), ff(0.f));
+        r.tm = C<ff>(ff(1.f), ff(0.f));
+        return r;
+    }
+    // the general form above with its products and sums joined
+    const cx<ff> ec = C<ff>(m.eps_r, -(m.sigma * ieps)), z = C<ff>(fma(ct, ct, ec.re - ff(1.f)), ec.im);
+    const cx<ff> sq = csqrt_(z), ecct = C<ff>(ec.re * ct, ec.im * ct);
+    const cx<ff> a1 = C<ff>(ct - sq.re, -sq.im), b1 = C<ff>(ct + sq.re, sq.im), a2 = ecct - sq, b2 = ecct + sq;
+    const ff n1 = cabs2(b1), n2 = cabs2(b2), q = ff(1.f) / (n1 * n2), i1 = n2 * q, i2 = n1 * q;
+    r.te = C<ff>(det2(a1.re, b1.re, -a1.im, b1.im) * i1, det2(a1.im, b1.re, a1.re, b1.im) * i1);
+    r.tm = C<ff>(det2(a2.re, b2.re, -a2.im, b2.im) * i2, det2(a2.im, b2.re, a2.re, b2.im) * i2);
+    return r;
+}
+DRT_HD void fresnel(MatV<ff> m, ff ieps, ff ct, cx<ff> &rte, cx<ff> &rtm) {
+    const FresnelFF r = fresnel_ff(m, ieps, ct);
+    rte = r.te;
+    rtm = r.tm;
 }
 
 // UTD transition function F(X) = 2j sqrt(X) exp(jX) int_sqrt(X)^inf exp(-j u^2) du for X >= 0,
@@ -814,6 +930,30 @@ template <class T> DRT_OUTLINE cx<T> transition_F_near(T X) {
     const int depth = min(Cfg::n_cf, (int)ceil(T(Cfg::cf_a) + T(Cfg::cf_b) / X));
     for (int k = depth; k >= 1; --k) f = z + cdiv(C<T>(T(0.5) * T(k), T(0)), f);
     return cdiv(pre, f * sqpi);
+}
+
+// F(X) in two-float numbers: the asymptotic series, its terms from the fourth on (below (1 / 2X)^4 105 = 3e-6 from X = 40 on)
+// in FP32; nearer values, rare, in FP64
+DRT_NOINL1 cx<ff> transition_F(ff X) {
+    if (!(X.h > 0.f)) return C<ff>(ff(0.f), ff(0.f));
+    if (X.h < 40.f) {
+        const cx<double> F = transition_F_near<double>(to_double(X));
+        return C<ff>(from_double(F.re), from_double(F.im));
+    }
+    // sum_m (2m - 1)!! (j u)^m, u = 1 / (2 X): Re = 1 - 3 u^2 + 105 u^4 - .., Im = u - 15 u^3 + 945 u^5 - ..
+    const ff u = ff(0.5f) / X, u2 = u * u;
+    float re = 0.f, im = 0.f;
+    // tails in FP32, bottom up: 105 u^4 (1 - 9 11 u^2 (1 - 13 15 u^2 (..))), 945 u^5 (1 - 11 13 u^2 (..))
+    const float w = u2.h;
+    for (int m = 19; m >= 5; m -= 2) {   // terms 2m - 1 = 37 .. 9: ~1e-9 of the tail at X = 40
+        re = 1.f - (2 * m - 1) * (2 * m + 1) * w * re;
+        im = 1.f - (2 * m + 1) * (2 * m + 3) * w * im;
+    }
+    re = 105.f * w * w * re;
+    im = 945.f * w * w * im;
+    // the leading terms: Re = 1 - 3 u^2 + re, Im = u (1 - 15 u^2 + im)
+    const ff r = ff(1.f) + (u2 * -3.f + ff(re));
+    return C<ff>(r, u * (ff(1.f) + (u2 * -15.f + ff(im))));
 }
 
 template <class T> DRT_HD cx<T> transition_F(T X) {
@@ -969,6 +1109,9 @@ template <class T> DRT_HD v3<T> vertical_pol(v3<T> k) {
     return unit(p);
 }
 
+DRT_NOINL1 v3<ff> vertical_pol_ff(v3<ff> k) { return vertical_pol<ff>(k); }
+DRT_HD v3<ff> vertical_pol(v3<ff> k) { return vertical_pol_ff(k); }
+
 // complex amplitude a_p excluding exp(-j k d): (lambda / 4 pi) x ray spreading x polarimetric chain of
 // Fresnel / UTD / ER factors; TX and RX vertically polarised.  seg[1..n+1] are the segment vectors.
 // Spreading and UTD distance parameters per stretch between point sources (TX, tiles, RX), after
@@ -999,7 +1142,7 @@ DRT_HD c3<T> refl_field_inl(c3<T> E, v3<T> kin, v3<T> kout, v3<T> nf, MatV<T> m,
     v3<T> epin = cross(ep, kin), epout = cross(ep, kout);
     cx<T> rte, rtm;
     fresnel(m, ieps, ct, rte, rtm);
-    return cscale(ep, rte * cdot(E, ep) * m.spec) + cscale(epout, rtm * cdot(E, epin) * m.spec);
+    return mix(ep, rte * cdot(E, ep) * m.spec, epout, rtm * cdot(E, epin) * m.spec);
 }
 
 // e: edge direction; t0, n0: the 0-face tangent and normal; wn: wedge n; snp, cnp: sin(n pi), cos(n pi);
@@ -1029,6 +1172,80 @@ DRT_HD c3<T> diff_field_inl(c3<T> E, v3<T> kin, v3<T> kout, v3<T> e, v3<T> t0, v
     return cscale(bv, -(Ds * cdot(E, bpv))) + cscale(ph, -(Dh * cdot(E, php)));
 }
 
+// The same in two-float numbers.  phi and phi' enter the four terms by the sine and cosine of eps / 6 (right-angled wedge) or
+// of eps / 2 and eps / 2n; the numbers N of turns and the distance from a boundary need their FP32 values only.  Within 1e-5 rad
+// of a shadow or reflection boundary the result is NaN: the caller leaves the step to FP64.
+DRT_HD cx<ff> utd_term_ff(float eps, ff sh, ff s2, ff c2, ff kL) {
+    if (fabsf(eps) < 1e-5f) return C<ff>(ff(nanf(""), 0.f), ff(0.f));
+    const cx<ff> F = transition_F(twice(kL) * (sh * sh));
+    const ff cot = c2 / s2;
+    return C<ff>(F.re * cot, F.im * cot);
+}
+DRT_HD c3<ff> diff_field_inl(c3<ff> E, v3<ff> kin, v3<ff> kout, v3<ff> e, v3<ff> t0, v3<ff> n0, ff wn, ff snp, ff cnp,
+                             ff Lf, ff k, ff isk, MatV<ff> m, ff ieps) {
+    const v3<ff> wi = axpy(-kin, e, dot(kin, e)), wo = axpy(kout, e, -dot(kout, e));
+    const ff yi = dot(wi, n0), xi = dot(wi, t0), yo = dot(wo, n0), xo = dot(wo, t0);
+    const ff phip = angle2pi(yi, xi), phi = angle2pi(yo, xo);
+    const v3<ff> eki = cross(e, kin), eko = cross(e, kout);
+    const ff q = dot(eki, eki), rq = rsqrt(q);   // sin^2 b0
+    const ff kL = k * (Lf * q);
+    const bool ra = wn.h == 1.5f && wn.l == 0.f;
+    const ff inv2n = ra ? ff(1.0 / 3.0) : ff(0.5f) / wn;
+    const float tpn = 6.2831853f * wn.h, itpn = 1.f / tpn;
+    cx<ff> t[4];
+    const float bm = phi.h - phip.h, bp = phi.h + phip.h, pi = 3.14159265f;
+    // eps_i = pi + sg_i beta_i - sg_i 2 pi n N_i with (sg, beta) = (+, -), (-, -), (-, +), (+, +)
+    ff sa, ca, sb, cb;
+    if (ra) {
+        sincos_ff(phi * ff(1.0 / 6.0), sa, ca);
+        sincos_ff(phip * ff(1.0 / 6.0), sb, cb);
+    }
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {
+        const float sg = (i == 0 || i == 3) ? 1.f : -1.f, beta = i < 2 ? bm : bp;
+        const float N = sg * rintf((beta + sg * pi) * itpn);
+        const float eps = pi + sg * beta - tpn * N;
+        ff sh, s2, c2;
+        if (ra) {
+            // sin, cos of sg (phi -+ phi') / 6 + pi / 6 - N pi / 2
+            const ff sbi = i < 2 ? -sb : sb;
+            const ff S = fma(sa, cb, ca * sbi), Cq = fma(ca, cb, -(sa * sbi));
+            ff a, b;
+            ra_shift(sg > 0.f ? S : -S, Cq, (int)N, a, b);
+            const ff a2 = a * a;
+            sh = a * (ff(3.f) - ff(4.f * a2.h, 4.f * a2.l));
+            s2 = twice(a * b);
+            c2 = ff(1.f) - twice(a2);
+        } else {
+            const ff bt = i < 2 ? phi - phip : phi + phip;
+            const ff ee = (sg > 0.f ? bt : -bt) + (ff(PI) - (twice(wn) * ff(PI)) * N);
+            ff dummy;
+            sincos_ff(halve(ee), sh, dummy);
+            sincos_ff(ee * inv2n, s2, c2);
+        }
+        t[i] = utd_term_ff(eps, sh, s2, c2, kL);
+    }
+    // (one copy of the Fresnel code for the two faces)
+    cx<ff> r0s = C<ff>(ff(-1.f), ff(0.f)), r0h = C<ff>(ff(1.f), ff(0.f)), rns = r0s, rnh = r0h;
+    if (!m.pec) {
+        const ff ri2 = fma(xi, xi, yi * yi), ro2 = fma(xo, xo, yo * yo);
+        const FresnelFF f0 = fresnel_ff(m, ieps, fabs(yi) * rsqrt(ri2));
+        const FresnelFF fn = fresnel_ff(m, ieps, fabs(det2(snp, xo, cnp, yo)) * rsqrt(ro2));
+        r0s = f0.te;
+        r0h = f0.tm;
+        rns = fn.te;
+        rnh = fn.tm;
+    }
+    const cx<ff> base = t[0] + t[1];
+    // C = -exp(-j pi/4) / (2 n sqrt(2 pi k) sin b0)
+    const ff pref = inv2n * isk * rq * ff(0.70710678118654752440);
+    const cx<ff> Cc = C<ff>(-pref, pref);
+    const cx<ff> Ds = Cc * (base + r0s * t[2] + rns * t[3]), Dh = Cc * (base + r0h * t[2] + rnh * t[3]);
+    const v3<ff> php = eki * (-rq), bpv = cross(php, kin);
+    const v3<ff> ph = eko * rsqrt(dot(eko, eko)), bv = cross(ph, kout);
+    return mix(bv, -(Ds * cdot(E, bpv)), ph, -(Dh * cdot(E, php)));
+}
+
 template <class T>
 DRT_HD c3<T> tile_field_inl(c3<T> E, v3<T> kin, v3<T> kout, v3<T> nt, TileV<T> tl) {
     if (dot(nt, kin) > T(0)) nt = -nt;
@@ -1053,7 +1270,6 @@ DRT_HD c3<T> tile_field_inl(c3<T> E, v3<T> kin, v3<T> kout, v3<T> nt, TileV<T> t
     return cscale(Ep, ph * amp);
 }
 
-#define DRT_NOINL __host__ __device__ __noinline__
 template <class T> DRT_NOINL c3<T> refl_field_out(c3<T> E, v3<T> kin, v3<T> kout, v3<T> nf, MatV<T> m, T ieps) {
     return refl_field_inl(E, kin, kout, nf, m, ieps);
 }
@@ -1066,10 +1282,19 @@ template <class T> DRT_NOINL c3<T> tile_field_out(c3<T> E, v3<T> kin, v3<T> kout
     return tile_field_inl(E, kin, kout, nt, tl);
 }
 
+// per-call constants of the field: wavenumber k, 1 / sqrt(2 pi k), 1 / (2 pi f eps0), lambda / (4 pi)
+template <class T> struct FieldK { T k, isk, ieps, lam; };
+template <class T> DRT_HD FieldK<T> field_k(const FreqGridD &fg) {   // one division
+    const T fc = std::is_same<T, float>::value ? T(fg.fcf) : T(fg.fc);
+    const T ifc = T(1) / fc, k = fc * T(2 * PI / C0);
+    return {k, rsqrt(T(2 * PI) * k), ifc * T(1 / (2 * PI * EPS0)), ifc * T(C0 / (4 * PI))};
+}
+template <> DRT_HD FieldK<ff> field_k<ff>(const FreqGridD &fg) { return {fg.kq, fg.iskq, fg.iepsq, fg.lamq}; }
+
+// unit directions kd of the segments, per diffraction its distance parameter over sin^2 b0, and the ray spreading squared
 template <int N = -1, class S, class T = typename ST<S>::R>
-DRT_HD cx<T> amplitude(const LinkDev &L, const Prim<S> *pr, int n, const v3<T> *seg, T fc) {
+DRT_HD void field_spread(const Prim<S> *pr, int n, const v3<T> *seg, v3<T> *kd, T *Lfac, T &sp_num, T &sp_den) {
     const int nv = N >= 0 ? N : n;
-    v3<T> kd[MAXI + 2];
     T len[MAXI + 2];
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI + 1; ++i) {
@@ -1097,7 +1322,7 @@ DRT_HD cx<T> amplitude(const LinkDev &L, const Prim<S> *pr, int n, const v3<T> *
     }
     // spreading and, per diffraction, L / sin^2 b0
     // spread^2 = sp_num / sp_den, one square root per call
-    T sp_num = T(1), sp_den = T(1), Lfac[MAXI + 1];
+    sp_num = sp_den = T(1);
     {
         T d = T(0), re = T(0);          // distance since the point source or latest diffraction; its rho_e
         bool after_d = false;
@@ -1147,10 +1372,16 @@ DRT_HD cx<T> amplitude(const LinkDev &L, const Prim<S> *pr, int n, const v3<T> *
             d = T(0);
         }
     }
-    // one division per call: the wavenumber, eps_c = eps_r - j sigma ieps and lambda / (4 pi) from 1/fc
-    const T ifc = T(1) / fc;
-    const T k = fc * T(2 * PI / C0), isk = rsqrt(T(2 * PI) * k);
-    const T ieps = ifc * T(1 / (2 * PI * EPS0));
+}
+
+template <int N = -1, class S, class T = typename ST<S>::R>
+DRT_HD cx<T> amplitude(const LinkDev &L, const Prim<S> *pr, int n, const v3<T> *seg, const FreqGridD &fg) {
+    const int nv = N >= 0 ? N : n;
+    v3<T> kd[MAXI + 2];
+    T sp_num, sp_den, Lfac[MAXI + 1];
+    field_spread<N>(pr, n, seg, kd, Lfac, sp_num, sp_den);
+    const FieldK<T> fk = field_k<T>(fg);
+    const T k = fk.k, isk = fk.isk, ieps = fk.ieps;
     c3<T> E = cscale(vertical_pol(kd[1]), C<T>(T(1), T(0)));
     v3<T> klast = kd[1];
 #pragma unroll (N >= 0 ? 8 : 1)
@@ -1176,7 +1407,7 @@ DRT_HD cx<T> amplitude(const LinkDev &L, const Prim<S> *pr, int n, const v3<T> *
         }
     }
     const T spread = sqrt(sp_num / sp_den);
-    return cdot(E, vertical_pol(klast)) * (ifc * T(C0 / (4 * PI)) * spread);
+    return cdot(E, vertical_pol(klast)) * (fk.lam * spread);
 }
 
 // App. A Eq. doppler_freq: f' = f0 prod_i (c - v_i.k_i) / (c - v_{i-1}.k_i), evaluated without
@@ -1354,7 +1585,7 @@ DRT_HD void path_step_fp64_core(const LinkDev &L, const TimeGridD &tg, const Fre
     // are computed only when the caller asked for the amplitude output, which reports them for every
     // step (a degenerate chain has none)
     const bool field = !fl || (OUT && out.amp && !(fl & F_DEGEN));
-    cx<T> a = field ? amplitude<N>(L, pr, n, seg, T(fg.fc)) : C<T>(T(0), T(0));
+    cx<T> a = field ? amplitude<N>(L, pr, n, seg, fg) : C<T>(T(0), T(0));
     if constexpr (OUT) {
         if (out.tau || out.amp || out.doppler || out.angles || out.flags || out.points) {
             T fd = 0;
@@ -1989,7 +2220,7 @@ DRT_HD bool bulk_eval(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg
     }
     // as in the FP64 form: an invalid step's field coefficients only for the amplitude output
     const bool field = !fl || (OUT && out.amp && !(fl & F_DEGEN));
-    cx<T> a = field ? amplitude<N>(L, pr, n, seg, fg.fcf) : C<T>(T(0), T(0));
+    cx<T> a = field ? amplitude<N>(L, pr, n, seg, fg) : C<T>(T(0), T(0));
     if constexpr (OUT) {
         if (out.tau || out.amp || out.doppler || out.angles || out.flags || out.points) {
             T fd = 0.f;
@@ -2012,7 +2243,7 @@ DRT_HD bool bulk_eval(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg
     };
     phase_record(fg, B, a, rec);
     if (fg2) {
-        const cx<T> a2 = field ? amplitude<N>(L, pr, n, seg, fg2->fcf) : C<T>(T(0), T(0));
+        const cx<T> a2 = field ? amplitude<N>(L, pr, n, seg, *fg2) : C<T>(T(0), T(0));
         phase_record(*fg2, ld_row(R.base2[(size_t)(chunk - R.c0) * R.bstride]), a2, *rec2);
     }
     return true;
