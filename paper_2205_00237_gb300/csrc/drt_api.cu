@@ -307,15 +307,6 @@ Link *find_link(drt_ctx *c, uint64_t id) {
 TimeGridD tgd(const drt_time_grid *g, int chunk = 16) { return make_tgrid(g->t_start, g->dt, g->n_steps, chunk); }
 FreqGridD fgd(const drt_freq_grid *g) { return make_fgrid(g->fc, g->bandwidth, g->n_bins); }
 
-// Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
-// is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
-// as checked at load.  Beyond that the records are computed in FP64.
-bool ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
-    const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
-    const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T);
-    return v.ff_range && reach * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
-}
-
 // bracket one launch with events when tracing is on
 template <class F> drt_status traced(drt_ctx *c, int kind, cudaStream_t s, F &&launch) {
     if (!c->profiling) {
@@ -355,20 +346,21 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
         // which so do not wait for the warm starts; s joins side[1] at the end.
         cudaStream_t sa = c->side[0], sw = c->side[1];
         const int nb = L.dev.n_bulk;
+        const bool two = ff_applies(L.view, *tg, *fg);
         cudaEvent_t ev_p64 = c->ev_aux[0], ev_base0 = c->ev_aux[1], ev_pb = c->ev_aux[2];
         CUDA_TRY(cudaMemsetAsync(rd, 0, sizeof(int), s));   // the redo counter, before any kernel that queues
         CUDA_TRY(cudaEventRecord(c->ev_fork, s));
         CUDA_TRY(cudaStreamWaitEvent(sa, c->ev_fork, 0));
         CUDA_TRY(cudaStreamWaitEvent(sw, c->ev_fork, 0));
-        if (drt_status st = traced(c, 3, sw, [&] { return launch_warm_fp64(L.dev, t, warm, sw); })) return st;
-        if (drt_status st = traced(c, 3, sa, [&] { return launch_base_pose64(L.dev, t, p64, sa); })) return st;
+        if (drt_status st = traced(c, 3, sw, [&] { return launch_warm_fp64(L.dev, t, warm, sw, two); })) return st;
+        if (drt_status st = traced(c, 3, sa, [&] { return launch_base_pose64(L.dev, t, p64, sa, two); })) return st;
         CUDA_TRY(cudaEventRecord(ev_p64, sa));
-        if (drt_status st = traced(c, 3, sa, [&] { return launch_base_paths(L.dev, t, f, p64, bs, warm, 0, nb, sa); }))
+        if (drt_status st = traced(c, 3, sa, [&] { return launch_base_paths(L.dev, t, f, p64, bs, warm, 0, nb, sa, two); }))
             return st;
         CUDA_TRY(cudaEventRecord(ev_base0, sa));
         CUDA_TRY(cudaStreamWaitEvent(sw, ev_p64, 0));
         if (drt_status st = traced(c, 3, sw, [&] {
-                return launch_base_paths(L.dev, t, f, p64, bs, warm, nb, L.dev.n_paths, sw);
+                return launch_base_paths(L.dev, t, f, p64, bs, warm, nb, L.dev.n_paths, sw, two);
             }))
             return st;
         if (drt_status st = traced(c, 0, s, [&] { return launch_pose_bulk(L.dev, t, pb, s); })) return st;
@@ -387,7 +379,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
             }))
             return st;
         if (!defer_redo)   // else the caller runs the redo beside the synthesis (synth_into)
-            if (drt_status st = traced(c, 3, s, [&] { return launch_redo(L.dev, t, f, out, rec, rd, warm, s); }))
+            if (drt_status st = traced(c, 3, s, [&] { return launch_redo(L.dev, t, f, out, rd, warm, s, two); }))
                 return st;
         return DRT_OK;
     }
@@ -407,7 +399,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
             cudaError_t e = cudaEventRecord(c->ev_fork, s);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, c->ev_fork, 0);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s1, c->ev_fork, 0);
-            if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1);
+            if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1, true);
             if (e == cudaSuccess) e = launch_extrapolate_ff_generic(D, t, f, pose, rec, warm, s1);
             if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 2, warm, s0);
             if (e == cudaSuccess) e = launch_extrapolate_ff(D, t, f, pose, rec, 0, warm, s0);
@@ -433,7 +425,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
         cudaError_t e = cudaEventRecord(c->ev_fork, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, c->ev_fork, 0);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s1, c->ev_fork, 0);
-        if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1);
+        if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1, ff_applies(L.view, *tg, *fg));
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s1, ls[MAXI], -1, false, warm);
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s1, ls[1], ls[2], false, warm);
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s0, ls[2], ls[3], false, warm);
@@ -462,13 +454,14 @@ drt_status synth_into(drt_ctx *c, Link &L, const drt_time_grid *tg, const drt_fr
         if (drt_status st = ensure(c, c->redo3, (size_t)L.n_paths * tg->n_steps * 3 * sizeof(double) + 8)) return st;
         if (drt_status st = run_extrapolation(c, L, tg, fg, none, rec, precision, s, true)) return st;
         double *r3 = reinterpret_cast<double *>(c->redo3.ptr);
+        const bool two = ff_applies(L.view, *tg, *fg);
         void *rd = c->redo.ptr;
         const double *warm = reinterpret_cast<const double *>(c->warm.ptr);
         if (wm) CUDA_TRY(launch_select(L.dev, t, f, *wm, warm, s));
         cudaStream_t sb = c->side[1];
         CUDA_TRY(cudaEventRecord(c->ev_fork, s));
         CUDA_TRY(cudaStreamWaitEvent(sb, c->ev_fork, 0));
-        if (drt_status st = traced(c, 3, sb, [&] { return launch_redo_rec(L.dev, t, f, rd, warm, r3, sb); })) return st;
+        if (drt_status st = traced(c, 3, sb, [&] { return launch_redo_rec(L.dev, t, f, rd, warm, r3, sb, two); })) return st;
         if (wm) CUDA_TRY(launch_redo_window_mask(L.dev, t, rd, *wm, r3, sb));
         CUDA_TRY(cudaEventRecord(c->ev_join[1], sb));
         if (wm) CUDA_TRY(launch_window_mask(L.dev, t, rec, *wm, s));
@@ -485,6 +478,15 @@ drt_status synth_into(drt_ctx *c, Link &L, const drt_time_grid *tg, const drt_fr
 }
 
 }  // namespace
+
+// Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
+// is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
+// as checked at load.  Beyond that the records are computed in FP64.
+bool drt::ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
+    const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
+    const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T);
+    return v.ff_range && reach * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
+}
 
 // validated host-side structure-of-arrays image of one link (device pointers unset)
 drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink &H) {
@@ -644,6 +646,13 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
         h.alpha = (int32_t)g.alpha;
         h.mat = g.mat;
         h.pad = 0;
+    }
+    for (int k = 0; k < 2; ++k) {
+        const drt_terminal &m = k ? s->rx : s->tx;
+        TermQ &h = k ? d.rxq : d.txq;
+        q3(h.r, m.r);
+        q3(h.v, m.v);
+        q3(h.a, m.a);
     }
     H.bodiesQ.resize(s->n_bodies);
     for (int i = 0; i < s->n_bodies; ++i) {
@@ -896,7 +905,8 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     img.add(t0par, &d.t0par);
     drt_status st = img.upload(c, L);
     if (!st && n_t0) {
-        cudaError_t e = launch_t0par(d, const_cast<double *>(d.t0par), 0);
+        // at t = 0, whatever the grids of later calls: edge parameters only (1e-6 m is enough of a start)
+        cudaError_t e = launch_t0par(d, const_cast<double *>(d.t0par), 0, L.view.ff_range && L.view.extent < 1e5);
         if (e == cudaSuccess) e = cudaStreamSynchronize(0);
         if (e != cudaSuccess) st = fail(DRT_ECUDA, "t0 edge parameters: %s", cudaGetErrorString(e));
     }
@@ -1343,7 +1353,7 @@ extern "C" drt_status drt_synthesize_H_noalloc(drt_ctx *c, uint64_t link, const 
     // the same launches as drt_synthesize_H's FP64 form: pose table, multi-diffraction warm starts,
     // extrapolation into the records, synthesis
     CUDA_TRY(launch_pose(L->dev, t, pose, s));
-    CUDA_TRY(launch_warm_fp64(L->dev, t, warm, s));
+    CUDA_TRY(launch_warm_fp64(L->dev, t, warm, s, false));
     CUDA_TRY(launch_extrapolate_fp64(L->dev, t, f, pose, none, rec, s, 0, -1, false, warm));
     CUDA_TRY(launch_synth(rec, L->n_paths, t, f, reinterpret_cast<float2 *>(H), s));
     return DRT_OK;

@@ -110,6 +110,7 @@ struct BatchPlan {
     bool dual = false;  // some link asks for Doppler outputs: carry the rates
     bool any_out = false;   // some link asks for per-path-step records (all units then run generic code)
     bool any_pair = false;  // some entries form carrier pairs
+    bool two = true;        // two-float numbers apply to every link and grid
     int synth_run = 1;      // items in turn per synthesis block (see k_batch_synth)
     cudaGraphExec_t graph = nullptr;
     cudaStream_t capture = nullptr;   // private stream the graph is captured on (any caller stream,
@@ -134,6 +135,7 @@ static BatchDev dev_view(const BatchPlan &P, int l0, int l1, long long n_items, 
     B.counter = reinterpret_cast<unsigned long long *>(P.mem) + k;
     B.rec_a = reinterpret_cast<float4 *>(P.mem + P.off_rec);
     B.rec_b = reinterpret_cast<float *>(P.mem + P.off_rec + P.rec_count * sizeof(float4));
+    B.two = P.two;
     B.synth_run = P.synth_run;
     B.redo.count = reinterpret_cast<int *>(P.mem + P.off_redo);
     B.redo.items = reinterpret_cast<int4 *>(P.mem + P.off_redo + 256);
@@ -252,6 +254,7 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
     const int n = (int)links.size();
     BatchPlan *P = new BatchPlan();
     P->n_links = n;
+    for (int i = 0; i < n; ++i) P->two = P->two && ff_applies(views[i], tgs[i], fgs[i]);
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
     // largest links first: their units are claimed first

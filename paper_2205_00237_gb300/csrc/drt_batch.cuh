@@ -51,6 +51,7 @@ struct BatchDev {
     unsigned long long *counter;
     float4 *rec_a;
     float *rec_b;
+    bool two;            // two-float numbers apply to every link and grid of the batch (ff_applies)
     int synth_run;       // items a synthesis block (or, in small links, each of its warps) takes in turn
     RedoList redo;   // items (link, path, step)
 };

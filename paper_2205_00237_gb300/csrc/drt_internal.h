@@ -34,6 +34,7 @@ struct FaceQ { ff c[3], n[3], u[3], hu, hw; int32_t body, mat; };
 struct EdgeQ { ff a[3], e[3], t0[3], n0[3], len, wn, snp, cnp; int32_t body, mat; };
 struct TileQ { ff c[3], n[3], area, s, cph, sph; int32_t alpha, body, mat, pad; };
 struct BodyQ { ff o[3], v[3], a[3], k[3], w0, wdot; };
+struct TermQ { ff r[3], v[3], a[3]; };
 struct TermD { double r[3], v[3], a[3]; };
 struct BodyD { double o[3], v[3], a[3], k[3], w0, wdot; };
 
@@ -62,6 +63,7 @@ struct LinkDev {
     const EdgeQ *edgesQ;
     const TileQ *tilesQ;
     const BodyQ *bodiesQ;
+    TermQ txq, rxq;
     // paths in internal (signature-sorted) order
     const uint32_t *ptypes;   // byte j = type of vertex j (0 past the chain)
     const int4 *pprims;       // primitive index of vertex j
@@ -136,6 +138,7 @@ struct RecD { float4 *rec_a; float *rec_b; };
 // translation speed (m/s), largest acceleration (m/s^2), largest angular speed (rad/s)
 // and extent, the largest coordinate at t0 (m); ff_range: every length and material constant lies in the range of the two-float form
 struct drt_scene_view { double vmax, amax, wmax, extent; bool ff_range; };
+bool ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg);
 
 // a10 batch plans (drt_batch.cu)
 struct BatchPlan;
@@ -225,8 +228,9 @@ cudaError_t launch_extrapolate_ff_generic(const LinkDev &L, const TimeGridD &tg,
                                           const RecD &rec, const double *warm, cudaStream_t s);
 // the warm-start table of the multi-diffraction chains (FP64 dual-number solves at the chunk bases)
 // edge parameters and rates at t = 0 of the multi-diffraction paths (LinkDev::t0par), at load
-cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s);
-cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s);
+// two: in two-float numbers (the caller has checked that they apply), here and below
+cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s, bool two);
+cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two);
 // FP32-bulk form (CHUNK consecutive steps share FP64 anchors); see drt_physics.cuh.  Scratch:
 // per-(body or terminal, chunk) FP32 base poses and per-(path, chunk) FP64 anchors.
 size_t bulk_pose_bytes(const LinkDev &L, const TimeGridD &tg);
@@ -236,9 +240,9 @@ size_t bulk_pose64_bytes(const LinkDev &L, const TimeGridD &tg);
 size_t bulk_redo_bytes(const LinkDev &L, const TimeGridD &tg);
 // FP32-bulk anchors in parts: FP64 poses at the chunk bases, then the anchors of paths [p0, p1) (the
 // multi-diffraction paths [n_bulk, n_paths) need their warm starts, launch_warm_fp64, first)
-cudaError_t launch_base_pose64(const LinkDev &L, const TimeGridD &tg, double *pose64, cudaStream_t s);
+cudaError_t launch_base_pose64(const LinkDev &L, const TimeGridD &tg, double *pose64, cudaStream_t s, bool two);
 cudaError_t launch_base_paths(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const double *pose64,
-                              void *base, const double *warm, int p0, int p1, cudaStream_t s);
+                              void *base, const double *warm, int p0, int p1, cudaStream_t s, bool two);
 // the redo scratch holds an int counter (zeroed here, on s, when zero is set) followed by the
 // (path, step) list; lengths / generic select the launches of chain lengths 0..3 (on s) and of the
 // generic range (on s_multi, else s)
@@ -246,12 +250,12 @@ cudaError_t launch_extrapolate_bulk(const LinkDev &L, const TimeGridD &tg, const
                                     const void *base, const double *warm, const OutD &out, const RecD &rec,
                                     void *redo, cudaStream_t s, cudaStream_t s_multi = nullptr, bool lengths = true,
                                     bool generic = true, bool zero = true);
-cudaError_t launch_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, const RecD &rec,
-                        void *redo, const double *warm, cudaStream_t s);
+cudaError_t launch_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, void *redo,
+                        const double *warm, cudaStream_t s, bool two);
 // the redo for an H synthesis: (Re a, Im a, tau) per queued step into out3 ([cap][3] doubles), then
 // added into H after the synthesis
 cudaError_t launch_redo_rec(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, void *redo, const double *warm,
-                            double *out3, cudaStream_t s);
+                            double *out3, cudaStream_t s, bool two);
 cudaError_t launch_redo_add(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, void *redo, const double *in3,
                             float2 *H, cudaStream_t s, int ld = -1);
 // multipath lifetime: per-instant total |a|^2 of the valid paths (tot[T]) and major validity changes

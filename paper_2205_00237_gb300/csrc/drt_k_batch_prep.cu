@@ -2,11 +2,12 @@
 // multi-diffraction warm starts and FP64 chunk anchors, each a persistent launch over its
 // (link, item) list.
 #include "drt_batch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
-// stages 0-3: block-wide claims of blockDim.x consecutive items
-template <int STAGE>
+// stages 0-3: block-wide claims of blockDim.x consecutive items; TWO: stages 1-3 in two-float numbers (PoseQ rows)
+template <int STAGE, bool TWO>
 __global__ void __launch_bounds__(128) k_stage(const BatchDev B) {
     __shared__ long long s_start;
     const long long total = B.n_items;
@@ -30,25 +31,33 @@ __global__ void __launch_bounds__(128) k_stage(const BatchDev B) {
             else terminal_base(b == BL.L.n_bodies ? BL.L.tx : BL.L.rx, tb, BL.poseb[local]);
         } else if (STAGE == ST_POSE64) {
             int b = (int)(local / nch), c = (int)(local - (long long)b * nch);
-            body_pose_row(BL.L.bodies[b], BL.tg.t_start + (double)c * BL.tg.chunk * BL.tg.dt,
-                          BL.pose64 + local * POSE_W);
+            const double tb = BL.tg.t_start + (double)c * BL.tg.chunk * BL.tg.dt;
+            if constexpr (TWO) body_pose_ff(BL.L.bodiesQ[b], from_double(tb), reinterpret_cast<PoseQ *>(BL.pose64)[local]);
+            else body_pose_row(BL.L.bodies[b], tb, BL.pose64 + local * POSE_W);
         } else if (STAGE == ST_WARM) {   // rows 0..nch
             int p = BL.L.n_bulk + (int)(local / (nch + 1)), c = (int)(local % (nch + 1));
-            path_warm_fp64(BL.L, BL.tg, p, c, BL.warm);
+            if constexpr (TWO) path_warm_ff(BL.L, BL.tg, p, c, BL.warm);
+            else path_warm_fp64(BL.L, BL.tg, p, c, BL.warm);
         } else {
             int p = (int)(local / nch), c = (int)(local % nch);
-            path_base_fp64(BL.L, BL.tg, BL.fg, BL.pose64, p, c, BL.base, BL.warm);
+            if constexpr (TWO)
+                path_base_ff(BL.L, BL.tg, BL.fg, reinterpret_cast<const PoseQ *>(BL.pose64), p, c, BL.base, BL.warm);
+            else path_base_fp64(BL.L, BL.tg, BL.fg, BL.pose64, p, c, BL.base, BL.warm);
         }
     }
 }
 
-cudaError_t launch_batch_stage(int stage, const BatchDev &B, int grid, cudaStream_t s) {
+template <bool TWO> static void launch_stage(int stage, const BatchDev &B, int grid, cudaStream_t s) {
     switch (stage) {
-    case ST_POSEB: k_stage<ST_POSEB><<<grid, 128, 0, s>>>(B); break;
-    case ST_POSE64: k_stage<ST_POSE64><<<grid, 128, 0, s>>>(B); break;
-    case ST_WARM: k_stage<ST_WARM><<<grid, 128, 0, s>>>(B); break;
-    default: k_stage<ST_BASE><<<grid, 128, 0, s>>>(B); break;
+    case ST_POSEB: k_stage<ST_POSEB, false><<<grid, 128, 0, s>>>(B); break;
+    case ST_POSE64: k_stage<ST_POSE64, TWO><<<grid, 128, 0, s>>>(B); break;
+    case ST_WARM: k_stage<ST_WARM, TWO><<<grid, 128, 0, s>>>(B); break;
+    default: k_stage<ST_BASE, TWO><<<grid, 128, 0, s>>>(B); break;
     }
+}
+cudaError_t launch_batch_stage(int stage, const BatchDev &B, int grid, cudaStream_t s) {
+    if (B.two) launch_stage<true>(stage, B, grid, s);
+    else launch_stage<false>(stage, B, grid, s);
     return cudaGetLastError();
 }
 

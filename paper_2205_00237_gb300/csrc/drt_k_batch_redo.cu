@@ -2,16 +2,16 @@
 // in FP64 and its contribution added to H.  Compiled twice: values only, and (drt_k_batch_redo_dual.cu,
 // DRT_BATCH_REDO_DUAL) with the rates the Doppler output needs.
 #include "drt_batch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
 // FP64 redo of queued steps; their contribution is added to H (all bins) with atomics, for the entry
 // and, for a carrier pair, its partner
 template <bool DUAL>
-__device__ void redo_add_entry(const BatchLink &BL, int p, int ti) {
+__device__ void redo_add_entry(const BatchLink &BL, int p, int ti, bool two) {
     double r[3];
-    const RecD nor{nullptr, nullptr};
-    path_step_redo_as<DUAL>(BL.L, BL.tg, BL.fg, p, ti, BL.out, nor, BL.warm, r);
+    path_step_redo<DUAL>(BL.L, BL.tg, BL.fg, p, ti, BL.out, BL.warm, r, two);
     if (r[0] == 0.0 && r[1] == 0.0) return;
     // a exp(-j 2 pi f_k tau): FP64-reduced seed per 16-bin tile, FP32 rotation across the tile
     const double f0 = BL.fg.f0, df = BL.fg.df;
@@ -55,8 +55,8 @@ __global__ void __launch_bounds__(32) k_batch_redo(const BatchDev B) {   // one 
         const int4 itm = B.redo.items[k];
         const BatchLink &BL = B.links[itm.x];
         if (!one && chain_length(BL.L, itm.y) != (int)blockIdx.y) continue;
-        redo_add_entry<DUAL>(BL, itm.y, itm.z);
-        if (BL.partner >= 0 && itm.y >= BL.pair_p0) redo_add_entry<DUAL>(B.links[BL.partner], itm.y, itm.z);
+        redo_add_entry<DUAL>(BL, itm.y, itm.z, B.two);
+        if (BL.partner >= 0 && itm.y >= BL.pair_p0) redo_add_entry<DUAL>(B.links[BL.partner], itm.y, itm.z, B.two);
     }
 }
 

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "drt_launch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
@@ -29,6 +30,14 @@ k_warm_fp64(const LinkDev L, const TimeGridD tg, double *__restrict__ warm) {
     if (p >= L.n_paths || c > n_chunks_of(tg)) return;   // rows 0..n_chunks
     path_warm_fp64(L, tg, p, c, warm);
 }
+// the same in two-float numbers
+__global__ void __launch_bounds__(WARM_T)
+k_warm_ff(const __grid_constant__ LinkDev L, const TimeGridD tg, double *__restrict__ warm) {
+    int p = L.n_bulk + blockIdx.x;
+    int c = blockIdx.y * WARM_T + threadIdx.x;
+    if (p >= L.n_paths || c > n_chunks_of(tg)) return;
+    path_warm_ff(L, tg, p, c, warm);
+}
 
 // one path per warp (lane 0): the chains' lengths differ, and each length is its own code instance
 __global__ void __launch_bounds__(32) k_t0par(const LinkDev L, double *__restrict__ t0par) {
@@ -37,17 +46,25 @@ __global__ void __launch_bounds__(32) k_t0par(const LinkDev L, double *__restric
     path_t0par_fp64(L, p, t0par + (size_t)(p - L.n_bulk) * (2 * MAXI));
 }
 
-cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s) {
+__global__ void __launch_bounds__(32) k_t0par_ff(const __grid_constant__ LinkDev L, double *__restrict__ t0par) {
+    const int p = L.n_bulk + blockIdx.x;
+    if (threadIdx.x != 0 || p >= L.n_paths) return;
+    path_t0par_ff(L, p, t0par + (size_t)(p - L.n_bulk) * (2 * MAXI));
+}
+
+cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s, bool two) {
     const int n = L.n_paths - L.n_bulk;
     if (n <= 0) return cudaSuccess;
-    k_t0par<<<n, 32, 0, s>>>(L, t0par);
+    if (two) k_t0par_ff<<<n, 32, 0, s>>>(L, t0par);
+    else k_t0par<<<n, 32, 0, s>>>(L, t0par);
     return cudaGetLastError();
 }
 
-cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s) {
+cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two) {
     if (!warm || L.n_bulk >= L.n_paths || tg.n_steps == 0) return cudaSuccess;
     dim3 gw(L.n_paths - L.n_bulk, (n_chunks_of(tg) + 1 + WARM_T - 1) / WARM_T);
-    k_warm_fp64<<<gw, WARM_T, 0, s>>>(L, tg, warm);
+    if (two) k_warm_ff<<<gw, WARM_T, 0, s>>>(L, tg, warm);
+    else k_warm_fp64<<<gw, WARM_T, 0, s>>>(L, tg, warm);
     return cudaGetLastError();
 }
 

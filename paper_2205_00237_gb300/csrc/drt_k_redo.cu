@@ -1,6 +1,7 @@
 // drt_k_redo.cu -- the FP64 redo of the FP32-bulk path-steps that FP32 cannot resolve, beside the
 // synthesis, with their contributions added to H afterwards (the records form is in drt_k_redo_out.cu).
 #include "drt_launch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
@@ -11,23 +12,22 @@ namespace drt {
 // share a warp, so none waits for another's branches.  Otherwise grid row y takes the steps of chains
 // of length y (each length is its own code instance, which lanes of one warp would run in turn).
 __global__ void __launch_bounds__(32)
-k_redo_rec(const LinkDev L, const TimeGridD tg, const FreqGridD fg, const RedoList redo, const double *__restrict__ warm,
-           double *__restrict__ out3) {
+k_redo_rec(const __grid_constant__ LinkDev L, const __grid_constant__ TimeGridD tg, const __grid_constant__ FreqGridD fg,
+           const RedoList redo, const double *__restrict__ warm, double *__restrict__ out3, bool two) {
     const int n = min(*redo.count, redo.cap);
     const OutD none{};
-    const RecD nor{nullptr, nullptr};
     const int warp = blockIdx.y * gridDim.x + blockIdx.x;
     if (n <= (int)(gridDim.x * gridDim.y)) {
         if (threadIdx.x == 0 && warp < n) {
             const int4 it = redo.items[warp];
-            path_step_redo_as<false>(L, tg, fg, it.y, it.z, none, nor, warm, out3 + 3 * (size_t)warp);
+            path_step_redo<false>(L, tg, fg, it.y, it.z, none, warm, out3 + 3 * (size_t)warp, two);
         }
         return;
     }
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int4 it = redo.items[k];
         if (chain_length(L, it.y) != (int)blockIdx.y) continue;
-        path_step_redo_as<false>(L, tg, fg, it.y, it.z, none, nor, warm, out3 + 3 * (size_t)k);
+        path_step_redo<false>(L, tg, fg, it.y, it.z, none, warm, out3 + 3 * (size_t)k, two);
     }
 }
 
@@ -59,9 +59,9 @@ k_redo_add(const FreqGridD fg, const RedoList redo, const double *__restrict__ i
 }
 
 cudaError_t launch_redo_rec(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, void *redo, const double *warm,
-                            double *out3, cudaStream_t s) {
+                            double *out3, cudaStream_t s, bool two) {
     if (L.n_paths == 0 || tg.n_steps == 0) return cudaSuccess;
-    k_redo_rec<<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, redo_list(redo, L, tg), warm, out3);
+    k_redo_rec<<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, redo_list(redo, L, tg), warm, out3, two);
     return cudaGetLastError();
 }
 

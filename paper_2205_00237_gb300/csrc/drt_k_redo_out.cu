@@ -1,6 +1,7 @@
 // drt_k_redo_out.cu -- the FP64 redo of the FP32-bulk path-steps that FP32 cannot resolve, written in
 // place into the caller's per-path-step outputs and records.
 #include "drt_launch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
@@ -9,33 +10,41 @@ namespace drt {
 // chains of length y (one code instance per length: a warp runs one of them)
 template <bool DUAL>
 __global__ void __launch_bounds__(32)
-k_redo(const LinkDev L, const TimeGridD tg, const FreqGridD fg, const OutD out, const RecD rec, const RedoList redo,
-       const double *__restrict__ warm) {
+k_redo(const __grid_constant__ LinkDev L, const __grid_constant__ TimeGridD tg, const __grid_constant__ FreqGridD fg,
+       const OutD out, const RedoList redo, const double *__restrict__ warm, bool two) {
     int n = min(*redo.count, redo.cap);
     const int warp = blockIdx.y * gridDim.x + blockIdx.x;
     if (n <= (int)(gridDim.x * gridDim.y)) {   // few queued steps: one per warp (see k_redo_rec)
         if (threadIdx.x == 0 && warp < n) {
             const int4 it = redo.items[warp];
-            if constexpr (DUAL) path_step_redo_as<true>(L, tg, fg, it.y, it.z, out, rec, warm);
-            else path_step_redo_as<false>(L, tg, fg, it.y, it.z, out, rec, warm);
+            path_step_redo<DUAL>(L, tg, fg, it.y, it.z, out, warm, nullptr, two);
         }
         return;
     }
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const int4 it = redo.items[k];
         if (chain_length(L, it.y) != (int)blockIdx.y) continue;
-        if constexpr (DUAL) path_step_redo_as<true>(L, tg, fg, it.y, it.z, out, rec, warm);
-        else path_step_redo_as<false>(L, tg, fg, it.y, it.z, out, rec, warm);
+        path_step_redo<DUAL>(L, tg, fg, it.y, it.z, out, warm, nullptr, two);
     }
 }
 
-cudaError_t launch_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, const RecD &rec,
-                        void *redo, const double *warm, cudaStream_t s) {
-    if (L.n_paths == 0 || tg.n_steps == 0) return cudaSuccess;
-    const dim3 grid(152 * 4, MAXI + 1);
-    if (out.doppler) k_redo<true><<<grid, 32, 0, s>>>(L, tg, fg, out, rec, redo_list(redo, L, tg), warm);
-    else k_redo<false><<<grid, 32, 0, s>>>(L, tg, fg, out, rec, redo_list(redo, L, tg), warm);
+#ifdef DRT_REDO_DUAL   // drt_k_redo_out_dual.cu: with the rates the Doppler output needs
+cudaError_t launch_redo_dual(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, void *redo,
+                             const double *warm, cudaStream_t s, bool two) {
+    k_redo<true><<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
     return cudaGetLastError();
 }
+#else
+cudaError_t launch_redo_dual(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, void *redo,
+                             const double *warm, cudaStream_t s, bool two);
+
+cudaError_t launch_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, void *redo,
+                        const double *warm, cudaStream_t s, bool two) {
+    if (L.n_paths == 0 || tg.n_steps == 0) return cudaSuccess;
+    if (out.doppler) return launch_redo_dual(L, tg, fg, out, redo, warm, s, two);
+    k_redo<false><<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
+    return cudaGetLastError();
+}
+#endif
 
 }  // namespace drt

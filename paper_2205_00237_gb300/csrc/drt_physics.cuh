@@ -281,6 +281,9 @@ template <> DRT_HD void clamp_positive<float>(float &x, float eps) {
 template <> DRT_HD void clamp_positive<ff>(ff &x, ff eps) {
     if (!(x > eps)) x = eps;
 }
+template <> DRT_HD void clamp_positive<dl<ff>>(dl<ff> &x, ff eps) {
+    if (!(x.v > eps)) x.v = eps;
+}
 template <> DRT_HD void clamp_positive<de>(de &x, float eps) {
     if (!(x.b + x.d > eps)) {
         x.b = eps;
@@ -297,6 +300,9 @@ template <> DRT_HD void clamp_positive<dd>(dd &x, float eps) {
 // Newton start for an edge parameter from its value `base` + `delta` and rate: for delta numbers
 // the base part is `base` (the chunk-base solution) and the delta `delta`
 template <class S> DRT_HD S newton_start(double base, double delta, double rate);
+template <> DRT_HD dl<ff> newton_start<dl<ff>>(double base, double delta, double rate) {
+    return {from_double(base + delta), from_double(rate)};
+}
 template <> DRT_HD ff newton_start<ff>(double base, double delta, double) { return from_double(base + delta); }
 template <> DRT_HD double newton_start<double>(double base, double delta, double) { return base + delta; }
 template <> DRT_HD float newton_start<float>(double base, double delta, double) { return (float)(base + delta); }
@@ -312,6 +318,9 @@ template <> DRT_HD dd newton_start<dd>(double base, double delta, double rate) {
 template <class S> DRT_HD S newton_start_f(double base, float delta, float rate);
 template <> DRT_HD de newton_start_f<de>(double base, float delta, float) { return {(float)base, delta}; }
 template <> DRT_HD dd newton_start_f<dd>(double base, float delta, float rate) { return {(float)base, delta, rate}; }
+template <> DRT_HD dl<ff> newton_start_f<dl<ff>>(double base, float delta, float rate) {
+    return {from_double(base) + ff(delta), ff(rate)};
+}
 template <> DRT_HD ff newton_start_f<ff>(double base, float delta, float) { return from_double(base) + ff(delta); }
 
 // chain length of path p (vertices before the first empty type byte)
@@ -1965,25 +1974,21 @@ DRT_HD Prim<double> load_prim_value(const LinkDev &L, const double *Pr, int type
 
 // (path, chunk) FP64 anchors: path length and segment vectors at the chunk's first instant, phase
 // seed and per-bin step.  N < 0: the chain length is read at run time (one instance per length).
-template <int N = -1>
-DRT_HD void path_base_fp64(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const double *pose64, int p,
-                           int chunk, BaseRec *out, const double *warm = nullptr) {
+template <int N = -1, class Loader>
+DRT_HD void path_base_fp64_core(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int chunk,
+                                BaseRec *out, const double *warm, Loader load) {
     if constexpr (N < 0) {
         with_length(chain_length(L, p), [&](auto NC) {
-            path_base_fp64<decltype(NC)::value>(L, tg, fg, pose64, p, chunk, out, warm);
+            path_base_fp64_core<decltype(NC)::value>(L, tg, fg, p, chunk, out, warm, load);
         });
     } else {
         const double tb = tg.t_start + (double)chunk * tg.chunk * tg.dt;
-        const int n_chunks = (tg.n_steps + tg.chunk - 1) / tg.chunk;
         const uint32_t code = L.ptypes[p];
         const int4 pi = L.pprims[p];
         const int prim[MAXI] = {pi.x, pi.y, pi.z, pi.w};
         Prim<double> pr[N > 0 ? N : 1];
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const int ty = (code >> (8 * j)) & 0xff;
-            pr[j] = load_prim_value(L, pose_at(pose64, n_chunks, prim_body(L, ty, prim[j]), chunk), ty, prim[j]);
-        }
+        for (int j = 0; j < N; ++j) pr[j] = load((code >> (8 * j)) & 0xff, prim[j]);
         v3<double> V[N + 2];
         V[0] = val(terminal<double>(L.tx, tb));
         V[N + 1] = val(terminal<double>(L.rx, tb));
@@ -2014,6 +2019,13 @@ DRT_HD void path_base_fp64(const LinkDev &L, const TimeGridD &tg, const FreqGrid
         r.pad = 0.f;
         out[(size_t)chunk * L.n_paths + p] = r;
     }
+}
+DRT_HD void path_base_fp64(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const double *pose64, int p,
+                           int chunk, BaseRec *out, const double *warm) {
+    const int n_chunks = (tg.n_steps + tg.chunk - 1) / tg.chunk;
+    path_base_fp64_core(L, tg, fg, p, chunk, out, warm, [&](int ty, int idx) {
+        return load_prim_value(L, pose_at(pose64, n_chunks, prim_body(L, ty, idx), chunk), ty, idx);
+    });
 }
 
 

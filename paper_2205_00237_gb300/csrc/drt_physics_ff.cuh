@@ -42,11 +42,11 @@ DRT_HD void body_pose_ff(const BodyQ &B, ff t, PoseQ &q) {
     for (int j = 0; j < 3; ++j) q.O[j] = fma(B.a[j], t2, fma(B.v[j], t, B.o[j]));
 }
 
-DRT_HD Prim<ff> load_prim_ff(const LinkDev &L, const PoseQ *pose, int n_steps, int ti, int type, int idx) {
-    Prim<ff> q;
+// the primitive as stored: placed in the world when its body is at rest (returns -1), else relative to the rotation centre of
+// the body returned
+DRT_HD int load_prim_rest(const LinkDev &L, int type, int idx, Prim<ff> &q) {
     q.type = type;
     q.idx = idx;
-    int body;
     if (type == T_R) {
         const FaceQ &f = L.facesQ[idx];
         q.p = vq(f.c);
@@ -55,8 +55,9 @@ DRT_HD Prim<ff> load_prim_ff(const LinkDev &L, const PoseQ *pose, int n_steps, i
         q.h1 = f.hu;
         q.h2 = f.hw;
         q.mat = f.mat;
-        body = f.body;
-    } else if (type == T_D) {
+        return f.body;
+    }
+    if (type == T_D) {
         const EdgeQ &e = L.edgesQ[idx];
         q.p = vq(e.a);
         q.a = vq(e.e);
@@ -67,22 +68,92 @@ DRT_HD Prim<ff> load_prim_ff(const LinkDev &L, const PoseQ *pose, int n_steps, i
         q.h3 = e.snp;
         q.h4 = e.cnp;
         q.mat = e.mat;
-        body = e.body;
-    } else {
-        const TileQ &tl = L.tilesQ[idx];
-        q.p = vq(tl.c);
-        q.a = vq(tl.n);
-        q.mat = tl.mat;
-        body = tl.body;
+        return e.body;
     }
+    const TileQ &tl = L.tilesQ[idx];
+    q.p = vq(tl.c);
+    q.a = vq(tl.n);
+    q.mat = tl.mat;
+    return tl.body;
+}
+DRT_HD void pose_prim(const PoseQ &P, Prim<ff> &q) {
+    q.p = vq(P.O) + rotq(P, q.p);
+    q.a = rotq(P, q.a);
+    if (q.type != T_S) q.b = rotq(P, q.b);
+    if (q.type == T_D) q.c = rotq(P, q.c);
+}
+// posed from a table of rows [body][row]
+DRT_HD Prim<ff> load_prim_ff(const LinkDev &L, const PoseQ *pose, int n_rows, int row, int type, int idx) {
+    Prim<ff> q;
+    const int body = load_prim_rest(L, type, idx, q);
+    if (body >= 0) pose_prim(pose[(size_t)body * n_rows + row], q);
+    return q;
+}
+// posed from the body's kinematics at t
+DRT_HD Prim<ff> load_prim_ff_direct(const LinkDev &L, ff t, int type, int idx) {
+    Prim<ff> q;
+    const int body = load_prim_rest(L, type, idx, q);
     if (body >= 0) {
-        const PoseQ &P = pose[(size_t)body * n_steps + ti];
-        q.p = vq(P.O) + rotq(P, q.p);
-        q.a = rotq(P, q.a);
-        if (type != T_S) q.b = rotq(P, q.b);
-        if (type == T_D) q.c = rotq(P, q.c);
+        PoseQ P;
+        body_pose_ff(L.bodiesQ[body], t, P);
+        pose_prim(P, q);
     }
     return q;
+}
+// the same with rates
+DRT_HD Prim<dl<ff>> load_prim_ff_dual(const LinkDev &L, ff t, int type, int idx) {
+    Prim<ff> q;
+    const int body = load_prim_rest(L, type, idx, q);
+    v3<ff> dp = V3<ff>(ff(0.f), ff(0.f), ff(0.f)), da = dp;
+    if (body >= 0) {
+        const BodyQ &B = L.bodiesQ[body];
+        PoseQ P;
+        body_pose_ff(B, t, P);
+        pose_prim(P, q);
+        const v3<ff> w = vq(B.k) * fma(B.wdot, t, B.w0);
+        dp = axpy(vq(B.v), vq(B.a), t) + cross(w, q.p - vq(P.O));
+        da = cross(w, q.a);
+    }
+    Prim<dl<ff>> r;
+    r.type = q.type;
+    r.mat = q.mat;
+    r.idx = q.idx;
+    r.p = dual(q.p, dp);
+    r.a = dual(q.a, da);
+    r.b = q.b;
+    r.c = q.c;
+    r.h1 = q.h1;
+    r.h2 = q.h2;
+    r.h3 = q.h3;
+    r.h4 = q.h4;
+    return r;
+}
+DRT_HD Prim<ff> val_prim(const Prim<dl<ff>> &q) {
+    Prim<ff> r;
+    r.type = q.type;
+    r.mat = q.mat;
+    r.idx = q.idx;
+    r.p = val(q.p);
+    r.a = val(q.a);
+    r.b = q.b;
+    r.c = q.c;
+    r.h1 = q.h1;
+    r.h2 = q.h2;
+    r.h3 = q.h3;
+    r.h4 = q.h4;
+    return r;
+}
+DRT_HD v3<float> f32v(v3<ff> a) { return V3<float>(a.x.h, a.y.h, a.z.h); }
+DRT_HD Prim<float> f32_prim(const Prim<dl<ff>> &q) {   // the Newton solve reads no more than this
+    Prim<float> r;
+    r.type = q.type;
+    r.p = f32v(val(q.p));
+    r.a = f32v(val(q.a));
+    return r;
+}
+DRT_HD v3<dl<ff>> terminal_dual_ff(const TermQ &m, ff t) {
+    const v3<ff> v = vq(m.v), a = vq(m.a);
+    return dual(axpy(axpy(vq(m.r), v, t), a, halve(t * t)), axpy(v, a, t));
 }
 
 // amplitude 0 and all-zero phases for a path that does not exist; phases in turns from the path length d
@@ -175,6 +246,302 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
     if (!sure) path_step_ff_fallback<N, MULTI>(L, tg, fg, p, ti, rec, warm);
 }
 
+// ------------------------------------------------------------------------------------------------
+// The FP64 parts of the FP32-bulk form in two-float numbers: warm starts, anchors at the chunk bases, and the redo of the steps FP32
+// cannot resolve.  They are short dependent chains (a few solves per path), so what they cost is latency: 65 cycles per FP64
+// instruction, a few per FP32 one.
+
+// The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, one two-float dual step for the
+// rates.  False where it did not converge (the caller runs the FP64 solve).
+template <int N> DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
+    const uint32_t code = L.ptypes[p];
+    const int4 pi = L.pprims[p];
+    const int prim[MAXI] = {pi.x, pi.y, pi.z, pi.w};
+    const ff tq = from_double(t);
+    Prim<dl<ff>> pr[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) pr[j] = load_prim_ff_dual(L, tq, (code >> (8 * j)) & 0xff, prim[j]);
+    v3<dl<ff>> V[N + 2];
+    V[0] = terminal_dual_ff(L.txq, tq);
+    V[N + 1] = terminal_dual_ff(L.rxq, tq);
+    bool nv[N + 1];   // the unknowns: diffractions of a stretch with several of them
+    int cf[N + 1], c = 0, run = -1;
+#pragma unroll
+    for (int i = 1; i <= N; ++i) {
+        c = pr[i - 1].type == T_S ? 0 : c + (pr[i - 1].type == T_D ? 1 : 0);
+        cf[i] = c;
+    }
+#pragma unroll
+    for (int i = N; i >= 1; --i) {
+        if (pr[i - 1].type == T_S) run = -1;
+        else if (run < 0) run = cf[i];
+        nv[i] = pr[i - 1].type == T_D && run >= 2;
+    }
+    place_tiles<N>(pr, V);
+    double s1[MAXI];
+#pragma unroll
+    for (int j = 0; j < MAXI; ++j) s1[j] = sin[j];
+    {
+        Prim<float> pf[N];
+        v3<float> Vf[N + 2];
+        uint32_t ff_ = 0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) pf[j] = f32_prim(pr[j]);
+#pragma unroll
+        for (int i = 0; i <= N + 1; ++i) Vf[i] = f32v(val(V[i]));
+        newton_diffractions<N>(pf, Vf, nv, s1, (const double *)nullptr, (const double *)nullptr, ff_);
+        if (!(ff_ & F_NOCONV))
+#pragma unroll
+            for (int j = 0; j < N; ++j)
+                if (nv[j + 1]) s1[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
+    }
+    uint32_t fl = 0;
+    {
+        Prim<ff> pd[N];
+        v3<ff> Vd[N + 2];
+#pragma unroll
+        for (int j = 0; j < N; ++j) pd[j] = val_prim(pr[j]);
+#pragma unroll
+        for (int i = 0; i <= N + 1; ++i) Vd[i] = val(V[i]);
+        newton_diffractions<N>(pd, Vd, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (nv[j + 1]) s1[j] = to_double(dot(Vd[j + 1] - pd[j].p, pd[j].a));
+    }
+    newton_diffractions<N>(pr, V, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
+    bool ok = !(fl & F_NOCONV);
+    // the diffractions alone in their stretch: on their Keller cones
+    bool single = false;
+#pragma unroll
+    for (int i = 1; i <= N; ++i) single = single || (pr[i - 1].type == T_D && !nv[i]);
+    if (single) place_keller<N>(pr, V, fl, nv);
+#pragma unroll
+    for (int j = 0; j < MAXI; ++j) {
+        sv[j] = sin[j];
+        sd[j] = 0.0;
+        if (j < N && pr[j].type == T_D) {
+            const dl<ff> sj = dot(V[j + 1] - pr[j].p, pr[j].a);
+            ok = ok && isfinite(sj.v.h) && isfinite(sj.d.h);
+            sv[j] = to_double(sj.v);
+            sd[j] = to_double(sj.d);
+        }
+    }
+    return ok;
+}
+template <int N> DRT_NOINL void solve_edge_params_fp64(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
+    solve_edge_params<N>(L, p, t, sin, sv, sd, [&](int ty, int idx) { return load_prim_direct<double>(L, t, ty, idx); });
+}
+DRT_HD void edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
+    with_length<2>(chain_length(L, p), [&](auto NC) {
+        constexpr int N = decltype(NC)::value;
+        double start[MAXI];
+        for (int j = 0; j < MAXI; ++j) start[j] = sin[j];
+        if (!solve_edge_params_ff<N>(L, p, t, start, sv, sd)) solve_edge_params_fp64<N>(L, p, t, start, sv, sd);
+    });
+}
+// path_t0par_fp64 and path_warm_fp64 (drt_physics.cuh) on it
+DRT_HD void path_t0par_ff(const LinkDev &L, int p, double *out) {
+    edge_params_ff(L, p, 0.0, L.ps0 + (size_t)p * MAXI, out, out + MAXI);
+}
+DRT_HD void path_warm_ff(const LinkDev &L, const TimeGridD &tg, int p, int row, double *warm) {
+    const double t = tg.t_start + (double)row * tg.chunk * tg.dt;
+    const double *q = L.t0par + (size_t)(p - L.n_bulk) * (2 * MAXI);
+    double start[MAXI];
+    for (int j = 0; j < MAXI; ++j) start[j] = q[j] + q[MAXI + j] * t;
+    double *w = warm + ((size_t)row * (L.n_paths - L.n_bulk) + (p - L.n_bulk)) * (2 * MAXI);
+    edge_params_ff(L, p, t, start, w, w + MAXI);
+}
+
+// path_base_fp64 (drt_physics.cuh): anchors of a (path, chunk) from the poses at the chunk bases [body][chunk]
+template <int N> DRT_NOINL void path_base_ff_fallback(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int chunk,
+                                                      BaseRec *out, const double *warm) {
+    const double tb = tg.t_start + (double)chunk * tg.chunk * tg.dt;
+    path_base_fp64_core<N>(L, tg, fg, p, chunk, out, warm,
+                           [&](int ty, int idx) { return val_prim(load_prim_direct<double>(L, tb, ty, idx)); });
+}
+template <int N = -1>
+DRT_HD void path_base_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const PoseQ *pose, int p, int chunk,
+                         BaseRec *out, const double *warm) {
+    if constexpr (N < 0) {
+        with_length(chain_length(L, p), [&](auto NC) {
+            path_base_ff<decltype(NC)::value>(L, tg, fg, pose, p, chunk, out, warm);
+        });
+    } else {
+        const ff tb = from_double(tg.t_start + (double)chunk * tg.chunk * tg.dt);
+        const int n_chunks = (tg.n_steps + tg.chunk - 1) / tg.chunk;
+        const uint32_t code = L.ptypes[p];
+        const int4 pi = L.pprims[p];
+        const int prim[MAXI] = {pi.x, pi.y, pi.z, pi.w};
+        Prim<ff> pr[N > 0 ? N : 1];
+#pragma unroll
+        for (int j = 0; j < N; ++j) pr[j] = load_prim_ff(L, pose, n_chunks, chunk, (code >> (8 * j)) & 0xff, prim[j]);
+        v3<ff> V[N + 2];
+        V[0] = val(terminal_dual_ff(L.txq, tb));
+        V[N + 1] = val(terminal_dual_ff(L.rxq, tb));
+        uint32_t fl = 0;
+        const double *s0 = L.ps0 + (size_t)p * MAXI;
+        if (warm && p >= L.n_bulk) s0 = warm_row(L, warm, chunk, p);
+        solve_geometry_any<N>(pr, V, s0, fl);
+        BaseRec r;
+        ff d = ff(0.f);
+#pragma unroll
+        for (int i = 0; i <= MAXI; ++i) r.seg[i][0] = r.seg[i][1] = r.seg[i][2] = 0.f;
+#pragma unroll
+        for (int i = 1; i <= N + 1; ++i) {
+            const v3<ff> sg = V[i] - V[i - 1];
+            d = d + norm(sg);
+            r.seg[i - 1][0] = sg.x.h;
+            r.seg[i - 1][1] = sg.y.h;
+            r.seg[i - 1][2] = sg.z.h;
+        }
+        if ((fl & (F_REDO64 | F_NOCONV | F_DEGEN)) || !isfinite(d.h)) {
+            path_base_ff_fallback<N>(L, tg, fg, p, chunk, out, warm);
+            return;
+        }
+        const ff x = d * fg.f0c_q, y = d * fg.dfc_q;
+        const float st = y.h - floorf(y.h);
+        r.d = to_double(d);
+        r.ph0 = (x.h - floorf(x.h)) + x.l;
+        r.st_hi = rintf((st + y.l) * 4096.f) * (1.f / 4096.f);
+        r.st_lo = (st - r.st_hi) + y.l;
+        r.pad = 0.f;
+        out[(size_t)chunk * L.n_paths + p] = r;
+    }
+}
+
+// App. A Eq. doppler_freq (doppler<N>, drt_physics.cuh) to second order in v / c: sum_i log1p(-u_i) - log1p(-u_{i-1}) with u = v.k / c of
+// ~1e-6, whose third-order terms are below 1e-17, and expm1 alike
+template <int N> DRT_HD float doppler_ff(const v3<dl<ff>> *V, const v3<ff> *seg, const FreqGridD &fg) {
+    ff s1 = ff(0.f);
+    float s2 = 0.f;
+#pragma unroll
+    for (int i = 1; i <= N + 1; ++i) {
+        const v3<ff> k = unit(seg[i]);
+        const ff u1 = dot(der(V[i]), k), u0 = dot(der(V[i - 1]), k);
+        s1 = s1 + (u0 - u1);
+        s2 += (u0.h - u1.h) * (u0.h + u1.h);
+    }
+    const ff S = s1 * ff(1 / C0) + ff(s2 * (float)(0.5 / (C0 * C0)));
+    return (fg.kq * ff(C0 / (2 * PI)) * (S + halve(S * S))).h;   // fc = k c / 2 pi
+}
+
+// FP64 redo of one queued FP32-bulk path-step (path_step_redo_as, drt_physics.cuh) in two-float numbers: FP32 output formats and
+// (Re a, Im a, tau) in rec64, a = 0 where the path does not exist.  False where two-float numbers cannot decide the step.
+template <int N, bool DUAL>
+DRT_HD bool path_step_redo_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti, const OutD &out,
+                              const double *warm, double *rec64) {
+    typedef std::conditional_t<DUAL, dl<ff>, ff> S;
+    const ff t = from_double(tg.t_start + ti * tg.dt);
+    const uint32_t code = L.ptypes[p];
+    const int4 pi = L.pprims[p];
+    const int prim[MAXI] = {pi.x, pi.y, pi.z, pi.w};
+    Prim<S> pr[N > 0 ? N : 1];
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        if constexpr (DUAL) pr[j] = load_prim_ff_dual(L, t, (code >> (8 * j)) & 0xff, prim[j]);
+        else pr[j] = load_prim_ff_direct(L, t, (code >> (8 * j)) & 0xff, prim[j]);
+    }
+    v3<S> V[N + 2];
+    if constexpr (DUAL) {
+        V[0] = terminal_dual_ff(L.txq, t);
+        V[N + 1] = terminal_dual_ff(L.rxq, t);
+    } else {
+        V[0] = val(terminal_dual_ff(L.txq, t));
+        V[N + 1] = val(terminal_dual_ff(L.rxq, t));
+    }
+    uint32_t fl = 0;
+    if (warm && p >= L.n_bulk) {
+        WarmStart32 ws;
+        warm_start_at32(L, tg, warm, p, ti, ws);
+        solve_geometry_any<N>(pr, V, ws.s, fl, ws.ds, ws.rate);
+    } else {
+        solve_geometry_any<N>(pr, V, L.ps0 + (size_t)p * MAXI, fl);
+    }
+    v3<ff> P[N + 2], seg[N + 2];
+    ff d = ff(0.f);
+    P[0] = val(V[0]);
+#pragma unroll
+    for (int i = 1; i <= N + 1; ++i) {
+        P[i] = val(V[i]);
+        seg[i] = P[i] - P[i - 1];
+        d = d + norm(seg[i]);
+    }
+    fl |= validity<N>(pr, N, P);
+    if ((fl & (F_REDO64 | F_NOCONV | F_DEGEN)) || !isfinite(d.h)) return false;
+    cx<ff> a = C<ff>(ff(0.f), ff(0.f));
+    if (!fl || out.amp) {
+        Prim<ff> pv[N > 0 ? N : 1];
+        if constexpr (DUAL) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) pv[j] = val_prim(pr[j]);
+            a = amplitude_ff<N>(L, pv, seg, fg);
+        } else {
+            a = amplitude_ff<N>(L, pr, seg, fg);
+        }
+        if (!isfinite(a.re.h) || !isfinite(a.im.h)) return false;
+    }
+    const double tau = to_double(d) * (1 / C0);
+    if (rec64) {
+        rec64[0] = fl ? 0.0 : to_double(a.re);
+        rec64[1] = fl ? 0.0 : to_double(a.im);
+        rec64[2] = tau;
+    }
+    const size_t oi = (size_t)ti * L.n_paths + L.perm[p];
+    if (out.tau) out.tau[oi] = tau;
+    if (out.amp) {
+        float *q = reinterpret_cast<float *>(out.amp) + 2 * oi;
+        q[0] = a.re.h;
+        q[1] = a.im.h;
+    }
+    if constexpr (DUAL)
+        if (out.doppler) reinterpret_cast<float *>(out.doppler)[oi] = doppler_ff<N>(V, seg, fg);
+    if (out.angles) {
+        const v3<float> kd = f32v(unit(seg[1])), ka = f32v(-unit(seg[N + 1]));
+        float *q = out.angles + 4 * oi;
+        q[0] = atan2f(kd.y, kd.x);
+        q[1] = atan2f(kd.z, hypotf(kd.x, kd.y));
+        q[2] = atan2f(ka.y, ka.x);
+        q[3] = atan2f(ka.z, hypotf(ka.x, ka.y));
+    }
+    if (out.flags) out.flags[oi] = (uint8_t)fl;
+    if (out.points) {
+        double *q = out.points + oi * (MAXI * 3);
+        const double qn = nan("");
+#pragma unroll
+        for (int j = 0; j < MAXI; ++j) {
+            q[3 * j + 0] = j < N ? to_double(P[j + 1 < N + 1 ? j + 1 : N].x) : qn;
+            q[3 * j + 1] = j < N ? to_double(P[j + 1 < N + 1 ? j + 1 : N].y) : qn;
+            q[3 * j + 2] = j < N ? to_double(P[j + 1 < N + 1 ? j + 1 : N].z) : qn;
+        }
+    }
+    return true;
+}
+template <int N, bool DUAL>
+DRT_NOINL void path_step_redo_fp64(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti, const OutD &out,
+                                   const double *warm, double *rec64) {
+    const double t = tg.t_start + ti * tg.dt;
+    const RecD nor{nullptr, nullptr};
+    if constexpr (DUAL)
+        path_step_fp64_core<N, true, true, dl<double>>(
+            L, tg, fg, p, ti, out, nor, true, [&](int ty, int idx) { return load_prim_direct<double>(L, t, ty, idx); },
+            warm, rec64);
+    else
+        path_step_fp64_core<N, true, true, double>(
+            L, tg, fg, p, ti, out, nor, true,
+            [&](int ty, int idx) { return val_prim(load_prim_direct<double>(L, t, ty, idx)); }, warm, rec64);
+}
+// two: two-float numbers apply to the link and grid (ff_applies), else the step is computed in FP64
+template <bool DUAL>
+DRT_HD void path_step_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti, const OutD &out,
+                           const double *warm, double *rec64, bool two) {
+    with_length(chain_length(L, p), [&](auto NC) {
+        constexpr int N = decltype(NC)::value;
+        if (!two || !path_step_redo_ff<N, DUAL>(L, tg, fg, p, ti, out, warm, rec64))
+            path_step_redo_fp64<N, DUAL>(L, tg, fg, p, ti, out, warm, rec64);
+    });
+}
+
+// ------------------------------------------------------------------------------------------------
 // A block covers consecutive (path, 32 steps) warps in path-major order, so neighbouring blocks, which run at the same time, are
 // on paths of the same signature
 template <int N, bool MULTI> struct FFBlock { static constexpr int v = 128, per_sm = N <= 1 ? 5 : N == 2 && !MULTI ? 4 : 3; };
