@@ -1051,20 +1051,34 @@ drt_status drt_lifetime_windows(drt_ctx *c, uint64_t link, const drt_time_grid *
     if (T == 0) return DRT_OK;
     const size_t n = (size_t)T * L->n_paths;
     const size_t fsz = precision == DRT_FP64 ? sizeof(double) : sizeof(float);
-    if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
-    if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
     if (drt_status st = ensure(c, c->lt_tot, (size_t)T * sizeof(double))) return st;
-    if (drt_status st = ensure(c, c->lt_major, (size_t)T)) return st;
-    OutD o{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
-    cudaStream_t s = (cudaStream_t)stream;
-    RecD none{nullptr, nullptr};
-    if (drt_status st = run_extrapolation(c, *L, tg, fg, o, none, precision, s)) return st;
+    if (drt_status st = ensure(c, c->lt_major, (size_t)T + 1)) return st;
     uint8_t *mj = reinterpret_cast<uint8_t *>(c->lt_major.ptr);
-    CUDA_TRY(launch_lifetime(precision == DRT_FP64, o, T, L->n_paths, lp->share,
-                             reinterpret_cast<double *>(c->lt_tot.ptr), mj, s));
-    std::vector<uint8_t> m(T);
-    CUDA_TRY(cudaMemcpyAsync(m.data(), mj, T, cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
+    double *tot = reinterpret_cast<double *>(c->lt_tot.ptr);
+    cudaStream_t s = (cudaStream_t)stream;
+    const RecD none{nullptr, nullptr};
+    std::vector<uint8_t> m((size_t)T + 1);
+    bool decided = false;
+    // FP64 form: the changes from the synthesis records (two-float arithmetic, a quarter of the FP64 outputs' time), unless one of
+    // them lies within the records' rounding of the threshold
+    if (precision == DRT_FP64 && lp->share >= 1e-12 && ff_applies(L->view, *tg, *fg) &&
+        ensure(c, c->rec_a, n * sizeof(float4)) == DRT_OK && ensure(c, c->rec_b, n * sizeof(float)) == DRT_OK) {
+        const RecD rec{reinterpret_cast<float4 *>(c->rec_a.ptr), reinterpret_cast<float *>(c->rec_b.ptr)};
+        if (drt_status st = run_extrapolation(c, *L, tg, fg, OutD{}, rec, precision, s)) return st;
+        CUDA_TRY(launch_lifetime_rec(rec, T, L->n_paths, lp->share, tot, mj, s));
+        CUDA_TRY(cudaMemcpyAsync(m.data(), mj, (size_t)T + 1, cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(cudaStreamSynchronize(s));
+        decided = m[T] == 0;
+    }
+    if (!decided) {
+        if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
+        if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
+        OutD o{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
+        if (drt_status st = run_extrapolation(c, *L, tg, fg, o, none, precision, s)) return st;
+        CUDA_TRY(launch_lifetime(precision == DRT_FP64, o, T, L->n_paths, lp->share, tot, mj, s));
+        CUDA_TRY(cudaMemcpyAsync(m.data(), mj, T, cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(cudaStreamSynchronize(s));
+    }
     if (major) std::memcpy(major, m.data(), T);
     // windows: from start w, the first major change in [w + min_steps, w + max_steps], else w + max_steps
     std::vector<int32_t> w{0};
@@ -1147,19 +1161,23 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
                       cudaStream_t s) {
     const long long n_cand = trace_candidates(L.dev, max_order, with_tiles);
     const int cap_dev = (int)std::min<long long>(n_cand, 1 << 22);
+    const bool two = L.view.ff_range && L.view.extent + std::fabs(t) * (L.view.vmax + 0.5 * L.view.amax * std::fabs(t)) < 1e5;
     if (drt_status st = ensure(c, c->tr_faces, (size_t)std::max(L.dev.n_faces, 1) * trace_face_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);
-    CUDA_TRY(launch_trace(L.dev, t, max_order, with_tiles, c->tr_faces.ptr, c->tr_rays.ptr, cap_dev, cnt, s));
+    // with two-float numbers the list holds the candidates that FP64 has dropped, too: more than it holds is tried again without
     int count = 0;
-    CUDA_TRY(cudaMemcpyAsync(&count, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(cudaStreamSynchronize(s));
+    for (int pass = two ? 0 : 1; pass < 2; ++pass) {
+        CUDA_TRY(launch_trace(L.dev, t, max_order, with_tiles, c->tr_faces.ptr, c->tr_rays.ptr, cap_dev, cnt, s, pass == 0));
+        CUDA_TRY(cudaMemcpyAsync(&count, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(cudaStreamSynchronize(s));
+        if (count <= cap_dev) break;
+    }
     if (count > cap_dev) return fail(DRT_ENOMEM, "ray tracing found %d rays, more than %d", count, cap_dev);
     std::vector<char> rays((size_t)count * trace_ray_bytes());
     if (count) CUDA_TRY(cudaMemcpy(rays.data(), c->tr_rays.ptr, rays.size(), cudaMemcpyDeviceToHost));
-    out->n_found = count;
-    trace_unpack(rays.data(), count, out->n_int, out->types, out->prims, out->s0, out->cap);
+    out->n_found = trace_unpack(rays.data(), count, out->n_int, out->types, out->prims, out->s0, out->cap);
     return DRT_OK;
 }
 

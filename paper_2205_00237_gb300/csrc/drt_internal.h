@@ -262,6 +262,10 @@ cudaError_t launch_redo_add(const LinkDev &L, const TimeGridD &tg, const FreqGri
 // (major[T], 1 at instant n when a path with >= share of the power at its valid side changes validity)
 cudaError_t launch_lifetime(bool fp64, const OutD &rec, int n_steps, int n_paths, double share, double *tot,
                             uint8_t *major, cudaStream_t s);
+// the same from synthesis records of the FP64 form (share >= 1e-12); major[n_steps] is set when a decision lies within the rounding
+// of the records and the FP64 outputs have to decide
+cudaError_t launch_lifetime_rec(const RecD &rec, int n_steps, int n_paths, double share, double *tot, uint8_t *major,
+                                cudaStream_t s);
 // T_C windows: window w starts at step starts[w] (starts[0] = 0, increasing); sel is [T][P] (caller
 // path order) and holds, in the rows of the window starts, the path's FP64 flags at that instant
 // (0: in the window's multipath); launch_select writes those rows
@@ -290,9 +294,11 @@ cudaError_t launch_probe(int kind, int blocks, double *sink, cudaStream_t s, flo
 long long trace_candidates(const LinkDev &L, int max_order, int with_tiles);
 size_t trace_ray_bytes();
 size_t trace_face_bytes();
+// two: candidates are solved in two-float numbers first, and FP64 decides what those leave open (see drt_trace.cu); trace_unpack returns
+// the number of rays
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s);
-void trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0,
+                         int *count, cudaStream_t s, bool two);
+int trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0,
                   int cap);
 
 }  // namespace drt

@@ -150,6 +150,50 @@ cudaError_t launch_lifetime(bool fp64, const OutD &rec, int n_steps, int n_paths
     return cudaGetLastError();
 }
 
+// The same from the FP32 amplitudes of synthesis records, for the FP64 form: their squares and sums are within 2.4e-7 of the FP64 ones,
+// so a share within 1e-6 of the threshold is not decided here but marks amb[0], as does an instant whose power is too small for
+// FP32 amplitudes; a record without amplitude is a path that is not valid there.
+__global__ void __launch_bounds__(256)
+k_step_power_rec(const float4 *__restrict__ rec, int n_steps, int n_paths, double *__restrict__ tot, uint8_t *__restrict__ amb) {
+    const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (n >= n_steps) return;   // warp-uniform
+    double acc = 0.0;
+    for (int p = lane; p < n_paths; p += 32) {
+        const float2 a = *reinterpret_cast<const float2 *>(rec + (size_t)n * n_paths + p);
+        acc += (double)a.x * a.x + (double)a.y * a.y;
+    }
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+        tot[n] = acc;
+        if (!(acc > 1e-50)) amb[0] = 1;
+    }
+}
+__global__ void __launch_bounds__(256)
+k_toggle_rec(const float4 *__restrict__ rec, const double *__restrict__ tot, int n_steps, int n_paths, double share,
+             uint8_t *__restrict__ major, uint8_t *__restrict__ amb) {
+    const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (q >= (long long)(n_steps - 1) * n_paths) return;
+    const float2 a0 = *reinterpret_cast<const float2 *>(rec + q), a1 = *reinterpret_cast<const float2 *>(rec + q + n_paths);
+    const bool v0 = a0.x != 0.f || a0.y != 0.f, v1 = a1.x != 0.f || a1.y != 0.f;
+    if (v1 == v0) return;
+    const int n = 1 + (int)(q / n_paths);
+    const float2 a = v1 ? a1 : a0;
+    const double pw = (double)a.x * a.x + (double)a.y * a.y, thr = share * tot[v1 ? n : n - 1];
+    if (!(fabs(pw - thr) > 1e-6 * thr)) amb[0] = 1;
+    else if (pw > thr) major[n] = 1;
+}
+cudaError_t launch_lifetime_rec(const RecD &rec, int n_steps, int n_paths, double share, double *tot, uint8_t *major,
+                                cudaStream_t s) {
+    if (cudaError_t e = cudaMemsetAsync(major, 0, (size_t)n_steps + 1, s)) return e;
+    if (n_paths == 0) return cudaSuccess;
+    const long long nq = (long long)(n_steps - 1) * n_paths;
+    k_step_power_rec<<<(unsigned)((n_steps + 7) / 8), 256, 0, s>>>(rec.rec_a, n_steps, n_paths, tot, major + n_steps);
+    if (nq)
+        k_toggle_rec<<<(unsigned)((nq + 255) / 256), 256, 0, s>>>(rec.rec_a, tot, n_steps, n_paths, share, major,
+                                                                  major + n_steps);
+    return cudaGetLastError();
+}
+
 // DRT over T_C windows: a path that is not valid at the first instant of its window is outside that
 // window's multipath (sel[start][caller index] != 0, its FP64 flags at the window start) and its
 // records carry a = 0; the same holds for the FP64 redo contributions of the FP32-bulk form.

@@ -10,11 +10,13 @@
 #include <vector>
 
 #include "drt_launch.cuh"
+#include "drt_physics_ff.cuh"
 
 namespace drt {
 
 // a face posed at the instant: centre, unit normal, in-plane axes, half extents
 struct PosedFace { double c[3], n[3], u[3], w[3], hu, hw; };
+struct PosedFaceQ { ff c[3], n[3], u[3], w[3], hu, hw; };   // the same in two-float numbers, in a table behind the first
 
 DRT_HD void pose_face(const LinkDev &L, double t, int f, PosedFace *out_f) {
     const FaceD &F = L.faces[f];
@@ -32,9 +34,22 @@ DRT_HD void pose_face(const LinkDev &L, double t, int f, PosedFace *out_f) {
     *out_f = r;
 }
 
-__global__ void k_pose_faces(const LinkDev L, double t, PosedFace *__restrict__ out) {
+__global__ void k_pose_faces(const LinkDev L, double t, PosedFace *__restrict__ out, PosedFaceQ *__restrict__ outq) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f < L.n_faces) pose_face(L, t, f, out + f);
+    if (f >= L.n_faces) return;
+    pose_face(L, t, f, out + f);
+    if (!outq) return;
+    const PosedFace F = out[f];
+    PosedFaceQ q;
+    for (int j = 0; j < 3; ++j) {
+        q.c[j] = from_double(F.c[j]);
+        q.n[j] = from_double(F.n[j]);
+        q.u[j] = from_double(F.u[j]);
+        q.w[j] = from_double(F.w[j]);
+    }
+    q.hu = L.facesQ[f].hu;
+    q.hw = L.facesQ[f].hw;
+    outq[f] = q;
 }
 
 // Does the face block the segment A -> B?  It does when the segment crosses the face's plane
@@ -51,7 +66,9 @@ DRT_HD bool face_blocks(const PosedFace &F, v3<double> A, v3<double> B) {
 }
 
 // one ray found: its enumeration index, chain and diffraction parameters at the instant
-struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; };
+// (state: how far it is decided; index -1: FP64 found that it is none)
+enum { RAY_FINAL = 0, RAY_POLISH = 1, RAY_OPEN = 2 };
+struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; int32_t state, pad; };
 
 constexpr int TRACE_T = 128;
 
@@ -93,6 +110,7 @@ DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code
         for (int f = 0; f < L.n_faces; ++f)
             if (face_blocks(faces[f], V[i - 1], V[i])) return false;
     r->index = k;
+    r->state = RAY_FINAL;
     r->n = N;
     r->types = types;
 #pragma unroll
@@ -137,33 +155,202 @@ k_trace(const LinkDev L, double t, long long n_cand, int with_tiles, const Posed
     if (slot < cap) out[slot] = r;
 }
 
+// ------------------------------------------------------------------------------------------------
+// The same in two passes.  Nearly every candidate is no ray by a clear margin, and in FP64 the solves and the segment-face tests of all of
+// them wait on the FP64 pipe (1.13 ms for the canyon's 97206).  k_trace_ff decides the candidates in two-float numbers, with margins
+// as in path_step_ff; what is a ray or open goes to the list, and k_trace_finish, in FP64, tries the open ones again and solves the
+// rays' diffraction parameters from the two-float ones (one Newton step), so that the list ends as k_trace's.
+
+// 1: the face blocks the segment, 0: it does not, -1: within the margins
+DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B) {
+    const v3<ff> c = vq(F.c), n = vq(F.n);
+    const ff ha = dot(A - c, n), hb = dot(B - c, n);
+    const float fa = fabsf(ha.h), fb = fabsf(hb.h), scale = fmaxf(fmaxf(amax3(A), amax3(B)), amax3(c));
+    // an end within 1e-9 m of the plane: the points of a chain lie on its own faces to ~2^-46 of the coordinates, which 2^-42 bounds
+    const float tol = ff_margin_tol(scale), e = fmaxf(2.3e-13f * (scale + 1.f), 1e-10f);
+    if (fabsf(fa - 1e-9f) <= e || fabsf(fb - 1e-9f) <= e || e > 5e-10f) return -1;
+    if (fa < 1e-9f || fb < 1e-9f) return 0;
+    if ((ha.h > 0.f) == (hb.h > 0.f)) return 0;
+    const v3<ff> r = axpy(A, B - A, ha / (ha - hb)) - c;
+    const float mu = ff_within(dot(r, vq(F.u)), F.hu), mw = ff_within(dot(r, vq(F.w)), F.hw);
+    // the point moves along the plane with the error of h over the segment's slope
+    const v3<ff> d = B - A;
+    const float lim = tol * (1.f + (fabsf(d.x.h) + fabsf(d.y.h) + fabsf(d.z.h)) / (fa + fb));
+    if (mu < -lim || mw < -lim) return 0;
+    return mu > lim && mw > lim ? 1 : -1;
+}
+
+template <int N>
+DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const PosedFaceQ *faces, TracedRay *r) {
+    const int NP = L.n_faces + L.n_edges;
+    const ff tq = from_double(t);
+    Prim<ff> pr[N > 0 ? N : 1];
+    double s0[MAXI] = {0.0, 0.0, 0.0, 0.0};
+    uint32_t types = 0;
+    bool any_d = false;
+    r->n = N;
+#pragma unroll
+    for (int j = 0; j < MAXI; ++j) {
+        r->prims[j] = 0;
+        r->s[j] = 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const int c = code[j];
+        int ty, idx;
+        if (c < L.n_faces) { ty = T_R; idx = c; }
+        else if (c < NP) { ty = T_D; idx = c - L.n_faces; s0[j] = 0.5 * L.edges[idx].len; }
+        else { ty = T_S; idx = c - NP; }
+        pr[j] = load_prim_ff_direct(L, tq, ty, idx);
+        types |= (uint32_t)ty << (8 * j);
+        r->prims[j] = idx;
+        any_d = any_d || ty == T_D;
+    }
+    r->types = types;
+    v3<ff> V[N + 2];
+    V[0] = val(terminal_dual_ff(L.txq, tq));
+    V[N + 1] = val(terminal_dual_ff(L.rxq, tq));
+    uint32_t fl = 0;
+    if constexpr (N == 2) {
+        // two diffractions: FP32 Newton from the midpoints first
+        if (pr[0].type == T_D && pr[1].type == T_D) {
+            Prim<float> pf[2];
+            v3<float> Vf[4];
+            const bool nv[3] = {false, true, true};
+            for (int j = 0; j < 2; ++j) {
+                pf[j].type = T_D;
+                pf[j].p = f32v(pr[j].p);
+                pf[j].a = f32v(pr[j].a);
+            }
+            Vf[0] = f32v(V[0]);
+            Vf[3] = f32v(V[3]);
+            Vf[1] = Vf[2] = Vf[0];
+            uint32_t f0 = 0;
+            newton_diffractions<2>(pf, Vf, nv, s0, (const double *)nullptr, (const double *)nullptr, f0);
+            if (!(f0 & F_NOCONV))
+                for (int j = 0; j < 2; ++j) s0[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
+        }
+    }
+    solve_geometry_any<N>(pr, V, s0, fl);
+    fl |= validity<N>(pr, N, V);
+    if (fl & (F_REDO64 | F_NOCONV | F_DEGEN)) return RAY_OPEN;
+#pragma unroll
+    for (int i = 1; i <= N; ++i)
+        if (!(isfinite(V[i].x.h) && isfinite(V[i].y.h) && isfinite(V[i].z.h))) return RAY_OPEN;
+    if (fl) return -1;
+    bool open = false;
+#pragma unroll
+    for (int i = 1; i <= N + 1; ++i)
+        for (int f = 0; f < L.n_faces; ++f) {
+            const int b = face_blocks_ff(faces[f], V[i - 1], V[i]);
+            if (b > 0) return -1;
+            open = open || b < 0;
+        }
+    if (open) return RAY_OPEN;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        if (pr[j].type == T_D) r->s[j] = to_double(dot(V[j + 1] - pr[j].p, pr[j].a));
+    return any_d ? RAY_POLISH : RAY_FINAL;
+}
+
+__global__ void __launch_bounds__(TRACE_T)
+k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int with_tiles, const PosedFaceQ *__restrict__ faces,
+           TracedRay *__restrict__ out, int cap, int *__restrict__ count) {
+    const long long k = blockIdx.x * (long long)TRACE_T + threadIdx.x;
+    if (k >= n_cand) return;
+    const int NP = L.n_faces + L.n_edges, NT = with_tiles ? L.n_tiles : 0;
+    TracedRay r;
+    r.pad = 0;
+    int code[2] = {0, 0}, state;
+    if (k == 0) {
+        state = trace_chain_ff<0>(L, t, code, faces, &r);
+    } else if (k - 1 < NP + NT) {
+        code[0] = (int)(k - 1);
+        state = trace_chain_ff<1>(L, t, code, faces, &r);
+    } else {
+        const long long q = k - 1 - NP - NT;
+        code[0] = (int)(q / NP);
+        code[1] = (int)(q % NP);
+        if (code[0] == code[1]) return;
+        state = trace_chain_ff<2>(L, t, code, faces, &r);
+    }
+    if (state < 0) return;
+    r.index = k;
+    r.state = state;
+    const int slot = atomicAdd(count, 1);
+    if (slot < cap) out[slot] = r;
+}
+
+// the diffraction parameters of a ray in FP64, from the two-float ones
+template <int N> DRT_HD void polish_ray(const LinkDev &L, double t, TracedRay *r) {
+    Prim<double> pr[N];
+    double s0[MAXI] = {r->s[0], r->s[1], 0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j < N; ++j) pr[j] = val_prim(load_prim_direct<double>(L, t, (r->types >> (8 * j)) & 0xff, r->prims[j]));
+    v3<double> V[N + 2];
+    V[0] = val(terminal<double>(L.tx, t));
+    V[N + 1] = val(terminal<double>(L.rx, t));
+    uint32_t fl = 0;
+    solve_geometry_any<N>(pr, V, s0, fl);
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        if (pr[j].type == T_D) r->s[j] = dot(V[j + 1] - pr[j].p, pr[j].a);
+}
+
+__global__ void __launch_bounds__(32)
+k_trace_finish(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
+               TracedRay *__restrict__ out, int cap, const int *__restrict__ count) {
+    const int n = min(*count, cap);
+    for (int k = blockIdx.x * 32 + threadIdx.x; k < n; k += gridDim.x * 32) {
+        TracedRay *r = out + k;
+        if (r->state == RAY_POLISH) {
+            if (r->n == 1) polish_ray<1>(L, t, r);
+            else polish_ray<2>(L, t, r);
+        } else if (r->state == RAY_OPEN) {
+            TracedRay q;
+            if (trace_eval(L, t, r->index, with_tiles, faces, &q)) *r = q;
+            else r->index = -1;
+        }
+    }
+}
+
 long long trace_candidates(const LinkDev &L, int max_order, int with_tiles) {
     const long long NP = L.n_faces + L.n_edges, NT = with_tiles ? L.n_tiles : 0;
     return 1 + (max_order >= 1 ? NP + NT : 0) + (max_order >= 2 ? NP * NP : 0);
 }
 
 size_t trace_ray_bytes() { return sizeof(TracedRay); }
-size_t trace_face_bytes() { return sizeof(PosedFace); }
+size_t trace_face_bytes() { return sizeof(PosedFace) + sizeof(PosedFaceQ); }
 
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s) {
+                         int *count, cudaStream_t s, bool two) {
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
-    if (L.n_faces > 0) k_pose_faces<<<(L.n_faces + 127) / 128, 128, 0, s>>>(L, t, reinterpret_cast<PosedFace *>(faces));
+    PosedFace *F = reinterpret_cast<PosedFace *>(faces);
+    PosedFaceQ *Q = reinterpret_cast<PosedFaceQ *>(F + L.n_faces);
+    TracedRay *out = reinterpret_cast<TracedRay *>(rays);
+    if (L.n_faces > 0) k_pose_faces<<<(L.n_faces + 127) / 128, 128, 0, s>>>(L, t, F, two ? Q : nullptr);
     const long long n = trace_candidates(L, max_order, with_tiles);
-    k_trace<<<(unsigned)((n + TRACE_T - 1) / TRACE_T), TRACE_T, 0, s>>>(
-        L, t, n, with_tiles, reinterpret_cast<const PosedFace *>(faces), reinterpret_cast<TracedRay *>(rays), cap, count);
+    const unsigned grid = (unsigned)((n + TRACE_T - 1) / TRACE_T);
+    if (two) {
+        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, Q, out, cap, count);
+        k_trace_finish<<<152 * 8, 32, 0, s>>>(L, t, with_tiles, F, out, cap, count);
+    } else {
+        k_trace<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, F, out, cap, count);
+    }
     return cudaGetLastError();
 }
 
-// the found rays (count of them, in any order) to host arrays in enumeration order
-void trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0,
-                  int cap) {
+// the rays in a list of `count` (in any order) to host arrays in enumeration order; returns their number
+int trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0, int cap) {
     const TracedRay *R = reinterpret_cast<const TracedRay *>(rays_host);
-    std::vector<int> order(count);
-    for (int i = 0; i < count; ++i) order[i] = i;
+    std::vector<int> order;
+    order.reserve(count);
+    for (int i = 0; i < count; ++i)
+        if (R[i].index >= 0) order.push_back(i);
+    const int n = (int)order.size();
     std::sort(order.begin(), order.end(), [&](int a, int b) { return R[a].index < R[b].index; });
-    for (int q = 0; q < count && q < cap; ++q) {
+    for (int q = 0; q < n && q < cap; ++q) {
         const TracedRay &r = R[order[q]];
         n_int[q] = (uint8_t)r.n;
         for (int j = 0; j < MAXI; ++j) {
@@ -172,6 +359,7 @@ void trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *typ
             s0[q * MAXI + j] = r.s[j];
         }
     }
+    return n;
 }
 
 }  // namespace drt
