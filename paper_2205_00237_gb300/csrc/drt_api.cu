@@ -1162,7 +1162,7 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
     const long long n_cand = trace_candidates(L.dev, max_order, with_tiles);
     const int cap_dev = (int)std::min<long long>(n_cand, 1 << 22);
     const bool two = L.view.ff_range && L.view.extent + std::fabs(t) * (L.view.vmax + 0.5 * L.view.amax * std::fabs(t)) < 1e5;
-    if (drt_status st = ensure(c, c->tr_faces, (size_t)std::max(L.dev.n_faces, 1) * trace_face_bytes())) return st;
+    if (drt_status st = ensure(c, c->tr_faces, trace_prim_bytes(L.dev))) return st;
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);

@@ -24,6 +24,8 @@ enum : uint32_t { F_FACE = 1, F_EDGE = 2, F_SIDE = 4, F_NOCONV = 8, F_DEGEN = 16
 // internal: the FP32-bulk solve met a geometry it cannot resolve in FP32 (near-grazing Keller cone,
 // unconverged Newton, non-finite value); the path-step is redone in FP64.  Never written out.
 constexpr uint32_t F_REDO64 = 128;
+// internal (two-float form): a flag is set whose own margin is clear: the chain is no ray, whatever the undecided tests say
+constexpr uint32_t F_CLEAR = 32;
 // internal: some FP32 validity margin lies within 100x the FP32 error bound (fp32_margin_tol)
 constexpr uint32_t F_NEAR100 = 64;
 
@@ -246,7 +248,7 @@ DRT_HD S keller_s(v3<S> Sv, v3<S> Rv, const Prim<S> &e, uint32_t &fl) {
     }
     // two-float numbers: within 1 um of the edge line
     if constexpr (std::is_same<T, ff>::value)
-        if (!(ra2.h > 1e-12f) || !(rb2.h > 1e-12f)) fl |= F_REDO64;
+        if (!(ra2.h > 1e-12f) || !(rb2.h > 1e-12f)) fl |= F_NOCONV;
     // near grazing (a virtual terminal within 1 mm of the edge line) FP32 cannot resolve the cone
     if (sizeof(T) == 4 && (ra2 < T(1e-6) || rb2 < T(1e-6))) fl |= F_REDO64;
     S ra = norm(pa), rb = norm(pb);
@@ -663,37 +665,37 @@ template <class T> struct VertexCheck { uint32_t fl; T m; };
 DRT_NOINL1 VertexCheck<float> vertex_validity_inl(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
                                               v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
     uint32_t fl = 0;
-    float m, scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), amax3(Pi));
+    float scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), amax3(Pi));
+    if (ty != T_S) scale = fmaxf(scale, amax3(c));
+    const float tol = ff_margin_tol(scale);
+    // a test passes with margin v > 0; within the bound (or not a number) it is undecided
+    auto test = [&](float v, uint32_t bit) {
+        if (!(v > 0.f)) fl |= v < -tol ? bit | F_CLEAR : bit;
+        if (!(fabsf(v) > tol)) fl |= F_REDO64;
+    };
     if (ty == T_D) {
-        scale = fmaxf(scale, amax3(c));
         const ff s = dot(Pi - c, nn);
-        const float up = (h1.h - s.h) + (h1.l - s.l);
-        if (s.h < 0.f || up < 0.f) fl |= F_EDGE;
-        m = fminf(fabsf(s.h), fabsf(up));
+        test(s.h, F_EDGE);
+        test((h1.h - s.h) + (h1.l - s.l), F_EDGE);
 #pragma unroll
         for (int side = -1; side <= 1; side += 2) {   // see the general form below
             const v3<ff> r = (side < 0 ? Pm : Pp) - Pi;
             const v3<ff> rp = axpy(r, nn, -dot(r, nn));
             const ff y = dot(rp, cc), x = dot(rp, b);
             const float sn = det2(h3, x, h4, y).h;
-            if (!(y.h > 0.f) && !(sn > 0.f)) fl |= F_SIDE;   // zero of either is within the margin
-            m = fminf(m, fminf(fabsf(y.h), fabsf(sn)));
+            if (!(fabsf(y.h) > tol) || !(fabsf(sn) > tol)) fl |= F_REDO64;
+            if (!(y.h > 0.f) && !(sn > 0.f)) fl |= y.h < -tol && sn < -tol ? F_SIDE | F_CLEAR : F_SIDE;
         }
     } else {
-        m = 1e30f;
         if (ty == T_R) {
-            scale = fmaxf(scale, amax3(c));
             const v3<ff> r = Pi - c;
-            const float mu = ff_within(dot(r, b), h1), mw = ff_within(dot(r, cross(b, nn)), h2);
-            if (mu < 0.f || mw < 0.f) fl |= F_FACE;
-            m = fminf(fabsf(mu), fabsf(mw));
+            test(ff_within(dot(r, b), h1), F_FACE);
+            test(ff_within(dot(r, cross(b, nn)), h2), F_FACE);
         }
-        const float dp = dot(Pm - c, nn).h, dn = dot(Pp - c, nn).h;   // a tile is its own point
-        if (!(dp > 0.f) || !(dn > 0.f)) fl |= F_SIDE;
-        m = fminf(m, fminf(fabsf(dp), fabsf(dn)));
+        test(dot(Pm - c, nn).h, F_SIDE);   // a tile is its own point
+        test(dot(Pp - c, nn).h, F_SIDE);
     }
-    // written so that a margin that is not a number is inside the bound
-    return VertexCheck<float>{fl, m > ff_margin_tol(scale) ? 2.f : 0.f};
+    return VertexCheck<float>{fl, 2.f};
 }
 template <class T>
 DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3<T> cc, T h1, T h2, T h3, T h4,
@@ -761,7 +763,10 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
     for (int i = 1; i <= MAXI + 1; ++i) {
         if (i > nv + 1) break;
         v3<T> d = P[i] - P[i - 1];
-        if (!(dot(d, d) >= T(1e-18))) fl |= F_DEGEN;
+        const T q = dot(d, d);
+        if (!(q >= T(1e-18))) fl |= F_DEGEN;
+        if constexpr (FF)   // shorter than half of that bound: clear of it
+            if (q.h < 2.5e-19f) fl |= F_CLEAR;
     }
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI; ++i) {
@@ -776,8 +781,6 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         if (mmin < T(1)) fl |= F_REDO64;
         if (mmin < T(100)) fl |= F_NEAR100;
     }
-    if constexpr (FF)
-        if (mmin < 1.f) fl |= F_REDO64;
     return fl;
 }
 

@@ -234,7 +234,7 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
         d = d + norm(seg[i]);
     }
     fl |= validity<N>(pr, N, V);
-    bool sure = !(fl & (F_REDO64 | F_NOCONV | F_DEGEN)) && isfinite(d.h);
+    bool sure = !(fl & F_NOCONV) && (!(fl & (F_REDO64 | F_DEGEN)) || (fl & F_CLEAR)) && isfinite(d.h);
     if (sure && !fl) {
         const cx<ff> a = amplitude_ff<N>(L, pr, seg, fg);
         sure = isfinite(a.re.h) && isfinite(a.im.h);
@@ -467,7 +467,8 @@ DRT_HD bool path_step_redo_ff(const LinkDev &L, const TimeGridD &tg, const FreqG
         d = d + norm(seg[i]);
     }
     fl |= validity<N>(pr, N, P);
-    if ((fl & (F_REDO64 | F_NOCONV | F_DEGEN)) || !isfinite(d.h)) return false;
+    if ((fl & (F_REDO64 | F_NOCONV | F_DEGEN)) || !isfinite(d.h)) return false;   // every bit is written out: all decided
+    fl &= ~F_CLEAR;
     cx<ff> a = C<ff>(ff(0.f), ff(0.f));
     if (!fl || out.amp) {
         Prim<ff> pv[N > 0 ? N : 1];

@@ -68,7 +68,7 @@ DRT_HD bool face_blocks(const PosedFace &F, v3<double> A, v3<double> B) {
 // one ray found: its enumeration index, chain and diffraction parameters at the instant
 // (state: how far it is decided; index -1: FP64 found that it is none)
 enum { RAY_FINAL = 0, RAY_POLISH = 1, RAY_OPEN = 2 };
-struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; int32_t state, pad; };
+struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; int32_t state, pad; ff v[2][3]; };
 
 constexpr int TRACE_T = 128;
 
@@ -76,9 +76,9 @@ constexpr int TRACE_T = 128;
 // pairs of faces / edges, the same primitive twice excluded) solved at t: true when it is a ray, which
 // then fills *r
 // the candidate's chain of N interactions (codes c[0..N-1]): solved, checked and, if it is a ray, stored
-template <int N>
-DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code, const PosedFace *faces,
-                        TracedRay *r) {
+// (blocked(A, B): whether a face blocks a segment)
+template <int N, class Blocked>
+DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code, TracedRay *r, Blocked blocked) {
     const int NP = L.n_faces + L.n_edges;
     Prim<double> pr[N > 0 ? N : 1];
     double s0[MAXI] = {0.0, 0.0, 0.0, 0.0};
@@ -107,8 +107,7 @@ DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code
     if (fl) return false;
 #pragma unroll
     for (int i = 1; i <= N + 1; ++i)
-        for (int f = 0; f < L.n_faces; ++f)
-            if (face_blocks(faces[f], V[i - 1], V[i])) return false;
+        if (blocked(V[i - 1], V[i])) return false;
     r->index = k;
     r->state = RAY_FINAL;
     r->n = N;
@@ -123,7 +122,8 @@ DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code
     return true;
 }
 
-DRT_HD bool trace_eval(const LinkDev &L, double t, long long k, int with_tiles, const PosedFace *faces, TracedRay *r) {
+template <class Blocked>
+DRT_HD bool trace_eval(const LinkDev &L, double t, long long k, int with_tiles, TracedRay *r, Blocked blocked) {
     const int NP = L.n_faces + L.n_edges, NT = with_tiles ? L.n_tiles : 0;
     int n = 0, code[2] = {0, 0};
     if (k > 0) {
@@ -139,9 +139,9 @@ DRT_HD bool trace_eval(const LinkDev &L, double t, long long k, int with_tiles, 
             n = 2;
         }
     }
-    if (n == 0) return trace_chain<0>(L, t, k, code, faces, r);
-    if (n == 1) return trace_chain<1>(L, t, k, code, faces, r);
-    return trace_chain<2>(L, t, k, code, faces, r);
+    if (n == 0) return trace_chain<0>(L, t, k, code, r, blocked);
+    if (n == 1) return trace_chain<1>(L, t, k, code, r, blocked);
+    return trace_chain<2>(L, t, k, code, r, blocked);
 }
 
 __global__ void __launch_bounds__(TRACE_T)
@@ -150,16 +150,22 @@ k_trace(const LinkDev L, double t, long long n_cand, int with_tiles, const Posed
     const long long k = blockIdx.x * (long long)TRACE_T + threadIdx.x;
     if (k >= n_cand) return;
     TracedRay r;
-    if (!trace_eval(L, t, k, with_tiles, faces, &r)) return;
+    if (!trace_eval(L, t, k, with_tiles, &r, [&](v3<double> A, v3<double> B) {
+            for (int f = 0; f < L.n_faces; ++f)
+                if (face_blocks(faces[f], A, B)) return true;
+            return false;
+        }))
+        return;
     const int slot = atomicAdd(count, 1);
     if (slot < cap) out[slot] = r;
 }
 
 // ------------------------------------------------------------------------------------------------
-// The same in two passes.  Nearly every candidate is no ray by a clear margin, and in FP64 the solves and the segment-face tests of all of
-// them wait on the FP64 pipe (1.13 ms for the canyon's 97206).  k_trace_ff decides the candidates in two-float numbers, with margins
-// as in path_step_ff; what is a ray or open goes to the list, and k_trace_finish, in FP64, tries the open ones again and solves the
-// rays' diffraction parameters from the two-float ones (one Newton step), so that the list ends as k_trace's.
+// The same in three passes.  Nearly every candidate is no ray by a clear margin, and in FP64 all of them wait on the FP64 pipe, and the few
+// that reach the segment-face tests on one thread's loop over the faces (1.13 ms for the canyon's 97206 candidates).  k_trace_ff
+// solves and checks the candidates in two-float numbers, with margins as in path_step_ff, and lists those that may be rays;
+// k_trace_block, a warp per listed candidate, spreads the (segment, face) tests over its lanes and tries what is still open in FP64;
+// k_trace_polish solves the rays' diffraction parameters in FP64 from the two-float ones (one Newton step).  The list ends as k_trace's.
 
 // 1: the face blocks the segment, 0: it does not, -1: within the margins
 DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B) {
@@ -180,8 +186,34 @@ DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B) {
     return mu > lim && mw > lim ? 1 : -1;
 }
 
+// the faces, then the edges, posed
+__global__ void __launch_bounds__(128)
+k_pose_prims(const __grid_constant__ LinkDev L, double t, Prim<ff> *__restrict__ prims) {
+    const int i = blockIdx.x * 128 + threadIdx.x;
+    if (i >= L.n_faces + L.n_edges) return;
+    prims[i] = load_prim_ff_direct(L, from_double(t), i < L.n_faces ? T_R : T_D, i < L.n_faces ? i : i - L.n_faces);
+}
+
+// Two edges whose lines meet in a point C (a corner of a box or of a facade): the shortest path over both runs through C when the length
+// has its minimum at that kink, where the Newton solve does not converge or ends on a path without a middle segment; either way the
+// chain is no ray.  The minimum is there when the pulls of the outer segments along the edges can be balanced by a vector z of length
+// below 1 (the subgradient of the middle segment's length): z.e1 = -p, z.e2 = -q with p = u.e1, q = w.e2 for the unit directions u
+// from A to C and w from C to B.  The length is convex, so a kink minimum with |z| clear of 1 is its only stationary point.
+DRT_HD bool corner_path(const Prim<ff> &E1, const Prim<ff> &E2, v3<ff> A, v3<ff> B) {
+    const v3<ff> x = cross(E1.a, E2.a), d = E2.p - E1.p;
+    const ff xx = dot(x, x), gap = dot(d, x);
+    if (!(xx.h > 1e-4f) || !(gap.h * gap.h < 2.5e-19f * xx.h)) return false;   // the lines meet within 5e-10 m
+    const v3<ff> C = axpy(E1.p, E1.a, dot(cross(d, E2.a), x) / xx);
+    const v3<float> e1 = f32v(E1.a), e2 = f32v(E2.a), ac = f32v(C - A), cb = f32v(B - C);
+    if (!(dot(ac, ac) > 0.01f) || !(dot(cb, cb) > 0.01f)) return false;
+    const v3<float> u = unit(ac), w = unit(cb);
+    const float c = dot(e1, e2), p = dot(u, e1), q = dot(w, e2), det = 1.f - c * c;
+    const float a = (c * q - p) / det, b = (c * p - q) / det;   // z = a e1 + b e2
+    return -(a * p + b * q) < 0.99f;                            // |z|^2
+}
+
 template <int N>
-DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const PosedFaceQ *faces, TracedRay *r) {
+DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Prim<ff> *prims, TracedRay *r) {
     const int NP = L.n_faces + L.n_edges;
     const ff tq = from_double(t);
     Prim<ff> pr[N > 0 ? N : 1];
@@ -201,7 +233,8 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pos
         if (c < L.n_faces) { ty = T_R; idx = c; }
         else if (c < NP) { ty = T_D; idx = c - L.n_faces; s0[j] = 0.5 * L.edges[idx].len; }
         else { ty = T_S; idx = c - NP; }
-        pr[j] = load_prim_ff_direct(L, tq, ty, idx);
+        if (ty == T_S) pr[j] = load_prim_ff_direct(L, tq, ty, idx);
+        else pr[j] = prims[c];
         types |= (uint32_t)ty << (8 * j);
         r->prims[j] = idx;
         any_d = any_d || ty == T_D;
@@ -212,49 +245,65 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pos
     V[N + 1] = val(terminal_dual_ff(L.rxq, tq));
     uint32_t fl = 0;
     if constexpr (N == 2) {
-        // two diffractions: FP32 Newton from the midpoints first
-        if (pr[0].type == T_D && pr[1].type == T_D) {
-            Prim<float> pf[2];
-            v3<float> Vf[4];
-            const bool nv[3] = {false, true, true};
-            for (int j = 0; j < 2; ++j) {
-                pf[j].type = T_D;
-                pf[j].p = f32v(pr[j].p);
-                pf[j].a = f32v(pr[j].a);
-            }
-            Vf[0] = f32v(V[0]);
-            Vf[3] = f32v(V[3]);
-            Vf[1] = Vf[2] = Vf[0];
-            uint32_t f0 = 0;
-            newton_diffractions<2>(pf, Vf, nv, s0, (const double *)nullptr, (const double *)nullptr, f0);
-            if (!(f0 & F_NOCONV))
-                for (int j = 0; j < 2; ++j) s0[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
+        if (pr[0].type == T_D && pr[1].type == T_D && corner_path(pr[0], pr[1], V[0], V[3])) return -1;
+        // FP32 first.  A chain whose FP32 solve fails a test, with every margin (the failed one's too) above 1000 times the FP32
+        // bound 2e-6 of the coordinates, is none: an error of the solved points is that bound times (leg / height), and the
+        // heights are among the margins, so it is at most 1 / 60 of them.
+        Prim<float> pf[2];
+        v3<float> Vf[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            pf[j].type = pr[j].type;
+            pf[j].p = f32v(pr[j].p);
+            pf[j].a = f32v(pr[j].a);
+            pf[j].b = f32v(pr[j].b);
+            pf[j].c = f32v(pr[j].c);
+            pf[j].h1 = pr[j].h1.h;
+            pf[j].h2 = pr[j].h2.h;
+            pf[j].h3 = pr[j].h3.h;
+            pf[j].h4 = pr[j].h4.h;
         }
+        Vf[0] = f32v(V[0]);
+        Vf[3] = f32v(V[3]);
+        uint32_t f0 = 0, bad = 0;
+        solve_geometry_any<2>(pf, Vf, s0, f0);
+        float margin = 1e30f;
+        bool fine = true;
+#pragma unroll
+        for (int i = 1; i <= 2; ++i) {
+            const Prim<float> &q = pf[i - 1];
+            const VertexCheck<float> v = vertex_validity_inl(q.type, q.p, q.a, q.b, q.c, q.h1, q.h2, q.h3, q.h4, Vf[i - 1], Vf[i], Vf[i + 1]);
+            bad |= v.fl;
+            margin = fminf(margin, v.m);
+            fine = fine && isfinite(Vf[i].x) && isfinite(Vf[i].y) && isfinite(Vf[i].z) && v.m > 1000.f;
+        }
+        if (fine && bad && margin > 1000.f && !(f0 & (F_NOCONV | F_REDO64 | F_DEGEN))) return -1;
+        if (!(f0 & F_NOCONV))   // the two-float Newton solve starts from the FP32 one's
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (pf[j].type == T_D) s0[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
     }
     solve_geometry_any<N>(pr, V, s0, fl);
     fl |= validity<N>(pr, N, V);
-    if (fl & (F_REDO64 | F_NOCONV | F_DEGEN)) return RAY_OPEN;
+    if (fl & F_NOCONV) return RAY_OPEN;
 #pragma unroll
     for (int i = 1; i <= N; ++i)
         if (!(isfinite(V[i].x.h) && isfinite(V[i].y.h) && isfinite(V[i].z.h))) return RAY_OPEN;
+    if (fl & F_CLEAR) return -1;
+    if (fl & (F_REDO64 | F_DEGEN)) return RAY_OPEN;
     if (fl) return -1;
-    bool open = false;
 #pragma unroll
-    for (int i = 1; i <= N + 1; ++i)
-        for (int f = 0; f < L.n_faces; ++f) {
-            const int b = face_blocks_ff(faces[f], V[i - 1], V[i]);
-            if (b > 0) return -1;
-            open = open || b < 0;
-        }
-    if (open) return RAY_OPEN;
-#pragma unroll
-    for (int j = 0; j < N; ++j)
+    for (int j = 0; j < N; ++j) {
+        r->v[j][0] = V[j + 1].x;
+        r->v[j][1] = V[j + 1].y;
+        r->v[j][2] = V[j + 1].z;
         if (pr[j].type == T_D) r->s[j] = to_double(dot(V[j + 1] - pr[j].p, pr[j].a));
+    }
     return any_d ? RAY_POLISH : RAY_FINAL;
 }
 
 __global__ void __launch_bounds__(TRACE_T)
-k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int with_tiles, const PosedFaceQ *__restrict__ faces,
+k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int with_tiles, const Prim<ff> *__restrict__ prims,
            TracedRay *__restrict__ out, int cap, int *__restrict__ count) {
     const long long k = blockIdx.x * (long long)TRACE_T + threadIdx.x;
     if (k >= n_cand) return;
@@ -263,22 +312,62 @@ k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int wi
     r.pad = 0;
     int code[2] = {0, 0}, state;
     if (k == 0) {
-        state = trace_chain_ff<0>(L, t, code, faces, &r);
+        state = trace_chain_ff<0>(L, t, code, prims, &r);
     } else if (k - 1 < NP + NT) {
         code[0] = (int)(k - 1);
-        state = trace_chain_ff<1>(L, t, code, faces, &r);
+        state = trace_chain_ff<1>(L, t, code, prims, &r);
     } else {
         const long long q = k - 1 - NP - NT;
         code[0] = (int)(q / NP);
         code[1] = (int)(q % NP);
         if (code[0] == code[1]) return;
-        state = trace_chain_ff<2>(L, t, code, faces, &r);
+        state = trace_chain_ff<2>(L, t, code, prims, &r);
     }
     if (state < 0) return;
     r.index = k;
     r.state = state;
     const int slot = atomicAdd(count, 1);
     if (slot < cap) out[slot] = r;
+}
+
+__global__ void __launch_bounds__(128)
+k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
+              const PosedFaceQ *__restrict__ facesq, TracedRay *__restrict__ out, int cap, const int *__restrict__ count) {
+    const int n = min(*count, cap), lane = threadIdx.x & 31;
+    const ff tq = from_double(t);
+    for (int k = blockIdx.x * 4 + (threadIdx.x >> 5); k < n; k += gridDim.x * 4) {   // warp-uniform
+        TracedRay *r = out + k;
+        int state = r->state;
+        if (state != RAY_OPEN) {
+            const int N = r->n;
+            const v3<ff> tx = val(terminal_dual_ff(L.txq, tq)), rx = val(terminal_dual_ff(L.rxq, tq));
+            bool hit = false, open = false;
+            for (int q = lane; q < (N + 1) * L.n_faces; q += 32) {
+                const int i = q / L.n_faces, f = q - i * L.n_faces;
+                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(r->v[i - 1]), i == N ? rx : vq(r->v[i]));
+                hit = hit || b > 0;
+                open = open || b < 0;
+            }
+            hit = __any_sync(0xffffffffu, hit);
+            open = __any_sync(0xffffffffu, open);
+            if (hit) {
+                if (lane == 0) r->index = -1;
+                continue;
+            }
+            if (!open) continue;
+        }
+        TracedRay q;
+        const bool ray = trace_eval(L, t, r->index, with_tiles, &q, [&](v3<double> A, v3<double> B) {
+            bool hit = false;
+            for (int f = lane; f < L.n_faces; f += 32) hit = hit || face_blocks(faces[f], A, B);
+            return __any_sync(0xffffffffu, hit) != 0;
+        });
+        __syncwarp();   // every lane has read the entry
+        if (lane == 0) {
+            if (ray) *r = q;
+            else r->index = -1;
+        }
+    }
 }
 
 // the diffraction parameters of a ray in FP64, from the two-float ones
@@ -298,19 +387,13 @@ template <int N> DRT_HD void polish_ray(const LinkDev &L, double t, TracedRay *r
 }
 
 __global__ void __launch_bounds__(32)
-k_trace_finish(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
-               TracedRay *__restrict__ out, int cap, const int *__restrict__ count) {
+k_trace_polish(const __grid_constant__ LinkDev L, double t, TracedRay *__restrict__ out, int cap, const int *__restrict__ count) {
     const int n = min(*count, cap);
     for (int k = blockIdx.x * 32 + threadIdx.x; k < n; k += gridDim.x * 32) {
         TracedRay *r = out + k;
-        if (r->state == RAY_POLISH) {
-            if (r->n == 1) polish_ray<1>(L, t, r);
-            else polish_ray<2>(L, t, r);
-        } else if (r->state == RAY_OPEN) {
-            TracedRay q;
-            if (trace_eval(L, t, r->index, with_tiles, faces, &q)) *r = q;
-            else r->index = -1;
-        }
+        if (r->state != RAY_POLISH || r->index < 0) continue;
+        if (r->n == 1) polish_ray<1>(L, t, r);
+        else polish_ray<2>(L, t, r);
     }
 }
 
@@ -320,7 +403,9 @@ long long trace_candidates(const LinkDev &L, int max_order, int with_tiles) {
 }
 
 size_t trace_ray_bytes() { return sizeof(TracedRay); }
-size_t trace_face_bytes() { return sizeof(PosedFace) + sizeof(PosedFaceQ); }
+size_t trace_prim_bytes(const LinkDev &L) {
+    return (size_t)L.n_faces * (sizeof(PosedFace) + sizeof(PosedFaceQ)) + (size_t)(L.n_faces + L.n_edges) * sizeof(Prim<ff>) + 256;
+}
 
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
                          int *count, cudaStream_t s, bool two) {
@@ -333,8 +418,12 @@ cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_til
     const long long n = trace_candidates(L, max_order, with_tiles);
     const unsigned grid = (unsigned)((n + TRACE_T - 1) / TRACE_T);
     if (two) {
-        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, Q, out, cap, count);
-        k_trace_finish<<<152 * 8, 32, 0, s>>>(L, t, with_tiles, F, out, cap, count);
+        Prim<ff> *prims = reinterpret_cast<Prim<ff> *>(Q + L.n_faces);
+        const int np = L.n_faces + L.n_edges;
+        if (np) k_pose_prims<<<(np + 127) / 128, 128, 0, s>>>(L, t, prims);
+        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, prims, out, cap, count);
+        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, out, cap, count);
+        k_trace_polish<<<152 * 8, 32, 0, s>>>(L, t, out, cap, count);
     } else {
         k_trace<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, F, out, cap, count);
     }
