@@ -112,6 +112,10 @@ struct drt_ctx {
     // links in a loop then costs no cudaMalloc / cudaFree; the blocks count against the HBM budget
     std::multimap<size_t, void *> link_pool;
     size_t link_pool_bytes = 0;
+    // pinned host image of the link being loaded (grows with the largest one; the context lock is held from its filling to the end
+    // of its copy): a fresh pageable image per load costs its page faults and a staged copy
+    char *stage = nullptr;
+    size_t stage_cap = 0;
 };
 
 namespace {
@@ -186,22 +190,35 @@ drt_status ensure(drt_ctx *c, Scratch &s, size_t bytes) {
 // the arrays of one link packed at 256-byte offsets into one host image, uploaded as one device
 // allocation with one copy (separate allocations cost a cudaMalloc / cudaFree per array per link)
 struct LinkImage {
-    std::vector<char> host;
-    std::vector<std::function<void(char *)>> bind;
+    struct Part { const void *src; size_t bytes, off; void *dst; };   // dst: the device pointer to set
+    std::vector<Part> parts;
+    size_t size = 0;
     template <class X> void add(const std::vector<X> &v, const X **dst) {
-        const size_t off = (host.size() + 255) & ~(size_t)255;
-        host.resize(off + v.size() * sizeof(X));
-        if (!v.empty()) std::memcpy(host.data() + off, v.data(), v.size() * sizeof(X));
-        bind.push_back([dst, off](char *base) { *dst = reinterpret_cast<const X *>(base + off); });
+        const size_t off = (size + 255) & ~(size_t)255;
+        size = off + v.size() * sizeof(X);
+        parts.push_back(Part{v.data(), v.size() * sizeof(X), off, dst});
     }
+    // queued on the default stream; the staging image may be filled again once the stream has been waited for
     drt_status upload(drt_ctx *c, Link &L) {
         void *p = nullptr;
         size_t got = 0;
-        if (drt_status st = link_block_alloc(c, host.size(), &p, &got)) return st;
+        if (drt_status st = link_block_alloc(c, size, &p, &got)) return st;
         L.allocs.push_back(p);
         L.bytes += got;
-        if (!host.empty()) CUDA_TRY(cudaMemcpy(p, host.data(), host.size(), cudaMemcpyHostToDevice));
-        for (auto &b : bind) b(reinterpret_cast<char *>(p));
+        if (c->stage_cap < size) {
+            if (c->stage) cudaFreeHost(c->stage);
+            c->stage = nullptr;
+            c->stage_cap = 0;
+            const size_t want = std::max(size + size / 2, (size_t)1 << 20);
+            CUDA_TRY(cudaMallocHost(reinterpret_cast<void **>(&c->stage), want));
+            c->stage_cap = want;
+        }
+        for (const Part &q : parts) {
+            if (q.bytes) std::memcpy(c->stage + q.off, q.src, q.bytes);
+            const char *at = reinterpret_cast<const char *>(p) + q.off;
+            std::memcpy(q.dst, &at, sizeof at);
+        }
+        if (size) CUDA_TRY(cudaMemcpyAsync(p, c->stage, size, cudaMemcpyHostToDevice, 0));
         return DRT_OK;
     }
 };
@@ -840,6 +857,7 @@ void drt_destroy(drt_ctx *c) {
                        &c->tr_faces, &c->tr_rays, &c->tr_count})
         if (s->ptr) cudaFree(s->ptr);
     cudaFree(c->probe_sink);
+    if (c->stage) cudaFreeHost(c->stage);
     for (int i = 0; i < 2; ++i) {
         if (c->side[i]) cudaStreamDestroy(c->side[i]);
         if (c->ev_join[i]) cudaEventDestroy(c->ev_join[i]);
@@ -861,27 +879,27 @@ namespace {
 // validate, pack and upload one link (the caller holds the context lock and set the device)
 void free_link(drt_ctx *c, Link &L);
 
-drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Link &L) {
+// scene: the host copy that *s is a view of, when there is one already
+drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Link &L,
+                     std::shared_ptr<HostScene> scene = nullptr) {
     PackedLink H;
     if (drt_status st = pack_link(s, ps, H)) return st;
-    auto hs = std::make_shared<HostScene>();
-    hs->tx = s->tx;
-    hs->rx = s->rx;
-    hs->bodies.assign(s->bodies, s->bodies + s->n_bodies);
-    hs->mats.assign(s->materials, s->materials + s->n_materials);
-    hs->faces.assign(s->faces, s->faces + s->n_faces);
-    hs->edges.assign(s->edges, s->edges + s->n_edges);
-    hs->tiles.assign(s->tiles, s->tiles + s->n_tiles);
+    auto hs = scene ? scene : std::make_shared<HostScene>();
+    if (!scene) {
+        hs->tx = s->tx;
+        hs->rx = s->rx;
+        hs->bodies.assign(s->bodies, s->bodies + s->n_bodies);
+        hs->mats.assign(s->materials, s->materials + s->n_materials);
+        hs->faces.assign(s->faces, s->faces + s->n_faces);
+        hs->edges.assign(s->edges, s->edges + s->n_edges);
+        hs->tiles.assign(s->tiles, s->tiles + s->n_tiles);
+    }
     L.scene = hs;
     L.dev = H.dev;
     L.view = H.view;
     L.n_paths = ps->n_paths;
     LinkDev &d = L.dev;
     LinkImage img;
-    auto bytes = [](const auto &...v) { return ((v.size() * sizeof(v[0]) + 256) + ...); };
-    img.host.reserve(bytes(H.bodies, H.body_fixed, H.faces, H.edges, H.tiles, H.mats, H.facesF, H.edgesF, H.tilesF, H.facesQ,
-                           H.edgesQ, H.tilesQ, H.bodiesQ, H.ptypes, H.pprims, H.ps0, H.perm) +
-                     (size_t)(d.n_paths - d.n_bulk) * 2 * MAXI * sizeof(double) + 256);
     img.add(H.bodies, &d.bodies);
     img.add(H.body_fixed, &d.body_fixed);
     img.add(H.faces, &d.faces);
@@ -907,8 +925,11 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     if (!st && n_t0) {
         // at t = 0, whatever the grids of later calls: edge parameters only (1e-6 m is enough of a start)
         cudaError_t e = launch_t0par(d, const_cast<double *>(d.t0par), 0, L.view.ff_range && L.view.extent < 1e5);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
         if (e != cudaSuccess) st = fail(DRT_ECUDA, "t0 edge parameters: %s", cudaGetErrorString(e));
+    }
+    {   // the copy and the solve are done when the call returns, whatever stream uses the link next
+        cudaError_t e = cudaStreamSynchronize(0);
+        if (!st && e != cudaSuccess) st = fail(DRT_ECUDA, "link upload: %s", cudaGetErrorString(e));
     }
     if (st) {
         free_link(c, L);
@@ -1157,7 +1178,7 @@ drt_status drt_synthesize_H_wideband(drt_ctx *c, uint64_t link, const drt_time_g
 namespace {
 
 // conventional ray tracing at t over a link's scene into host arrays (the context lock is held)
-drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_tiles, drt_traced_paths *out,
+drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_tiles, std::vector<char> &rays, int *n_rays,
                       cudaStream_t s) {
     const long long n_cand = trace_candidates(L.dev, max_order, with_tiles);
     const int cap_dev = (int)std::min<long long>(n_cand, 1 << 22);
@@ -1175,9 +1196,9 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
         if (count <= cap_dev) break;
     }
     if (count > cap_dev) return fail(DRT_ENOMEM, "ray tracing found %d rays, more than %d", count, cap_dev);
-    std::vector<char> rays((size_t)count * trace_ray_bytes());
+    rays.resize((size_t)count * trace_ray_bytes());
     if (count) CUDA_TRY(cudaMemcpy(rays.data(), c->tr_rays.ptr, rays.size(), cudaMemcpyDeviceToHost));
-    out->n_found = trace_unpack(rays.data(), count, out->n_int, out->types, out->prims, out->s0, out->cap);
+    *n_rays = count;
     return DRT_OK;
 }
 
@@ -1201,7 +1222,11 @@ drt_status drt_trace_paths(drt_ctx *c, uint64_t link, double t, int32_t max_orde
     Link *L = find_link(c, link);
     if (!L) return fail(DRT_ENOTFOUND, "unknown link %llu", (unsigned long long)link);
     CUDA_TRY(cudaSetDevice(c->device));
-    return trace_into(c, *L, t, max_order, with_tiles != 0, out, (cudaStream_t)stream);
+    std::vector<char> rays;
+    int n = 0;
+    if (drt_status st = trace_into(c, *L, t, max_order, with_tiles != 0, rays, &n, (cudaStream_t)stream)) return st;
+    out->n_found = trace_unpack(rays.data(), n, out->n_int, out->types, out->prims, out->s0, out->cap);
+    return DRT_OK;
 }
 
 drt_status drt_synthesize_H_retraced(drt_ctx *c, uint64_t link, const drt_time_grid *tg, const drt_freq_grid *fg,
@@ -1225,21 +1250,26 @@ drt_status drt_synthesize_H_retraced(drt_ctx *c, uint64_t link, const drt_time_g
     cudaStream_t s = (cudaStream_t)stream;
     const int F = fg->n_bins;
     const drt_scene scene = L->scene->view();
+    std::vector<char> rays;
+    std::vector<uint8_t> n_int, types;
+    std::vector<int32_t> prims;
+    std::vector<double> s0;
     for (int w = 0; w < n_windows && T > 0; ++w) {
         const int k0 = starts[w], k1 = w + 1 < n_windows ? starts[w + 1] : T;
         const double tw = tg->t_start + k0 * tg->dt;
         // the window's chains: a ray-tracing run at its first instant
-        const long long n_cand = trace_candidates(L->dev, max_order, with_tiles != 0);
-        const int cap = (int)std::min<long long>(n_cand, 1 << 22);
-        std::vector<uint8_t> n_int(cap), types((size_t)cap * MAXI);
-        std::vector<int32_t> prims((size_t)cap * MAXI);
-        std::vector<double> s0((size_t)cap * MAXI);
-        drt_traced_paths tp{cap, 0, n_int.data(), types.data(), prims.data(), s0.data()};
-        if (drt_status st = trace_into(c, *L, tw, max_order, with_tiles != 0, &tp, s)) return st;
+        int listed = 0;
+        if (drt_status st = trace_into(c, *L, tw, max_order, with_tiles != 0, rays, &listed, s)) return st;
+        n_int.resize(listed);
+        types.resize((size_t)listed * MAXI);
+        prims.resize((size_t)listed * MAXI);
+        s0.resize((size_t)listed * MAXI);
+        drt_traced_paths tp{listed, 0, n_int.data(), types.data(), prims.data(), s0.data()};
+        tp.n_found = trace_unpack(rays.data(), listed, tp.n_int, tp.types, tp.prims, tp.s0, tp.cap);
         // extrapolated over the window's instants into its rows of H
         const drt_path_set ps{tp.n_found, 0, n_int.data(), types.data(), prims.data(), s0.data()};
         Link W;
-        if (drt_status st = load_link(c, &scene, &ps, W)) return st;
+        if (drt_status st = load_link(c, &scene, &ps, W, L->scene)) return st;
         const drt_time_grid tw_grid{tw, tg->dt, k1 - k0, 0};
         drt_status st = synth_into(c, W, &tw_grid, fg, reinterpret_cast<float2 *>(H) + (size_t)k0 * F, precision, s,
                                    nullptr, F);
