@@ -409,18 +409,25 @@ DRT_HD void path_base_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
     }
 }
 
-// App. A Eq. doppler_freq (doppler<N>, drt_physics.cuh) to second order in v / c: sum_i log1p(-u_i) - log1p(-u_{i-1}) with u = v.k / c of
-// ~1e-6, whose third-order terms are below 1e-17, and expm1 alike
+// App. A Eq. doppler_freq (doppler<N>, drt_physics.cuh): sum_i log1p(-u_i) - log1p(-u_{i-1}) with u = v.k / c, to second order while every
+// |u| is below 1e-5 (the third-order terms are then below 1e-10 of the first).  The points of a chain that is no ray may run faster
+// than that: FP64 logarithms there.
 template <int N> DRT_HD float doppler_ff(const v3<dl<ff>> *V, const v3<ff> *seg, const FreqGridD &fg) {
     ff s1 = ff(0.f);
-    float s2 = 0.f;
+    float s2 = 0.f, big = 0.f;
+    double full = 0.0;
 #pragma unroll
     for (int i = 1; i <= N + 1; ++i) {
         const v3<ff> k = unit(seg[i]);
         const ff u1 = dot(der(V[i]), k), u0 = dot(der(V[i - 1]), k);
         s1 = s1 + (u0 - u1);
         s2 += (u0.h - u1.h) * (u0.h + u1.h);
+        const float m = fmaxf(fabsf(u0.h), fabsf(u1.h));
+        big = fmaxf(big, m);
+        if (!(m < 1e-5f * (float)C0)) full += log1p(-to_double(u1) * (1 / C0)) - log1p(-to_double(u0) * (1 / C0));
+        else full += to_double(u0 - u1) * (1 / C0);
     }
+    if (!(big < 1e-5f * (float)C0)) return (float)(fg.fc * expm1(full));
     const ff S = s1 * ff(1 / C0) + ff(s2 * (float)(0.5 / (C0 * C0)));
     return (fg.kq * ff(C0 / (2 * PI)) * (S + halve(S * S))).h;   // fc = k c / 2 pi
 }

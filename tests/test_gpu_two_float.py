@@ -101,3 +101,26 @@ def test_large_scene_keeps_fp64():
         want = torch.empty_like(H)
         link.synthesize_H_noalloc(tg, fg, want)
         assert bool(H.abs().max() > 0) and torch.equal(H, want)
+
+
+@pytest.mark.parametrize("name,k", [("link", 0), ("link", 1), ("link", 2), ("link", 3), ("canyon", 0)])
+def test_doppler_of_redone_steps(name, k):
+    """The FP32-bulk records' redone steps (their delay is the FP64 one to 1e-12; an FP32 step's is within 1e-9 of it, but for the first
+    step of a chunk, a multiple of 4, whose delay is an FP64 anchor while its Doppler shift is FP32) have the FP64 Doppler shift to FP32 rounding, also where a point of a chain that is no ray runs at a good part of the speed of light: 1e-6
+    covers the rounding of the result and of the velocities (2^-40)."""
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2205_00237_gb300 import drt
+    scene, paths = base(name, k)
+    tg, fg = I.TimeGrid(0.0, 1e-3, 1237), I.FreqGrid(60e9 if name == "canyon" else 28e9, 400e6, 1)
+    with drt.Context(0) as ctx:
+        link = ctx.load(scene, paths)
+        a = {q: v.cpu().numpy() for q, v in link.extrapolate(tg, fg, drt.FP64).items() if v is not None}
+        b = {q: v.cpu().numpy() for q, v in link.extrapolate(tg, fg, drt.FP32_BULK).items() if v is not None}
+    fine = (a["flags"] & 24) == 0   # converged and not degenerate
+    redone = fine & (np.abs(b["tau"] / a["tau"] - 1) < 1e-12) & (a["flags"] == b["flags"])
+    redone[::4] = False
+    assert redone.any()
+    err = np.abs(b["doppler"] - a["doppler"])[redone]
+    # a step of FP32 geometry whose delay agrees by chance keeps the FP32 form's 0.1 Hz
+    assert (err <= np.maximum(1e-6 * np.abs(a["doppler"][redone]), 0.1)).all(), err.max()
