@@ -6,29 +6,39 @@
 
 namespace drt {
 
-// FP64 redo of queued steps; their contribution is added to H (all bins) with atomics, for the entry
-// and, for a carrier pair, its partner
+// The lanes' steps (link li, path p, step ti; `on`: the lane has one) recomputed, then added to H by the whole warp, one after
+// another: lane l takes the bins l, l + 32, .. (with a lane per step, 32 rows were written at once and the lanes without a step
+// idled through it).  second: the step's carrier partner instead, where it shares the geometry.
 template <bool DUAL>
-__device__ void redo_add_entry(const BatchLink &BL, int p, int ti, bool two) {
-    double r[3];
-    path_step_redo<DUAL>(BL.L, BL.tg, BL.fg, p, ti, BL.out, BL.warm, r, two);
-    if (r[0] == 0.0 && r[1] == 0.0) return;
-    // a exp(-j 2 pi f_k tau): FP64-reduced seed per 16-bin tile, FP32 rotation across the tile
-    const double f0 = BL.fg.f0, df = BL.fg.df;
-    const int F = BL.fg.n_bins;
-    float2 *row = BL.H + (size_t)ti * F;
-    double xs = df * r[2];
-    float ws, wc;
-    sincospif(2.f * (float)(xs - floor(xs)), &ws, &wc);
-    for (int k0 = 0; k0 < F; k0 += 16) {
-        double x = (f0 + k0 * df) * r[2];
-        float sn, cs;
+__device__ void redo_add_warp(const BatchDev &B, int4 itm, bool on, bool second) {
+    int li = itm.x;
+    if (second) {
+        li = on ? B.links[itm.x].partner : -1;
+        on = on && li >= 0 && itm.y >= B.links[itm.x].pair_p0;
+    }
+    double r[3] = {0.0, 0.0, 0.0};
+    if (on) {
+        const BatchLink &BL = B.links[li];
+        path_step_redo<DUAL>(BL.L, BL.tg, BL.fg, itm.y, itm.z, BL.out, BL.warm, r, B.two);
+    }
+    __syncwarp();
+    const int lane = threadIdx.x;
+    for (unsigned left = __ballot_sync(0xffffffffu, r[0] != 0.0 || r[1] != 0.0); left; left &= left - 1) {
+        const int l = __ffs(left) - 1;
+        const float ar = (float)__shfl_sync(0xffffffffu, r[0], l), ai = (float)__shfl_sync(0xffffffffu, r[1], l);
+        const double tau = __shfl_sync(0xffffffffu, r[2], l);
+        const int step = __shfl_sync(0xffffffffu, itm.z, l);
+        const BatchLink &BL = B.links[__shfl_sync(0xffffffffu, li, l)];
+        // a exp(-j 2 pi f_k tau): FP64-reduced seed at the lane's first bin, FP32 rotation by 32 bins
+        const double f0 = BL.fg.f0, df = BL.fg.df, x = (f0 + lane * df) * tau, xs = 32 * df * tau;
+        const int F = BL.fg.n_bins;
+        float2 *row = BL.H + (size_t)step * F;
+        float sn, cs, ws, wc;
         sincospif(2.f * (float)(x - floor(x)), &sn, &cs);
-        const float ar = (float)r[0], ai = (float)r[1];
+        sincospif(2.f * (float)(xs - floor(xs)), &ws, &wc);
         float zr = fmaf(ar, cs, ai * sn), zi = fmaf(ai, cs, -ar * sn);
-        for (int j = 0; j < 16 && k0 + j < F; ++j) {
-            atomicAdd(&row[k0 + j].x, zr);
-            atomicAdd(&row[k0 + j].y, zi);
+        for (int k = lane; k < F; k += 32) {
+            atomicAdd(row + k, make_float2(zr, zi));
             const float nr = fmaf(zr, wc, zi * ws);
             zi = fmaf(zi, wc, -zr * ws);
             zr = nr;
@@ -43,20 +53,24 @@ __global__ void __launch_bounds__(32) k_batch_redo(const BatchDev B) {   // one 
         atomicAdd(hdr + 1, (unsigned long long)*B.redo.count);
         if (*B.redo.count > B.redo.cap) atomicOr(hdr + 2, 1ull);
     }
-    const int n = min(*B.redo.count, B.redo.cap);
-    // few queued steps: one per warp, on one lane (a step is one long dependent FP64 chain; lanes of
-    // different chains would wait for each other's branches); otherwise grid row y takes the chains of
-    // length y, whose code is one instance
-    const bool one = n <= (int)(gridDim.x * gridDim.y);
-    const int k0 = one ? blockIdx.y * gridDim.x + blockIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
-    const int kstep = one ? n + 1 : gridDim.x * blockDim.x;
-    if (one && threadIdx.x != 0) return;
-    for (int k = k0; k < n; k += kstep) {
-        const int4 itm = B.redo.items[k];
-        const BatchLink &BL = B.links[itm.x];
-        if (!one && chain_length(BL.L, itm.y) != (int)blockIdx.y) continue;
-        redo_add_entry<DUAL>(BL, itm.y, itm.z, B.two);
-        if (BL.partner >= 0 && itm.y >= BL.pair_p0) redo_add_entry<DUAL>(B.links[BL.partner], itm.y, itm.z, B.two);
+    // Grid row y takes the chains of y vertices, so that warps that run at the same time run the same code.  Few queued steps: a run
+    // (steps of one path, see for_redo_runs) per warp, the shortest latency.  Many: 32 list places per warp, whose chains'
+    // branches run in turn but which keep the lanes filled (126 000 steps of a 128-link batch: 0.8 ms against 1.4 ms by runs).
+    const int count = *B.redo.count, n = count < B.redo.cap ? count : B.redo.cap, lane = threadIdx.x, y = blockIdx.y;
+    const bool packed = n > 64 * (int)gridDim.x;
+    for (int k = packed ? 32 * blockIdx.x : blockIdx.x; k < n; k += packed ? 32 * gridDim.x : gridDim.x) {
+        int4 itm = make_int4(-1, 0, 0, 0);
+        bool on = k + lane < n;
+        if (!packed) {
+            const int run = B.redo.items[k].w;
+            if (run & 255) continue;   // inside another's run
+            on = on && lane < (run >> 8);
+        }
+        if (on) itm = B.redo.items[k + lane];
+        on = on && chain_length(B.links[itm.x].L, itm.y) == y;
+        if (!__any_sync(0xffffffffu, on)) continue;
+        redo_add_warp<DUAL>(B, itm, on, false);
+        if (__any_sync(0xffffffffu, on && B.links[itm.x].partner >= 0)) redo_add_warp<DUAL>(B, itm, on, true);
     }
 }
 

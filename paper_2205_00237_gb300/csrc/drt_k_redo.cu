@@ -7,28 +7,14 @@ namespace drt {
 
 // The same redo beside the H synthesis: each queued step's (Re a, Im a, tau) goes to out3 (its record
 // keeps a = 0, so the synthesis skips it), and k_redo_add then adds a exp(-j 2 pi f tau) into H.
-// A queued step is one long dependent FP64 chain, so the kernel's time is the latency of its slowest
-// warp.  With no more queued steps than warps, each warp takes one step on one lane: no two chains
-// share a warp, so none waits for another's branches.  Otherwise grid row y takes the steps of chains
-// of length y (each length is its own code instance, which lanes of one warp would run in turn).
+// A queued step is one long dependent chain, so the kernel's time is the latency of its slowest warp (see for_redo_runs).
 __global__ void __launch_bounds__(32)
 k_redo_rec(const __grid_constant__ LinkDev L, const __grid_constant__ TimeGridD tg, const __grid_constant__ FreqGridD fg,
            const RedoList redo, const double *__restrict__ warm, double *__restrict__ out3, bool two) {
-    const int n = min(*redo.count, redo.cap);
     const OutD none{};
-    const int warp = blockIdx.y * gridDim.x + blockIdx.x;
-    if (n <= (int)(gridDim.x * gridDim.y)) {
-        if (threadIdx.x == 0 && warp < n) {
-            const int4 it = redo.items[warp];
-            path_step_redo<false>(L, tg, fg, it.y, it.z, none, warm, out3 + 3 * (size_t)warp, two);
-        }
-        return;
-    }
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int4 it = redo.items[k];
-        if (chain_length(L, it.y) != (int)blockIdx.y) continue;
+    for_redo_runs(redo, blockIdx.x, gridDim.x, threadIdx.x, [&](int k, int4 it) {
         path_step_redo<false>(L, tg, fg, it.y, it.z, none, warm, out3 + 3 * (size_t)k, two);
-    }
+    });
 }
 
 // one thread per (queued step, 16-bin tile): FP64-reduced seed, FP32 rotation across the tile
@@ -61,7 +47,7 @@ k_redo_add(const FreqGridD fg, const RedoList redo, const double *__restrict__ i
 cudaError_t launch_redo_rec(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, void *redo, const double *warm,
                             double *out3, cudaStream_t s, bool two) {
     if (L.n_paths == 0 || tg.n_steps == 0) return cudaSuccess;
-    k_redo_rec<<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, redo_list(redo, L, tg), warm, out3, two);
+    k_redo_rec<<<152 * 16, 32, 0, s>>>(L, tg, fg, redo_list(redo, L, tg), warm, out3, two);
     return cudaGetLastError();
 }
 

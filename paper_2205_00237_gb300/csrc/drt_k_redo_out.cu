@@ -5,33 +5,20 @@
 
 namespace drt {
 
-// FP64 redo of the queued path-steps: a fixed grid strides over the device-side count, one warp per
-// block (the few queued steps spread over all SMs; each is a long FP64 chain), grid row y taking the
-// chains of length y (one code instance per length: a warp runs one of them)
+// redo of the queued path-steps: a fixed grid strides over the device-side count, one warp per block (see for_redo_runs)
 template <bool DUAL>
 __global__ void __launch_bounds__(32)
 k_redo(const __grid_constant__ LinkDev L, const __grid_constant__ TimeGridD tg, const __grid_constant__ FreqGridD fg,
        const OutD out, const RedoList redo, const double *__restrict__ warm, bool two) {
-    int n = min(*redo.count, redo.cap);
-    const int warp = blockIdx.y * gridDim.x + blockIdx.x;
-    if (n <= (int)(gridDim.x * gridDim.y)) {   // few queued steps: one per warp (see k_redo_rec)
-        if (threadIdx.x == 0 && warp < n) {
-            const int4 it = redo.items[warp];
-            path_step_redo<DUAL>(L, tg, fg, it.y, it.z, out, warm, nullptr, two);
-        }
-        return;
-    }
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int4 it = redo.items[k];
-        if (chain_length(L, it.y) != (int)blockIdx.y) continue;
+    for_redo_runs(redo, blockIdx.x, gridDim.x, threadIdx.x, [&](int, int4 it) {
         path_step_redo<DUAL>(L, tg, fg, it.y, it.z, out, warm, nullptr, two);
-    }
+    });
 }
 
 #ifdef DRT_REDO_DUAL   // drt_k_redo_out_dual.cu: with the rates the Doppler output needs
 cudaError_t launch_redo_dual(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const OutD &out, void *redo,
                              const double *warm, cudaStream_t s, bool two) {
-    k_redo<true><<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
+    k_redo<true><<<152 * 16, 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
     return cudaGetLastError();
 }
 #else
@@ -42,7 +29,7 @@ cudaError_t launch_redo(const LinkDev &L, const TimeGridD &tg, const FreqGridD &
                         const double *warm, cudaStream_t s, bool two) {
     if (L.n_paths == 0 || tg.n_steps == 0) return cudaSuccess;
     if (out.doppler) return launch_redo_dual(L, tg, fg, out, redo, warm, s, two);
-    k_redo<false><<<dim3(152 * 4, MAXI + 1), 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
+    k_redo<false><<<152 * 16, 32, 0, s>>>(L, tg, fg, out, redo_list(redo, L, tg), warm, two);
     return cudaGetLastError();
 }
 #endif
