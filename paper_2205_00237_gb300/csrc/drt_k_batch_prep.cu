@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(128) k_stage(const BatchDev B) {
             else body_pose_row(BL.L.bodies[b], tb, BL.pose64 + local * POSE_W);
         } else if (STAGE == ST_WARM) {   // rows 0..nch
             int p = BL.L.n_bulk + (int)(local / (nch + 1)), c = (int)(local % (nch + 1));
-            if constexpr (TWO) path_warm_ff(BL.L, BL.tg, p, c, BL.warm);
+            if constexpr (TWO) path_warm_ff<true>(BL.L, BL.tg, p, c, BL.warm);
             else path_warm_fp64(BL.L, BL.tg, p, c, BL.warm);
         } else {
             int p = (int)(local / nch), c = (int)(local % nch);

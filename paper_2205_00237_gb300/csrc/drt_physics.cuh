@@ -283,6 +283,9 @@ template <> DRT_HD void clamp_positive<float>(float &x, float eps) {
 template <> DRT_HD void clamp_positive<ff>(ff &x, ff eps) {
     if (!(x > eps)) x = eps;
 }
+template <> DRT_HD void clamp_positive<dl<float>>(dl<float> &x, float eps) {
+    if (!(x.v > eps)) x.v = eps;
+}
 template <> DRT_HD void clamp_positive<dl<ff>>(dl<ff> &x, ff eps) {
     if (!(x.v > eps)) x.v = eps;
 }
@@ -302,6 +305,9 @@ template <> DRT_HD void clamp_positive<dd>(dd &x, float eps) {
 // Newton start for an edge parameter from its value `base` + `delta` and rate: for delta numbers
 // the base part is `base` (the chunk-base solution) and the delta `delta`
 template <class S> DRT_HD S newton_start(double base, double delta, double rate);
+template <> DRT_HD dl<float> newton_start<dl<float>>(double base, double delta, double rate) {
+    return {(float)(base + delta), (float)rate};
+}
 template <> DRT_HD dl<ff> newton_start<dl<ff>>(double base, double delta, double rate) {
     return {from_double(base + delta), from_double(rate)};
 }

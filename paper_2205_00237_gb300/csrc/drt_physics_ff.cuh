@@ -251,9 +251,12 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
 // cannot resolve.  They are short dependent chains (a few solves per path), so what they cost is latency: 65 cycles per FP64
 // instruction, a few per FP32 one.
 
-// The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, one two-float dual step for the
-// rates.  False where it did not converge (the caller runs the FP64 solve).
-template <int N> DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
+// The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, a dual-number step for the rates.  False
+// where it did not converge (the caller runs the FP64 solve).  RATE32: the rates in FP32 dual numbers, for the FP32-bulk form, where
+// they only place the Newton starts between the chunk bases (an error of 1e-5 of 10 m/s is 1e-6 m over a chunk, the size of
+// the FP32 rounding of the coordinates), and the unknowns only.
+template <int N, bool RATE32>
+DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     const uint32_t code = L.ptypes[p];
     const int4 pi = L.pprims[p];
     const int prim[MAXI] = {pi.x, pi.y, pi.z, pi.w};
@@ -308,6 +311,30 @@ template <int N> DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, doubl
         for (int j = 0; j < N; ++j)
             if (nv[j + 1]) s1[j] = to_double(dot(Vd[j + 1] - pd[j].p, pd[j].a));
     }
+    if constexpr (RATE32) {
+        Prim<dl<float>> pf[N];
+        v3<dl<float>> Vf[N + 2];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            pf[j].type = pr[j].type;
+            pf[j].p = dual(f32v(val(pr[j].p)), f32v(der(pr[j].p)));
+            pf[j].a = dual(f32v(val(pr[j].a)), f32v(der(pr[j].a)));
+        }
+#pragma unroll
+        for (int i = 0; i <= N + 1; ++i) Vf[i] = dual(f32v(val(V[i])), f32v(der(V[i])));
+        newton_diffractions<N>(pf, Vf, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
+        bool ok = !(fl & F_NOCONV);
+#pragma unroll
+        for (int j = 0; j < MAXI; ++j) {
+            sv[j] = s1[j];
+            sd[j] = 0.0;
+            if (j < N && nv[j + 1 < N + 1 ? j + 1 : N]) {
+                sd[j] = dot(Vf[j + 1 < N + 1 ? j + 1 : N] - pf[j < N ? j : 0].p, pf[j < N ? j : 0].a).d;
+                ok = ok && isfinite(sv[j]) && isfinite(sd[j]);
+            }
+        }
+        return ok;
+    }
     newton_diffractions<N>(pr, V, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
     bool ok = !(fl & F_NOCONV);
     // the diffractions alone in their stretch: on their Keller cones
@@ -331,25 +358,27 @@ template <int N> DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, doubl
 template <int N> DRT_NOINL void solve_edge_params_fp64(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     solve_edge_params<N>(L, p, t, sin, sv, sd, [&](int ty, int idx) { return load_prim_direct<double>(L, t, ty, idx); });
 }
+template <bool RATE32>
 DRT_HD void edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     with_length<2>(chain_length(L, p), [&](auto NC) {
         constexpr int N = decltype(NC)::value;
         double start[MAXI];
         for (int j = 0; j < MAXI; ++j) start[j] = sin[j];
-        if (!solve_edge_params_ff<N>(L, p, t, start, sv, sd)) solve_edge_params_fp64<N>(L, p, t, start, sv, sd);
+        if (!solve_edge_params_ff<N, RATE32>(L, p, t, start, sv, sd)) solve_edge_params_fp64<N>(L, p, t, start, sv, sd);
     });
 }
 // path_t0par_fp64 and path_warm_fp64 (drt_physics.cuh) on it
 DRT_HD void path_t0par_ff(const LinkDev &L, int p, double *out) {
-    edge_params_ff(L, p, 0.0, L.ps0 + (size_t)p * MAXI, out, out + MAXI);
+    edge_params_ff<false>(L, p, 0.0, L.ps0 + (size_t)p * MAXI, out, out + MAXI);
 }
+template <bool RATE32>
 DRT_HD void path_warm_ff(const LinkDev &L, const TimeGridD &tg, int p, int row, double *warm) {
     const double t = tg.t_start + (double)row * tg.chunk * tg.dt;
     const double *q = L.t0par + (size_t)(p - L.n_bulk) * (2 * MAXI);
     double start[MAXI];
     for (int j = 0; j < MAXI; ++j) start[j] = q[j] + q[MAXI + j] * t;
     double *w = warm + ((size_t)row * (L.n_paths - L.n_bulk) + (p - L.n_bulk)) * (2 * MAXI);
-    edge_params_ff(L, p, t, start, w, w + MAXI);
+    edge_params_ff<RATE32>(L, p, t, start, w, w + MAXI);
 }
 
 // path_base_fp64 (drt_physics.cuh): anchors of a (path, chunk) from the poses at the chunk bases [body][chunk]
