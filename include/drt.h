@@ -174,7 +174,8 @@ drt_status drt_synthesize_H_host(drt_ctx *ctx, uint64_t link, const drt_time_gri
  * that cannot allocate device memory at call time: latency-bound anticipative-prediction loops,
  * where cudaMalloc / cudaFree may synchronise the device and stall for milliseconds, and processes
  * whose device memory is already fully reserved by another allocator).  Same inputs, output and
- * result as drt_synthesize_H's FP64 form (the same launches), but the pose table, the warm-start
+ * result as drt_synthesize_H's FP64 form, computed in FP64 throughout (the FP64 form's records take
+ * two-float arithmetic where that gives the same FP32 records), but the pose table, the warm-start
  * table of the chains with several diffractions in one segment and the synthesis records live in one
  * static device array of DRT_NOALLOC_SCRATCH_BYTES (32 MiB) that the library reserves on every
  * device that loads it, until the process exits; the call makes no cudaMalloc, cudaFree or other

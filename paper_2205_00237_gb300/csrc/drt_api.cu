@@ -369,7 +369,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
         CUDA_TRY(cudaEventRecord(c->ev_fork, s));
         CUDA_TRY(cudaStreamWaitEvent(sa, c->ev_fork, 0));
         CUDA_TRY(cudaStreamWaitEvent(sw, c->ev_fork, 0));
-        if (drt_status st = traced(c, 3, sw, [&] { return launch_warm_fp64(L.dev, t, warm, sw, two, true); })) return st;
+        if (drt_status st = traced(c, 3, sw, [&] { return launch_warm_fp64(L.dev, t, warm, sw, two); })) return st;
         if (drt_status st = traced(c, 3, sa, [&] { return launch_base_pose64(L.dev, t, p64, sa, two); })) return st;
         CUDA_TRY(cudaEventRecord(ev_p64, sa));
         if (drt_status st = traced(c, 3, sa, [&] { return launch_base_paths(L.dev, t, f, p64, bs, warm, 0, nb, sa, two); }))
@@ -442,7 +442,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
         cudaError_t e = cudaEventRecord(c->ev_fork, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s0, c->ev_fork, 0);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s1, c->ev_fork, 0);
-        if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1, ff_applies(L.view, *tg, *fg));
+        if (e == cudaSuccess) e = launch_warm_fp64(D, t, warm, s1, false);   // FP64 Newton steps follow: FP64 starts
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s1, ls[MAXI], -1, false, warm);
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s1, ls[1], ls[2], false, warm);
         if (e == cudaSuccess) e = launch_extrapolate_fp64(D, t, f, pose, out, rec, s0, ls[2], ls[3], false, warm);
@@ -1398,7 +1398,7 @@ extern "C" drt_status drt_synthesize_H_noalloc(drt_ctx *c, uint64_t link, const 
              reinterpret_cast<float *>(base + pose_bytes + warm_sz + reca_bytes)};
     cudaStream_t s = (cudaStream_t)stream;
     OutD none{};
-    // the same launches as drt_synthesize_H's FP64 form: pose table, multi-diffraction warm starts,
+    // drt_synthesize_H's FP64 form on the FP64 kernels: pose table, multi-diffraction warm starts,
     // extrapolation into the records, synthesis
     CUDA_TRY(launch_pose(L->dev, t, pose, s));
     CUDA_TRY(launch_warm_fp64(L->dev, t, warm, s, false));

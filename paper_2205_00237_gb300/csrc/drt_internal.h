@@ -230,9 +230,7 @@ cudaError_t launch_extrapolate_ff_generic(const LinkDev &L, const TimeGridD &tg,
 // edge parameters and rates at t = 0 of the multi-diffraction paths (LinkDev::t0par), at load
 // two: in two-float numbers (the caller has checked that they apply), here and below
 cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s, bool two);
-// rate32: the rates to FP32 accuracy (two only)
-cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two,
-                             bool rate32 = false);
+cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two);
 // FP32-bulk form (CHUNK consecutive steps share FP64 anchors); see drt_physics.cuh.  Scratch:
 // per-(body or terminal, chunk) FP32 base poses and per-(path, chunk) FP64 anchors.
 size_t bulk_pose_bytes(const LinkDev &L, const TimeGridD &tg);

@@ -31,13 +31,12 @@ k_warm_fp64(const LinkDev L, const TimeGridD tg, double *__restrict__ warm) {
     path_warm_fp64(L, tg, p, c, warm);
 }
 // the same in two-float numbers
-template <bool RATE32>
 __global__ void __launch_bounds__(WARM_T)
 k_warm_ff(const __grid_constant__ LinkDev L, const TimeGridD tg, double *__restrict__ warm) {
     int p = L.n_bulk + blockIdx.x;
     int c = blockIdx.y * WARM_T + threadIdx.x;
     if (p >= L.n_paths || c > n_chunks_of(tg)) return;
-    path_warm_ff<RATE32>(L, tg, p, c, warm);
+    path_warm_ff(L, tg, p, c, warm);
 }
 
 // one path per warp (lane 0): the chains' lengths differ, and each length is its own code instance
@@ -61,11 +60,10 @@ cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s, bool t
     return cudaGetLastError();
 }
 
-cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two, bool rate32) {
+cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two) {
     if (!warm || L.n_bulk >= L.n_paths || tg.n_steps == 0) return cudaSuccess;
     dim3 gw(L.n_paths - L.n_bulk, (n_chunks_of(tg) + 1 + WARM_T - 1) / WARM_T);
-    if (two && rate32) k_warm_ff<true><<<gw, WARM_T, 0, s>>>(L, tg, warm);
-    else if (two) k_warm_ff<false><<<gw, WARM_T, 0, s>>>(L, tg, warm);
+    if (two) k_warm_ff<<<gw, WARM_T, 0, s>>>(L, tg, warm);
     else k_warm_fp64<<<gw, WARM_T, 0, s>>>(L, tg, warm);
     return cudaGetLastError();
 }

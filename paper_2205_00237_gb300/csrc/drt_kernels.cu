@@ -216,8 +216,7 @@ k_select(const LinkDev L, const TimeGridD tg, const FreqGridD fg, WinMask wm, co
     const int w = (int)(q / L.n_paths), p = (int)(q % L.n_paths);
     OutD o{};
     o.flags = wm.sel;   // written at [starts[w]][caller index]
-    const RecD none{nullptr, nullptr};
-    path_step_redo_as<false>(L, tg, fg, p, wm.starts[w], o, none, warm);   // flags only: values suffice
+    path_step_fp64_at(L, tg, fg, p, wm.starts[w], o, warm);   // flags only: values suffice
 }
 
 cudaError_t launch_select(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, const WinMask &wm,

@@ -411,7 +411,7 @@ template <int N, class S> DRT_HD void place_reflections(const Prim<S> *pr, v3<S>
 // -- to the next, through the reflections in between) and eliminates each unknown of the
 // tridiagonal system at the anchor that closes its outgoing leg; the back substitution runs the
 // other way.  Nothing is indexed at run time.
-template <int N, class S, class D = double>
+template <int N, int MAXIT = 64, class S, class D = double>
 DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, const double *s0, const D *ds0,
                                 const D *rate0, uint32_t &fl) {
     typedef typename ST<S>::R T;
@@ -436,7 +436,7 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
     int halvings = 0;
     T Lprev = T(0), smax_prev = T(0);
     bool have_prev = false;
-    for (int it = 0; it < 64; ++it) {
+    for (int it = 0; it < MAXIT; ++it) {
         // cpS[i], dpS[i]: elimination of the unknown whose outgoing leg ends at anchor i (cl[i])
         S cpS[N + 2], dpS[N + 2];
         bool cl[N + 2];
@@ -2295,21 +2295,14 @@ DRT_HD void path_step_bulk(const LinkDev &L, const TimeGridD &tg, const FreqGrid
     }
 }
 
-// FP64 redo of one queued FP32-bulk path-step (FP32 output formats); DUAL: with the rates the Doppler
-// output needs (dual numbers), else values only
-template <bool DUAL>
-DRT_HD void path_step_redo_as(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti,
-                              const OutD &out, const RecD &rec, const double *warm, double *rec64 = nullptr) {
+// one FP64 path-step (values only, FP32 output formats) posed from the bodies' kinematics
+DRT_HD void path_step_fp64_at(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti, const OutD &out,
+                              const double *warm) {
     const double t = tg.t_start + ti * tg.dt;
-    if constexpr (DUAL) {
-        path_step_fp64_core<LEN_ANY, true, true, dl<double>>(
-            L, tg, fg, p, ti, out, rec, true, [&](int ty, int idx) { return load_prim_direct<double>(L, t, ty, idx); },
-            warm, rec64);
-    } else {
-        path_step_fp64_core<LEN_ANY, true, true, double>(
-            L, tg, fg, p, ti, out, rec, true,
-            [&](int ty, int idx) { return val_prim(load_prim_direct<double>(L, t, ty, idx)); }, warm, rec64);
-    }
+    const RecD none{nullptr, nullptr};
+    path_step_fp64_core<LEN_ANY, true, true, double>(
+        L, tg, fg, p, ti, out, none, true,
+        [&](int ty, int idx) { return val_prim(load_prim_direct<double>(L, t, ty, idx)); }, warm);
 }
 
 // one (path, step) of the FP64 form from the per-step pose table; DUAL = false when no Doppler

@@ -4,6 +4,7 @@
 // carry the path length to ~1e-10 m and the decisions exactly.  Two-float arithmetic does the first with 47 bits; a step that it
 // cannot decide (a validity margin within 2^-36 of the coordinates, a virtual terminal on an edge line, a boundary of the
 // transition function, a Newton solve that did not converge, anything not finite) is computed in FP64 by the lane that met it.
+// Canyon call (512 paths x 2000 steps x 512 bins) 1.93 -> 0.54 ms against the FP64 kernels, 3 paths x 1000 steps 54 -> 33 us.
 #pragma once
 #include "drt_launch.cuh"
 
@@ -249,13 +250,13 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
 // ------------------------------------------------------------------------------------------------
 // The FP64 parts of the FP32-bulk form in two-float numbers: warm starts, anchors at the chunk bases, and the redo of the steps FP32
 // cannot resolve.  They are short dependent chains (a few solves per path), so what they cost is latency: 65 cycles per FP64
-// instruction, a few per FP32 one.
+// instruction, a few per FP32 one.  Canyon: anchors 33 + 23 -> 13 + 21 us, warm starts 77 -> 57, redo 135 -> 94.
 
-// The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, a dual-number step for the rates.  False
-// where it did not converge (the caller runs the FP64 solve).  RATE32: the rates in FP32 dual numbers, for the FP32-bulk form, where
-// they only place the Newton starts between the chunk bases (an error of 1e-5 of 10 m/s is 1e-6 m over a chunk, the size of
-// the FP32 rounding of the coordinates), and the unknowns only.
-template <int N, bool RATE32>
+// The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, one dual-number step for the rates.  False
+// where it did not converge (the caller runs the FP64 solve).  The rates only place Newton starts between the chunk bases and predict
+// them from t = 0, so FP32 dual numbers give them (an error of 1e-5 of 10 m/s is 1e-6 m over a chunk, the size of the FP32
+// rounding of the coordinates; a two-float step took half of the solve's latency) unless FP32 does not resolve the step.
+template <int N>
 DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     const uint32_t code = L.ptypes[p];
     const int4 pi = L.pprims[p];
@@ -311,7 +312,7 @@ DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double
         for (int j = 0; j < N; ++j)
             if (nv[j + 1]) s1[j] = to_double(dot(Vd[j + 1] - pd[j].p, pd[j].a));
     }
-    if constexpr (RATE32) {
+    {
         Prim<dl<float>> pf[N];
         v3<dl<float>> Vf[N + 2];
 #pragma unroll
@@ -322,18 +323,20 @@ DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double
         }
 #pragma unroll
         for (int i = 0; i <= N + 1; ++i) Vf[i] = dual(f32v(val(V[i])), f32v(der(V[i])));
-        newton_diffractions<N>(pf, Vf, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
+        uint32_t f32 = 0;   // one step from the root gives the rates; its value part is the FP32 rounding
+        newton_diffractions<N, 1>(pf, Vf, nv, s1, (const double *)nullptr, (const double *)nullptr, f32);
         bool ok = !(fl & F_NOCONV);
 #pragma unroll
         for (int j = 0; j < MAXI; ++j) {
             sv[j] = s1[j];
             sd[j] = 0.0;
             if (j < N && nv[j + 1 < N + 1 ? j + 1 : N]) {
-                sd[j] = dot(Vf[j + 1 < N + 1 ? j + 1 : N] - pf[j < N ? j : 0].p, pf[j < N ? j : 0].a).d;
-                ok = ok && isfinite(sv[j]) && isfinite(sd[j]);
+                const dl<float> sj = dot(Vf[j + 1 < N + 1 ? j + 1 : N] - pf[j < N ? j : 0].p, pf[j < N ? j : 0].a);
+                sd[j] = sj.d;
+                ok = ok && isfinite(sj.d) && fabsf(sj.v - (float)s1[j]) < 1e-3f;
             }
         }
-        return ok;
+        if (ok) return true;   // else (FP32 does not settle: near grazing) the step below
     }
     newton_diffractions<N>(pr, V, nv, s1, (const double *)nullptr, (const double *)nullptr, fl);
     bool ok = !(fl & F_NOCONV);
@@ -358,27 +361,25 @@ DRT_HD bool solve_edge_params_ff(const LinkDev &L, int p, double t, const double
 template <int N> DRT_NOINL void solve_edge_params_fp64(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     solve_edge_params<N>(L, p, t, sin, sv, sd, [&](int ty, int idx) { return load_prim_direct<double>(L, t, ty, idx); });
 }
-template <bool RATE32>
 DRT_HD void edge_params_ff(const LinkDev &L, int p, double t, const double *sin, double *sv, double *sd) {
     with_length<2>(chain_length(L, p), [&](auto NC) {
         constexpr int N = decltype(NC)::value;
         double start[MAXI];
         for (int j = 0; j < MAXI; ++j) start[j] = sin[j];
-        if (!solve_edge_params_ff<N, RATE32>(L, p, t, start, sv, sd)) solve_edge_params_fp64<N>(L, p, t, start, sv, sd);
+        if (!solve_edge_params_ff<N>(L, p, t, start, sv, sd)) solve_edge_params_fp64<N>(L, p, t, start, sv, sd);
     });
 }
-// path_t0par_fp64 and path_warm_fp64 (drt_physics.cuh) on it
+// path_t0par_fp64 and path_warm_fp64 (drt_physics.cuh) on it; the former's rates serve a linear predictor
 DRT_HD void path_t0par_ff(const LinkDev &L, int p, double *out) {
-    edge_params_ff<false>(L, p, 0.0, L.ps0 + (size_t)p * MAXI, out, out + MAXI);
+    edge_params_ff(L, p, 0.0, L.ps0 + (size_t)p * MAXI, out, out + MAXI);
 }
-template <bool RATE32>
 DRT_HD void path_warm_ff(const LinkDev &L, const TimeGridD &tg, int p, int row, double *warm) {
     const double t = tg.t_start + (double)row * tg.chunk * tg.dt;
     const double *q = L.t0par + (size_t)(p - L.n_bulk) * (2 * MAXI);
     double start[MAXI];
     for (int j = 0; j < MAXI; ++j) start[j] = q[j] + q[MAXI + j] * t;
     double *w = warm + ((size_t)row * (L.n_paths - L.n_bulk) + (p - L.n_bulk)) * (2 * MAXI);
-    edge_params_ff<RATE32>(L, p, t, start, w, w + MAXI);
+    edge_params_ff(L, p, t, start, w, w + MAXI);
 }
 
 // path_base_fp64 (drt_physics.cuh): anchors of a (path, chunk) from the poses at the chunk bases [body][chunk]
@@ -461,7 +462,7 @@ template <int N> DRT_HD float doppler_ff(const v3<dl<ff>> *V, const v3<ff> *seg,
     return (fg.kq * ff(C0 / (2 * PI)) * (S + halve(S * S))).h;   // fc = k c / 2 pi
 }
 
-// FP64 redo of one queued FP32-bulk path-step (path_step_redo_as, drt_physics.cuh) in two-float numbers: FP32 output formats and
+// Redo of one queued FP32-bulk path-step in two-float numbers: FP32 output formats and
 // (Re a, Im a, tau) in rec64, a = 0 where the path does not exist.  False where two-float numbers cannot decide the step.
 template <int N, bool DUAL>
 DRT_HD bool path_step_redo_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int ti, const OutD &out,
