@@ -93,7 +93,7 @@ struct drt_ctx {
     std::map<uint64_t, Link> links;
     uint64_t next_link = 1;
     Scratch pose, rec_a, rec_b, h, poseb, base, pose64, redo, warm, redo3, pp_tau, pp_amp, pp_fd, pp_fl, lt_tot,
-        lt_major, win_sel, win_starts, tr_faces, tr_rays, tr_count;
+        lt_major, win_sel, win_starts, tr_faces, tr_rays, tr_count, tr_prims;
     double *probe_sink = nullptr;
     // side streams for work that overlaps within one call (FP32-bulk: anchors and the FP64
     // multi-diffraction paths run beside the FP32 kernel), joined back with events
@@ -125,7 +125,10 @@ drt_status dev_alloc(drt_ctx *c, size_t bytes, void **out) {
         return fail(DRT_ENOMEM, "HBM budget exceeded: %llu + %llu > %llu bytes", (unsigned long long)c->used,
                     (unsigned long long)bytes, (unsigned long long)c->budget);
     cudaError_t e = cudaMalloc(out, bytes ? bytes : 16);
-    if (e != cudaSuccess) return fail(DRT_ENOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // the call may go on another way: the launch checks after it must not see this error
+        return fail(DRT_ENOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
+    }
     c->used += bytes;
     return DRT_OK;
 }
@@ -185,6 +188,12 @@ drt_status ensure(drt_ctx *c, Scratch &s, size_t bytes) {
     if (st) return st;
     s.cap = want;
     return DRT_OK;
+}
+
+void release(drt_ctx *c, Scratch &s) {
+    cudaDeviceSynchronize();
+    dev_free(c, s.ptr, s.cap);
+    s = Scratch{};
 }
 
 // the arrays of one link packed at 256-byte offsets into one host image, uploaded as one device
@@ -854,7 +863,7 @@ void drt_destroy(drt_ctx *c) {
     for (auto &kv : c->link_pool) cudaFree(kv.second);
     for (Scratch *s : {&c->pose, &c->rec_a, &c->rec_b, &c->h, &c->poseb, &c->base, &c->pose64, &c->redo, &c->warm, &c->redo3, &c->pp_tau,
                        &c->pp_amp, &c->pp_fd, &c->pp_fl, &c->lt_tot, &c->lt_major, &c->win_sel, &c->win_starts,
-                       &c->tr_faces, &c->tr_rays, &c->tr_count})
+                       &c->tr_faces, &c->tr_rays, &c->tr_count, &c->tr_prims})
         if (s->ptr) cudaFree(s->ptr);
     cudaFree(c->probe_sink);
     if (c->stage) cudaFreeHost(c->stage);
@@ -899,29 +908,38 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     L.view = H.view;
     L.n_paths = ps->n_paths;
     LinkDev &d = L.dev;
-    LinkImage img;
-    img.add(H.bodies, &d.bodies);
-    img.add(H.body_fixed, &d.body_fixed);
-    img.add(H.faces, &d.faces);
-    img.add(H.edges, &d.edges);
-    img.add(H.tiles, &d.tiles);
-    img.add(H.mats, &d.mats);
-    img.add(H.facesF, &d.facesF);
-    img.add(H.edgesF, &d.edgesF);
-    img.add(H.tilesF, &d.tilesF);
-    img.add(H.facesQ, &d.facesQ);
-    img.add(H.edgesQ, &d.edgesQ);
-    img.add(H.tilesQ, &d.tilesQ);
-    img.add(H.bodiesQ, &d.bodiesQ);
-    img.add(H.ptypes, &d.ptypes);
-    img.add(H.pprims, &d.pprims);
-    img.add(H.ps0, &d.ps0);
-    img.add(H.perm, &d.perm);
-    // multi-diffraction edge parameters and rates at t = 0 (warm-start predictor), solved below
     const size_t n_t0 = (size_t)(d.n_paths - d.n_bulk) * 2 * MAXI;
     std::vector<double> t0par(n_t0, 0.0);
-    img.add(t0par, &d.t0par);
-    drt_status st = img.upload(c, L);
+    auto image = [&](bool two) {
+        LinkImage img;
+        img.add(H.bodies, &d.bodies);
+        img.add(H.body_fixed, &d.body_fixed);
+        img.add(H.faces, &d.faces);
+        img.add(H.edges, &d.edges);
+        img.add(H.tiles, &d.tiles);
+        img.add(H.mats, &d.mats);
+        img.add(H.facesF, &d.facesF);
+        img.add(H.edgesF, &d.edgesF);
+        img.add(H.tilesF, &d.tilesF);
+        if (two) {   // the two-float copies
+            img.add(H.facesQ, &d.facesQ);
+            img.add(H.edgesQ, &d.edgesQ);
+            img.add(H.tilesQ, &d.tilesQ);
+            img.add(H.bodiesQ, &d.bodiesQ);
+        }
+        img.add(H.ptypes, &d.ptypes);
+        img.add(H.pprims, &d.pprims);
+        img.add(H.ps0, &d.ps0);
+        img.add(H.perm, &d.perm);
+        // multi-diffraction edge parameters and rates at t = 0 (warm-start predictor), solved below
+        img.add(t0par, &d.t0par);
+        return img;
+    };
+    drt_status st = image(true).upload(c, L);
+    if (st == DRT_ENOMEM) {   // no room for the two-float copies: FP64 everywhere
+        L.view.ff_range = false;
+        st = image(false).upload(c, L);
+    }
     if (!st && n_t0) {
         // at t = 0, whatever the grids of later calls: edge parameters only (1e-6 m is enough of a start)
         cudaError_t e = launch_t0par(d, const_cast<double *>(d.t0par), 0, L.view.ff_range && L.view.extent < 1e5);
@@ -1085,17 +1103,30 @@ drt_status drt_lifetime_windows(drt_ctx *c, uint64_t link, const drt_time_grid *
     if (precision == DRT_FP64 && lp->share >= 1e-12 && ff_applies(L->view, *tg, *fg) &&
         ensure(c, c->rec_a, n * sizeof(float4)) == DRT_OK && ensure(c, c->rec_b, n * sizeof(float)) == DRT_OK) {
         const RecD rec{reinterpret_cast<float4 *>(c->rec_a.ptr), reinterpret_cast<float *>(c->rec_b.ptr)};
-        if (drt_status st = run_extrapolation(c, *L, tg, fg, OutD{}, rec, precision, s)) return st;
-        CUDA_TRY(launch_lifetime_rec(rec, T, L->n_paths, lp->share, tot, mj, s));
-        CUDA_TRY(cudaMemcpyAsync(m.data(), mj, (size_t)T + 1, cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-        decided = m[T] == 0;
+        const drt_status st = run_extrapolation(c, *L, tg, fg, OutD{}, rec, precision, s);
+        if (st && st != DRT_ENOMEM) return st;
+        if (!st) {
+            CUDA_TRY(launch_lifetime_rec(rec, T, L->n_paths, lp->share, tot, mj, s));
+            CUDA_TRY(cudaMemcpyAsync(m.data(), mj, (size_t)T + 1, cudaMemcpyDeviceToHost, s));
+            CUDA_TRY(cudaStreamSynchronize(s));
+            decided = m[T] == 0;
+        }
     }
     if (!decided) {
-        if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
-        if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
-        OutD o{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
-        if (drt_status st = run_extrapolation(c, *L, tg, fg, o, none, precision, s)) return st;
+        OutD o{};
+        auto outputs = [&]() -> drt_status {
+            if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
+            if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
+            o = OutD{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
+            return run_extrapolation(c, *L, tg, fg, o, none, precision, s);
+        };
+        drt_status st = outputs();
+        if (st == DRT_ENOMEM) {   // the records taken above (or by an earlier call) may be what exceeds the budget
+            release(c, c->rec_a);
+            release(c, c->rec_b);
+            st = outputs();
+        }
+        if (st) return st;
         CUDA_TRY(launch_lifetime(precision == DRT_FP64, o, T, L->n_paths, lp->share, tot, mj, s));
         CUDA_TRY(cudaMemcpyAsync(m.data(), mj, T, cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
@@ -1182,15 +1213,18 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
                       cudaStream_t s) {
     const long long n_cand = trace_candidates(L.dev, max_order, with_tiles);
     const int cap_dev = (int)std::min<long long>(n_cand, 1 << 22);
-    const bool two = L.view.ff_range && L.view.extent + std::fabs(t) * (L.view.vmax + 0.5 * L.view.amax * std::fabs(t)) < 1e5;
-    if (drt_status st = ensure(c, c->tr_faces, trace_prim_bytes(L.dev))) return st;
+    if (drt_status st = ensure(c, c->tr_faces, (size_t)std::max(L.dev.n_faces, 1) * trace_face_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
+    const bool two = L.view.ff_range && L.view.extent + std::fabs(t) * (L.view.vmax + 0.5 * L.view.amax * std::fabs(t)) < 1e5;
+    // without room for their scratch the FP64 pass alone
+    void *prims = two && ensure(c, c->tr_prims, trace_prim_bytes(L.dev, cap_dev)) == DRT_OK ? c->tr_prims.ptr : nullptr;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);
     // with two-float numbers the list holds the candidates that FP64 has dropped, too: more than it holds is tried again without
     int count = 0;
-    for (int pass = two ? 0 : 1; pass < 2; ++pass) {
-        CUDA_TRY(launch_trace(L.dev, t, max_order, with_tiles, c->tr_faces.ptr, c->tr_rays.ptr, cap_dev, cnt, s, pass == 0));
+    for (int pass = prims ? 0 : 1; pass < 2; ++pass) {
+        CUDA_TRY(launch_trace(L.dev, t, max_order, with_tiles, c->tr_faces.ptr, c->tr_rays.ptr, cap_dev, cnt, s,
+                              pass == 0 ? prims : nullptr));
         CUDA_TRY(cudaMemcpyAsync(&count, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
         if (count <= cap_dev) break;

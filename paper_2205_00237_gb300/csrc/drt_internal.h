@@ -293,11 +293,12 @@ cudaError_t launch_probe(int kind, int blocks, double *sink, cudaStream_t s, flo
 // `count` rays into path-set arrays in enumeration order
 long long trace_candidates(const LinkDev &L, int max_order, int with_tiles);
 size_t trace_ray_bytes();
-size_t trace_prim_bytes(const LinkDev &L);   // faces and edges posed at the instant
-// two: candidates are solved in two-float numbers first, and FP64 decides what those leave open (see drt_trace.cu); trace_unpack returns
-// the number of rays
+size_t trace_face_bytes();
+size_t trace_prim_bytes(const LinkDev &L, int cap);   // scratch of the two-float passes
+// prims (trace_prim_bytes) non-null: candidates are solved in two-float numbers first, and FP64 decides what those leave open (see
+// drt_trace.cu); trace_unpack returns the number of rays
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s, bool two);
+                         int *count, cudaStream_t s, void *prims);
 int trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0,
                   int cap);
 

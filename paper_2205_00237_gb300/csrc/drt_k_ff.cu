@@ -18,7 +18,7 @@ k_pose_ff(const BodyQ *__restrict__ bodies, int n_bodies, TermD tx, TermD rx, do
         body_pose_ff(bodies[b], from_double(t), pose[i]);
     } else {
         const v3<double> r = val(terminal<double>(b == n_bodies ? tx : rx, t));
-        term[i - n_bodies * n_steps] = PointQ{{from_double(r.x), from_double(r.y), from_double(r.z)}, ff(0.f)};
+        term[i - n_bodies * n_steps] = PointQ{{from_double(r.x), from_double(r.y), from_double(r.z)}};
     }
 }
 

@@ -12,7 +12,7 @@ namespace drt {
 
 // per (body, step): rotation rows and rotation centre; per (terminal, step): position
 struct PoseQ { ff R[9], O[3]; };      // 96 B
-struct PointQ { ff r[3], pad; };      // 32 B
+struct PointQ { ff r[3]; };           // 24 B: with it a row is no larger than the FP64 table's
 
 DRT_HD v3<ff> vq(const ff *a) { return V3<ff>(a[0], a[1], a[2]); }
 DRT_NOINL1 v3<ff> rotq(const PoseQ &P, v3<ff> x) {

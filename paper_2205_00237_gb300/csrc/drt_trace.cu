@@ -66,9 +66,10 @@ DRT_HD bool face_blocks(const PosedFace &F, v3<double> A, v3<double> B) {
 }
 
 // one ray found: its enumeration index, chain and diffraction parameters at the instant
-// (state: how far it is decided; index -1: FP64 found that it is none)
+// (n: the vertices, and from bit 8 on how far it is decided; index -1: FP64 found that it is none)
 enum { RAY_FINAL = 0, RAY_POLISH = 1, RAY_OPEN = 2 };
-struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; int32_t state, pad; ff v[2][3]; };
+struct RayPoints { ff v[2][3]; };   // the solved vertices of a listed candidate
+struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; };
 
 constexpr int TRACE_T = 128;
 
@@ -109,7 +110,6 @@ DRT_HD bool trace_chain(const LinkDev &L, double t, long long k, const int *code
     for (int i = 1; i <= N + 1; ++i)
         if (blocked(V[i - 1], V[i])) return false;
     r->index = k;
-    r->state = RAY_FINAL;
     r->n = N;
     r->types = types;
 #pragma unroll
@@ -213,7 +213,8 @@ DRT_HD bool corner_path(const Prim<ff> &E1, const Prim<ff> &E2, v3<ff> A, v3<ff>
 }
 
 template <int N>
-DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Prim<ff> *prims, TracedRay *r) {
+DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Prim<ff> *prims, TracedRay *r,
+                          RayPoints *v) {
     const int NP = L.n_faces + L.n_edges;
     const ff tq = from_double(t);
     Prim<ff> pr[N > 0 ? N : 1];
@@ -294,9 +295,9 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pri
     if (fl) return -1;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        r->v[j][0] = V[j + 1].x;
-        r->v[j][1] = V[j + 1].y;
-        r->v[j][2] = V[j + 1].z;
+        v->v[j][0] = V[j + 1].x;
+        v->v[j][1] = V[j + 1].y;
+        v->v[j][2] = V[j + 1].z;
         if (pr[j].type == T_D) r->s[j] = to_double(dot(V[j + 1] - pr[j].p, pr[j].a));
     }
     return any_d ? RAY_POLISH : RAY_FINAL;
@@ -304,47 +305,50 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pri
 
 __global__ void __launch_bounds__(TRACE_T)
 k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int with_tiles, const Prim<ff> *__restrict__ prims,
-           TracedRay *__restrict__ out, int cap, int *__restrict__ count) {
+           TracedRay *__restrict__ out, RayPoints *__restrict__ points, int cap, int *__restrict__ count) {
     const long long k = blockIdx.x * (long long)TRACE_T + threadIdx.x;
     if (k >= n_cand) return;
     const int NP = L.n_faces + L.n_edges, NT = with_tiles ? L.n_tiles : 0;
     TracedRay r;
-    r.pad = 0;
+    RayPoints v{};
     int code[2] = {0, 0}, state;
     if (k == 0) {
-        state = trace_chain_ff<0>(L, t, code, prims, &r);
+        state = trace_chain_ff<0>(L, t, code, prims, &r, &v);
     } else if (k - 1 < NP + NT) {
         code[0] = (int)(k - 1);
-        state = trace_chain_ff<1>(L, t, code, prims, &r);
+        state = trace_chain_ff<1>(L, t, code, prims, &r, &v);
     } else {
         const long long q = k - 1 - NP - NT;
         code[0] = (int)(q / NP);
         code[1] = (int)(q % NP);
         if (code[0] == code[1]) return;
-        state = trace_chain_ff<2>(L, t, code, prims, &r);
+        state = trace_chain_ff<2>(L, t, code, prims, &r, &v);
     }
     if (state < 0) return;
     r.index = k;
-    r.state = state;
+    r.n |= state << 8;
     const int slot = atomicAdd(count, 1);
-    if (slot < cap) out[slot] = r;
+    if (slot >= cap) return;
+    out[slot] = r;
+    points[slot] = v;
 }
 
 __global__ void __launch_bounds__(128)
 k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
-              const PosedFaceQ *__restrict__ facesq, TracedRay *__restrict__ out, int cap, const int *__restrict__ count) {
+              const PosedFaceQ *__restrict__ facesq, TracedRay *__restrict__ out, const RayPoints *__restrict__ points, int cap,
+              const int *__restrict__ count) {
     const int n = min(*count, cap), lane = threadIdx.x & 31;
     const ff tq = from_double(t);
     for (int k = blockIdx.x * 4 + (threadIdx.x >> 5); k < n; k += gridDim.x * 4) {   // warp-uniform
         TracedRay *r = out + k;
-        int state = r->state;
-        if (state != RAY_OPEN) {
-            const int N = r->n;
+        if (r->n >> 8 != RAY_OPEN) {
+            const int N = r->n & 255;
+            const RayPoints &v = points[k];
             const v3<ff> tx = val(terminal_dual_ff(L.txq, tq)), rx = val(terminal_dual_ff(L.rxq, tq));
             bool hit = false, open = false;
             for (int q = lane; q < (N + 1) * L.n_faces; q += 32) {
                 const int i = q / L.n_faces, f = q - i * L.n_faces;
-                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(r->v[i - 1]), i == N ? rx : vq(r->v[i]));
+                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(v.v[i - 1]), i == N ? rx : vq(v.v[i]));
                 hit = hit || b > 0;
                 open = open || b < 0;
             }
@@ -391,8 +395,8 @@ k_trace_polish(const __grid_constant__ LinkDev L, double t, TracedRay *__restric
     const int n = min(*count, cap);
     for (int k = blockIdx.x * 32 + threadIdx.x; k < n; k += gridDim.x * 32) {
         TracedRay *r = out + k;
-        if (r->state != RAY_POLISH || r->index < 0) continue;
-        if (r->n == 1) polish_ray<1>(L, t, r);
+        if (r->n >> 8 != RAY_POLISH || r->index < 0) continue;
+        if ((r->n & 255) == 1) polish_ray<1>(L, t, r);
         else polish_ray<2>(L, t, r);
     }
 }
@@ -403,26 +407,29 @@ long long trace_candidates(const LinkDev &L, int max_order, int with_tiles) {
 }
 
 size_t trace_ray_bytes() { return sizeof(TracedRay); }
-size_t trace_prim_bytes(const LinkDev &L) {
-    return (size_t)L.n_faces * (sizeof(PosedFace) + sizeof(PosedFaceQ)) + (size_t)(L.n_faces + L.n_edges) * sizeof(Prim<ff>) + 256;
+size_t trace_face_bytes() { return sizeof(PosedFace); }
+size_t trace_prim_bytes(const LinkDev &L, int cap) {   // posed faces and primitives, then the points of `cap` listed candidates
+    return (size_t)L.n_faces * sizeof(PosedFaceQ) + (size_t)(L.n_faces + L.n_edges) * sizeof(Prim<ff>) + cap * sizeof(RayPoints);
 }
 
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s, bool two) {
+                         int *count, cudaStream_t s, void *prims_mem) {
+    const bool two = prims_mem != nullptr;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
     PosedFace *F = reinterpret_cast<PosedFace *>(faces);
-    PosedFaceQ *Q = reinterpret_cast<PosedFaceQ *>(F + L.n_faces);
+    PosedFaceQ *Q = reinterpret_cast<PosedFaceQ *>(prims_mem);
     TracedRay *out = reinterpret_cast<TracedRay *>(rays);
-    if (L.n_faces > 0) k_pose_faces<<<(L.n_faces + 127) / 128, 128, 0, s>>>(L, t, F, two ? Q : nullptr);
+    if (L.n_faces > 0) k_pose_faces<<<(L.n_faces + 127) / 128, 128, 0, s>>>(L, t, F, Q);
     const long long n = trace_candidates(L, max_order, with_tiles);
     const unsigned grid = (unsigned)((n + TRACE_T - 1) / TRACE_T);
     if (two) {
         Prim<ff> *prims = reinterpret_cast<Prim<ff> *>(Q + L.n_faces);
         const int np = L.n_faces + L.n_edges;
+        RayPoints *points = reinterpret_cast<RayPoints *>(prims + np);
         if (np) k_pose_prims<<<(np + 127) / 128, 128, 0, s>>>(L, t, prims);
-        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, prims, out, cap, count);
-        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, out, cap, count);
+        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, prims, out, points, cap, count);
+        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, out, points, cap, count);
         k_trace_polish<<<152 * 8, 32, 0, s>>>(L, t, out, cap, count);
     } else {
         k_trace<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, F, out, cap, count);
@@ -437,18 +444,19 @@ int trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *type
     order.reserve(count);
     for (int i = 0; i < count; ++i)
         if (R[i].index >= 0) order.push_back(i);
-    const int n = (int)order.size();
+    const int found = (int)order.size();
     std::sort(order.begin(), order.end(), [&](int a, int b) { return R[a].index < R[b].index; });
-    for (int q = 0; q < n && q < cap; ++q) {
+    for (int q = 0; q < found && q < cap; ++q) {
         const TracedRay &r = R[order[q]];
-        n_int[q] = (uint8_t)r.n;
+        const int n = r.n & 255;
+        n_int[q] = (uint8_t)n;
         for (int j = 0; j < MAXI; ++j) {
             types[q * MAXI + j] = (uint8_t)((r.types >> (8 * j)) & 0xff);
-            prims[q * MAXI + j] = j < r.n ? r.prims[j] : -1;
+            prims[q * MAXI + j] = j < n ? r.prims[j] : -1;
             s0[q * MAXI + j] = r.s[j];
         }
     }
-    return n;
+    return found;
 }
 
 }  // namespace drt
