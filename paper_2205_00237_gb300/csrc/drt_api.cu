@@ -505,13 +505,19 @@ drt_status synth_into(drt_ctx *c, Link &L, const drt_time_grid *tg, const drt_fr
 
 }  // namespace
 
+// The largest coordinate (m) that two-float numbers have to carry for instants within T of t = 0: the scene's extent, what its bodies
+// and terminals cover, and the rotation of a primitive, whose angle in radians has the same 47 bits as a length, times
+// that.  Infinite past 4096 rad: up to there the FP32 count of whole turns (body_pose_ff) leaves a remainder below 3.15.
+double drt::ff_reach(const drt_scene_view &v, double T) {
+    const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T), turn = T * (v.w0max + 0.5 * v.wdotmax * T);
+    return turn <= 4096.0 ? reach * (1.0 + turn) : HUGE_VAL;
+}
 // Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
 // is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
 // as checked at load.  Beyond that the records are computed in FP64.
 bool drt::ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
     const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
-    const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T);
-    return v.ff_range && reach * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
+    return v.ff_range && ff_reach(v, T) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
 }
 
 // validated host-side structure-of-arrays image of one link (device pointers unset)
@@ -519,7 +525,7 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
     if (drt_status st = validate(s, ps)) return st;
     {
         auto n3 = [](const double *x) { return std::sqrt(dot3(x, x)); };
-        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0, 0.0, true};
+        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0, 0.0, 0.0, 0.0, true};
         auto reach = [&](const double *x) { v.extent = std::max(v.extent, n3(x)); };
         reach(s->tx.r);
         reach(s->rx.r);
@@ -544,6 +550,8 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
             v.vmax = std::max(v.vmax, n3(b.v));
             v.amax = std::max(v.amax, n3(b.a));
             v.wmax = std::max(v.wmax, std::fabs(b.w0) + std::fabs(b.wdot));
+            v.w0max = std::max(v.w0max, std::fabs(b.w0));
+            v.wdotmax = std::max(v.wdotmax, std::fabs(b.wdot));
         }
         H.view = v;
     }
@@ -1216,7 +1224,7 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
     if (drt_status st = ensure(c, c->tr_faces, (size_t)std::max(L.dev.n_faces, 1) * trace_face_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
-    const bool two = L.view.ff_range && L.view.extent + std::fabs(t) * (L.view.vmax + 0.5 * L.view.amax * std::fabs(t)) < 1e5;
+    const bool two = L.view.ff_range && ff_reach(L.view, std::fabs(t)) < 1e5;
     // without room for their scratch the FP64 pass alone
     void *prims = two && ensure(c, c->tr_prims, trace_prim_bytes(L.dev, cap_dev)) == DRT_OK ? c->tr_prims.ptr : nullptr;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);
