@@ -514,10 +514,12 @@ double drt::ff_reach(const drt_scene_view &v, double T) {
 }
 // Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
 // is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
-// as checked at load.  Beyond that the records are computed in FP64.
+// as checked at load, and no permittivity |eps_c| = |eps_r - j sigma / (2 pi fc eps0)| above 1e15 (copper below 1 kHz), so that |eps_c|^2 is
+// a divisor that FP32 can invert (1 / x is 0 from x = 2^126 on).  Beyond that the records are computed in FP64.
 bool drt::ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
     const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
-    return v.ff_range && ff_reach(v, T) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
+    return v.ff_range && 1e6 + v.sigma_max / (2 * 3.14159265358979323846 * 8.8541878128e-12 * fg.fc) <= 1e15 &&
+           ff_reach(v, T) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
 }
 
 // validated host-side structure-of-arrays image of one link (device pointers unset)
@@ -525,7 +527,7 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
     if (drt_status st = validate(s, ps)) return st;
     {
         auto n3 = [](const double *x) { return std::sqrt(dot3(x, x)); };
-        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0, 0.0, 0.0, 0.0, true};
+        drt_scene_view v{std::max(n3(s->tx.v), n3(s->rx.v)), std::max(n3(s->tx.a), n3(s->rx.a)), 0.0, 0.0, 0.0, 0.0, 0.0, true};
         auto reach = [&](const double *x) { v.extent = std::max(v.extent, n3(x)); };
         reach(s->tx.r);
         reach(s->rx.r);
@@ -545,6 +547,7 @@ drt_status drt::pack_link(const drt_scene *s, const drt_path_set *ps, PackedLink
         }
         for (int i = 0; i < s->n_materials; ++i)
             v.ff_range = v.ff_range && s->materials[i].eps_r < 1e6 && s->materials[i].sigma < 1e8;
+        for (int i = 0; i < s->n_materials; ++i) v.sigma_max = std::max(v.sigma_max, s->materials[i].sigma);
         for (int i = 0; i < s->n_bodies; ++i) {
             const drt_body &b = s->bodies[i];
             v.vmax = std::max(v.vmax, n3(b.v));

@@ -137,8 +137,8 @@ struct RecD { float4 *rec_a; float *rec_b; };
 // kinematic bounds of a link used by the batch planner's chunk model: fastest terminal / body
 // translation speed (m/s), largest acceleration (m/s^2), largest angular speed (rad/s)
 // and extent, the largest coordinate at t0 (m), and the largest angular speed at t = 0 (rad/s) and angular acceleration (rad/s^2)
-// apart; ff_range: every length and material constant lies in the range of the two-float form
-struct drt_scene_view { double vmax, amax, wmax, extent, w0max, wdotmax; bool ff_range; };
+// apart; the largest conductivity (S/m); ff_range: every length and material constant lies in the range of the two-float form
+struct drt_scene_view { double vmax, amax, wmax, extent, w0max, wdotmax, sigma_max; bool ff_range; };
 double ff_reach(const drt_scene_view &v, double T);
 bool ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg);
 

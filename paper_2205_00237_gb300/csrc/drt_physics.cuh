@@ -846,7 +846,8 @@ DRT_NOINL1 FresnelFF fresnel_ff(MatV<ff> m, ff ieps, ff ct) {
     const cx<ff> ec = C<ff>(m.eps_r, -(m.sigma * ieps)), z = C<ff>(fma(ct, ct, ec.re - ff(1.f)), ec.im);
     const cx<ff> sq = csqrt_(z), ecct = C<ff>(ec.re * ct, ec.im * ct);
     const cx<ff> a1 = C<ff>(ct - sq.re, -sq.im), b1 = C<ff>(ct + sq.re, sq.im), a2 = ecct - sq, b2 = ecct + sq;
-    const ff n1 = cabs2(b1), n2 = cabs2(b2), q = ff(1.f) / (n1 * n2), i1 = n2 * q, i2 = n1 * q;
+    // (a quotient each: their common divisor ~ |eps_c|^3 leaves the range of FP32 for a metal at a low carrier)
+    const ff i1 = ff(1.f) / cabs2(b1), i2 = ff(1.f) / cabs2(b2);
     r.te = C<ff>(det2(a1.re, b1.re, -a1.im, b1.im) * i1, det2(a1.im, b1.re, a1.re, b1.im) * i1);
     r.tm = C<ff>(det2(a2.re, b2.re, -a2.im, b2.im) * i2, det2(a2.im, b2.re, a2.re, b2.im) * i2);
     return r;
