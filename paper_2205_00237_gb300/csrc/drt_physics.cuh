@@ -647,8 +647,8 @@ template <int N> constexpr int len_min() { return N == LEN_GEN ? 2 : 0; }
 // that bound (the FP32-bulk step uses it to keep the FP32 flags of invalid steps that moved far).
 template <class T> DRT_HD T amax3(v3<T> a) { return fmax(fmax(fabs(a.x), fabs(a.y)), fabs(a.z)); }
 DRT_HD float amax3(v3<ff> a) { return fmaxf(fmaxf(fabsf(a.x.h), fabsf(a.y.h)), fabsf(a.z.h)); }
-// The two-float form (H of the FP64 form) leaves margins within 2^-36 of the coordinates (1.5e-9 m at 100 m: ~2000 times the
-// rounding of a coordinate) to FP64 in the same way.
+// The two-float form (H of the FP64 form) leaves margins within 2^-36 of the coordinates (1.5e-9 m at 100 m: ~1000 times the
+// rounding of a coordinate) to FP64 in the same way, and larger ones in a chain close to grazing (validity).
 DRT_HD float ff_margin_tol(float scale) { return 1.4551915e-11f * (scale + 1.f); }
 // the margin b - |a| (b may be infinite) and the sign-exact value of a normalised number
 DRT_HD float ff_within(ff a, ff b) {
@@ -668,16 +668,24 @@ DRT_HD float fp32_margin_tol(float scale) { return 2e-6f * (scale + 1.f); }
 // error bound.  (Called out of line in the FP32 kernels it measured no faster, unlike the field
 // updates, so it stays inline.)
 template <class T> struct VertexCheck { uint32_t fl; T m; };
-DRT_NOINL1 VertexCheck<float> vertex_validity_inl(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
-                                              v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
-    uint32_t fl = 0;
+// The same in two-float numbers: the flags, the smallest margin over the bound on a coordinate's error, the largest margin by which a
+// test fails, and amp, by how much the point's place is less certain than a coordinate: leg / height for a reflection,
+// (leg / distance from the edge line)^2 for a diffraction, whose Newton step divides by sin^2 of the angle to the edge.
+// the smaller of m and |v|, -1 from the first that is not a number on
+DRT_HD float least(float m, float v) { return ::fabsf(v) < m ? ::fabsf(v) : v == v ? m : -1.f; }
+struct VertexMargins { uint32_t fl; float m, out, amp; };
+DRT_NOINL1 VertexMargins vertex_margins(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
+                                        v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
+    VertexMargins r{0, 1e30f, 0.f, 1.f};
     float scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), amax3(Pi));
     if (ty != T_S) scale = fmaxf(scale, amax3(c));
-    const float tol = ff_margin_tol(scale);
-    // a test passes with margin v > 0; within the bound (or not a number) it is undecided
+    // a test passes with margin v > 0 (not a number: undecided)
     auto test = [&](float v, uint32_t bit) {
-        if (!(v > 0.f)) fl |= v < -tol ? bit | F_CLEAR : bit;
-        if (!(fabsf(v) > tol)) fl |= F_REDO64;
+        if (!(v > 0.f)) {
+            r.fl |= bit;
+            r.out = fmaxf(r.out, -v);
+        }
+        r.m = least(r.m, v);
     };
     if (ty == T_D) {
         const ff s = dot(Pi - c, nn);
@@ -685,23 +693,37 @@ DRT_NOINL1 VertexCheck<float> vertex_validity_inl(int ty, v3<ff> c, v3<ff> nn, v
         test((h1.h - s.h) + (h1.l - s.l), F_EDGE);
 #pragma unroll
         for (int side = -1; side <= 1; side += 2) {   // see the general form below
-            const v3<ff> r = (side < 0 ? Pm : Pp) - Pi;
-            const v3<ff> rp = axpy(r, nn, -dot(r, nn));
+            const v3<ff> d = (side < 0 ? Pm : Pp) - Pi;
+            const v3<ff> rp = axpy(d, nn, -dot(d, nn));
             const ff y = dot(rp, cc), x = dot(rp, b);
-            const float sn = det2(h3, x, h4, y).h;
-            if (!(fabsf(y.h) > tol) || !(fabsf(sn) > tol)) fl |= F_REDO64;
-            if (!(y.h > 0.f) && !(sn > 0.f)) fl |= y.h < -tol && sn < -tol ? F_SIDE | F_CLEAR : F_SIDE;
+            const float sn = det2(h3, x, h4, y).h, near = fabsf(y.h) < fabsf(sn) ? fabsf(y.h) : fabsf(sn);
+            r.m = least(r.m, near);
+            if (!(y.h > 0.f) && !(sn > 0.f)) {
+                r.fl |= F_SIDE;
+                r.out = fmaxf(r.out, near);
+            }
+            const float l2 = fmaf(d.x.h, d.x.h, fmaf(d.y.h, d.y.h, d.z.h * d.z.h));
+            const float a = l2 / fmaf(x.h, x.h, y.h * y.h);
+            if (l2 > 1e-17f && !(a <= r.amp)) r.amp = a == a ? a : HUGE_VALF;   // (a leg of no length is a test of its own)
         }
     } else {
         if (ty == T_R) {
-            const v3<ff> r = Pi - c;
-            test(ff_within(dot(r, b), h1), F_FACE);
-            test(ff_within(dot(r, cross(b, nn)), h2), F_FACE);
+            const v3<ff> d = Pi - c;
+            test(ff_within(dot(d, b), h1), F_FACE);
+            test(ff_within(dot(d, cross(b, nn)), h2), F_FACE);
         }
-        test(dot(Pm - c, nn).h, F_SIDE);   // a tile is its own point
-        test(dot(Pp - c, nn).h, F_SIDE);
+        const float hm = dot(Pm - c, nn).h, hp = dot(Pp - c, nn).h;
+        test(hm, F_SIDE);   // a tile is its own point
+        test(hp, F_SIDE);
+        if (ty == T_R) {
+            const float leg = fabsf(Pm.x.h - Pp.x.h) + fabsf(Pm.y.h - Pp.y.h) + fabsf(Pm.z.h - Pp.z.h);
+            r.amp = 1.f + (leg + 1e-6f * scale) / (fabsf(hm) + fabsf(hp));
+        }
     }
-    return VertexCheck<float>{fl, 2.f};
+    const float itol = 1.f / ff_margin_tol(scale);
+    r.m *= itol;
+    r.out *= itol;
+    return r;
 }
 template <class T>
 DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3<T> cc, T h1, T h2, T h3, T h4,
@@ -757,35 +779,62 @@ DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3
     return VertexCheck<T>{fl, mmin};
 }
 
+// (amp_out, two-float only: how much less certain than a coordinate a point of the chain is along its face or edge)
 template <int N = -1, class S>
-DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P) {
+DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P, float *amp_out = nullptr) {
     typedef typename ST<S>::R T;
     constexpr bool F32 = sizeof(T) == 4, FF = std::is_same<T, ff>::value;
     typedef std::conditional_t<FF, float, T> M;
     const int nv = N >= 0 ? N : n;
     uint32_t fl = 0;
     M mmin = M(1e30);    // FP32 and two-float only: the smallest margin over its bound
+    float out = 0.f, amp = 1.f;   // two-float only (vertex_margins)
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI + 1; ++i) {
         if (i > nv + 1) break;
         v3<T> d = P[i] - P[i - 1];
         const T q = dot(d, d);
-        if (!(q >= T(1e-18))) fl |= F_DEGEN;
-        if constexpr (FF)   // shorter than half of that bound: clear of it
-            if (q.h < 2.5e-19f) fl |= F_CLEAR;
+        if constexpr (FF) {
+            // the margin of a length is held against the error bound itself, 2^-42: points that coincide shall be decided
+            const float v = ::sqrtf(q.h) - 1e-9f, w = 64.f / ff_margin_tol(fmaxf(amax3(P[i]), amax3(P[i - 1])));
+            mmin = least(mmin, v * w);
+            if (!(v >= 0.f)) {
+                fl |= F_DEGEN;
+                out = ::fmaxf(out, -v * w);
+            }
+        } else {
+            if (!(q >= T(1e-18))) fl |= F_DEGEN;
+        }
     }
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI; ++i) {
         if (i > nv) break;
         const Prim<S> &q = pr[i - 1];
-        const VertexCheck<M> v =
-            vertex_validity_inl(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
-        fl |= v.fl;
-        mmin = fmin(mmin, v.m);
+        if constexpr (FF) {
+            const VertexMargins v =
+                vertex_margins(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
+            fl |= v.fl;
+            mmin = ::fminf(mmin, v.m);
+            out = ::fmaxf(out, v.out);
+            amp *= v.amp;
+        } else {
+            const VertexCheck<T> v =
+                vertex_validity_inl(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
+            fl |= v.fl;
+            mmin = fmin(mmin, v.m);
+        }
     }
     if constexpr (F32) {
         if (mmin < T(1)) fl |= F_REDO64;
         if (mmin < T(100)) fl |= F_NEAR100;
+    }
+    if constexpr (FF) {
+        // The bound is 1000 times the rounding of a coordinate (2^-46); 64 of that are for the amplification of a usual chain
+        const float need = ::fmaxf(1.f, amp * (1.f / 64.f));
+        if (!(mmin > need)) fl |= F_REDO64;
+        if (out > need) fl |= F_CLEAR;
+        if (amp_out) *amp_out = amp;
+        if (!(amp < 1e30f)) fl = (fl | F_REDO64) & ~F_CLEAR;
     }
     return fl;
 }

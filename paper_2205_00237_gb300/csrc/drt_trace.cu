@@ -68,7 +68,7 @@ DRT_HD bool face_blocks(const PosedFace &F, v3<double> A, v3<double> B) {
 // one ray found: its enumeration index, chain and diffraction parameters at the instant
 // (n: the vertices, and from bit 8 on how far it is decided; index -1: FP64 found that it is none)
 enum { RAY_FINAL = 0, RAY_POLISH = 1, RAY_OPEN = 2 };
-struct RayPoints { ff v[2][3]; };   // the solved vertices of a listed candidate
+struct RayPoints { ff v[2][3]; float amp, pad; };   // the solved vertices of a listed candidate, and its amp (validity)
 struct TracedRay { long long index; int32_t n; uint32_t types; int32_t prims[MAXI]; double s[MAXI]; };
 
 constexpr int TRACE_T = 128;
@@ -167,23 +167,32 @@ k_trace(const LinkDev L, double t, long long n_cand, int with_tiles, const Posed
 // k_trace_block, a warp per listed candidate, spreads the (segment, face) tests over its lanes and tries what is still open in FP64;
 // k_trace_polish solves the rays' diffraction parameters in FP64 from the two-float ones (one Newton step).  The list ends as k_trace's.
 
-// 1: the face blocks the segment, 0: it does not, -1: within the margins
-DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B) {
+// 1: the face blocks the segment, 0: it does not, -1: within the margins.  The ends' heights over the face are less certain than a
+// coordinate by upA and upB, their places along it by amp
+DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B, float upA, float upB, float amp) {
     const v3<ff> c = vq(F.c), n = vq(F.n);
     const ff ha = dot(A - c, n), hb = dot(B - c, n);
     const float fa = fabsf(ha.h), fb = fabsf(hb.h), scale = fmaxf(fmaxf(amax3(A), amax3(B)), amax3(c));
     // an end within 1e-9 m of the plane: the points of a chain lie on its own faces to ~2^-46 of the coordinates, which 2^-42 bounds
     const float tol = ff_margin_tol(scale), e = fmaxf(2.3e-13f * (scale + 1.f), 1e-10f);
-    if (fabsf(fa - 1e-9f) <= e || fabsf(fb - 1e-9f) <= e || e > 5e-10f) return -1;
+    if (!(fabsf(fa - 1e-9f) > e * upA) || !(fabsf(fb - 1e-9f) > e * upB)) return -1;
     if (fa < 1e-9f || fb < 1e-9f) return 0;
     if ((ha.h > 0.f) == (hb.h > 0.f)) return 0;
     const v3<ff> r = axpy(A, B - A, ha / (ha - hb)) - c;
     const float mu = ff_within(dot(r, vq(F.u)), F.hu), mw = ff_within(dot(r, vq(F.w)), F.hw);
     // the point moves along the plane with the error of h over the segment's slope
     const v3<ff> d = B - A;
-    const float lim = tol * (1.f + (fabsf(d.x.h) + fabsf(d.y.h) + fabsf(d.z.h)) / (fa + fb));
+    const float lim = tol * fmaxf(1.f, amp * (1.f / 64.f)) * (1.f + (fabsf(d.x.h) + fabsf(d.y.h) + fabsf(d.z.h)) / (fa + fb));
     if (mu < -lim || mw < -lim) return 0;
     return mu > lim && mw > lim ? 1 : -1;
+}
+
+// how much less certain than a coordinate the height over a face of normal n is at a vertex on the primitive q, which may lie amp
+// coordinate errors from its place along its face or edge
+DRT_HD float height_amp(const Prim<ff> &q, v3<float> n, float amp) {
+    const v3<float> a = f32v(q.a);
+    const v3<float> x = cross(a, n);
+    return 1.f + amp * (q.type == T_D ? fabsf(dot(a, n)) : sqrtf(dot(x, x)));
 }
 
 // the faces, then the edges, posed
@@ -285,7 +294,7 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pri
                 if (pf[j].type == T_D) s0[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
     }
     solve_geometry_any<N>(pr, V, s0, fl);
-    fl |= validity<N>(pr, N, V);
+    fl |= validity<N>(pr, N, V, &v->amp);
     if (fl & F_NOCONV) return RAY_OPEN;
 #pragma unroll
     for (int i = 1; i <= N; ++i)
@@ -335,7 +344,7 @@ k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int wi
 
 __global__ void __launch_bounds__(128)
 k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
-              const PosedFaceQ *__restrict__ facesq, TracedRay *__restrict__ out, const RayPoints *__restrict__ points, int cap,
+              const PosedFaceQ *__restrict__ facesq, const Prim<ff> *__restrict__ prims, TracedRay *__restrict__ out, const RayPoints *__restrict__ points, int cap,
               const int *__restrict__ count) {
     const int n = min(*count, cap), lane = threadIdx.x & 31;
     const ff tq = from_double(t);
@@ -348,7 +357,13 @@ k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const
             bool hit = false, open = false;
             for (int q = lane; q < (N + 1) * L.n_faces; q += 32) {
                 const int i = q / L.n_faces, f = q - i * L.n_faces;
-                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(v.v[i - 1]), i == N ? rx : vq(v.v[i]));
+                const v3<float> n = f32v(vq(facesq[f].n));
+                auto up = [&](int j) {   // of vertex j + 1 (terminals and tiles are where they are)
+                    const int ty = (r->types >> (8 * j)) & 0xff;
+                    return ty == T_S ? 1.f : height_amp(prims[r->prims[j] + (ty == T_D ? L.n_faces : 0)], n, v.amp);
+                };
+                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(v.v[i - 1]), i == N ? rx : vq(v.v[i]),
+                                             i == 0 ? 1.f : up(i - 1), i == N ? 1.f : up(i), v.amp);
                 hit = hit || b > 0;
                 open = open || b < 0;
             }
@@ -429,7 +444,7 @@ cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_til
         RayPoints *points = reinterpret_cast<RayPoints *>(prims + np);
         if (np) k_pose_prims<<<(np + 127) / 128, 128, 0, s>>>(L, t, prims);
         k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, prims, out, points, cap, count);
-        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, out, points, cap, count);
+        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, prims, out, points, cap, count);
         k_trace_polish<<<152 * 8, 32, 0, s>>>(L, t, out, cap, count);
     } else {
         k_trace<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, F, out, cap, count);

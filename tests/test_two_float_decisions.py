@@ -1,0 +1,31 @@
+"""What two-float numbers decide about a chain is what FP64 decides: random chains with points within 1e-13 m .. 1 m of a face rim, an edge
+end, a face plane or a wedge face, at grazing angles down to 1e-7 rad, where an error of a coordinate moves the point by
+leg / height of it (a reflection) or by (leg / distance from the edge line)^2 (a diffraction).  On the CPU, whose
+additions, products and fused operations are the GPU's."""
+import os
+
+import pytest
+
+import host_program
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def decide(tmp_path_factory):
+    with open(os.path.join(HERE, "two_float_decisions.cu")) as f:
+        exe = host_program.build(f.read(), tmp_path_factory.mktemp("decide"))
+
+    def call(**q):
+        order = ("most_diffractions", "extent", "shortest", "angle", "come_from", "seed", "n")
+        return [int(x) for x in host_program.run(exe, [[q[k] for k in order]])[0]]
+    return call
+
+
+@pytest.mark.parametrize("extent", [20, 500])
+@pytest.mark.parametrize("shortest,angle,least", [(1, 0.2, 0.7), (0.01, 0.01, 0.7), (0.01, 1e-4, 0.5), (1e-4, 1e-7, 0.25)])
+def test_chains_with_one_diffraction(decide, extent, shortest, angle, least):
+    """(least: the share that is still decided without FP64)"""
+    n, decided, rays, wrong, unconverged = decide(most_diffractions=1, extent=extent, shortest=shortest, angle=angle,
+                                                  come_from=0, seed=11, n=30000)
+    assert wrong == 0 and unconverged == 0 and rays > 1000 and decided > least * n
