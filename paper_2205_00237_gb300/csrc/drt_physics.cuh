@@ -416,7 +416,8 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
                                 const D *rate0, uint32_t &fl) {
     typedef typename ST<S>::R T;
     // convergence threshold on the Newton step (m): near round-off of the working precision
-    // (two-float numbers stop at a step of 1 um: the next one would be ~1e-12 / leg length, below their resolution)
+    // (two-float numbers stop at a step of 1 um, less where a leg is short: the next one is ~step^2 / leg length, which is held
+    // below 1e-12 m, their resolution)
     const T tol = std::is_same<T, ff>::value ? T(1e-6) : sizeof(T) == 8 ? T(1e-10) : T(1e-4);
     // below this step (m) the length change of a Newton step is at round-off of the ~100 m path
     // length, so the backtracking test is only applied to larger steps
@@ -445,6 +446,7 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
         // gk, hk: gradient and Hessian diagonal of the unknown starting the current leg; hop: its
         // coupling to the unknown before it; cpP, dpP: elimination of that previous unknown
         S Lc = zero, gk = zero, hk = zero, hop = zero, cpP = zero, dpP = zero;
+        float lmin = 1e30f;   // two-float only: the shortest leg
 #pragma unroll
         for (int i = 1; i <= N + 1; ++i) {
             cl[i] = false;
@@ -463,6 +465,7 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
             if (startN || var) {
                 const v3<S> r = X - Y;
                 const S l = norm(r);
+                if constexpr (std::is_same<S, ff>::value) lmin = ::fminf(lmin, l.h);
                 Lc = Lc + l;
                 const S il = one / l;
                 const v3<S> rh = r * il;
@@ -552,7 +555,9 @@ DRT_HD void newton_diffractions(const Prim<S> *pr, v3<S> *V, const bool *nv, con
         // warm starts the first step is ~1e-6..1e-5 m (the FP32 rounding of the coordinates), so the
         // remaining error is far below that rounding.
         if (conv) break;
-        if (smax < tol) {
+        bool small = smax < tol;
+        if constexpr (std::is_same<S, ff>::value) small = small && smax.h * smax.h < 1e-12f * lmin;
+        if (small) {
             conv = true;
             if (sizeof(T) == 8 || std::is_same<S, de>::value) break;
         }
@@ -788,7 +793,8 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
     const int nv = N >= 0 ? N : n;
     uint32_t fl = 0;
     M mmin = M(1e30);    // FP32 and two-float only: the smallest margin over its bound
-    float out = 0.f, amp = 1.f;   // two-float only (vertex_margins)
+    float out = 0.f, amp = 1.f, steep = 0.f;   // two-float only (vertex_margins)
+    int nd = 0;
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI + 1; ++i) {
         if (i > nv + 1) break;
@@ -817,6 +823,10 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
             mmin = ::fminf(mmin, v.m);
             out = ::fmaxf(out, v.out);
             amp *= v.amp;
+            if (N >= 2 && q.type == T_D) {
+                ++nd;
+                steep = ::fmaxf(steep, v.amp * (amax3(P[i]) + 1.f));
+            }
         } else {
             const VertexCheck<T> v =
                 vertex_validity_inl(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
@@ -834,7 +844,9 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         if (!(mmin > need)) fl |= F_REDO64;
         if (out > need) fl |= F_CLEAR;
         if (amp_out) *amp_out = amp;
-        if (!(amp < 1e30f)) fl = (fl | F_REDO64) & ~F_CLEAR;
+        // Several diffractions in a row where the FP64 Newton solve may not reach its step of 1e-10 m, 2^-53 of the coordinates times
+        // 9 amp: whether it does is a flag of its own
+        if (!(amp < 1e30f) || (nd > 1 && steep > 1e5f)) fl = (fl | F_REDO64) & ~F_CLEAR;
     }
     return fl;
 }

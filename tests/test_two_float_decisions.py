@@ -29,3 +29,13 @@ def test_chains_with_one_diffraction(decide, extent, shortest, angle, least):
     n, decided, rays, wrong, unconverged = decide(most_diffractions=1, extent=extent, shortest=shortest, angle=angle,
                                                   come_from=0, seed=11, n=30000)
     assert wrong == 0 and unconverged == 0 and rays > 1000 and decided > least * n
+
+
+@pytest.mark.parametrize("extent", [20, 500])
+@pytest.mark.parametrize("shortest,angle,least", [(1, 0.2, 0.7), (0.01, 0.01, 0.6), (0.01, 1e-4, 0.45), (1e-4, 1e-7, 0.25)])
+def test_chains_with_several_diffractions(decide, extent, shortest, angle, least):
+    """Newton solves: the two-float one has to have arrived where it stops, also over short legs, and a chain whose FP64 solve does not
+    converge is left to it.  That one may fail by a chance of its line search (steps at its rounding): 1 in 20000."""
+    n, decided, rays, wrong, unconverged = decide(most_diffractions=3, extent=extent, shortest=shortest, angle=angle,
+                                                  come_from=0, seed=12, n=30000)
+    assert wrong == 0 and unconverged <= n // 20000 and rays > 1000 and decided > least * n
