@@ -330,7 +330,9 @@ Link *find_link(drt_ctx *c, uint64_t id) {
 
 // chunk of 16 steps (FP64 warm starts); the FP32-bulk form takes its chunk from the phase-error
 // model (choose_chunk)
-TimeGridD tgd(const drt_time_grid *g, int chunk = 16) { return make_tgrid(g->t_start, g->dt, g->n_steps, chunk); }
+TimeGridD tgd(const drt_time_grid *g, const drt_scene_view &v, int chunk = 16) {
+    return make_tgrid(g->t_start, g->dt, g->n_steps, chunk, ff_reach(v, *g));
+}
 FreqGridD fgd(const drt_freq_grid *g) { return make_fgrid(g->fc, g->bandwidth, g->n_bins); }
 
 // bracket one launch with events when tracing is on
@@ -354,7 +356,7 @@ drt_status run_extrapolation(drt_ctx *c, Link &L, const drt_time_grid *tg, const
                              const OutD &out, const RecD &rec, int32_t precision, cudaStream_t s,
                              bool defer_redo = false) {
     // FP32-bulk chunk length from the same phase-error model as the batch planner
-    TimeGridD t = precision == DRT_FP32_BULK ? tgd(tg, choose_chunk(L.view, *tg, *fg)) : tgd(tg);
+    TimeGridD t = precision == DRT_FP32_BULK ? tgd(tg, L.view, choose_chunk(L.view, *tg, *fg)) : tgd(tg, L.view);
     FreqGridD f = fgd(fg);
     if (precision == DRT_FP32_BULK) {
         if (drt_status st = ensure(c, c->poseb, bulk_pose_bytes(L.dev, t))) return st;
@@ -472,7 +474,7 @@ drt_status synth_into(drt_ctx *c, Link &L, const drt_time_grid *tg, const drt_fr
     if (drt_status st = ensure(c, c->rec_b, n * sizeof(float))) return st;
     RecD rec{reinterpret_cast<float4 *>(c->rec_a.ptr), reinterpret_cast<float *>(c->rec_b.ptr)};
     OutD none{};
-    TimeGridD t = precision == DRT_FP32_BULK ? tgd(tg, choose_chunk(L.view, *tg, *fg)) : tgd(tg);
+    TimeGridD t = precision == DRT_FP32_BULK ? tgd(tg, L.view, choose_chunk(L.view, *tg, *fg)) : tgd(tg, L.view);
     FreqGridD f = fgd(fg);
     if (precision == DRT_FP32_BULK) {
         // the FP64 redo of the few steps FP32 cannot resolve runs beside the synthesis (their records
@@ -512,14 +514,16 @@ double drt::ff_reach(const drt_scene_view &v, double T) {
     const double reach = v.extent + T * (v.vmax + 0.5 * v.amax * T), turn = T * (v.w0max + 0.5 * v.wdotmax * T);
     return turn <= 4096.0 ? reach * (1.0 + turn) : HUGE_VAL;
 }
+double drt::ff_reach(const drt_scene_view &v, const drt_time_grid &tg) {
+    return ff_reach(v, std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps)));
+}
 // Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
 // is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
 // as checked at load, and no permittivity |eps_c| = |eps_r - j sigma / (2 pi fc eps0)| above 1e15 (copper below 1 kHz), so that |eps_c|^2 is
 // a divisor that FP32 can invert (1 / x is 0 from x = 2^126 on).  Beyond that the records are computed in FP64.
 bool drt::ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
-    const double T = std::max(std::fabs(tg.t_start), std::fabs(tg.t_start + tg.dt * tg.n_steps));
     return v.ff_range && 1e6 + v.sigma_max / (2 * 3.14159265358979323846 * 8.8541878128e-12 * fg.fc) <= 1e15 &&
-           ff_reach(v, T) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
+           ff_reach(v, tg) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
 }
 
 // validated host-side structure-of-arrays image of one link (device pointers unset)
@@ -1227,7 +1231,8 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
     if (drt_status st = ensure(c, c->tr_faces, (size_t)std::max(L.dev.n_faces, 1) * trace_face_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
-    const bool two = L.view.ff_range && ff_reach(L.view, std::fabs(t)) < 1e5;
+    const double far = ff_reach(L.view, std::fabs(t));
+    const bool two = L.view.ff_range && far < 1e5;
     // without room for their scratch the FP64 pass alone
     void *prims = two && ensure(c, c->tr_prims, trace_prim_bytes(L.dev, cap_dev)) == DRT_OK ? c->tr_prims.ptr : nullptr;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);
@@ -1235,7 +1240,7 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
     int count = 0;
     for (int pass = prims ? 0 : 1; pass < 2; ++pass) {
         CUDA_TRY(launch_trace(L.dev, t, max_order, with_tiles, c->tr_faces.ptr, c->tr_rays.ptr, cap_dev, cnt, s,
-                              pass == 0 ? prims : nullptr));
+                              pass == 0 ? prims : nullptr, far));
         CUDA_TRY(cudaMemcpyAsync(&count, cnt, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_TRY(cudaStreamSynchronize(s));
         if (count <= cap_dev) break;
@@ -1422,7 +1427,7 @@ extern "C" drt_status drt_synthesize_H_noalloc(drt_ctx *c, uint64_t link, const 
     std::lock_guard<std::mutex> lk(c->mu);
     Link *L = find_link(c, link);
     if (!L) return fail(DRT_ENOTFOUND, "unknown link %llu", (unsigned long long)link);
-    TimeGridD t = tgd(tg);
+    TimeGridD t = tgd(tg, L->view);
     FreqGridD f = fgd(fg);
     size_t pose_bytes = round256((size_t)tg->n_steps * L->dev.n_bodies * POSE_W * sizeof(double));
     size_t warm_sz = round256(warm_bytes(L->dev, t));

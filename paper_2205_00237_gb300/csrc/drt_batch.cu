@@ -339,7 +339,7 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
         int chunk = choose_chunk(views[i], tgs[i], fgs[i]);
         if (mate[i] >= 0) chunk = std::min(chunk, choose_chunk(views[i], tgs[i], fgs[mate[i]]));
         chunk = std::max(4, chunk / std::max(1, chunk_div));
-        B.tg = make_tgrid(tgs[i].t_start, tgs[i].dt, tgs[i].n_steps, chunk);
+        B.tg = make_tgrid(tgs[i].t_start, tgs[i].dt, tgs[i].n_steps, chunk, ff_reach(views[i], tgs[i]));
         B.fg = make_fgrid(fgs[i].fc, fgs[i].bandwidth, fgs[i].n_bins);
         B.H = reinterpret_cast<float2 *>(H[i]);
         if (outs) B.out = outs[i];

@@ -82,6 +82,7 @@ struct TimeGridD {
     double t_start, dt;
     int32_t n_steps, chunk;
     float dtf;   // dt
+    float far;   // two-float form: the largest coordinate that a place is computed from (ff_reach; m)
 };
 struct FreqGridD {
     double fc, bandwidth;
@@ -93,8 +94,8 @@ struct FreqGridD {
     ff f0c_q, dfc_q;            // f0 / c, df / c
     double f0, df;    // first bin fc - B/2 and bin step B / n_bins (Hz), so that no kernel divides per step
 };
-inline TimeGridD make_tgrid(double t_start, double dt, int32_t n_steps, int32_t chunk) {
-    return TimeGridD{t_start, dt, n_steps, chunk, (float)dt};
+inline TimeGridD make_tgrid(double t_start, double dt, int32_t n_steps, int32_t chunk, double far = 0.0) {
+    return TimeGridD{t_start, dt, n_steps, chunk, (float)dt, (float)far};
 }
 inline FreqGridD make_fgrid(double fc, double bandwidth, int32_t n_bins) {
     const double c0 = 299792458.0, pi = 3.14159265358979323846, eps0 = 8.8541878128e-12, k = 2 * pi * fc / c0;
@@ -140,6 +141,7 @@ struct RecD { float4 *rec_a; float *rec_b; };
 // apart; the largest conductivity (S/m); ff_range: every length and material constant lies in the range of the two-float form
 struct drt_scene_view { double vmax, amax, wmax, extent, w0max, wdotmax, sigma_max; bool ff_range; };
 double ff_reach(const drt_scene_view &v, double T);
+double ff_reach(const drt_scene_view &v, const drt_time_grid &tg);
 bool ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg);
 
 // a10 batch plans (drt_batch.cu)
@@ -300,7 +302,7 @@ size_t trace_prim_bytes(const LinkDev &L, int cap);   // scratch of the two-floa
 // prims (trace_prim_bytes) non-null: candidates are solved in two-float numbers first, and FP64 decides what those leave open (see
 // drt_trace.cu); trace_unpack returns the number of rays
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s, void *prims);
+                         int *count, cudaStream_t s, void *prims, double far);
 int trace_unpack(const void *rays_host, int count, uint8_t *n_int, uint8_t *types, int32_t *prims, double *s0,
                   int cap);
 

@@ -653,7 +653,8 @@ template <int N> constexpr int len_min() { return N == LEN_GEN ? 2 : 0; }
 template <class T> DRT_HD T amax3(v3<T> a) { return fmax(fmax(fabs(a.x), fabs(a.y)), fabs(a.z)); }
 DRT_HD float amax3(v3<ff> a) { return fmaxf(fmaxf(fabsf(a.x.h), fabsf(a.y.h)), fabsf(a.z.h)); }
 // The two-float form (H of the FP64 form) leaves margins within 2^-36 of the coordinates (1.5e-9 m at 100 m: ~1000 times the
-// rounding of a coordinate) to FP64 in the same way, and larger ones in a chain close to grazing (validity).
+// rounding of a coordinate) to FP64 in the same way, and larger ones in a chain close to grazing (validity).  The coordinates are
+// also those that the motion has cancelled: a place o + v t keeps the rounding of o and of v t.
 DRT_HD float ff_margin_tol(float scale) { return 1.4551915e-11f * (scale + 1.f); }
 // the margin b - |a| (b may be infinite) and the sign-exact value of a normalised number
 DRT_HD float ff_within(ff a, ff b) {
@@ -680,9 +681,9 @@ template <class T> struct VertexCheck { uint32_t fl; T m; };
 DRT_HD float least(float m, float v) { return ::fabsf(v) < m ? ::fabsf(v) : v == v ? m : -1.f; }
 struct VertexMargins { uint32_t fl; float m, out, amp; };
 DRT_NOINL1 VertexMargins vertex_margins(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
-                                        v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
+                                        v3<ff> Pm, v3<ff> Pi, v3<ff> Pp, float far) {
     VertexMargins r{0, 1e30f, 0.f, 1.f};
-    float scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), amax3(Pi));
+    float scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), fmaxf(amax3(Pi), far));
     if (ty != T_S) scale = fmaxf(scale, amax3(c));
     // a test passes with margin v > 0 (not a number: undecided)
     auto test = [&](float v, uint32_t bit) {
@@ -784,9 +785,9 @@ DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3
     return VertexCheck<T>{fl, mmin};
 }
 
-// (amp_out, two-float only: how much less certain than a coordinate a point of the chain is along its face or edge)
+// (two-float only: far, the largest coordinate that a place is computed from; amp_out, how much less certain than a coordinate a point of the chain is along its face or edge)
 template <int N = -1, class S>
-DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P, float *amp_out = nullptr) {
+DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P, float far = 0.f, float *amp_out = nullptr) {
     typedef typename ST<S>::R T;
     constexpr bool F32 = sizeof(T) == 4, FF = std::is_same<T, ff>::value;
     typedef std::conditional_t<FF, float, T> M;
@@ -802,7 +803,7 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         const T q = dot(d, d);
         if constexpr (FF) {
             // the margin of a length is held against the error bound itself, 2^-42: points that coincide shall be decided
-            const float v = ::sqrtf(q.h) - 1e-9f, w = 64.f / ff_margin_tol(fmaxf(amax3(P[i]), amax3(P[i - 1])));
+            const float v = ::sqrtf(q.h) - 1e-9f, w = 64.f / ff_margin_tol(fmaxf(fmaxf(amax3(P[i]), amax3(P[i - 1])), far));
             mmin = least(mmin, v * w);
             if (!(v >= 0.f)) {
                 fl |= F_DEGEN;
@@ -818,7 +819,7 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         const Prim<S> &q = pr[i - 1];
         if constexpr (FF) {
             const VertexMargins v =
-                vertex_margins(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
+                vertex_margins(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1], far);
             fl |= v.fl;
             mmin = ::fminf(mmin, v.m);
             out = ::fmaxf(out, v.out);

@@ -234,7 +234,7 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
         seg[i] = V[i] - V[i - 1];
         d = d + norm(seg[i]);
     }
-    fl |= validity<N>(pr, N, V);
+    fl |= validity<N>(pr, N, V, tg.far);
     bool sure = !(fl & F_NOCONV) && (!(fl & (F_REDO64 | F_DEGEN)) || (fl & F_CLEAR)) && isfinite(d.h);
     if (sure && !fl) {
         const cx<ff> a = amplitude_ff<N>(L, pr, seg, fg);
@@ -503,7 +503,7 @@ DRT_HD bool path_step_redo_ff(const LinkDev &L, const TimeGridD &tg, const FreqG
         seg[i] = P[i] - P[i - 1];
         d = d + norm(seg[i]);
     }
-    fl |= validity<N>(pr, N, P);
+    fl |= validity<N>(pr, N, P, tg.far);
     if ((fl & (F_REDO64 | F_NOCONV | F_DEGEN)) || !isfinite(d.h)) return false;   // every bit is written out: all decided
     fl &= ~F_CLEAR;
     cx<ff> a = C<ff>(ff(0.f), ff(0.f));

@@ -169,10 +169,10 @@ k_trace(const LinkDev L, double t, long long n_cand, int with_tiles, const Posed
 
 // 1: the face blocks the segment, 0: it does not, -1: within the margins.  The ends' heights over the face are less certain than a
 // coordinate by upA and upB, their places along it by amp
-DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B, float upA, float upB, float amp) {
+DRT_NOINL1 int face_blocks_ff(const PosedFaceQ &F, v3<ff> A, v3<ff> B, float upA, float upB, float amp, float far) {
     const v3<ff> c = vq(F.c), n = vq(F.n);
     const ff ha = dot(A - c, n), hb = dot(B - c, n);
-    const float fa = fabsf(ha.h), fb = fabsf(hb.h), scale = fmaxf(fmaxf(amax3(A), amax3(B)), amax3(c));
+    const float fa = fabsf(ha.h), fb = fabsf(hb.h), scale = fmaxf(fmaxf(amax3(A), amax3(B)), fmaxf(amax3(c), far));
     // an end within 1e-9 m of the plane: the points of a chain lie on its own faces to ~2^-46 of the coordinates, which 2^-42 bounds
     const float tol = ff_margin_tol(scale), e = fmaxf(2.3e-13f * (scale + 1.f), 1e-10f);
     if (!(fabsf(fa - 1e-9f) > e * upA) || !(fabsf(fb - 1e-9f) > e * upB)) return -1;
@@ -222,7 +222,7 @@ DRT_HD bool corner_path(const Prim<ff> &E1, const Prim<ff> &E2, v3<ff> A, v3<ff>
 }
 
 template <int N>
-DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Prim<ff> *prims, TracedRay *r,
+DRT_HD int trace_chain_ff(const LinkDev &L, double t, float far, const int *code, const Prim<ff> *prims, TracedRay *r,
                           RayPoints *v) {
     const int NP = L.n_faces + L.n_edges;
     const ff tq = from_double(t);
@@ -294,7 +294,7 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pri
                 if (pf[j].type == T_D) s0[j] = (double)dot(Vf[j + 1] - pf[j].p, pf[j].a);
     }
     solve_geometry_any<N>(pr, V, s0, fl);
-    fl |= validity<N>(pr, N, V, &v->amp);
+    fl |= validity<N>(pr, N, V, far, &v->amp);
     if (fl & F_NOCONV) return RAY_OPEN;
 #pragma unroll
     for (int i = 1; i <= N; ++i)
@@ -313,7 +313,7 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, const int *code, const Pri
 }
 
 __global__ void __launch_bounds__(TRACE_T)
-k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int with_tiles, const Prim<ff> *__restrict__ prims,
+k_trace_ff(const __grid_constant__ LinkDev L, double t, float far, long long n_cand, int with_tiles, const Prim<ff> *__restrict__ prims,
            TracedRay *__restrict__ out, RayPoints *__restrict__ points, int cap, int *__restrict__ count) {
     const long long k = blockIdx.x * (long long)TRACE_T + threadIdx.x;
     if (k >= n_cand) return;
@@ -322,16 +322,16 @@ k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int wi
     RayPoints v{};
     int code[2] = {0, 0}, state;
     if (k == 0) {
-        state = trace_chain_ff<0>(L, t, code, prims, &r, &v);
+        state = trace_chain_ff<0>(L, t, far, code, prims, &r, &v);
     } else if (k - 1 < NP + NT) {
         code[0] = (int)(k - 1);
-        state = trace_chain_ff<1>(L, t, code, prims, &r, &v);
+        state = trace_chain_ff<1>(L, t, far, code, prims, &r, &v);
     } else {
         const long long q = k - 1 - NP - NT;
         code[0] = (int)(q / NP);
         code[1] = (int)(q % NP);
         if (code[0] == code[1]) return;
-        state = trace_chain_ff<2>(L, t, code, prims, &r, &v);
+        state = trace_chain_ff<2>(L, t, far, code, prims, &r, &v);
     }
     if (state < 0) return;
     r.index = k;
@@ -343,7 +343,7 @@ k_trace_ff(const __grid_constant__ LinkDev L, double t, long long n_cand, int wi
 }
 
 __global__ void __launch_bounds__(128)
-k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const PosedFace *__restrict__ faces,
+k_trace_block(const __grid_constant__ LinkDev L, double t, float far, int with_tiles, const PosedFace *__restrict__ faces,
               const PosedFaceQ *__restrict__ facesq, const Prim<ff> *__restrict__ prims, TracedRay *__restrict__ out, const RayPoints *__restrict__ points, int cap,
               const int *__restrict__ count) {
     const int n = min(*count, cap), lane = threadIdx.x & 31;
@@ -363,7 +363,7 @@ k_trace_block(const __grid_constant__ LinkDev L, double t, int with_tiles, const
                     return ty == T_S ? 1.f : height_amp(prims[r->prims[j] + (ty == T_D ? L.n_faces : 0)], n, v.amp);
                 };
                 const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(v.v[i - 1]), i == N ? rx : vq(v.v[i]),
-                                             i == 0 ? 1.f : up(i - 1), i == N ? 1.f : up(i), v.amp);
+                                             i == 0 ? 1.f : up(i - 1), i == N ? 1.f : up(i), v.amp, far);
                 hit = hit || b > 0;
                 open = open || b < 0;
             }
@@ -428,7 +428,7 @@ size_t trace_prim_bytes(const LinkDev &L, int cap) {   // posed faces and primit
 }
 
 cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_tiles, void *faces, void *rays, int cap,
-                         int *count, cudaStream_t s, void *prims_mem) {
+                         int *count, cudaStream_t s, void *prims_mem, double far) {
     const bool two = prims_mem != nullptr;
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
     if (e != cudaSuccess) return e;
@@ -443,8 +443,8 @@ cudaError_t launch_trace(const LinkDev &L, double t, int max_order, int with_til
         const int np = L.n_faces + L.n_edges;
         RayPoints *points = reinterpret_cast<RayPoints *>(prims + np);
         if (np) k_pose_prims<<<(np + 127) / 128, 128, 0, s>>>(L, t, prims);
-        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, prims, out, points, cap, count);
-        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, with_tiles, F, Q, prims, out, points, cap, count);
+        k_trace_ff<<<grid, TRACE_T, 0, s>>>(L, t, (float)far, n, with_tiles, prims, out, points, cap, count);
+        k_trace_block<<<152 * 4, 128, 0, s>>>(L, t, (float)far, with_tiles, F, Q, prims, out, points, cap, count);
         k_trace_polish<<<152 * 8, 32, 0, s>>>(L, t, out, cap, count);
     } else {
         k_trace<<<grid, TRACE_T, 0, s>>>(L, t, n, with_tiles, F, out, cap, count);

@@ -14,7 +14,7 @@ def build(source, folder):
     with open(src, "w") as f:
         f.write(source)
     r = subprocess.run([os.environ.get("NVCC", "nvcc"), *B.ARCH, "-O1", "-std=c++17", "--expt-relaxed-constexpr",
-                        "-Xcompiler", "-ffp-contract=off", "-I", CSRC, "-I", os.path.join(ROOT, "include"), src, "-o", exe,
+                        "-Xcompiler", "-ffp-contract=off", "-I", CSRC, "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "tests"), src, "-o", exe,
                         lib, "-Xlinker", "-rpath=" + os.path.dirname(lib)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout + r.stderr
     return exe

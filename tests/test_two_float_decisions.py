@@ -39,3 +39,11 @@ def test_chains_with_several_diffractions(decide, extent, shortest, angle, least
     n, decided, rays, wrong, unconverged = decide(most_diffractions=3, extent=extent, shortest=shortest, angle=angle,
                                                   come_from=0, seed=12, n=30000)
     assert wrong == 0 and unconverged <= n // 20000 and rays > 1000 and decided > least * n
+
+
+@pytest.mark.parametrize("come_from", [1e3, 1e5, 1e7])
+def test_chains_that_have_come_far(decide, come_from):
+    """A place keeps the rounding of the coordinates it is the difference of: o + v t of bodies and terminals that have driven far."""
+    n, decided, rays, wrong, unconverged = decide(most_diffractions=3, extent=20, shortest=1, angle=0.2, come_from=come_from, seed=13,
+                                                  n=30000)
+    assert wrong == 0 and unconverged == 0 and rays > 1000 and decided > 0.5 * n
