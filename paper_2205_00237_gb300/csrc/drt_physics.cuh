@@ -845,9 +845,10 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         if (!(mmin > need)) fl |= F_REDO64;
         if (out > need) fl |= F_CLEAR;
         if (amp_out) *amp_out = amp;
+        if (!(amp < 1e30f)) fl = (fl | F_REDO64) & ~F_CLEAR;
         // Several diffractions in a row where the FP64 Newton solve may not reach its step of 1e-10 m, 2^-53 of the coordinates times
-        // 9 amp: whether it does is a flag of its own
-        if (!(amp < 1e30f) || (nd > 1 && steep > 1e5f)) fl = (fl | F_REDO64) & ~F_CLEAR;
+        // 9 amp: whether it does is a flag of its own (a chain that is clearly none is none either way)
+        if (nd > 1 && steep > 1e5f) fl |= F_REDO64;
     }
     return fl;
 }
