@@ -674,17 +674,14 @@ DRT_HD float fp32_margin_tol(float scale) { return 2e-6f * (scale + 1.f); }
 // error bound.  (Called out of line in the FP32 kernels it measured no faster, unlike the field
 // updates, so it stays inline.)
 template <class T> struct VertexCheck { uint32_t fl; T m; };
-// The same in two-float numbers: the flags, the smallest margin over the bound on a coordinate's error, the largest margin by which a
-// test fails, and amp, by how much the point's place is less certain than a coordinate: leg / height for a reflection,
+// The same in two-float numbers: the flags, the smallest margin and the largest one by which a test fails (m), and amp, by how much the point's place is less certain than a coordinate: leg / height for a reflection,
 // (leg / distance from the edge line)^2 for a diffraction, whose Newton step divides by sin^2 of the angle to the edge.
 // the smaller of m and |v|, -1 from the first that is not a number on
 DRT_HD float least(float m, float v) { return ::fabsf(v) < m ? ::fabsf(v) : v == v ? m : -1.f; }
 struct VertexMargins { uint32_t fl; float m, out, amp; };
 DRT_NOINL1 VertexMargins vertex_margins(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v3<ff> cc, ff h1, ff h2, ff h3, ff h4,
-                                        v3<ff> Pm, v3<ff> Pi, v3<ff> Pp, float far) {
+                                        v3<ff> Pm, v3<ff> Pi, v3<ff> Pp) {
     VertexMargins r{0, 1e30f, 0.f, 1.f};
-    float scale = fmaxf(fmaxf(amax3(Pm), amax3(Pp)), fmaxf(amax3(Pi), far));
-    if (ty != T_S) scale = fmaxf(scale, amax3(c));
     // a test passes with margin v > 0 (not a number: undecided)
     auto test = [&](float v, uint32_t bit) {
         if (!(v > 0.f)) {
@@ -723,12 +720,9 @@ DRT_NOINL1 VertexMargins vertex_margins(int ty, v3<ff> c, v3<ff> nn, v3<ff> b, v
         test(hp, F_SIDE);
         if (ty == T_R) {
             const float leg = fabsf(Pm.x.h - Pp.x.h) + fabsf(Pm.y.h - Pp.y.h) + fabsf(Pm.z.h - Pp.z.h);
-            r.amp = 1.f + (leg + 1e-6f * scale) / (fabsf(hm) + fabsf(hp));
+            r.amp = 1.f + (leg + 1e-6f * amax3(Pi)) / (fabsf(hm) + fabsf(hp));
         }
     }
-    const float itol = 1.f / ff_margin_tol(scale);
-    r.m *= itol;
-    r.out *= itol;
     return r;
 }
 template <class T>
@@ -794,7 +788,7 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
     const int nv = N >= 0 ? N : n;
     uint32_t fl = 0;
     M mmin = M(1e30);    // FP32 and two-float only: the smallest margin over its bound
-    float out = 0.f, amp = 1.f, steep = 0.f;   // two-float only (vertex_margins)
+    float out = 0.f, amp = 1.f, steep = 0.f, scale = 0.f;   // two-float only (vertex_margins; scale: the largest coordinate)
     int nd = 0;
 #pragma unroll (N >= 0 ? 8 : 1)
     for (int i = 1; i <= MAXI + 1; ++i) {
@@ -803,11 +797,12 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         const T q = dot(d, d);
         if constexpr (FF) {
             // the margin of a length is held against the error bound itself, 2^-42: points that coincide shall be decided
-            const float v = ::sqrtf(q.h) - 1e-9f, w = 64.f / ff_margin_tol(fmaxf(fmaxf(amax3(P[i]), amax3(P[i - 1])), far));
-            mmin = least(mmin, v * w);
+            const float v = ::sqrtf(q.h) - 1e-9f;
+            scale = ::fmaxf(scale, i == 1 ? ::fmaxf(amax3(P[0]), amax3(P[1])) : amax3(P[i]));
+            mmin = least(mmin, 64.f * v);
             if (!(v >= 0.f)) {
                 fl |= F_DEGEN;
-                out = ::fmaxf(out, -v * w);
+                out = ::fmaxf(out, -64.f * v);
             }
         } else {
             if (!(q >= T(1e-18))) fl |= F_DEGEN;
@@ -819,14 +814,14 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
         const Prim<S> &q = pr[i - 1];
         if constexpr (FF) {
             const VertexMargins v =
-                vertex_margins(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1], far);
+                vertex_margins(q.type, val(q.p), val(q.a), q.b, q.c, q.h1, q.h2, q.h3, q.h4, P[i - 1], P[i], P[i + 1]);
             fl |= v.fl;
             mmin = ::fminf(mmin, v.m);
             out = ::fmaxf(out, v.out);
             amp *= v.amp;
             if (N >= 2 && q.type == T_D) {
                 ++nd;
-                steep = ::fmaxf(steep, v.amp * (amax3(P[i]) + 1.f));
+                steep = ::fmaxf(steep, v.amp);
             }
         } else {
             const VertexCheck<T> v =
@@ -841,14 +836,14 @@ DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *
     }
     if constexpr (FF) {
         // The bound is 1000 times the rounding of a coordinate (2^-46); 64 of that are for the amplification of a usual chain
-        const float need = ::fmaxf(1.f, amp * (1.f / 64.f));
+        const float need = ff_margin_tol(::fmaxf(scale, far)) * ::fmaxf(1.f, amp * (1.f / 64.f));
         if (!(mmin > need)) fl |= F_REDO64;
         if (out > need) fl |= F_CLEAR;
         if (amp_out) *amp_out = amp;
         if (!(amp < 1e30f)) fl = (fl | F_REDO64) & ~F_CLEAR;
         // Several diffractions in a row where the FP64 Newton solve may not reach its step of 1e-10 m, 2^-53 of the coordinates times
         // 9 amp: whether it does is a flag of its own (a chain that is clearly none is none either way)
-        if (nd > 1 && steep > 1e5f) fl |= F_REDO64;
+        if (nd > 1 && steep * (scale + 1.f) > 1e5f) fl |= F_REDO64;
     }
     return fl;
 }
