@@ -211,7 +211,8 @@ k_pose_prims(const __grid_constant__ LinkDev L, double t, Prim<ff> *__restrict__
 DRT_HD bool corner_path(const Prim<ff> &E1, const Prim<ff> &E2, v3<ff> A, v3<ff> B) {
     const v3<ff> x = cross(E1.a, E2.a), d = E2.p - E1.p;
     const ff xx = dot(x, x), gap = dot(d, x);
-    if (!(xx.h > 1e-4f) || !(gap.h * gap.h < 2.5e-19f * xx.h)) return false;   // the lines meet within 5e-10 m
+    // the lines meet within 5e-11 m: with |z|^2 < 0.99 the middle segment of the shortest path is then below 5e-10 m, no segment
+    if (!(xx.h > 1e-4f) || !(gap.h * gap.h < 2.5e-21f * xx.h)) return false;
     const v3<ff> C = axpy(E1.p, E1.a, dot(cross(d, E2.a), x) / xx);
     const v3<float> e1 = f32v(E1.a), e2 = f32v(E2.a), ac = f32v(C - A), cb = f32v(B - C);
     if (!(dot(ac, ac) > 0.01f) || !(dot(cb, cb) > 0.01f)) return false;
@@ -219,6 +220,45 @@ DRT_HD bool corner_path(const Prim<ff> &E1, const Prim<ff> &E2, v3<ff> A, v3<ff>
     const float c = dot(e1, e2), p = dot(u, e1), q = dot(w, e2), det = 1.f - c * c;
     const float a = (c * q - p) / det, b = (c * p - q) / det;   // z = a e1 + b e2
     return -(a * p + b * q) < 0.99f;                            // |z|^2
+}
+
+// A pair solved in FP32 first: whether the solve fails a test with every margin (the failed one's too) clear of the FP32 error, so that the
+// chain is none.  A coordinate's error moves a point by the amplification of vertex_margins at each vertex; the points' errors were at most
+// 0.08 of that product times 2e-6 of the coordinates (2e6 random pairs), so an eighth of it, and 1000 in any case, bounds the margins.
+struct Fp32Check { bool none; float margin, amp; };
+DRT_HD Fp32Check fp32_first(const Prim<ff> *pr, const v3<ff> *V, const double *s0, Prim<float> *pf, v3<float> *Vf, uint32_t &f0) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        pf[j].type = pr[j].type;
+        pf[j].p = f32v(pr[j].p);
+        pf[j].a = f32v(pr[j].a);
+        pf[j].b = f32v(pr[j].b);
+        pf[j].c = f32v(pr[j].c);
+        pf[j].h1 = pr[j].h1.h;
+        pf[j].h2 = pr[j].h2.h;
+        pf[j].h3 = pr[j].h3.h;
+        pf[j].h4 = pr[j].h4.h;
+    }
+    Vf[0] = f32v(V[0]);
+    Vf[3] = f32v(V[3]);
+    uint32_t bad = 0;
+    solve_geometry_any<2>(pf, Vf, s0, f0);
+    float margin = 1e30f, amp = 1.f;
+    bool fine = true;
+#pragma unroll
+    for (int i = 1; i <= 2; ++i) {
+        const Prim<float> &q = pf[i - 1];
+        const VertexCheck<float> v = vertex_validity_inl(q.type, q.p, q.a, q.b, q.c, q.h1, q.h2, q.h3, q.h4, Vf[i - 1], Vf[i], Vf[i + 1]);
+        bad |= v.fl;
+        margin = fminf(margin, v.m);
+        fine = fine && isfinite(Vf[i].x) && isfinite(Vf[i].y) && isfinite(Vf[i].z) && v.m > 1000.f;
+        // of a leg and its part along the normal or the edge: leg / height, or (leg / distance from the edge line)^2
+        const v3<float> dm = Vf[i - 1] - Vf[i], dp = Vf[i + 1] - Vf[i];
+        const float hm = dot(dm, q.a), hp = dot(dp, q.a), lm = dot(dm, dm), lp = dot(dp, dp);
+        if (q.type == T_R) amp *= 1.f + sqrtf(2.f * (lm + lp)) / (fabsf(hm) + fabsf(hp));
+        else amp *= 1.f / fmaxf(1.f - fmaxf(hm * hm / lm, hp * hp / lp), 0.f);
+    }
+    return Fp32Check{fine && bad && margin > 1000.f && margin > 0.125f * amp && !(f0 & (F_NOCONV | F_REDO64 | F_DEGEN)), margin, amp};
 }
 
 template <int N>
@@ -256,38 +296,10 @@ DRT_HD int trace_chain_ff(const LinkDev &L, double t, float far, const int *code
     uint32_t fl = 0;
     if constexpr (N == 2) {
         if (pr[0].type == T_D && pr[1].type == T_D && corner_path(pr[0], pr[1], V[0], V[3])) return -1;
-        // FP32 first.  A chain whose FP32 solve fails a test, with every margin (the failed one's too) above 1000 times the FP32
-        // bound 2e-6 of the coordinates, is none: an error of the solved points is that bound times (leg / height), and the
-        // heights are among the margins, so it is at most 1 / 60 of them.
         Prim<float> pf[2];
         v3<float> Vf[4];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            pf[j].type = pr[j].type;
-            pf[j].p = f32v(pr[j].p);
-            pf[j].a = f32v(pr[j].a);
-            pf[j].b = f32v(pr[j].b);
-            pf[j].c = f32v(pr[j].c);
-            pf[j].h1 = pr[j].h1.h;
-            pf[j].h2 = pr[j].h2.h;
-            pf[j].h3 = pr[j].h3.h;
-            pf[j].h4 = pr[j].h4.h;
-        }
-        Vf[0] = f32v(V[0]);
-        Vf[3] = f32v(V[3]);
-        uint32_t f0 = 0, bad = 0;
-        solve_geometry_any<2>(pf, Vf, s0, f0);
-        float margin = 1e30f;
-        bool fine = true;
-#pragma unroll
-        for (int i = 1; i <= 2; ++i) {
-            const Prim<float> &q = pf[i - 1];
-            const VertexCheck<float> v = vertex_validity_inl(q.type, q.p, q.a, q.b, q.c, q.h1, q.h2, q.h3, q.h4, Vf[i - 1], Vf[i], Vf[i + 1]);
-            bad |= v.fl;
-            margin = fminf(margin, v.m);
-            fine = fine && isfinite(Vf[i].x) && isfinite(Vf[i].y) && isfinite(Vf[i].z) && v.m > 1000.f;
-        }
-        if (fine && bad && margin > 1000.f && !(f0 & (F_NOCONV | F_REDO64 | F_DEGEN))) return -1;
+        uint32_t f0 = 0;
+        if (fp32_first(pr, V, s0, pf, Vf, f0).none) return -1;
         if (!(f0 & F_NOCONV))   // the two-float Newton solve starts from the FP32 one's
 #pragma unroll
             for (int j = 0; j < 2; ++j)
@@ -357,13 +369,17 @@ k_trace_block(const __grid_constant__ LinkDev L, double t, float far, int with_t
             bool hit = false, open = false;
             for (int q = lane; q < (N + 1) * L.n_faces; q += 32) {
                 const int i = q / L.n_faces, f = q - i * L.n_faces;
-                const v3<float> n = f32v(vq(facesq[f].n));
-                auto up = [&](int j) {   // of vertex j + 1 (terminals and tiles are where they are)
-                    const int ty = (r->types >> (8 * j)) & 0xff;
-                    return ty == T_S ? 1.f : height_amp(prims[r->prims[j] + (ty == T_D ? L.n_faces : 0)], n, v.amp);
-                };
-                const int b = face_blocks_ff(facesq[f], i == 0 ? tx : vq(v.v[i - 1]), i == N ? rx : vq(v.v[i]),
-                                             i == 0 ? 1.f : up(i - 1), i == N ? 1.f : up(i), v.amp, far);
+                const v3<ff> A = i == 0 ? tx : vq(v.v[i - 1]), B = i == N ? rx : vq(v.v[i]);
+                // (terminals and tiles are where they are; for nearly every face the most that a height can be off is enough)
+                int b = face_blocks_ff(facesq[f], A, B, i == 0 ? 1.f : 1.f + v.amp, i == N ? 1.f : 1.f + v.amp, v.amp, far);
+                if (b < 0) {
+                    const v3<float> n = f32v(vq(facesq[f].n));
+                    auto up = [&](int j) {   // of vertex j + 1
+                        const int ty = (r->types >> (8 * j)) & 0xff;
+                        return ty == T_S ? 1.f : height_amp(prims[r->prims[j] + (ty == T_D ? L.n_faces : 0)], n, v.amp);
+                    };
+                    b = face_blocks_ff(facesq[f], A, B, i == 0 ? 1.f : up(i - 1), i == N ? 1.f : up(i), v.amp, far);
+                }
                 hit = hit || b > 0;
                 open = open || b < 0;
             }
