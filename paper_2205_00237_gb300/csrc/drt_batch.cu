@@ -110,7 +110,7 @@ struct BatchPlan {
     bool dual = false;  // some link asks for Doppler outputs: carry the rates
     bool any_out = false;   // some link asks for per-path-step records (all units then run generic code)
     bool any_pair = false;  // some entries form carrier pairs
-    bool two = true;        // two-float numbers apply to every link and grid
+    bool any_two = false, any_64 = false;   // some link has two-float preparation and redo, some link FP64
     int synth_run = 1;      // items in turn per synthesis block (see k_batch_synth)
     cudaGraphExec_t graph = nullptr;
     cudaStream_t capture = nullptr;   // private stream the graph is captured on (any caller stream,
@@ -135,7 +135,6 @@ static BatchDev dev_view(const BatchPlan &P, int l0, int l1, long long n_items, 
     B.counter = reinterpret_cast<unsigned long long *>(P.mem) + k;
     B.rec_a = reinterpret_cast<float4 *>(P.mem + P.off_rec);
     B.rec_b = reinterpret_cast<float *>(P.mem + P.off_rec + P.rec_count * sizeof(float4));
-    B.two = P.two;
     B.synth_run = P.synth_run;
     B.redo.count = reinterpret_cast<int *>(P.mem + P.off_redo);
     B.redo.items = reinterpret_cast<int4 *>(P.mem + P.off_redo + 256);
@@ -152,23 +151,27 @@ static cudaError_t launch_synth_variant(int v, const BatchDev &B, int grid, cuda
     return cudaGetLastError();
 }
 
-// counters: 12 per wave (stages 0-3, bulk per chain length 0..3, generic bulk, synthesis, bulk of the
-// multi-diffraction chains of 2 and 3 vertices)
-constexpr int N_COUNTERS = 12;
+// counters: 15 per wave (stages 0-3, bulk per chain length 0..3, generic bulk, synthesis, bulk of the
+// multi-diffraction chains of 2 and 3 vertices, FP64 stages 1-3 beside two-float ones)
+constexpr int N_COUNTERS = 15;
 static size_t counter_of(size_t w, int slot) { return N_COUNTERS * w + slot; }
 
 // stages 0-3 of wave w
 static cudaError_t run_prep(BatchPlan &P, size_t w, cudaStream_t s) {
     const int grid = sm_count() * 4;
     const Wave &W = P.waves[w];
-    auto view = [&](int st) {
-        BatchDev B = dev_view(P, W.l0, W.l1, W.n_prep[st], counter_of(w, st));
+    auto launch = [&](int st, bool two, int slot) {
+        BatchDev B = dev_view(P, W.l0, W.l1, W.n_prep[st], counter_of(w, slot));
         B.it_base = W.prep0[st];
-        return B;
+        return launch_batch_stage(st, two, B, grid, s);
     };
-    for (int st = ST_POSEB; st <= ST_BASE; ++st)
-        if (W.n_prep[st])
-            if (cudaError_t e = launch_batch_stage(st, view(st), grid, s)) return e;
+    for (int st = ST_POSEB; st <= ST_BASE; ++st) {
+        if (!W.n_prep[st]) continue;
+        if (st == ST_POSEB || P.any_two)
+            if (cudaError_t e = launch(st, true, st)) return e;
+        if (st != ST_POSEB && P.any_64)
+            if (cudaError_t e = launch(st, false, 11 + st)) return e;
+    }
     return cudaSuccess;
 }
 
@@ -254,7 +257,6 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
     const int n = (int)links.size();
     BatchPlan *P = new BatchPlan();
     P->n_links = n;
-    for (int i = 0; i < n; ++i) P->two = P->two && ff_applies(views[i], tgs[i], fgs[i]);
     std::vector<int> order(n);
     std::iota(order.begin(), order.end(), 0);
     // largest links first: their units are claimed first
@@ -341,6 +343,8 @@ cudaError_t batch_build(const std::vector<const LinkDev *> &links, const std::ve
         chunk = std::max(4, chunk / std::max(1, chunk_div));
         B.tg = make_tgrid(tgs[i].t_start, tgs[i].dt, tgs[i].n_steps, chunk, ff_reach(views[i], tgs[i]));
         B.fg = make_fgrid(fgs[i].fc, fgs[i].bandwidth, fgs[i].n_bins);
+        B.two = ff_applies(views[i], tgs[i], fgs[i]);
+        (B.two ? P->any_two : P->any_64) = true;
         B.H = reinterpret_cast<float2 *>(H[i]);
         if (outs) B.out = outs[i];
         P->dual = P->dual || B.out.doppler != nullptr;

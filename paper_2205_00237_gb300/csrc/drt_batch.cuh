@@ -40,6 +40,7 @@ struct alignas(16) BatchLink {
     int32_t skip_p0, skip_p1;   // paths of that range with units of their own (the multi-diffraction
                                 // chains of 2 and 3 vertices; empty when the batch writes records)
     int32_t pair_p0;   // a pair's first entry also evaluates its partner's paths [pair_p0, n_paths)
+    int32_t two;       // two-float numbers apply to the link and its grids (ff_applies)
 };
 
 // one launch: the links [l0, l1) of its stage or wave, its item count and claim counter
@@ -51,7 +52,6 @@ struct BatchDev {
     unsigned long long *counter;
     float4 *rec_a;
     float *rec_b;
-    bool two;            // two-float numbers apply to every link and grid of the batch (ff_applies)
     int synth_run;       // items a synthesis block (or, in small links, each of its warps) takes in turn
     RedoList redo;   // items (link, path, step)
 };
@@ -76,7 +76,8 @@ cudaError_t launch_batch_bulk_multi(int N, bool pair, const BatchDev &B, int gri
 int batch_bulk_blocks(int N, bool multi = false);
 
 // the stage kernels in their own translation units
-cudaError_t launch_batch_stage(int stage, const BatchDev &B, int grid, cudaStream_t s);   // stages 0-3
+// stages 0-3; two: the links that two-float numbers apply to, else the others (stage 0: all)
+cudaError_t launch_batch_stage(int stage, bool two, const BatchDev &B, int grid, cudaStream_t s);
 cudaError_t launch_batch_redo(bool dual, const BatchDev &B, int grid, cudaStream_t s);
 
 }  // namespace drt

@@ -6,8 +6,9 @@
 
 namespace drt {
 
-// stages 0-3: block-wide claims of blockDim.x consecutive items; TWO: stages 1-3 in two-float numbers (PoseQ rows), the anchors at 4
-// blocks per SM (128 registers; 0.65 -> 0.52 ms of a 128-link batch against 2 blocks without spills)
+// stages 0-3: block-wide claims of blockDim.x consecutive items.  TWO: stages 1-3 of the links that two-float numbers apply to (PoseQ
+// rows), else of the others; a batch that has both runs both over all items, so that what a link gets does not depend on which
+// others are in its batch.  The two-float anchors at 4 blocks per SM (128 registers; 0.65 -> 0.52 ms of a 128-link batch against 2 blocks without spills)
 template <int STAGE, bool TWO>
 __global__ void __launch_bounds__(128, TWO && STAGE == ST_BASE ? 4 : 1) k_stage(const BatchDev B) {
     __shared__ long long s_start;
@@ -23,6 +24,7 @@ __global__ void __launch_bounds__(128, TWO && STAGE == ST_BASE ? 4 : 1) k_stage(
         const long long it = B.it_base + q;
         int li = find_link(B, STAGE, it);
         const BatchLink &BL = B.links[li];
+        if (STAGE != ST_POSEB && (BL.two != 0) != TWO) continue;
         long long local = it - BL.it0[STAGE];
         int nch = chunks_of(BL.tg);
         if (STAGE == ST_POSEB) {
@@ -56,8 +58,8 @@ template <bool TWO> static void launch_stage(int stage, const BatchDev &B, int g
     default: k_stage<ST_BASE, TWO><<<grid, 128, 0, s>>>(B); break;
     }
 }
-cudaError_t launch_batch_stage(int stage, const BatchDev &B, int grid, cudaStream_t s) {
-    if (B.two) launch_stage<true>(stage, B, grid, s);
+cudaError_t launch_batch_stage(int stage, bool two, const BatchDev &B, int grid, cudaStream_t s) {
+    if (two) launch_stage<true>(stage, B, grid, s);
     else launch_stage<false>(stage, B, grid, s);
     return cudaGetLastError();
 }

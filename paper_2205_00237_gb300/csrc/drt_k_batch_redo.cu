@@ -19,7 +19,7 @@ __device__ void redo_add_warp(const BatchDev &B, int4 itm, bool on, bool second)
     double r[3] = {0.0, 0.0, 0.0};
     if (on) {
         const BatchLink &BL = B.links[li];
-        path_step_redo<DUAL>(BL.L, BL.tg, BL.fg, itm.y, itm.z, BL.out, BL.warm, r, B.two);
+        path_step_redo<DUAL>(BL.L, BL.tg, BL.fg, itm.y, itm.z, BL.out, BL.warm, r, BL.two != 0);
     }
     __syncwarp();
     const int lane = threadIdx.x;
