@@ -73,8 +73,9 @@ struct Link {
     drt_scene_view view{};
     std::shared_ptr<std::atomic<int>> inflight = std::make_shared<std::atomic<int>>(0);   // serving
     std::shared_ptr<HostScene> scene;
-    std::vector<void *> allocs;
-    size_t bytes = 0;
+    // device blocks: the link's arrays, and their two-float copies (optional: make_room gives them back)
+    struct Block { void *ptr = nullptr; size_t bytes = 0; } block, two;
+    int plans = 0;   // batch plans that hold the device pointers
     int32_t n_paths = 0;
 };
 
@@ -110,7 +111,8 @@ struct drt_ctx {
     size_t arena_bytes = 0;
     // device blocks of unloaded links, kept for the next loads (size -> block): loading and unloading
     // links in a loop then costs no cudaMalloc / cudaFree; the blocks count against the HBM budget
-    std::multimap<size_t, void *> link_pool;
+    // ([0]: links' arrays, [1]: their two-float copies, whose sizes recur)
+    std::multimap<size_t, void *> link_pool[2];
     size_t link_pool_bytes = 0;
     // pinned host image of the link being loaded (grows with the largest one; the context lock is held from its filling to the end
     // of its copy): a fresh pageable image per load costs its page faults and a staged copy
@@ -144,31 +146,32 @@ void dev_free(drt_ctx *c, void *p, size_t bytes) {
 // large blocks), else a new allocation, after returning pooled blocks to the device when the budget
 // needs the room.  *got receives the block's size.
 constexpr size_t LINK_POOL_CAP = (size_t)1 << 30;   // pooled bytes kept at most
-drt_status link_block_alloc(drt_ctx *c, size_t bytes, void **out, size_t *got) {
+drt_status link_block_alloc(drt_ctx *c, int kind, size_t bytes, void **out, size_t *got) {
     bytes = std::max<size_t>(bytes, 256);
-    auto it = c->link_pool.lower_bound(bytes);
-    if (it != c->link_pool.end() && it->first <= 2 * bytes) {
+    auto it = c->link_pool[kind].lower_bound(bytes);
+    if (it != c->link_pool[kind].end() && it->first <= 2 * bytes) {
         *out = it->second;
         *got = it->first;
         c->link_pool_bytes -= it->first;
-        c->link_pool.erase(it);
+        c->link_pool[kind].erase(it);
         return DRT_OK;
     }
-    while (c->budget && c->used + bytes > c->budget && !c->link_pool.empty()) {
-        auto last = std::prev(c->link_pool.end());
-        cudaFree(last->second);
-        c->used -= last->first;
-        c->link_pool_bytes -= last->first;
-        c->link_pool.erase(last);
-    }
+    for (auto &pool : c->link_pool)
+        while (c->budget && c->used + bytes > c->budget && !pool.empty()) {
+            auto last = std::prev(pool.end());
+            cudaFree(last->second);
+            c->used -= last->first;
+            c->link_pool_bytes -= last->first;
+            pool.erase(last);
+        }
     *got = bytes;
     return dev_alloc(c, bytes, out);
 }
 // the caller has made sure that no queued work still reads the block
-void link_block_free(drt_ctx *c, void *p, size_t bytes) {
+void link_block_free(drt_ctx *c, int kind, void *p, size_t bytes) {
     if (!p) return;
     if (c->link_pool_bytes + bytes <= LINK_POOL_CAP) {
-        c->link_pool.emplace(bytes, p);
+        c->link_pool[kind].emplace(bytes, p);
         c->link_pool_bytes += bytes;
     } else {
         cudaFree(p);
@@ -196,7 +199,34 @@ void release(drt_ctx *c, Scratch &s) {
     s = Scratch{};
 }
 
-// the arrays of one link packed at 256-byte offsets into one host image, uploaded as one device
+// Give back what only makes calls faster: pooled link blocks, the two-float scratch of the ray tracer, the two-float copies of links
+// that no batch plan and no pending request uses (which run in FP64 from then on).  Whether there was any.
+bool make_room(drt_ctx *c) {
+    cudaDeviceSynchronize();
+    bool any = c->tr_prims.ptr || c->link_pool_bytes;
+    release(c, c->tr_prims);
+    for (auto &pool : c->link_pool) {
+        for (auto &kv : pool) dev_free(c, kv.second, kv.first);
+        pool.clear();
+    }
+    c->link_pool_bytes = 0;
+    for (auto &kv : c->links) {
+        Link &L = kv.second;
+        if (!L.two.ptr || L.plans || L.inflight->load() > 0) continue;
+        dev_free(c, L.two.ptr, L.two.bytes);
+        L.two = Link::Block{};
+        L.view.ff_range = false;
+        any = true;
+    }
+    return any;
+}
+// a call that finds no device memory is tried again after that, from its start: it takes its routes anew (again = true)
+template <class F> drt_status with_room(drt_ctx *c, F &&call) {
+    const drt_status st = call(false);
+    return st == DRT_ENOMEM && make_room(c) ? call(true) : st;
+}
+
+// arrays of one link packed at 256-byte offsets into one host image, uploaded as one device
 // allocation with one copy (separate allocations cost a cudaMalloc / cudaFree per array per link)
 struct LinkImage {
     struct Part { const void *src; size_t bytes, off; void *dst; };   // dst: the device pointer to set
@@ -207,30 +237,29 @@ struct LinkImage {
         size = off + v.size() * sizeof(X);
         parts.push_back(Part{v.data(), v.size() * sizeof(X), off, dst});
     }
-    // queued on the default stream; the staging image may be filled again once the stream has been waited for
-    drt_status upload(drt_ctx *c, Link &L) {
-        void *p = nullptr;
-        size_t got = 0;
-        if (drt_status st = link_block_alloc(c, size, &p, &got)) return st;
-        L.allocs.push_back(p);
-        L.bytes += got;
-        if (c->stage_cap < size) {
-            if (c->stage) cudaFreeHost(c->stage);
-            c->stage = nullptr;
-            c->stage_cap = 0;
-            const size_t want = std::max(size + size / 2, (size_t)1 << 20);
-            CUDA_TRY(cudaMallocHost(reinterpret_cast<void **>(&c->stage), want));
-            c->stage_cap = want;
-        }
+    // through the staging image from offset `at` on (stage_reserve), queued on the default stream; the staging image may be filled again
+    // once the stream has been waited for
+    drt_status upload(drt_ctx *c, int kind, Link::Block &b, size_t at) {
+        if (drt_status st = link_block_alloc(c, kind, size, &b.ptr, &b.bytes)) return st;
         for (const Part &q : parts) {
-            if (q.bytes) std::memcpy(c->stage + q.off, q.src, q.bytes);
-            const char *at = reinterpret_cast<const char *>(p) + q.off;
-            std::memcpy(q.dst, &at, sizeof at);
+            if (q.bytes) std::memcpy(c->stage + at + q.off, q.src, q.bytes);
+            const char *to = reinterpret_cast<const char *>(b.ptr) + q.off;
+            std::memcpy(q.dst, &to, sizeof to);
         }
-        if (size) CUDA_TRY(cudaMemcpyAsync(p, c->stage, size, cudaMemcpyHostToDevice, 0));
+        if (size) CUDA_TRY(cudaMemcpyAsync(b.ptr, c->stage + at, size, cudaMemcpyHostToDevice, 0));
         return DRT_OK;
     }
 };
+drt_status stage_reserve(drt_ctx *c, size_t size) {
+    if (c->stage_cap >= size) return DRT_OK;
+    if (c->stage) cudaFreeHost(c->stage);
+    c->stage = nullptr;
+    c->stage_cap = 0;
+    const size_t want = std::max(size + size / 2, (size_t)1 << 20);
+    CUDA_TRY(cudaMallocHost(reinterpret_cast<void **>(&c->stage), want));
+    c->stage_cap = want;
+    return DRT_OK;
+}
 
 bool finite3(const double *v) { return std::isfinite(v[0]) && std::isfinite(v[1]) && std::isfinite(v[2]); }
 double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
@@ -874,8 +903,9 @@ void drt_destroy(drt_ctx *c) {
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
     for (auto &kv : c->links)
-        for (void *p : kv.second.allocs) cudaFree(p);
-    for (auto &kv : c->link_pool) cudaFree(kv.second);
+        for (const Link::Block *b : {&kv.second.block, &kv.second.two}) cudaFree(b->ptr);
+    for (auto &pool : c->link_pool)
+        for (auto &kv : pool) cudaFree(kv.second);
     for (Scratch *s : {&c->pose, &c->rec_a, &c->rec_b, &c->h, &c->poseb, &c->base, &c->pose64, &c->redo, &c->warm, &c->redo3, &c->pp_tau,
                        &c->pp_amp, &c->pp_fd, &c->pp_fl, &c->lt_tot, &c->lt_major, &c->win_sel, &c->win_starts,
                        &c->tr_faces, &c->tr_rays, &c->tr_count, &c->tr_prims})
@@ -904,8 +934,9 @@ namespace {
 void free_link(drt_ctx *c, Link &L);
 
 // scene: the host copy that *s is a view of, when there is one already
+// copies_too: with the two-float copies, where they apply and there is room
 drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Link &L,
-                     std::shared_ptr<HostScene> scene = nullptr) {
+                     std::shared_ptr<HostScene> scene = nullptr, bool copies_too = true) {
     PackedLink H;
     if (drt_status st = pack_link(s, ps, H)) return st;
     auto hs = scene ? scene : std::make_shared<HostScene>();
@@ -925,35 +956,36 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     LinkDev &d = L.dev;
     const size_t n_t0 = (size_t)(d.n_paths - d.n_bulk) * 2 * MAXI;
     std::vector<double> t0par(n_t0, 0.0);
-    auto image = [&](bool two) {
-        LinkImage img;
-        img.add(H.bodies, &d.bodies);
-        img.add(H.body_fixed, &d.body_fixed);
-        img.add(H.faces, &d.faces);
-        img.add(H.edges, &d.edges);
-        img.add(H.tiles, &d.tiles);
-        img.add(H.mats, &d.mats);
-        img.add(H.facesF, &d.facesF);
-        img.add(H.edgesF, &d.edgesF);
-        img.add(H.tilesF, &d.tilesF);
-        if (two) {   // the two-float copies
-            img.add(H.facesQ, &d.facesQ);
-            img.add(H.edgesQ, &d.edgesQ);
-            img.add(H.tilesQ, &d.tilesQ);
-            img.add(H.bodiesQ, &d.bodiesQ);
+    LinkImage img, copies;
+    img.add(H.bodies, &d.bodies);
+    img.add(H.body_fixed, &d.body_fixed);
+    img.add(H.faces, &d.faces);
+    img.add(H.edges, &d.edges);
+    img.add(H.tiles, &d.tiles);
+    img.add(H.mats, &d.mats);
+    img.add(H.facesF, &d.facesF);
+    img.add(H.edgesF, &d.edgesF);
+    img.add(H.tilesF, &d.tilesF);
+    img.add(H.ptypes, &d.ptypes);
+    img.add(H.pprims, &d.pprims);
+    img.add(H.ps0, &d.ps0);
+    img.add(H.perm, &d.perm);
+    // multi-diffraction edge parameters and rates at t = 0 (warm-start predictor), solved below
+    img.add(t0par, &d.t0par);
+    copies.add(H.facesQ, &d.facesQ);
+    copies.add(H.edgesQ, &d.edgesQ);
+    copies.add(H.tilesQ, &d.tilesQ);
+    copies.add(H.bodiesQ, &d.bodiesQ);
+    const size_t at = (img.size + 255) & ~(size_t)255;
+    drt_status st = stage_reserve(c, at + copies.size);
+    if (!st) st = img.upload(c, 0, L.block, 0);
+    L.view.ff_range = L.view.ff_range && copies_too;
+    if (!st && L.view.ff_range) {
+        st = copies.upload(c, 1, L.two, at);
+        if (st == DRT_ENOMEM) {   // no room for them: FP64 everywhere
+            L.view.ff_range = false;
+            st = DRT_OK;
         }
-        img.add(H.ptypes, &d.ptypes);
-        img.add(H.pprims, &d.pprims);
-        img.add(H.ps0, &d.ps0);
-        img.add(H.perm, &d.perm);
-        // multi-diffraction edge parameters and rates at t = 0 (warm-start predictor), solved below
-        img.add(t0par, &d.t0par);
-        return img;
-    };
-    drt_status st = image(true).upload(c, L);
-    if (st == DRT_ENOMEM) {   // no room for the two-float copies: FP64 everywhere
-        L.view.ff_range = false;
-        st = image(false).upload(c, L);
     }
     if (!st && n_t0) {
         // at t = 0, whatever the grids of later calls: edge parameters only (1e-6 m is enough of a start)
@@ -971,11 +1003,11 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     return DRT_OK;
 }
 
-// a link holds one block (see LinkImage); the caller has made sure no queued work reads it
+// the caller has made sure that no queued work reads the link's blocks
 void free_link(drt_ctx *c, Link &L) {
-    for (void *p : L.allocs) link_block_free(c, p, L.bytes);
-    L.allocs.clear();
-    L.bytes = 0;
+    link_block_free(c, 0, L.block.ptr, L.block.bytes);
+    link_block_free(c, 1, L.two.ptr, L.two.bytes);
+    L.block = L.two = Link::Block{};
 }
 
 }  // namespace
@@ -988,7 +1020,7 @@ drt_status drt_load_paths(drt_ctx *c, const drt_scene *s, const drt_path_set *ps
     std::lock_guard<std::mutex> lk(c->mu);
     CUDA_TRY(cudaSetDevice(c->device));
     Link L;
-    if (drt_status st = load_link(c, s, ps, L)) return st;
+    if (drt_status st = with_room(c, [&](bool) { return load_link(c, s, ps, L); })) return st;
     uint64_t id = c->next_link++;
     c->links.emplace(id, std::move(L));
     *out_link = id;
@@ -1028,7 +1060,7 @@ drt_status drt_extrapolate(drt_ctx *c, uint64_t link, const drt_time_grid *tg, c
     CUDA_TRY(cudaSetDevice(c->device));
     OutD o{out->tau, out->amp, out->doppler, out->angles, out->flags, out->points};
     RecD none{nullptr, nullptr};
-    return run_extrapolation(c, *L, tg, fg, o, none, precision, (cudaStream_t)stream);
+    return with_room(c, [&](bool) { return run_extrapolation(c, *L, tg, fg, o, none, precision, (cudaStream_t)stream); });
 }
 
 drt_status drt_synthesize_H(drt_ctx *c, uint64_t link, const drt_time_grid *tg, const drt_freq_grid *fg, void *H,
@@ -1039,7 +1071,7 @@ drt_status drt_synthesize_H(drt_ctx *c, uint64_t link, const drt_time_grid *tg, 
     Link *L = find_link(c, link);
     if (!L) return fail(DRT_ENOTFOUND, "unknown link %llu", (unsigned long long)link);
     CUDA_TRY(cudaSetDevice(c->device));
-    return synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(H), precision, (cudaStream_t)stream);
+    return with_room(c, [&](bool) { return synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(H), precision, (cudaStream_t)stream); });
 }
 
 drt_status drt_synthesize_H_host(drt_ctx *c, uint64_t link, const drt_time_grid *tg, const drt_freq_grid *fg,
@@ -1051,9 +1083,12 @@ drt_status drt_synthesize_H_host(drt_ctx *c, uint64_t link, const drt_time_grid 
     if (!L) return fail(DRT_ENOTFOUND, "unknown link %llu", (unsigned long long)link);
     CUDA_TRY(cudaSetDevice(c->device));
     size_t bytes = (size_t)tg->n_steps * fg->n_bins * sizeof(float2);
-    if (drt_status st = ensure(c, c->h, bytes)) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    if (drt_status st = synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(c->h.ptr), precision, s)) return st;
+    if (drt_status st = with_room(c, [&](bool) -> drt_status {
+            if (drt_status q = ensure(c, c->h, bytes)) return q;
+            return synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(c->h.ptr), precision, s);
+        }))
+        return st;
     CUDA_TRY(cudaMemcpyAsync(H_host, c->h.ptr, bytes, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     return DRT_OK;
@@ -1074,15 +1109,18 @@ drt_status drt_power_profile(drt_ctx *c, uint64_t link, const drt_time_grid *tg,
     CUDA_TRY(cudaSetDevice(c->device));
     const size_t n = (size_t)tg->n_steps * L->n_paths;
     const size_t fsz = precision == DRT_FP64 ? sizeof(double) : sizeof(float);
-    if (drt_status st = ensure(c, c->pp_tau, n * sizeof(double) + 8)) return st;
-    if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
-    if (drt_status st = ensure(c, c->pp_fd, n * fsz + 8)) return st;
-    if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
-    OutD o{reinterpret_cast<double *>(c->pp_tau.ptr), c->pp_amp.ptr, c->pp_fd.ptr, nullptr,
-           reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
     cudaStream_t s = (cudaStream_t)stream;
-    RecD none{nullptr, nullptr};
-    if (drt_status st = run_extrapolation(c, *L, tg, fg, o, none, precision, s)) return st;
+    OutD o{};
+    if (drt_status st = with_room(c, [&](bool) -> drt_status {
+            if (drt_status q = ensure(c, c->pp_tau, n * sizeof(double) + 8)) return q;
+            if (drt_status q = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return q;
+            if (drt_status q = ensure(c, c->pp_fd, n * fsz + 8)) return q;
+            if (drt_status q = ensure(c, c->pp_fl, n + 8)) return q;
+            o = OutD{reinterpret_cast<double *>(c->pp_tau.ptr), c->pp_amp.ptr, c->pp_fd.ptr, nullptr,
+                     reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
+            return run_extrapolation(c, *L, tg, fg, o, RecD{nullptr, nullptr}, precision, s);
+        }))
+        return st;
     CUDA_TRY(launch_power_bin(precision == DRT_FP64, o, tg->n_steps, L->n_paths, g->steps_per_bin, g->x0, g->dx,
                               g->n_bins, g->kind, P, s));
     return DRT_OK;
@@ -1105,47 +1143,51 @@ drt_status drt_lifetime_windows(drt_ctx *c, uint64_t link, const drt_time_grid *
     if (T == 0) return DRT_OK;
     const size_t n = (size_t)T * L->n_paths;
     const size_t fsz = precision == DRT_FP64 ? sizeof(double) : sizeof(float);
-    if (drt_status st = ensure(c, c->lt_tot, (size_t)T * sizeof(double))) return st;
-    if (drt_status st = ensure(c, c->lt_major, (size_t)T + 1)) return st;
-    uint8_t *mj = reinterpret_cast<uint8_t *>(c->lt_major.ptr);
-    double *tot = reinterpret_cast<double *>(c->lt_tot.ptr);
-    cudaStream_t s = (cudaStream_t)stream;
-    const RecD none{nullptr, nullptr};
     std::vector<uint8_t> m((size_t)T + 1);
-    bool decided = false;
-    // FP64 form: the changes from the synthesis records (two-float arithmetic, a quarter of the FP64 outputs' time), unless one of
-    // them lies within the records' rounding of the threshold
-    if (precision == DRT_FP64 && lp->share >= 1e-12 && ff_applies(L->view, *tg, *fg) &&
-        ensure(c, c->rec_a, n * sizeof(float4)) == DRT_OK && ensure(c, c->rec_b, n * sizeof(float)) == DRT_OK) {
-        const RecD rec{reinterpret_cast<float4 *>(c->rec_a.ptr), reinterpret_cast<float *>(c->rec_b.ptr)};
-        const drt_status st = run_extrapolation(c, *L, tg, fg, OutD{}, rec, precision, s);
-        if (st && st != DRT_ENOMEM) return st;
-        if (!st) {
-            CUDA_TRY(launch_lifetime_rec(rec, T, L->n_paths, lp->share, tot, mj, s));
-            CUDA_TRY(cudaMemcpyAsync(m.data(), mj, (size_t)T + 1, cudaMemcpyDeviceToHost, s));
-            CUDA_TRY(cudaStreamSynchronize(s));
-            decided = m[T] == 0;
-        }
-    }
-    if (!decided) {
-        OutD o{};
-        auto outputs = [&]() -> drt_status {
-            if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
-            if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
-            o = OutD{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
-            return run_extrapolation(c, *L, tg, fg, o, none, precision, s);
-        };
-        drt_status st = outputs();
-        if (st == DRT_ENOMEM) {   // the records taken above (or by an earlier call) may be what exceeds the budget
-            release(c, c->rec_a);
-            release(c, c->rec_b);
-            st = outputs();
-        }
-        if (st) return st;
-        CUDA_TRY(launch_lifetime(precision == DRT_FP64, o, T, L->n_paths, lp->share, tot, mj, s));
-        CUDA_TRY(cudaMemcpyAsync(m.data(), mj, T, cudaMemcpyDeviceToHost, s));
-        CUDA_TRY(cudaStreamSynchronize(s));
-    }
+    if (drt_status st = with_room(c, [&](bool) -> drt_status {
+            if (drt_status st = ensure(c, c->lt_tot, (size_t)T * sizeof(double))) return st;
+            if (drt_status st = ensure(c, c->lt_major, (size_t)T + 1)) return st;
+            uint8_t *mj = reinterpret_cast<uint8_t *>(c->lt_major.ptr);
+            double *tot = reinterpret_cast<double *>(c->lt_tot.ptr);
+            cudaStream_t s = (cudaStream_t)stream;
+            const RecD none{nullptr, nullptr};
+            bool decided = false;
+            // FP64 form: the changes from the synthesis records (two-float arithmetic, a quarter of the FP64 outputs' time), unless one of
+            // them lies within the records' rounding of the threshold
+            if (precision == DRT_FP64 && lp->share >= 1e-12 && ff_applies(L->view, *tg, *fg) &&
+                ensure(c, c->rec_a, n * sizeof(float4)) == DRT_OK && ensure(c, c->rec_b, n * sizeof(float)) == DRT_OK) {
+                const RecD rec{reinterpret_cast<float4 *>(c->rec_a.ptr), reinterpret_cast<float *>(c->rec_b.ptr)};
+                const drt_status st = run_extrapolation(c, *L, tg, fg, OutD{}, rec, precision, s);
+                if (st && st != DRT_ENOMEM) return st;
+                if (!st) {
+                    CUDA_TRY(launch_lifetime_rec(rec, T, L->n_paths, lp->share, tot, mj, s));
+                    CUDA_TRY(cudaMemcpyAsync(m.data(), mj, (size_t)T + 1, cudaMemcpyDeviceToHost, s));
+                    CUDA_TRY(cudaStreamSynchronize(s));
+                    decided = m[T] == 0;
+                }
+            }
+            if (!decided) {
+                OutD o{};
+                auto outputs = [&]() -> drt_status {
+                    if (drt_status st = ensure(c, c->pp_amp, 2 * n * fsz + 8)) return st;
+                    if (drt_status st = ensure(c, c->pp_fl, n + 8)) return st;
+                    o = OutD{nullptr, c->pp_amp.ptr, nullptr, nullptr, reinterpret_cast<uint8_t *>(c->pp_fl.ptr), nullptr};
+                    return run_extrapolation(c, *L, tg, fg, o, none, precision, s);
+                };
+                drt_status st = outputs();
+                if (st == DRT_ENOMEM) {   // the records taken above (or by an earlier call) may be what exceeds the budget
+                    release(c, c->rec_a);
+                    release(c, c->rec_b);
+                    st = outputs();
+                }
+                if (st) return st;
+                CUDA_TRY(launch_lifetime(precision == DRT_FP64, o, T, L->n_paths, lp->share, tot, mj, s));
+                CUDA_TRY(cudaMemcpyAsync(m.data(), mj, T, cudaMemcpyDeviceToHost, s));
+                CUDA_TRY(cudaStreamSynchronize(s));
+            }
+            return DRT_OK;
+        }))
+        return st;
     if (major) std::memcpy(major, m.data(), T);
     // windows: from start w, the first major change in [w + min_steps, w + max_steps], else w + max_steps
     std::vector<int32_t> w{0};
@@ -1189,12 +1231,14 @@ drt_status drt_synthesize_H_windows(drt_ctx *c, uint64_t link, const drt_time_gr
     cudaStream_t s = (cudaStream_t)stream;
     // re-initialisation at every window start: the paths valid there (FP64 flags of that instant,
     // one selection launch inside the synthesis)
-    if (drt_status st = ensure(c, c->win_sel, (size_t)T * P + 8)) return st;
-    if (drt_status st = ensure(c, c->win_starts, (size_t)n_windows * sizeof(int32_t))) return st;
-    int32_t *sd = reinterpret_cast<int32_t *>(c->win_starts.ptr);
-    CUDA_TRY(cudaMemcpyAsync(sd, starts, (size_t)n_windows * sizeof(int32_t), cudaMemcpyHostToDevice, s));
-    WinMask wm{sd, n_windows, reinterpret_cast<uint8_t *>(c->win_sel.ptr)};
-    return synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(H), precision, s, &wm);
+    return with_room(c, [&](bool) -> drt_status {
+        if (drt_status st = ensure(c, c->win_sel, (size_t)T * P + 8)) return st;
+        if (drt_status st = ensure(c, c->win_starts, (size_t)n_windows * sizeof(int32_t))) return st;
+        int32_t *sd = reinterpret_cast<int32_t *>(c->win_starts.ptr);
+        CUDA_TRY(cudaMemcpyAsync(sd, starts, (size_t)n_windows * sizeof(int32_t), cudaMemcpyHostToDevice, s));
+        WinMask wm{sd, n_windows, reinterpret_cast<uint8_t *>(c->win_sel.ptr)};
+        return synth_into(c, *L, tg, fg, reinterpret_cast<float2 *>(H), precision, s, &wm);
+    });
 }
 
 drt_status drt_synthesize_H_wideband(drt_ctx *c, uint64_t link, const drt_time_grid *tg, const drt_freq_grid *fg,
@@ -1214,7 +1258,10 @@ drt_status drt_synthesize_H_wideband(drt_ctx *c, uint64_t link, const drt_time_g
         const int k0 = (int)((long long)sb * N / n_sub), k1 = (int)((long long)(sb + 1) * N / n_sub);
         const int n = k1 - k0;
         drt_freq_grid fs{fg->fc - 0.5 * fg->bandwidth + (k0 + 0.5 * n) * df, n * df, n, 0};
-        if (drt_status st = synth_into(c, *L, tg, &fs, h + k0, precision, (cudaStream_t)stream, nullptr, N)) return st;
+        if (drt_status st = with_room(c, [&](bool) {
+                return synth_into(c, *L, tg, &fs, h + k0, precision, (cudaStream_t)stream, nullptr, N);
+            }))
+            return st;
     }
     return DRT_OK;
 }
@@ -1274,7 +1321,10 @@ drt_status drt_trace_paths(drt_ctx *c, uint64_t link, double t, int32_t max_orde
     CUDA_TRY(cudaSetDevice(c->device));
     std::vector<char> rays;
     int n = 0;
-    if (drt_status st = trace_into(c, *L, t, max_order, with_tiles != 0, rays, &n, (cudaStream_t)stream)) return st;
+    if (drt_status st = with_room(c, [&](bool) {
+            return trace_into(c, *L, t, max_order, with_tiles != 0, rays, &n, (cudaStream_t)stream);
+        }))
+        return st;
     out->n_found = trace_unpack(rays.data(), n, out->n_int, out->types, out->prims, out->s0, out->cap);
     return DRT_OK;
 }
@@ -1307,26 +1357,30 @@ drt_status drt_synthesize_H_retraced(drt_ctx *c, uint64_t link, const drt_time_g
     for (int w = 0; w < n_windows && T > 0; ++w) {
         const int k0 = starts[w], k1 = w + 1 < n_windows ? starts[w + 1] : T;
         const double tw = tg->t_start + k0 * tg->dt;
-        // the window's chains: a ray-tracing run at its first instant
-        int listed = 0;
-        if (drt_status st = trace_into(c, *L, tw, max_order, with_tiles != 0, rays, &listed, s)) return st;
-        n_int.resize(listed);
-        types.resize((size_t)listed * MAXI);
-        prims.resize((size_t)listed * MAXI);
-        s0.resize((size_t)listed * MAXI);
-        drt_traced_paths tp{listed, 0, n_int.data(), types.data(), prims.data(), s0.data()};
-        tp.n_found = trace_unpack(rays.data(), listed, tp.n_int, tp.types, tp.prims, tp.s0, tp.cap);
-        // extrapolated over the window's instants into its rows of H
-        const drt_path_set ps{tp.n_found, 0, n_int.data(), types.data(), prims.data(), s0.data()};
-        Link W;
-        if (drt_status st = load_link(c, &scene, &ps, W, L->scene)) return st;
-        const drt_time_grid tw_grid{tw, tg->dt, k1 - k0, 0};
-        drt_status st = synth_into(c, W, &tw_grid, fg, reinterpret_cast<float2 *>(H) + (size_t)k0 * F, precision, s,
-                                   nullptr, F);
-        cudaError_t e = cudaStreamSynchronize(s);
-        free_link(c, W);
-        if (st) return st;
-        if (e != cudaSuccess) return fail(DRT_ECUDA, "window %d: %s", w, cudaGetErrorString(e));
+        if (drt_status st = with_room(c, [&](bool again) -> drt_status {
+                // the window's chains: a ray-tracing run at its first instant
+                int listed = 0;
+                if (drt_status st = trace_into(c, *L, tw, max_order, with_tiles != 0, rays, &listed, s)) return st;
+                n_int.resize(listed);
+                types.resize((size_t)listed * MAXI);
+                prims.resize((size_t)listed * MAXI);
+                s0.resize((size_t)listed * MAXI);
+                drt_traced_paths tp{listed, 0, n_int.data(), types.data(), prims.data(), s0.data()};
+                tp.n_found = trace_unpack(rays.data(), listed, tp.n_int, tp.types, tp.prims, tp.s0, tp.cap);
+                // extrapolated over the window's instants into its rows of H
+                const drt_path_set ps{tp.n_found, 0, n_int.data(), types.data(), prims.data(), s0.data()};
+                Link W;
+                if (drt_status st = load_link(c, &scene, &ps, W, L->scene, !again)) return st;
+                const drt_time_grid tw_grid{tw, tg->dt, k1 - k0, 0};
+                drt_status st = synth_into(c, W, &tw_grid, fg, reinterpret_cast<float2 *>(H) + (size_t)k0 * F, precision, s,
+                                           nullptr, F);
+                cudaError_t e = cudaStreamSynchronize(s);
+                free_link(c, W);
+                if (st) return st;
+                if (e != cudaSuccess) return fail(DRT_ECUDA, "window %d: %s", w, cudaGetErrorString(e));
+                return DRT_OK;
+            }))
+            return st;
     }
     return DRT_OK;
 }
@@ -1467,7 +1521,11 @@ struct drt_batch {
     int32_t chunk_div = 1;                  // chosen divisor of the phase-error model's chunk
     float chunk_ns[3] = {0.f, 0.f, 0.f};    // first wave's preparation + extrapolation, ns per path-step,
                                             // at the model's chunk, 1/2 and 1/4 of it
+    std::vector<uint64_t> links;            // whose device pointers the plan holds (Link::plans)
 };
+
+static drt_status batch_create_locked(drt_ctx *c, int32_t n_links, const uint64_t *links, const drt_time_grid *tgrids,
+                                      const drt_freq_grid *fgrids, void *const *H, int32_t precision, drt_batch **out);
 
 extern "C" drt_status drt_batch_create(drt_ctx *c, int32_t n_links, const uint64_t *links, const drt_time_grid *tgrids,
                                        const drt_freq_grid *fgrids, void *const *H, int32_t precision,
@@ -1479,6 +1537,11 @@ extern "C" drt_status drt_batch_create(drt_ctx *c, int32_t n_links, const uint64
                                 "per link for DRT_FP64");
     *out = nullptr;
     std::lock_guard<std::mutex> lk(c->mu);
+    return with_room(c, [&](bool) { return batch_create_locked(c, n_links, links, tgrids, fgrids, H, precision, out); });
+}
+
+static drt_status batch_create_locked(drt_ctx *c, int32_t n_links, const uint64_t *links, const drt_time_grid *tgrids,
+                                      const drt_freq_grid *fgrids, void *const *H, int32_t precision, drt_batch **out) {
     std::vector<const LinkDev *> devs(n_links);
     std::vector<drt_scene_view> views(n_links);
     for (int i = 0; i < n_links; ++i) {
@@ -1519,6 +1582,7 @@ extern "C" drt_status drt_batch_create(drt_ctx *c, int32_t n_links, const uint64
     void *mem = nullptr;
     cudaError_t e = cudaMalloc(&mem, std::max<size_t>(bytes, 256));
     if (e != cudaSuccess) {
+        cudaGetLastError();   // as in dev_alloc
         drop(-1);
         return fail(DRT_ENOMEM, "batch allocation of %zu bytes: %s", bytes, cudaGetErrorString(e));
     }
@@ -1549,6 +1613,8 @@ extern "C" drt_status drt_batch_create(drt_ctx *c, int32_t n_links, const uint64
         delete b;
         return fail(DRT_ECUDA, "batch autotune: %s", cudaGetErrorString(e));
     }
+    b->links.assign(links, links + n_links);
+    for (uint64_t id : b->links) ++find_link(c, id)->plans;
     *out = b;
     return DRT_OK;
 }
@@ -1597,6 +1663,8 @@ extern "C" void drt_batch_destroy(drt_ctx *c, drt_batch *b) {
     cudaDeviceSynchronize();
     batch_free(b->plan);
     c->used -= b->bytes;
+    for (uint64_t id : b->links)
+        if (Link *L = find_link(c, id)) --L->plans;
     delete b;
 }
 
@@ -1612,7 +1680,7 @@ static drt_status serve_start_locked(drt_ctx *c, uint64_t pool_bytes, int32_t n_
     if (pool_bytes < (1u << 20)) return fail(DRT_ENOMEM, "no HBM budget left for the serving arena");
     CUDA_TRY(cudaSetDevice(c->device));
     void *arena = nullptr;
-    if (drt_status st = dev_alloc(c, pool_bytes, &arena)) return st;
+    if (drt_status st = with_room(c, [&](bool) { return dev_alloc(c, pool_bytes, &arena); })) return st;
     Server *S = server_start(c->device, arena, pool_bytes, n_slots, max_batch);
     if (!S) {
         dev_free(c, arena, pool_bytes);
