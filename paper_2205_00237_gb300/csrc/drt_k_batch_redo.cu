@@ -29,19 +29,24 @@ __device__ void redo_add_warp(const BatchDev &B, int4 itm, bool on, bool second)
         const double tau = __shfl_sync(0xffffffffu, r[2], l);
         const int step = __shfl_sync(0xffffffffu, itm.z, l);
         const BatchLink &BL = B.links[__shfl_sync(0xffffffffu, li, l)];
-        // a exp(-j 2 pi f_k tau): FP64-reduced seed at the lane's first bin, FP32 rotation by 32 bins
-        const double f0 = BL.fg.f0, df = BL.fg.df, x = (f0 + lane * df) * tau, xs = 32 * df * tau;
+        // a exp(-j 2 pi f_k tau): FP64-reduced seed at the lane's bin of every 512, between them at most 15 FP32 rotations by 32 bins
+        // (each adds the rounding of its angle: one seed for 4096 bins was 2e-5 off at the last ones)
+        const double f0 = BL.fg.f0, df = BL.fg.df, xs = 32 * df * tau;
         const int F = BL.fg.n_bins;
         float2 *row = BL.H + (size_t)step * F;
-        float sn, cs, ws, wc;
-        sincospif(2.f * (float)(x - floor(x)), &sn, &cs);
+        float ws, wc;
         sincospif(2.f * (float)(xs - floor(xs)), &ws, &wc);
-        float zr = fmaf(ar, cs, ai * sn), zi = fmaf(ai, cs, -ar * sn);
-        for (int k = lane; k < F; k += 32) {
-            atomicAdd(row + k, make_float2(zr, zi));
-            const float nr = fmaf(zr, wc, zi * ws);
-            zi = fmaf(zi, wc, -zr * ws);
-            zr = nr;
+        for (int k0 = lane; k0 < F; k0 += 512) {
+            const double x = (f0 + k0 * df) * tau;
+            float sn, cs;
+            sincospif(2.f * (float)(x - floor(x)), &sn, &cs);
+            float zr = fmaf(ar, cs, ai * sn), zi = fmaf(ai, cs, -ar * sn);
+            for (int k = k0; k < F && k < k0 + 512; k += 32) {
+                atomicAdd(row + k, make_float2(zr, zi));
+                const float nr = fmaf(zr, wc, zi * ws);
+                zi = fmaf(zi, wc, -zr * ws);
+                zr = nr;
+            }
         }
     }
 }
