@@ -200,4 +200,13 @@ inline __host__ __device__ __noinline__ ff angle2pi(ff y, ff x) {
     return quick(t, fmul(num.h, rsqrtf(ffma(x.h, x.h, fmul(y.h, y.h)))));
 }
 
+// the angle of (x, y) as atan2f gives it, to its FP32 rounding: the FP32 angle and the angle from it
+inline __host__ __device__ __noinline__ float atan2_ff(ff y, ff x) {
+    const float t = atan2f(y.h, x.h), q = ffma(x.h, x.h, fmul(y.h, y.h));
+    if (!(q > 0.f)) return t;
+    ff s, c;
+    sincos_ff(ff(t, 0.f), s, c);
+    return fadd(t, fmul(det2(y, c, x, s).h, rsqrtf(q)));
+}
+
 }  // namespace drt

@@ -534,12 +534,16 @@ DRT_HD bool path_step_redo_ff(const LinkDev &L, const TimeGridD &tg, const FreqG
     if constexpr (DUAL)
         if (out.doppler) reinterpret_cast<float *>(out.doppler)[oi] = doppler_ff<N>(V, seg, fg);
     if (out.angles) {
-        const v3<float> kd = f32v(unit(seg[1])), ka = f32v(-unit(seg[N + 1]));
+        const v3<ff> kd = seg[1], ka = -seg[N + 1];
+        auto flat = [](v3<ff> k) {   // length of the horizontal part
+            const ff r2 = fma(k.x, k.x, k.y * k.y);
+            return r2.h > 0.f ? sqrt(r2) : ff(0.f);
+        };
         float *q = out.angles + 4 * oi;
-        q[0] = atan2f(kd.y, kd.x);
-        q[1] = atan2f(kd.z, hypotf(kd.x, kd.y));
-        q[2] = atan2f(ka.y, ka.x);
-        q[3] = atan2f(ka.z, hypotf(ka.x, ka.y));
+        q[0] = atan2_ff(kd.y, kd.x);
+        q[1] = atan2_ff(kd.z, flat(kd));
+        q[2] = atan2_ff(ka.y, ka.x);
+        q[3] = atan2_ff(ka.z, flat(ka));
     }
     if (out.flags) out.flags[oi] = (uint8_t)fl;
     if (out.points) {

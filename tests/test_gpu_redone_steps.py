@@ -31,6 +31,40 @@ def plates(n, seed):
     return b.build((list(TX), list(VT), [0, 0, 0]), (list(RX), list(VR), [0, 0, 0]))
 
 
+@pytest.fixture(scope="module")
+def redone():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2205_00237_gb300 import drt
+    n = 300
+    scene, paths = plates(n, 1), I.chains_to_pathset([[(I.T_R, i)] for i in range(n)])
+    tg, fg = I.TimeGrid(0.0, 1e-8, 8), I.FreqGrid(28e9, 400e6, 4)   # microns of motion
+    with drt.Context(0) as ctx:
+        link = ctx.load(scene, paths)
+        H = torch.empty(tg.n_steps, fg.n_bins, dtype=torch.complex64, device="cuda")
+        with ctx.batch([link], [tg], [fg], [H]) as b:
+            b.run()
+            assert b.info(redo=True)["redo_steps"] == n * tg.n_steps
+        out = [{k: v.cpu().numpy() for k, v in link.extrapolate(tg, fg, p).items() if v is not None}
+               for p in (drt.FP64, drt.FP32_BULK)]
+    assert not out[0]["flags"].any() and not out[1]["flags"].any()
+    return out
+
+
+def test_delay_and_doppler(redone):
+    """Delay in two-float numbers (2^-46 an operation, some ten of them); Doppler shift to its FP32 rounding (2^-24) and as much again."""
+    a, b = redone
+    assert (np.abs(b["tau"] / a["tau"] - 1) <= 2.0 ** -42).all()
+    assert (np.abs(b["doppler"] - a["doppler"]) <= 2.0 ** -23 * np.abs(a["doppler"])).all()
+
+
+def test_angles(redone):
+    """Both forms round an angle to FP32: to the same or to neighbouring numbers."""
+    a, b = redone
+    assert (np.abs(b["angles"].astype(np.float64) - a["angles"]) <= np.spacing(np.abs(a["angles"]))).all()
+
+
 @pytest.mark.parametrize("bins,bandwidth", [(4096, 3.7e8), (4096, 1.3e9), (4096, 2.9e9), (1500, 2.1e9), (600, 9e8)])
 def test_contribution_to_wide_grids(bins, bandwidth):
     """H of one redone path, bin by bin.  A seed is within 2e-7 rad (phase rounded to FP32) and 1e-7 (sine, cosine) of its place, each of the
