@@ -6,7 +6,8 @@ vehicles, 512 ray chains of <= 3 interactions (R:D:S = 6:2:2, committed t0 path 
 2000 steps x 0.5 ms, 512 frequency bins over 1 GHz, FP64 form.
 
 One step = one drt_synthesize_H call on the resident link: pose table (a2), extrapolation of every
-(path, time-step) with field coefficients (a3-a8), H(t, f) synthesis (a9).  value = path-timesteps/s
+(path, time-step) with field coefficients (a3-a8; two-float FP32 pairs of 47 bits, FP64 for the steps that
+they cannot decide), H(t, f) synthesis (a9).  value = path-timesteps/s
 over all ranks (each rank runs its own link: weak scaling, no data-path collective).  L2 (129 MB) is
 flushed by a 256 MB write between timed steps, outside the events.  `error` compares 16 sampled rows
 of the timed run's H with the FP64 oracle.
@@ -50,25 +51,24 @@ WORKLOAD = "canyon"
 PATHSET = os.path.join(ROOT, "tests", "golden", "pathset_canyon_seed0.npz")
 
 # Roofline constants of the extrapolation kernels, from one ncu capture of one call on this workload
-# (profiles/k_extrapolate_fp64_canyon.md, profiles/k_extrapolate_bulk_canyon.md): FP64 / FP32 FLOPs
-# executed per path-step (DADD + DMUL + 2 DFMA, or FADD + FMUL + 2 FFMA, thread-instructions summed over
-# the call's extrapolation launches), their DRAM bytes and FP64-pipe activity.  They hold for the kernel
-# sources whose hash is KERNEL_HASH; after any change to the sources the bench reports them as null
-# until they are measured again.  FP64 peak of the GB300 derived from its unit counts: 152 SMs x 2
-# DFMA/clk x 2 FLOP x 2.07 GHz = 1.26 TFLOP/s (no FP64 tensor path is used); FP32 peak 152 SMs x 128
-# lanes x 2 FLOP x 2.07 GHz = 80.5 TFLOP/s.  The synthesis is counted in issue slots: its kernel evaluates
-# the exponentials of 16 paths for a tile of 512 bins in 463 warp instructions (ncu), 1.81 slots of the
-# 128 lanes an SM issues per cycle for a term of H, so its roofline is 152 x 128 x 2.07 GHz / 1.81 =
-# 22.3e12 terms/s; the products and sums themselves (8 FLOP per term) run on the tensor cores.
-KERNEL_HASH = "8ff611f473138dd0"
-FP64_FLOP_PER_PATH_STEP = 1210.4
-K1_DRAM_BYTES_PER_CALL = 8.26e6
-K1_FP64_PIPE_ACTIVE = 0.861
-FP32_FLOP_PER_PATH_STEP = 1178.5
-# issue activity of k_extrapolate_bulk_n<3> (the largest FP32-bulk launch): share of the SM cycles in
-# which a sub-partition issued an instruction (ncu smsp__issue_active), the kernel's binding measure
-K2_ISSUE_ACTIVE = 0.429
-FP64_PEAK_FLOPS = 152 * 2 * 2 * 2.07e9
+# (profiles/k_extrapolate_ff_canyon.md, profiles/k_extrapolate_bulk_canyon.md), summed over the call's
+# extrapolation launches: warp instructions, FP32 FLOPs executed per path-step (FADD + FMUL + 2 FFMA,
+# thread-instructions), DRAM bytes, and the share of the SM cycles in which a sub-partition issued an
+# instruction (time-weighted).  The FP64 form's records come from two-float FP32 pairs, so both forms are
+# counted in issue slots: 152 SMs x 128 lanes x 2.07 GHz = 40.3e12 thread-instructions/s (FP32 peak 80.5
+# TFLOP/s at an FMA each).  The constants hold for the kernel sources whose hash is KERNEL_HASH; after any
+# change to the sources the bench reports them as null until they are measured again.  The synthesis
+# evaluates the exponentials of 16 paths for a tile of 512 bins in 463 warp instructions (ncu), 1.81
+# thread-instructions a term of H, so its roofline is 40.3e12 / 1.81 = 22.3e12 terms/s; the products and
+# sums themselves (8 FLOP per term) run on the tensor cores.
+KERNEL_HASH = None
+FF_WARP_INST_PER_CALL = None
+FF_FLOP_PER_PATH_STEP = None
+FF_DRAM_BYTES_PER_CALL = None
+FF_ISSUE_ACTIVE = None
+FP32_FLOP_PER_PATH_STEP = None
+BULK_WARP_INST_PER_CALL = None
+BULK_ISSUE_ACTIVE = None
 FP32_PEAK_FLOPS = 152 * 128 * 2 * 2.07e9
 SYNTH_FLOP_PER_TERM = 8.0
 SYNTH_SLOTS_PER_TERM = 463 * 32 / (16 * 512)
@@ -780,25 +780,27 @@ def run_ours(args):
                  "error": bulk_err}
     ke, kb = fp32_bulk["kernel_ms"].get("extrapolate"), fp32_bulk["kernel_ms"].get("synth")
     # k_synth is the same kernel on the same records in both forms: its roofline is taken where it runs
-    # alone (the FP64 call); in the FP32-bulk call it shares the GPU with the FP64 redo
+    # alone (the FP64 call); in the FP32-bulk call it shares the GPU with the redo
     ks = prof["synth"][1] / max(1, args.steps) if prof["synth"][0] else kb
     fresh = KERNEL_HASH is not None and KERNEL_HASH == kernel_source_hash()
     if ke and ks:
         a3 = SYNTH_FLOP_PER_TERM * P * T * F / (ks * 1e-3)
         slots = SYNTH_SLOTS_PER_TERM * P * T * F / (ks * 1e-3)
-        a1 = FP32_FLOP_PER_PATH_STEP * P * T / (ke * 1e-3) if fresh and FP32_FLOP_PER_PATH_STEP else None
+        a1 = 32 * BULK_WARP_INST_PER_CALL / (ke * 1e-3) if fresh else None
         fp32_bulk["rooflines"] = {
             "k_extrapolate_bulk": {"bound": "alu", "achieved": a1 / 1e12 if a1 else None,
-                                   "peak": FP32_PEAK_FLOPS / 1e12, "unit": "TFLOP/s",
-                                   "frac": a1 / FP32_PEAK_FLOPS if a1 else None,
-                                   "ncu_issue_active": K2_ISSUE_ACTIVE if fresh else None,
-                                   "note": None if a1 else "FLOP count not measured on this kernel build"},
+                                   "peak": FP32_ISSUE_PEAK / 1e12, "unit": "T issue slots/s",
+                                   "frac": a1 / FP32_ISSUE_PEAK if a1 else None,
+                                   "fp32_tflops": FP32_FLOP_PER_PATH_STEP * P * T / (ke * 1e-3) / 1e12 if fresh else None,
+                                   "fp32_peak_tflops": FP32_PEAK_FLOPS / 1e12,
+                                   "ncu_issue_active": BULK_ISSUE_ACTIVE if fresh else None,
+                                   "note": None if a1 else "instruction count not measured on this kernel build"},
             "k_synth": {"bound": "alu", "achieved": slots / 1e12, "peak": FP32_ISSUE_PEAK / 1e12,
                         "unit": "T issue slots/s (1.81 per term)", "frac": slots / FP32_ISSUE_PEAK,
                         "terms_per_s": P * T * F / (ks * 1e-3),
                         "roofline_terms_per_s": FP32_ISSUE_PEAK / SYNTH_SLOTS_PER_TERM,
                         "flop_tflops": a3 / 1e12,
-                        "ms": ks, "ms_beside_fp64_redo": kb}}
+                        "ms": ks, "ms_beside_redo": kb}}
 
     # end to end through the public API with host buffers: load (H2D) + synthesize to host (D2H)
     h2d = sum(np.ascontiguousarray(a).nbytes for a in (scene.bodies, scene.materials, scene.faces, scene.edges,
@@ -816,7 +818,8 @@ def run_ours(args):
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": max(3, args.warmup), "ms_per_step": 1e3 * total_s / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+            "scaling": "weak", "vs_baseline": None, "dtype": "f32x2", "data": "synthetic",
+            "dtype_note": "two-float FP32 pairs (47 bits), FP64 for the steps that they cannot decide; H complex64",
             "h_samples_per_s": world * T * F * args.steps / total_s,
             "config": {"workload": "canyon-512paths-2000x0.5ms-512bins-60GHz-fp64", "paths": P, "steps": T,
                        "bins": F, "fc_hz": fg.fc, "bandwidth_hz": fg.bandwidth, "precision": "DRT_FP64",
@@ -830,20 +833,20 @@ def run_ours(args):
             "kernel_ms_note": "device time per step of each kernel kind (all its launches)",
             "wall_s": wall, "clocks": clocks, "error": head_err, "fp32_bulk": fp32_bulk,
             "kernel_source_hash": kernel_source_hash()}
-    if fresh and FP64_FLOP_PER_PATH_STEP:
-        achieved = FP64_FLOP_PER_PATH_STEP * P * T / k1_avg_s
-        line["roofline"] = {"bound": "alu", "kernel": "k_extrapolate_fp64 (all launches of one call)",
-                            "achieved": achieved / 1e12,
-                            "peak": FP64_PEAK_FLOPS / 1e12, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_FLOPS,
-                            "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 FLOP x 2.07 GHz (no FP64 figure in "
-                                           "MEASURED_PEAKS.json)",
-                            "algorithmic": f"{FP64_FLOP_PER_PATH_STEP:.0f} FP64 FLOP per path-step x {P * T} path-steps",
-                            "traffic": K1_DRAM_BYTES_PER_CALL,
-                            "ncu_fp64_pipe_active": K1_FP64_PIPE_ACTIVE}
+    line["roofline"] = {"bound": "alu", "kernel": "k_extrapolate_ff (all launches of one call, warm starts included)",
+                        "achieved": None, "peak": FP32_ISSUE_PEAK / 1e12, "unit": "T issue slots/s", "frac": None,
+                        "peak_source": "derived: 152 SMs x 128 lanes x 2.07 GHz (no FP32 figure in MEASURED_PEAKS.json)",
+                        "fp32_peak_tflops": FP32_PEAK_FLOPS / 1e12, "traffic": None}
+    if fresh:
+        slots = 32 * FF_WARP_INST_PER_CALL / k1_avg_s
+        line["roofline"].update({
+            "achieved": slots / 1e12, "frac": slots / FP32_ISSUE_PEAK,
+            "fp32_tflops": FF_FLOP_PER_PATH_STEP * P * T / k1_avg_s / 1e12,
+            "algorithmic": f"{32 * FF_WARP_INST_PER_CALL / (P * T):.0f} thread-instructions ({FF_FLOP_PER_PATH_STEP:.0f} FP32 "
+                           f"FLOP) per path-step x {P * T} path-steps",
+            "traffic": FF_DRAM_BYTES_PER_CALL, "ncu_issue_active": FF_ISSUE_ACTIVE})
     else:
-        line["roofline"] = {"bound": "alu", "kernel": "k_extrapolate_fp64 (all launches of one call)",
-                            "achieved": None, "peak": FP64_PEAK_FLOPS / 1e12, "unit": "TFLOP/s", "frac": None,
-                            "traffic": None, "note": "per-path-step FLOP count not measured on this kernel build"}
+        line["roofline"]["note"] = "instruction count not measured on this kernel build"
     line["extrapolate_records"] = run_records(args, ctx, link, scene, paths, tg, fg, drt, flush)
     line["tiny"] = run_tiny(args, ctx, drt, flush)
     probe = ctx.probe_peak(0)

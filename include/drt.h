@@ -64,8 +64,14 @@ typedef int32_t drt_status;
 #define DRT_F_DEGEN 16   /* a zero-length segment or a degenerate diffraction geometry            */
 
 /* precision of a call */
-#define DRT_FP64 0        /* all per-path-step geometry, field and Doppler work in FP64           */
-#define DRT_FP32_BULK 1   /* FP32 work on deltas from per-chunk FP64 bases (delay, phase anchors) */
+/* DRT_FP64: per-path-step outputs (geometry, field, Doppler, flags) in FP64.  H and the T_C plan, whose
+ * per-path records are FP32, come from two-float FP32 pairs (47 bits; a step that they cannot decide is
+ * computed in FP64) while the scene's coordinates, motion and turns stay below 2^18 wavelengths, else
+ * from FP64; drt_synthesize_H_noalloc always from FP64.
+ * DRT_FP32_BULK: FP32 work on deltas from per-chunk bases (delay, phase anchors); the bases and the steps
+ * that FP32 cannot resolve in two-float numbers in the same range, else in FP64. */
+#define DRT_FP64 0
+#define DRT_FP32_BULK 1
 
 /* ---- dynamic environment database (Sec. II); all positions in world coordinates at t0 ---- */
 typedef struct { double o[3], v[3], a[3], k[3], w0, wdot; } drt_body;      /* 112 B: rotation centre o,
@@ -159,8 +165,10 @@ drt_status drt_extrapolate(drt_ctx *ctx, uint64_t link, const drt_time_grid *tgr
  * a2-a9: the whole hot path: extrapolation as above into context-owned scratch, then
  * H[t][k] = sum over valid paths of a_p(t) exp(-j 2 pi f_k tau_p(t)).  H is a caller-owned DEVICE
  * buffer of [tgrid->n_steps][fgrid->n_bins] complex64 (float re, im), in both precisions (the
- * synthesis accumulates in FP32 from phases reduced in FP64).  Scratch grows on demand within the
- * HBM budget.  Errors: DRT_EINVAL, DRT_ENOTFOUND, DRT_ENOMEM, DRT_ECUDA. */
+ * synthesis accumulates in FP32, from phases reduced in two-float numbers or FP64 and terms of 22 bits).
+ * Scratch grows on demand within the HBM budget; a call that finds no memory first frees what only
+ * makes calls faster (the two-float copies of links among it).  Errors: DRT_EINVAL, DRT_ENOTFOUND,
+ * DRT_ENOMEM, DRT_ECUDA. */
 drt_status drt_synthesize_H(drt_ctx *ctx, uint64_t link, const drt_time_grid *tgrid,
                             const drt_freq_grid *fgrid, void *H, int32_t precision, void *stream);
 
@@ -306,7 +314,7 @@ drt_status drt_synthesize_H_retraced(drt_ctx *ctx, uint64_t link, const drt_time
  * a10: batched synthesis over many resident links (FP32-bulk form).  drt_batch_create plans one
  * batch: link i is synthesised over tgrids[i] x fgrids[i] into the caller's DEVICE buffer H[i]
  * ([n_steps][n_bins] complex64).  Each stage (base poses, FP64 chunk poses, multi-diffraction warm
- * starts, FP64 chunk anchors, FP32-bulk extrapolation, H synthesis, FP64 redo) is one persistent
+ * starts, chunk anchors, FP32-bulk extrapolation, H synthesis, redo) is one persistent
  * launch over the (link, work unit) pairs of all links, claimed with atomic counters, largest links
  * first, so uneven links (8 to thousands of paths, 100 to thousands of steps) share one launch per
  * stage.  Extrapolation and synthesis stream through a record buffer of at most 4 GiB in waves of
@@ -326,7 +334,7 @@ drt_status drt_batch_create(drt_ctx *ctx, int32_t n_links, const uint64_t *links
 drt_status drt_batch_run(drt_ctx *ctx, drt_batch *batch, int32_t use_graph, void *stream);
 /* chosen synthesis variant (frequency tile of 0: 128, 1: 256, 2: 512 bins), scratch
  * bytes, the autotuner's best sample time (ms) and the path-steps of the last run that FP32 could
- * not resolve and the FP64 redo kernel recomputed (reading it waits for the device); any output
+ * not resolve and the redo kernel recomputed (reading it waits for the device); any output
  * may be NULL.  With redo_steps non-NULL the call returns DRT_ENOMEM when a wave of the last run
  * queued more redo steps than its list holds (2^22 + 1/128 of the wave's path-steps, or the value
  * of the environment variable DRT_BATCH_REDO_CAP when that is smaller, read when a plan is built):
@@ -365,8 +373,8 @@ typedef struct {
 } drt_request;
 typedef struct {
     drt_status status;          /* DRT_OK; DRT_ENOMEM when the request is larger than the arena, */
-                                /* or when its batch queued more FP64 redo steps than the redo    */
-                                /* list holds (H then misses them); DRT_EINVAL when the batch     */
+                                /* or when its batch queued more redo steps than its list holds */
+                                /* (H then misses them); DRT_EINVAL when the batch                */
                                 /* could not be planned; DRT_ECUDA                                */
     int32_t batch_requests;     /* requests in the launch that served this one                    */
     double t_submit, t_launch, t_done;   /* seconds on the library's steady clock                 */
@@ -396,9 +404,8 @@ drt_status drt_link_info(drt_ctx *ctx, uint64_t link, int32_t *n_paths);
 /* ---------------------------------------------------------------------------------------------
  * Tracing.  While enabled, every kernel the context launches is bracketed by CUDA events recorded
  * on the launch stream.  drt_profile_read synchronises the device and returns, per kernel kind
- * (0 = pose table, 1 = extrapolation, 2 = H synthesis, 3 = FP64 chunk anchors and FP64 redo of
- * the FP32-bulk form), the number of launches and
- * their summed device time in ms since the previous read, then clears the record.
+ * (0 = pose table, 1 = extrapolation, 2 = H synthesis, 3 = chunk anchors and redo of the FP32-bulk form), the
+ * number of launches and their summed device time in ms since the previous read, then clears the record.
  * Errors: DRT_EINVAL (NULL arguments), DRT_ECUDA. */
 drt_status drt_profile_enable(drt_ctx *ctx, int32_t on);
 drt_status drt_profile_read(drt_ctx *ctx, int64_t counts[4], double ms[4]);

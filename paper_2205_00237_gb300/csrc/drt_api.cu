@@ -506,7 +506,7 @@ drt_status synth_into(drt_ctx *c, Link &L, const drt_time_grid *tg, const drt_fr
     TimeGridD t = precision == DRT_FP32_BULK ? tgd(tg, L.view, choose_chunk(L.view, *tg, *fg)) : tgd(tg, L.view);
     FreqGridD f = fgd(fg);
     if (precision == DRT_FP32_BULK) {
-        // the FP64 redo of the few steps FP32 cannot resolve runs beside the synthesis (their records
+        // the redo of the few steps FP32 cannot resolve runs beside the synthesis (their records
         // stay zero) and adds its contributions to H afterwards
         if (drt_status st = ensure(c, c->redo3, (size_t)L.n_paths * tg->n_steps * 3 * sizeof(double) + 8)) return st;
         if (drt_status st = run_extrapolation(c, L, tg, fg, none, rec, precision, s, true)) return st;
@@ -548,8 +548,8 @@ double drt::ff_reach(const drt_scene_view &v, const drt_time_grid &tg) {
 }
 // Whether the records of H may be computed in two-float numbers: their 47 bits resolve a path's phase to 2e-7 rad while its length
 // is below 2^21 wavelengths, which a scene whose coordinates stay below 2^18 of them ensures (1.3 km at 60 GHz); materials and areas
-// as checked at load, and no permittivity |eps_c| = |eps_r - j sigma / (2 pi fc eps0)| above 1e15 (copper below 1 kHz), so that |eps_c|^2 is
-// a divisor that FP32 can invert (1 / x is 0 from x = 2^126 on).  Beyond that the records are computed in FP64.
+// as checked at load, and no permittivity |eps_c| = |eps_r - j sigma / (2 pi fc eps0)| above 1e15 (copper below 1 kHz), so that
+// |eps_c|^2 is a divisor that FP32 can invert (1 / x is 0 from x = 2^126 on).  Beyond that the records are computed in FP64.
 bool drt::ff_applies(const drt_scene_view &v, const drt_time_grid &tg, const drt_freq_grid &fg) {
     return v.ff_range && 1e6 + v.sigma_max / (2 * 3.14159265358979323846 * 8.8541878128e-12 * fg.fc) <= 1e15 &&
            ff_reach(v, tg) * (fg.fc + fg.bandwidth) <= 262144.0 * 299792458.0;
@@ -872,7 +872,7 @@ drt_status drt_create(drt_ctx **out, int32_t device, uint64_t hbm_budget_bytes) 
         return fail(DRT_ENOMEM, "cudaMalloc failed");
     }
     // side[1] carries the critical chain of a call (the latency-bound warm starts, then the chains that
-    // wait for them; in the FP32-bulk form also the FP64 redo beside the synthesis): at the greatest
+    // wait for them; in the FP32-bulk form also the redo beside the synthesis): at the greatest
     // stream priority its blocks are dispatched before those of the other streams' wide launches
     // (7-8 % off a canyon call in both forms)
     int prio_lo = 0, prio_hi = 0;
@@ -1554,7 +1554,7 @@ static drt_status batch_create_locked(drt_ctx *c, int32_t n_links, const uint64_
     }
     CUDA_TRY(cudaSetDevice(c->device));
     // Chunk autotuning: the phase-error model gives each link the longest chunk whose FP32 deltas stay
-    // within the phase bar; shorter chunks meet it too (more FP64 anchors, shorter deltas).  Plans with
+    // within the phase bar; shorter chunks meet it too (more anchors, shorter deltas).  Plans with
     // the model's chunk, half and a quarter of it share one allocation (the largest), the first wave's
     // preparation and extrapolation are timed in each (per path-step: the waves may differ), and the
     // fastest plan is kept.

@@ -16,7 +16,7 @@
 // All stages run in waves of links whose per-path-step records (20 B each) fit one record buffer and
 // whose poses, warm starts and anchors fit one scratch region, both reused by the next wave, so a
 // batch of any size streams through a bounded scratch.  Links are ordered by decreasing work so the
-// largest units are claimed first.  Steps FP32 cannot resolve go to an FP64 redo kernel at the end
+// largest units are claimed first.  Steps FP32 cannot resolve go to a redo kernel at the end
 // of their wave, which adds their contribution to H with atomics.  The frequency tile
 // width of stage 5 (128, 256 or 512 bins) is autotuned on the batch.  The whole sequence can
 // be captured in a CUDA graph.
@@ -549,13 +549,13 @@ void batch_set_variant(BatchPlan *P, int v) { P->variant = v; }
 int batch_chunk(const BatchPlan *P, int k) { return P->host[k].tg.chunk; }
 size_t batch_bytes(const BatchPlan *P) { return P->bytes; }
 
-// device address of the last run's redo overflow word (non-zero when a wave queued more FP64 redo
+// device address of the last run's redo overflow word (non-zero when a wave queued more redo
 // steps than its list holds, so that run's H misses their contributions)
 const unsigned long long *batch_redo_overflow(const BatchPlan *P) {
     return reinterpret_cast<const unsigned long long *>(P->mem + P->off_redo + 16);
 }
 
-// queued FP64 redo steps of the last completed run, all waves (a wave's count may exceed its list's
+// queued redo steps of the last completed run, all waves (a wave's count may exceed its list's
 // capacity; the total counts every queued step)
 cudaError_t batch_redo_count(const BatchPlan *P, long long *n, bool *overflow) {
     unsigned long long c[2] = {0, 0};

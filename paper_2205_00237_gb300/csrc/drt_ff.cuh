@@ -166,8 +166,9 @@ FF_D cx<ff> operator*(cx<ff> a, cx<ff> b) {
     return {det2(a.re, b.re, a.im, b.im), det2(a.re, b.im, -a.im, b.re)};
 }
 
-// sine and cosine of x (|x| < 6.4; beyond, or not a number: no angle's, but no read past the table): the nearest multiple r of 1/32 from a table, the remainder |d| <= 1/64 by its Taylor
-// terms (what is below 2^-24 of the result in FP32), joined by angle addition
+// sine and cosine of x (|x| < 6.4; beyond, or not a number: no angle's, but no read past the table): the nearest multiple
+// of 1/32 from a table, the remainder |d| <= 1/64 by its Taylor terms (what is below 2^-24 of the result in FP32), joined
+// by angle addition
 struct FFSinCos { ff s, c; };
 inline __host__ __device__ __noinline__ FFSinCos sincos_ff(ff x) {
     const float i = rintf(32.f * x.h);

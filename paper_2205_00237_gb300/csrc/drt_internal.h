@@ -74,7 +74,7 @@ struct LinkDev {
     const double *t0par;      // [n_paths - n_bulk][2 * MAXI]
 };
 
-// chunk: time steps per chunk (FP32-bulk FP64 anchors and multi-diffraction warm starts are taken
+// chunk: time steps per chunk (FP32-bulk anchors and multi-diffraction warm starts are taken
 // at the first step of every chunk); a power of two in [4, 64]
 // grids as kernels see them, with the FP32 constants of the FP32-bulk form derived once on the host
 // (per-step FP64 divisions of grid constants would occupy the FP64 pipe of the FP32 kernels)
@@ -235,8 +235,8 @@ cudaError_t launch_extrapolate_ff_generic(const LinkDev &L, const TimeGridD &tg,
 // two: in two-float numbers (the caller has checked that they apply), here and below
 cudaError_t launch_t0par(const LinkDev &L, double *t0par, cudaStream_t s, bool two);
 cudaError_t launch_warm_fp64(const LinkDev &L, const TimeGridD &tg, double *warm, cudaStream_t s, bool two);
-// FP32-bulk form (CHUNK consecutive steps share FP64 anchors); see drt_physics.cuh.  Scratch:
-// per-(body or terminal, chunk) FP32 base poses and per-(path, chunk) FP64 anchors.
+// FP32-bulk form (CHUNK consecutive steps share anchors); see drt_physics.cuh.  Scratch:
+// per-(body or terminal, chunk) FP32 base poses and per-(path, chunk) anchors.
 size_t bulk_pose_bytes(const LinkDev &L, const TimeGridD &tg);
 size_t bulk_base_bytes(const LinkDev &L, const TimeGridD &tg);
 cudaError_t launch_pose_bulk(const LinkDev &L, const TimeGridD &tg, void *poseb, cudaStream_t s);

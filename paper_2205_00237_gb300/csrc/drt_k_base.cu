@@ -1,5 +1,5 @@
-// drt_k_base.cu -- the FP32-bulk form's FP64 anchors: body poses at the chunk bases and, per (path,
-// chunk), the FP64 path length, segment vectors and phase seeds the FP32 deltas build on.
+// drt_k_base.cu -- the FP32-bulk form's anchors, in two-float numbers or FP64: body poses at the chunk bases and, per (path,
+// chunk), the path length, segment vectors and phase seeds the FP32 deltas build on.
 #include "drt_launch.cuh"
 #include "drt_physics_ff.cuh"
 

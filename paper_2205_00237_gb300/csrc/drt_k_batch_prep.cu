@@ -8,7 +8,8 @@ namespace drt {
 
 // stages 0-3: block-wide claims of blockDim.x consecutive items.  TWO: stages 1-3 of the links that two-float numbers apply to (PoseQ
 // rows), else of the others; a batch that has both runs both over all items, so that what a link gets does not depend on which
-// others are in its batch.  The two-float anchors at 4 blocks per SM (128 registers; 0.65 -> 0.52 ms of a 128-link batch against 2 blocks without spills)
+// others are in its batch.  The two-float anchors at 4 blocks per SM (128 registers; 0.65 -> 0.52 ms of a 128-link batch against
+// 2 blocks without spills)
 template <int STAGE, bool TWO>
 __global__ void __launch_bounds__(128, TWO && STAGE == ST_BASE ? 4 : 1) k_stage(const BatchDev B) {
     __shared__ long long s_start;

@@ -1,5 +1,5 @@
-// drt_k_batch_redo.cu -- the FP64 redo at the end of a batch wave: each queued path-step recomputed
-// in FP64 and its contribution added to H.  Compiled twice: values only, and (drt_k_batch_redo_dual.cu,
+// drt_k_batch_redo.cu -- the redo at the end of a batch wave: each queued path-step recomputed in two-float
+// numbers (or FP64) and its contribution added to H.  Compiled twice: values only, and (drt_k_batch_redo_dual.cu,
 // DRT_BATCH_REDO_DUAL) with the rates the Doppler output needs.
 #include "drt_batch.cuh"
 #include "drt_physics_ff.cuh"

@@ -1,6 +1,6 @@
 // drt_k_bulk.cu -- the FP32-bulk form's kernels: FP32 base poses per chunk of steps and the FP32
 // delta-number geometry and field per (path, step) for the chains of lengths 0..3 (the generic range
-// in drt_k_bulk_gen.cu, the FP64 anchors in drt_k_base.cu, the FP64 redo in drt_k_redo.cu).
+// in drt_k_bulk_gen.cu, the anchors in drt_k_base.cu, the redo in drt_k_redo.cu).
 #include <algorithm>
 #include <type_traits>
 
@@ -9,7 +9,7 @@
 namespace drt {
 
 // ------------------------------------------------------------------------------------------------
-// FP32-bulk form: base poses per (body or terminal, chunk), FP64 anchors per (path, chunk), then
+// FP32-bulk form: base poses per (body or terminal, chunk), anchors per (path, chunk), then
 // the per-(path, step) delta-number kernel with the same block mapping as the FP64 form
 size_t bulk_pose_bytes(const LinkDev &L, const TimeGridD &tg) {
     return (size_t)(L.n_bodies + 2) * n_chunks_of(tg) * sizeof(PoseB);

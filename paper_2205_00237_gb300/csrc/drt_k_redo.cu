@@ -1,4 +1,4 @@
-// drt_k_redo.cu -- the FP64 redo of the FP32-bulk path-steps that FP32 cannot resolve, beside the
+// drt_k_redo.cu -- the redo (two-float numbers, or FP64) of the FP32-bulk path-steps that FP32 cannot resolve, beside the
 // synthesis, with their contributions added to H afterwards (the records form is in drt_k_redo_out.cu).
 #include "drt_launch.cuh"
 #include "drt_physics_ff.cuh"

@@ -1,4 +1,4 @@
-// drt_k_redo_out.cu -- the FP64 redo of the FP32-bulk path-steps that FP32 cannot resolve, written in
+// drt_k_redo_out.cu -- the redo (two-float numbers, or FP64) of the FP32-bulk path-steps that FP32 cannot resolve, written in
 // place into the caller's per-path-step outputs and records.
 #include "drt_launch.cuh"
 #include "drt_physics_ff.cuh"

@@ -196,7 +196,7 @@ cudaError_t launch_lifetime_rec(const RecD &rec, int n_steps, int n_paths, doubl
 
 // DRT over T_C windows: a path that is not valid at the first instant of its window is outside that
 // window's multipath (sel[start][caller index] != 0, its FP64 flags at the window start) and its
-// records carry a = 0; the same holds for the FP64 redo contributions of the FP32-bulk form.
+// records carry a = 0; the same holds for the redo contributions of the FP32-bulk form.
 // k_select evaluates the FP64 flags of every (window start, path) in one launch (poses computed at the
 // instant, multi-diffraction warm starts from the grid's table).
 __device__ __forceinline__ int window_of(const int32_t *__restrict__ starts, int n_w, int n) {

@@ -647,7 +647,7 @@ template <int N> constexpr int len_min() { return N == LEN_GEN ? 2 : 0; }
 // In FP32 (the FP32-bulk form) the positions carry rounding errors of a few ulp of the coordinates,
 // amplified a little by the image construction, so a decision whose margin (the distance of the tested
 // point from the face rim, the edge end, the face plane or the wedge face) is within a bound on that
-// error is not taken here: the step gets F_REDO64 and the FP64 redo decides it, which makes the flags
+// error is not taken here: the step gets F_REDO64 and the redo decides it, which makes the flags
 // of the form exact outside the 1e-9 m band of the FP64 form.  F_NEAR100 marks margins within 100x
 // that bound (the FP32-bulk step uses it to keep the FP32 flags of invalid steps that moved far).
 template <class T> DRT_HD T amax3(v3<T> a) { return fmax(fmax(fabs(a.x), fabs(a.y)), fabs(a.z)); }
@@ -674,8 +674,9 @@ DRT_HD float fp32_margin_tol(float scale) { return 2e-6f * (scale + 1.f); }
 // error bound.  (Called out of line in the FP32 kernels it measured no faster, unlike the field
 // updates, so it stays inline.)
 template <class T> struct VertexCheck { uint32_t fl; T m; };
-// The same in two-float numbers: the flags, the smallest margin and the largest one by which a test fails (m), and amp, by how much the point's place is less certain than a coordinate: leg / height for a reflection,
-// (leg / distance from the edge line)^2 for a diffraction, whose Newton step divides by sin^2 of the angle to the edge.
+// The same in two-float numbers: the flags, the smallest margin and the largest one by which a test fails (m), and amp, by how much
+// the point's place is less certain than a coordinate: leg / height for a reflection, (leg / distance from the edge line)^2 for a
+// diffraction, whose Newton step divides by sin^2 of the angle to the edge.
 // the smaller of m and |v|, -1 from the first that is not a number on
 DRT_HD float least(float m, float v) { return ::fabsf(v) < m ? ::fabsf(v) : v == v ? m : -1.f; }
 struct VertexMargins { uint32_t fl; float m, out, amp; };
@@ -779,7 +780,8 @@ DRT_HD VertexCheck<T> vertex_validity_inl(int ty, v3<T> c, v3<T> nn, v3<T> b, v3
     return VertexCheck<T>{fl, mmin};
 }
 
-// (two-float only: far, the largest coordinate that a place is computed from; amp_out, how much less certain than a coordinate a point of the chain is along its face or edge)
+// (two-float only: far, the largest coordinate that a place is computed from; amp_out, how much less certain than a coordinate a
+// point of the chain is along its face or edge)
 template <int N = -1, class S>
 DRT_HD uint32_t validity(const Prim<S> *pr, int n, const v3<typename ST<S>::R> *P, float far = 0.f, float *amp_out = nullptr) {
     typedef typename ST<S>::R T;
@@ -1833,7 +1835,7 @@ DRT_HD void path_warm_fp64(const LinkDev &L, const TimeGridD &tg, int p, int row
 // delay is d_b + sum of the segment-length deltas, so the FP32 rounding acts on metre-scale
 // deltas, not on the ~100 m path length.
 
-// per (path, chunk) FP64 anchors
+// per (path, chunk) anchors
 struct alignas(16) BaseRec {
     double d;                  // path length at the chunk base (m)
     float ph0, st_hi, st_lo;   // frac(f_0 d / c); frac(df d / c) = st_hi + st_lo
@@ -2040,7 +2042,7 @@ DRT_HD Prim<double> load_prim_value(const LinkDev &L, const double *Pr, int type
     return q;
 }
 
-// (path, chunk) FP64 anchors: path length and segment vectors at the chunk's first instant, phase
+// (path, chunk) anchors: path length and segment vectors at the chunk's first instant, phase
 // seed and per-bin step.  N < 0: the chain length is read at run time (one instance per length).
 template <int N = -1, class Loader>
 DRT_HD void path_base_fp64_core(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg, int p, int chunk,
@@ -2188,7 +2190,7 @@ DRT_HD void write_outputs_bulk(const OutD &o, size_t oi, int n, const v3<S> *V, 
     }
 }
 
-// list of (link, path, step) triples the FP32-bulk kernels hand to the FP64 redo kernel
+// list of (link, path, step) triples the FP32-bulk kernels hand to the redo kernel
 struct RedoList { int *count; int4 *items; int cap; };
 // f(k, item) for the items of the list, a run of them (steps of one path) per warp: `warp` of `warps` takes the runs that start at its
 // places.  All lanes of a warp then run one chain's code, and no two chains share a warp; before, warps of 32 list places ran the
@@ -2208,7 +2210,7 @@ struct Rec5 { float ar, ai, ph, hi, lo; };
 // FP32-bulk (path, time-step): geometry in delta numbers on the chunk anchors, field in FP32.
 // Chains with >= 2 diffractions in a segment start their Newton solve from the FP64 chunk-base
 // parameters (warm, may be null for the others).  Returns false when the step was queued for the
-// FP64 redo (its record is then zero).  S = dd carries the rates the Doppler shift needs, S = de
+// redo (its record is then zero).  S = dd carries the rates the Doppler shift needs, S = de
 // (calls without Doppler output) leaves them out.  N, MULTI and OUT as for path_step_fp64_core.
 // A second carrier (fg2 with its anchors base2; the same time grid and chunks) shares the geometry:
 // its field coefficients and phase record go to *rec2.
@@ -2260,7 +2262,7 @@ DRT_HD bool bulk_eval(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg
         // and the delta rules multiply them by the deltas: the phase error grows with how far an
         // interaction point moved since the chunk base (~6e-4 rad per metre at 60 GHz when a
         // diffraction point slides fast near grazing).  Steps past 0.8 m at 60 GHz (scaled by
-        // 1/fc) are left to the FP64 redo.
+        // 1/fc) are left to the redo.
         float disp2 = 0.f;
         bool finite = true;
 #pragma unroll (N >= 0 ? 8 : 1)
@@ -2278,7 +2280,7 @@ DRT_HD bool bulk_eval(const LinkDev &L, const TimeGridD &tg, const FreqGridD &fg
         if (disp2 > dlim * dlim && !invalid_clear) fl |= F_REDO64;
         fl &= ~F_NEAR100;
         if (!finite || (fl & (F_REDO64 | F_NOCONV | F_DEGEN))) {
-            // geometry FP32 cannot resolve: queue this path-step for the FP64 redo kernel (rare,
+            // geometry FP32 cannot resolve: queue this path-step for the redo kernel (rare,
             // see F_REDO64); the list holds every path-step in the worst case
             if (redo.count) {
 #ifdef __CUDA_ARCH__

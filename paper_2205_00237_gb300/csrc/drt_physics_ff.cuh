@@ -2,8 +2,8 @@
 //
 // The records that the synthesis reads are FP32 (amplitude, phase seed and phase step in turns), so the geometry only has to
 // carry the path length to ~1e-10 m and the decisions exactly.  Two-float arithmetic does the first with 47 bits; a step that it
-// cannot decide (a validity margin within 2^-36 of the coordinates, more near grazing, a virtual terminal on an edge line, a boundary of the
-// transition function, a Newton solve that did not converge, anything not finite) is computed in FP64 by the lane that met it.
+// cannot decide (a validity margin within 2^-36 of the coordinates, more near grazing, a virtual terminal on an edge line, a boundary
+// of the transition function, a Newton solve that did not converge, anything not finite) is computed in FP64 by the lane that met it.
 // Canyon call (512 paths x 2000 steps x 512 bins) 1.93 -> 0.54 ms against the FP64 kernels, 3 paths x 1000 steps 54 -> 33 us.
 #pragma once
 #include "drt_launch.cuh"

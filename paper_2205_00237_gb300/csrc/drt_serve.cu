@@ -38,7 +38,7 @@ struct Slot {
     BatchPlan *plan = nullptr;
     size_t off = 0, size = 0;
     std::vector<uint64_t> tickets;
-    unsigned long long *overflow = nullptr;   // pinned: the batch's FP64 redo-overflow word, copied behind it
+    unsigned long long *overflow = nullptr;   // pinned: the batch's redo-overflow word, copied behind it
 };
 
 struct Request {
@@ -104,7 +104,7 @@ static void CUDART_CB on_batch_done(void *arg) {
     Slot *sl = static_cast<Slot *>(arg);
     Server *S = sl->srv;
     const double t = now_s();
-    // a wave that queued more FP64 redo steps than its list holds left those steps out of H
+    // a wave that queued more redo steps than its list holds left those steps out of H
     const drt_status st = (sl->overflow && *sl->overflow) ? DRT_ENOMEM : DRT_OK;
     {
         std::lock_guard<std::mutex> lk(S->m);

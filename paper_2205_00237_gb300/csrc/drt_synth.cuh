@@ -16,9 +16,9 @@
 //
 // Precision: FP32 operands split into two FP16 parts each, x = hi + lo with 22 bits, three products
 // hi hi + hi lo + lo hi into FP32 accumulators, which are added into FP32 sums every FLUSH steps (the
-// tensor cores' own additions truncate: without this the 20300 paths of a highway link lose 1.8e-5).  X is scaled by a power of two that keeps the largest amplitude
-// met so far in [2^11, 2^12) (a later, larger path rescales the sums exactly), so that paths 2^-25 of the
-// strongest one are still normal FP16 numbers.
+// tensor cores' own additions truncate: without this the 20300 paths of a highway link lose 1.8e-5).  X is
+// scaled by a power of two that keeps the largest amplitude met so far in [2^11, 2^12) (a later, larger
+// path rescales the sums exactly), so that paths 2^-25 of the strongest one are still normal FP16 numbers.
 //
 // m16n8k16 fragments (g = lane / 4, q = lane % 4): a lane evaluates the exponentials of the step's paths
 // 2 q, 2 q + 1, 2 q + 8, 2 q + 9 for its own rows u = g + 8 m (row g of row tile m: Re X, row g + 8: Im X)

@@ -161,8 +161,8 @@ k_trace(const LinkDev L, double t, long long n_cand, int with_tiles, const Posed
 }
 
 // ------------------------------------------------------------------------------------------------
-// The same in three passes.  Nearly every candidate is no ray by a clear margin, and in FP64 all of them wait on the FP64 pipe, and the few
-// that reach the segment-face tests on one thread's loop over the faces (1.13 ms for the canyon's 97206 candidates).  k_trace_ff
+// The same in three passes.  Nearly every candidate is no ray by a clear margin, and in FP64 all of them wait on the FP64 pipe, and
+// the few that reach the segment-face tests on one thread's loop over the faces (1.13 ms for the canyon's 97206 candidates).  k_trace_ff
 // solves and checks the candidates in two-float numbers, with margins as in path_step_ff, and lists those that may be rays;
 // k_trace_block, a warp per listed candidate, spreads the (segment, face) tests over its lanes and tries what is still open in FP64;
 // k_trace_polish solves the rays' diffraction parameters in FP64 from the two-float ones (one Newton step).  The list ends as k_trace's.
