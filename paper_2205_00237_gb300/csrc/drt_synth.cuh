@@ -9,8 +9,8 @@
 // columns (Re Y, Im Y).  Per path only rows + B / 2 exponentials are evaluated instead of a term per bin.
 //
 // What bounds it: the issue slots of the exponentials and their splits.  A step of 16 paths x 512 bins takes
-// 463 warp instructions (253 on the FMA pipe, 123 at two cycles on the ALU, 32 hardware sines and cosines at
-// eight) and 24 MMA of 8.2 cycles, against 16 x 512 x 6.3 / 32 = 1610 instructions term by term.  Measured
+// 455 warp instructions on the canyon's records (about 250 on the FMA pipe, 120 at two cycles on the ALU, 32
+// hardware sines and cosines at eight) and 24 MMA of 8.2 cycles, against 16 x 512 x 6.3 / 32 = 1610 term by term.  Measured
 // against the term-by-term kernel: 512 paths x 2000 steps x 512 bins 112 -> 45 us, 2048 x 1237 x 256 208 -> 72 us,
 // 20300 x 500 x 1024 2.40 -> 0.73 ms; error against FP64 1.7e-6 -> 0.7e-6 of the 2-norm.
 //
