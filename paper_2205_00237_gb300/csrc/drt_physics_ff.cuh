@@ -180,7 +180,7 @@ DRT_NOINL void path_step_ff_fallback(const LinkDev &L, const TimeGridD &tg, cons
 
 // Instruction fetch bounds this form as much as issue: a step is ~6000 instructions, and inlined at every vertex they gave 7 to 11
 // no-instruction stalls per issue (28 % of the issue slots used).  With the arithmetic's helpers out of line (one copy each) and
-// neighbouring blocks on neighbouring paths it is 2 to 3 (48 %).  Measured and left out: a barrier per stage, in blocks of 128 or one
+// neighbouring blocks on neighbouring paths it is 2 to 3 (41 to 59 % from one to three vertices).  Measured and left out: a barrier per stage, in blocks of 128 or one
 // of 384 threads per SM (1.0 stalls, but the same or a longer time); an order that gives each SM its own stretch of paths (25 to
 // 50 % slower: the SMs share instruction-cache lines).
 template <int N>
@@ -250,7 +250,7 @@ DRT_HD void path_step_ff(const LinkDev &L, const TimeGridD &tg, const FreqGridD 
 // ------------------------------------------------------------------------------------------------
 // The FP64 parts of the FP32-bulk form in two-float numbers: warm starts, anchors at the chunk bases, and the redo of the steps FP32
 // cannot resolve.  They are short dependent chains (a few solves per path), so what they cost is latency: 65 cycles per FP64
-// instruction, a few per FP32 one.  Canyon: anchors 33 + 23 -> 13 + 21 us, warm starts 77 -> 57, redo 135 -> 94.
+// instruction, a few per FP32 one.  Canyon: anchors 33 + 23 -> 15 + 22 us, warm starts 77 -> 31, redo 135 -> 59.
 
 // The three-stage solve of solve_edge_params (drt_physics.cuh): FP32 values, two-float values, one dual-number step for the rates.  False
 // where it did not converge (the caller runs the FP64 solve).  The rates only place Newton starts between the chunk bases and predict
