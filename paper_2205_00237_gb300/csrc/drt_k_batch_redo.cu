@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(32) k_batch_redo(const BatchDev B) {   // one 
     // branches run in turn but which keep the lanes filled (126 000 steps of a 128-link batch: 0.8 ms against 1.4 ms by runs).
     const int count = *B.redo.count, n = count < B.redo.cap ? count : B.redo.cap, lane = threadIdx.x, y = blockIdx.y;
     const bool packed = n > 64 * (int)gridDim.x;
-    for (int k = packed ? 32 * blockIdx.x : blockIdx.x; k < n; k += packed ? 32 * gridDim.x : gridDim.x) {
+    const int stride = packed ? 32 * (int)gridDim.x : redo_stride(gridDim.x), first = (packed ? 32 : 1) * (int)blockIdx.x;
+    for (int k = first < stride ? first : n; k < n; k += stride) {
         int4 itm = make_int4(-1, 0, 0, 0);
         bool on = k + lane < n;
         if (!packed) {
