@@ -1279,7 +1279,7 @@ drt_status trace_into(drt_ctx *c, Link &L, double t, int max_order, int with_til
     if (drt_status st = ensure(c, c->tr_rays, (size_t)cap_dev * trace_ray_bytes())) return st;
     if (drt_status st = ensure(c, c->tr_count, 256)) return st;
     const double far = ff_reach(L.view, std::fabs(t));
-    const bool two = L.view.ff_range && far < 1e5;
+    const bool two = L.view.ff_range && far < 1e5 && trace_two_float(L.dev, max_order, with_tiles);
     // without room for their scratch the FP64 pass alone
     void *prims = two && ensure(c, c->tr_prims, trace_prim_bytes(L.dev, cap_dev)) == DRT_OK ? c->tr_prims.ptr : nullptr;
     int *cnt = reinterpret_cast<int *>(c->tr_count.ptr);

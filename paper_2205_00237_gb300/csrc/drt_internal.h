@@ -296,6 +296,7 @@ cudaError_t launch_probe(int kind, int blocks, double *sink, cudaStream_t s, flo
 // scratch records (faces posed at the instant, rays found), the launch, and the host-side unpacking of
 // `count` rays into path-set arrays in enumeration order
 long long trace_candidates(const LinkDev &L, int max_order, int with_tiles);
+bool trace_two_float(const LinkDev &L, int max_order, int with_tiles);   // whether the two-float passes are the faster ones
 size_t trace_ray_bytes();
 size_t trace_face_bytes();
 size_t trace_prim_bytes(const LinkDev &L, int cap);   // scratch of the two-float passes

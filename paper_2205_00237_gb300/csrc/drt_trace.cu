@@ -437,6 +437,16 @@ long long trace_candidates(const LinkDev &L, int max_order, int with_tiles) {
     return 1 + (max_order >= 1 ? NP + NT : 0) + (max_order >= 2 ? NP * NP : 0);
 }
 
+// The three passes cost 25 us more in launches, and at order 2 the solves of what stays open come on top of the two-float ones
+// (560 + us against 435 for a handful of candidates); what they save is the FP64 pass's loop over the faces on one thread (per
+// face 0.9 us at order 0, 2.5 at 1, 3 at 2) and, where the candidates are more than the FP64 pipes take at once, its solves.
+// Measured on parts of the canyon and link scenes, FP64 | two-float us: order 0, 18 faces 90 | 102, 53 faces 118 | 101; order 1, 10
+// faces 116 | 124, 17 faces 134 | 107; order 2, 31 faces and 84 edges 530 | 725, 53 and 129 (33125 candidates) 826 | 717.
+bool trace_two_float(const LinkDev &L, int max_order, int with_tiles) {
+    const int least = max_order == 0 ? 31 : max_order == 1 ? 11 : 41;
+    return L.n_faces >= least || trace_candidates(L, max_order, with_tiles) > 16384;
+}
+
 size_t trace_ray_bytes() { return sizeof(TracedRay); }
 size_t trace_face_bytes() { return sizeof(PosedFace); }
 size_t trace_prim_bytes(const LinkDev &L, int cap) {   // posed faces and primitives, then the points of `cap` listed candidates
