@@ -118,6 +118,8 @@ struct drt_ctx {
     // of its copy): a fresh pageable image per load costs its page faults and a staged copy
     char *stage = nullptr;
     size_t stage_cap = 0;
+    // the image of a small link (STAGE_SMALL) in pageable memory: the driver takes so small a copy into its command buffer at once
+    std::vector<char> stage_small;
 };
 
 namespace {
@@ -237,27 +239,40 @@ struct LinkImage {
         size = off + v.size() * sizeof(X);
         parts.push_back(Part{v.data(), v.size() * sizeof(X), off, dst});
     }
-    // through the staging image from offset `at` on (stage_reserve), queued on the default stream; the staging image may be filled again
+    // through the staging image from `stage` on (stage_reserve), queued on the default stream; the staging image may be filled again
     // once the stream has been waited for
-    drt_status upload(drt_ctx *c, int kind, Link::Block &b, size_t at) {
+    drt_status upload(drt_ctx *c, int kind, Link::Block &b, char *stage) {
         if (drt_status st = link_block_alloc(c, kind, size, &b.ptr, &b.bytes)) return st;
         for (const Part &q : parts) {
-            if (q.bytes) std::memcpy(c->stage + at + q.off, q.src, q.bytes);
+            if (q.bytes) std::memcpy(stage + q.off, q.src, q.bytes);
             const char *to = reinterpret_cast<const char *>(b.ptr) + q.off;
             std::memcpy(q.dst, &to, sizeof to);
         }
-        if (size) CUDA_TRY(cudaMemcpyAsync(b.ptr, c->stage + at, size, cudaMemcpyHostToDevice, 0));
+        if (size) CUDA_TRY(cudaMemcpyAsync(b.ptr, stage, size, cudaMemcpyHostToDevice, 0));
         return DRT_OK;
     }
 };
-drt_status stage_reserve(drt_ctx *c, size_t size) {
-    if (c->stage_cap >= size) return DRT_OK;
+// room for an image of `size` bytes.  Small ones in pageable memory: load and unload of the tiny link (two copies of some KB) 33 us,
+// from pinned memory, where a copy is a transfer of its own, 36 us (29 us with the one copy that there was before the two-float
+// arrays)
+constexpr size_t STAGE_SMALL = 32 << 10;
+drt_status stage_reserve(drt_ctx *c, size_t size, char **stage) {
+    if (size <= STAGE_SMALL) {
+        c->stage_small.resize(STAGE_SMALL);
+        *stage = c->stage_small.data();
+        return DRT_OK;
+    }
+    if (c->stage_cap >= size) {
+        *stage = c->stage;
+        return DRT_OK;
+    }
     if (c->stage) cudaFreeHost(c->stage);
     c->stage = nullptr;
     c->stage_cap = 0;
     const size_t want = std::max(size + size / 2, (size_t)1 << 20);
     CUDA_TRY(cudaMallocHost(reinterpret_cast<void **>(&c->stage), want));
     c->stage_cap = want;
+    *stage = c->stage;
     return DRT_OK;
 }
 
@@ -977,11 +992,12 @@ drt_status load_link(drt_ctx *c, const drt_scene *s, const drt_path_set *ps, Lin
     copies.add(H.tilesQ, &d.tilesQ);
     copies.add(H.bodiesQ, &d.bodiesQ);
     const size_t at = (img.size + 255) & ~(size_t)255;
-    drt_status st = stage_reserve(c, at + copies.size);
-    if (!st) st = img.upload(c, 0, L.block, 0);
+    char *stage = nullptr;
+    drt_status st = stage_reserve(c, at + copies.size, &stage);
+    if (!st) st = img.upload(c, 0, L.block, stage);
     L.view.ff_range = L.view.ff_range && copies_too;
     if (!st && L.view.ff_range) {
-        st = copies.upload(c, 1, L.two, at);
+        st = copies.upload(c, 1, L.two, stage + at);
         if (st == DRT_ENOMEM) {   // no room for them: FP64 everywhere
             L.view.ff_range = false;
             st = DRT_OK;
