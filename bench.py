@@ -61,7 +61,7 @@ PATHSET = os.path.join(ROOT, "tests", "golden", "pathset_canyon_seed0.npz")
 # evaluates the exponentials of 16 paths for a tile of 512 bins in 455 warp instructions (ncu), 1.78
 # thread-instructions a term of H, so its roofline is 40.3e12 / 1.78 = 22.7e12 terms/s; the products and
 # sums themselves (8 FLOP per term) run on the tensor cores.
-KERNEL_HASH = "380309f997d3c175"
+KERNEL_HASH = "49de0ed32915576e"
 FF_WARP_INST_PER_CALL = 2.22347e8
 FF_FLOP_PER_PATH_STEP = 6764.8
 FF_DRAM_BYTES_PER_CALL = 1.179e7
